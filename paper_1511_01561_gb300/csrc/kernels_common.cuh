@@ -382,9 +382,9 @@ __host__ __device__ constexpr int line_group() {
 //     metric terms dxi_d/dx_c vanish for c != d and J is constant over the
 //     element, so -Jw div F at node (i,j,k) is w_i w_j w_k sum_d K_d (D F_d)
 //     along xi_d, with K_d = -J dxi_d/dx_d per element.  Folding K_d into the
-//     direction's copy of D (formed per element in shared memory) leaves the
-//     12 unweighted flux fields of (1) and 15 contractions, with no metric or
-//     Jw load per node.  The weight w_i w_j w_k is the same at every element
+//     direction's copy of D leaves the 12 unweighted flux fields of (1) and 15
+//     contractions, with no metric or Jw load per node; in FP64 these run in
+//     fixed point on the integer pipe (fixed64.cuh).  The weight w_i w_j w_k is the same at every element
 //     node of a global node (the Lobatto weights are symmetric and the box's
 //     elements meet face to face), so it moves out of the element kernel
 //     into the inverse mass of the DSS: the kernel writes
@@ -470,61 +470,6 @@ __device__ __forceinline__ void volume_element_nodal64(const VolumeArgs& a, long
   re[2 * Nl + n] = dym;
   re[3 * Nl + n] = dzm;
   re[4 * Nl + n] = dt;
-}
-
-// create_rhs of a rectilinear affine element in FP64 (see (2) above), one
-// thread per element node: 75 FP64 operations per node at N = 4 (the flux
-// components come from the update, formed once per global node).  It
-// writes the residual without its weight w_i w_j w_k, which the update
-// applies with the inverse mass.  a.affk holds K_d per element [3][Ne].
-// Shared memory: 12 (N+1)^3 + 3 (N+1)^2 doubles.
-template <int N>
-__device__ __forceinline__ void volume_element_rect(const VolumeArgs& a, long long e, unsigned char* smem_raw) {
-  constexpr int P = N + 1, PP = P * P, NP = PP * P;
-  double* F = reinterpret_cast<double*>(smem_raw);  // [kLF][NP]
-  double* Dk = F + kLF * NP;                         // [3][P][P]: K_d D
-  const int l = threadIdx.x;
-  for (int t = l; t < 3 * PP; t += blockDim.x) {
-    const int d = t / PP;
-    Dk[t] = a.affk[d * (long long)a.Ne + e] * a.D64[t - d * PP];
-  }
-  const long long Nl = a.Nl, n = (long long)e * NP + l;
-  if (l < NP) {
-    const FluxState64 z = gather_fluxes64(a, n);
-#pragma unroll
-    for (int f = 0; f < kLF; ++f) F[f * NP + l] = z.f[f];
-  }
-  __syncthreads();
-  if (l >= NP) return;
-  const int i = l % P, j = (l / P) % P, k = l / PP;
-  double dx[P], dy[P], dz[P];
-#pragma unroll
-  for (int m = 0; m < P; ++m) {
-    dx[m] = Dk[i * P + m];
-    dy[m] = Dk[PP + j * P + m];
-    dz[m] = Dk[2 * PP + k * P + m];
-  }
-  const int bx = P * (j + P * k), by = i + PP * k, bz = i + P * j;
-  // K_x D F_x along xi + K_y D F_y along eta + K_z D F_z along zeta
-  auto div = [&](int fx, int fy, int fz) {
-    const double* gx = F + fx * NP;
-    const double* gy = F + fy * NP;
-    const double* gz = F + fz * NP;
-    double t = dx[0] * gx[bx];
-#pragma unroll
-    for (int m = 1; m < P; ++m) t = fma(dx[m], gx[bx + m], t);
-#pragma unroll
-    for (int m = 0; m < P; ++m) t = fma(dy[m], gy[by + P * m], t);
-#pragma unroll
-    for (int m = 0; m < P; ++m) t = fma(dz[m], gz[bz + PP * m], t);
-    return t;
-  };
-  double* re = static_cast<double*>(a.re);
-  re[n] = div(lUx, lUy, lUz);
-  re[Nl + n] = div(lTxx, lTxy, lTxz);
-  re[2 * Nl + n] = div(lTxy, lTyy, lTyz);
-  re[3 * Nl + n] = div(lTxz, lTyz, lTzz);
-  re[4 * Nl + n] = div(lHx, lHy, lHz);
 }
 
 // create_rhs of element e in the FP32 form, organised by 1D lines of nodes
@@ -888,7 +833,7 @@ __device__ __forceinline__ void volume_element_pairs_affine(const VolumeArgs& a,
 }
 
 // create_rhs of a rectilinear affine element in the pairs mode: the folded
-// form of volume_element_rect (K_d D per direction, the weight w_i w_j w_k
+// form of volume_fx_rect (K_d D per direction, the weight w_i w_j w_k
 // left to the update's inverse mass, no metric or Jw per node) in (hi, lo)
 // float pairs.  The 12 unweighted fields are differentiated less their values at
 // element node 0 (K_d D annihilates constants as D does), and p' enters less
@@ -971,7 +916,6 @@ template <int N, typename T, bool AFF>
 constexpr size_t element_smem_bytes() {
   constexpr int P = N + 1, NP = P * P * P;
   if constexpr (std::is_same<T, float>::value) return sizeof(float) * (kNF > 15 ? kNF : 15) * NP;
-  if constexpr (AFF && std::is_same<T, double>::value) return sizeof(T) * (kLF * NP + 3 * P * P);
   if constexpr (std::is_same<T, double>::value) return sizeof(T) * (kLF * NP + P * P);
   if constexpr (AFF) return sizeof(T) * (15 * NP + P * P + 15);
   return sizeof(T) * (kLF * NP + P * P + kLF);
@@ -990,11 +934,8 @@ __device__ __forceinline__ void element_rhs(const VolumeArgs& a, long long e, un
     }
   } else if constexpr (std::is_same<T, float>::value) {
     volume_element_lines<N, AFF>(a, e, smem_raw);
-  } else if constexpr (AFF) {
-    // FP64 launches the affine instantiation for rectilinear elements only
-    // (volume_form); other affine meshes take the per-node form
-    volume_element_rect<N>(a, e, smem_raw);
   } else {
+    static_assert(!AFF, "rectilinear elements in FP64 take volume_fx_rect; other affine meshes the per-node form");
     volume_element_nodal64<N>(a, e, smem_raw);
   }
 }
@@ -1439,25 +1380,29 @@ int sm_count() {
 }
 
 // Persistent launch: as many CTAs as fit on the GPU at once.
-template <int N, typename T, bool AFF>
-cudaError_t launch_volume_ragged_t(const MemberDesc* d, const RaggedGroup* g, cudaStream_t s) {
-  constexpr int P = N + 1, NP = P * P * P;
-  constexpr int NT = (NP + 31) / 32 * 32;
-  const size_t smem = element_smem_bytes<N, T, AFF>();
-  static DeviceInts grids;  // per device, set up at its first launch there
+template <typename K>
+cudaError_t launch_persistent(K kernel, int threads, size_t smem, DeviceInts& grids, const MemberDesc* d,
+                              const RaggedGroup* g, cudaStream_t s) {
   int grid = grids.get();
   if (!grid) {
-    cudaError_t e =
-        cudaFuncSetAttribute(volume_ragged<N, T, AFF>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     int per_sm = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, volume_ragged<N, T, AFF>, NT, smem);
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, threads, smem);
     if (e != cudaSuccess) return e;
     grid = (per_sm > 0 ? per_sm : 1) * sm_count();
     grids.put(grid);
   }
-  volume_ragged<N, T, AFF><<<grid, NT, smem, s>>>(d, g);
+  kernel<<<grid, threads, smem, s>>>(d, g);
   return cudaGetLastError();
+}
+
+template <int N, typename T, bool AFF>
+cudaError_t launch_volume_ragged_t(const MemberDesc* d, const RaggedGroup* g, cudaStream_t s) {
+  constexpr int P = N + 1, NP = P * P * P;
+  static DeviceInts grids;  // per device, set up at its first launch there
+  return launch_persistent(volume_ragged<N, T, AFF>, (NP + 31) / 32 * 32, element_smem_bytes<N, T, AFF>(), grids, d,
+                           g, s);
 }
 
 template <typename T, bool AFF>

@@ -4,6 +4,7 @@
 // reference state and initial conditions.
 #include <algorithm>
 #include <cmath>
+#include <cstdlib>
 #include <cstring>
 #include <numeric>
 
@@ -275,6 +276,79 @@ void filter_matrix_host(int N, const double* xi, const double* w, int s, double 
       }
       F[i * P + m] = acc;
     }
+}
+
+// Lobatto points and D of order N in 113-bit arithmetic (the same IEEE format
+// on both host architectures), so that the fixed-point tables carry no
+// rounding of D.
+#if __LDBL_MANT_DIG__ == 113
+typedef long double Quad;
+#else
+typedef __float128 Quad;
+#endif
+
+static void lobatto_quad(int N, std::vector<Quad>& x) {
+  std::vector<double> xd, wd;
+  lobatto(N, xd, wd);
+  x.assign(xd.begin(), xd.end());
+  for (int i = 1; i < N; ++i)
+    for (int it = 0; it < 4; ++it) {  // Newton on x P_N - P_{N-1} from the double roots
+      Quad a = 1, b = x[i];
+      for (int k = 2; k <= N; ++k) {
+        const Quad c = ((2 * k - 1) * x[i] * b - (k - 1) * a) / k;
+        a = b;
+        b = c;
+      }
+      x[i] -= (x[i] * b - a) / ((N + 1) * b);
+    }
+}
+
+// The order of fx_line (fixed64.cuh): with H = P/2 and O = P%2, rows i < H of
+// (D_ij + D_i,N-j)/2 (j < H) and D_i,mid, rows i < H of (D_ij - D_i,N-j)/2,
+// and for odd P the middle row D_mid,j (j < H).  D 1 = 0 holds exactly in the
+// integers: a row's even part takes the rounding in its last entry (the
+// middle one), or for even P in its largest.
+int fx_table_host(int P, double a, double b, double c, int s, int2* out) {
+  const int N = P - 1, H = P / 2, O = P % 2;
+  std::vector<Quad> x, lam(P, Quad(1)), D(P * P, Quad(0));
+  lobatto_quad(N, x);
+  for (int j = 0; j < P; ++j)
+    for (int k = 0; k < P; ++k)
+      if (k != j) lam[j] *= x[j] - x[k];
+  Quad scale = (Quad)a * (Quad)b / (Quad)c;
+  for (int t = 0; t < s; ++t) scale *= 2;
+  for (int t = 0; t > s; --t) scale /= 2;
+  for (int i = 0; i < P; ++i) {
+    for (int j = 0; j < P; ++j)
+      if (j != i) {
+        D[i * P + j] = (lam[i] / lam[j]) / (x[i] - x[j]) * scale;
+        D[i * P + i] -= D[i * P + j];
+      }
+  }
+  auto whole = [](Quad v) { return (long long)(v < 0 ? v - Quad(0.5) : v + Quad(0.5)); };
+  int n = 0;
+  auto put = [&](long long v) {
+    const long long h = (v + (1LL << 28)) >> 29;
+    out[n++] = make_int2((int)(v - (h << 29)), (int)h);
+  };
+  std::vector<long long> ev(H + 1);
+  for (int i = 0; i < H; ++i) {
+    long long sum = 0;
+    int big = 0;
+    for (int j = 0; j < H; ++j) {
+      ev[j] = whole((D[i * P + j] + D[i * P + N - j]) / 2);
+      sum += ev[j];
+      if (std::llabs(ev[j]) > std::llabs(ev[big])) big = j;
+    }
+    if (O) ev[H] = -2 * sum;
+    else ev[big] -= sum;
+    for (int j = 0; j < H + O; ++j) put(ev[j]);
+  }
+  for (int i = 0; i < H; ++i)
+    for (int j = 0; j < H; ++j) put(whole((D[i * P + j] - D[i * P + N - j]) / 2));
+  if (O)
+    for (int j = 0; j < H; ++j) put(whole(D[H * P + j]));
+  return n;
 }
 
 bool build_host_mesh(const numa_config& c, HostMesh& m, std::string& err) {

@@ -2,6 +2,7 @@
 // life cycle, workspace binding, state I/O and the stage loop of code
 // example 1 in Sec. 7 (create_rhs, DSS with the inverse mass matrix, update
 // q), with one CUDA graph per RK step for numa_run.
+#include <algorithm>
 #include <cmath>
 #include <cstring>
 #include <new>
@@ -66,6 +67,9 @@ VolumeArgs volume_args(const numa_ctx* c, const double* q, const void* prim, voi
   a.D2 = c->L.D2;
   a.re = re;
   a.affk = c->L.affk;
+  a.fxD = c->fx ? c->L.fxD : nullptr;
+  a.fxD_host = c->fx ? c->fxD.data() : nullptr;
+  a.fxexp = c->fxexp;
   a.Ng = c->mesh.Ng;
   a.Nl = c->mesh.Nl;
   a.Ne = (int)c->mesh.Ne;
@@ -477,6 +481,7 @@ size_t layout_workspace(const numa_config& c, const HostMesh& m, char* base, Dev
   if ((c.precision == NUMA_FP64 || c.precision == NUMA_FP64_PAIRS) && affine_elements(c)) {
     d.affk = (double*)take(3 * (size_t)m.Ne * 8);
     d.Minv_r = (double*)take(Ng * 8);
+    d.fxD = (int2*)take(3 * kFxEntries * sizeof(int2));
   }
   d.D32 = (float*)take(PP * 4);
   d.D2 = (float2*)take(PP * 8);
@@ -624,7 +629,9 @@ int numa_bind(numa_ctx* c, void* ws, size_t bytes, void* stream) {
   // FP64 and pairs: the per-element constants of rectilinear elements; FP64:
   // the weighted metric of the per-node form, which it takes everywhere else
   std::vector<double> affk, w3, Minv_r;
-  bool rect = false;
+  std::vector<int2> fxD;
+  bool rect = false, fx = false;
+  int fxexp = 0;
   if (c->cfg.precision == NUMA_FP64 || c->cfg.precision == NUMA_FP64_PAIRS) {
     if (affine_elements(c->cfg)) {
       const int P = m.P;
@@ -640,6 +647,40 @@ int numa_bind(numa_ctx* c, void* ws, size_t bytes, void* stream) {
       for (int k = 0; k < P; ++k)
         for (int j = 0; j < P; ++j)
           for (int i = 0; i < P; ++i) w3[i + P * (j + P * k)] = m.w[i] * m.w[j] * m.w[k];
+      if (rect && c->cfg.precision == NUMA_FP64) {
+        // K_d = -J dxi_d/dx_d = -(area of the element's face normal to d) / 4,
+        // the same for all elements of a box (a mesh whose metric terms say
+        // otherwise is not treated as rectilinear).  One scale 2^s for the
+        // three directions: the largest row sum of |K_d D| below 2^60.
+        const double Lx[3] = {c->cfg.Lx, c->cfg.Ly, c->cfg.Lz};
+        const double ne[3] = {(double)c->cfg.nex, (double)c->cfg.ney, (double)c->cfg.nez};
+        double num[3][2], den[3], top = 0.0;
+        for (int d = 0; d < 3; ++d) {
+          const int p = (d + 1) % 3, r = (d + 2) % 3;
+          num[d][0] = -Lx[p];
+          num[d][1] = Lx[r];
+          den[d] = 4.0 * ne[p] * ne[r];
+          const double K = num[d][0] * num[d][1] / den[d];
+          for (long long el = 0; el < m.Ne; ++el)
+            if (!(std::fabs(affk[d * (size_t)m.Ne + el] - K) <= 1e-9 * std::fabs(K))) rect = false;
+          for (int i = 0; i < P; ++i) {
+            double row = 0.0;
+            for (int j = 0; j < P; ++j) row += std::fabs(K * m.D[i * P + j]);
+            top = std::max(top, row);
+          }
+        }
+        int e2 = 0;
+        std::frexp(top, &e2);  // top < 2^e2
+        const int s2 = 60 - e2;
+        fx = rect && top > 0.0 && std::isfinite(top) && s2 >= -250 && s2 <= 250;
+        if (fx) {
+          fxD.resize(3 * kFxEntries);
+          int n = 0;
+          for (int d = 0; d < 3; ++d) n += fx_table_host(P, num[d][0], num[d][1], den[d], s2, fxD.data() + n);
+          fxexp = 64 - s2;
+          up(L.fxD, fxD.data(), (size_t)n * sizeof(int2));
+        }
+      }
       // Minv_r: w_i w_j w_k of the node's first element node (its DSS list
       // is ascending), times 1/M.  Lobatto weights are symmetric, so every
       // element node of a global node of a box has that weight; a mesh
@@ -647,13 +688,16 @@ int numa_bind(numa_ctx* c, void* ws, size_t bytes, void* stream) {
       if (rect) {
         const long long Np = m.Np;
         Minv_r.resize((size_t)Ng);
+        const double rJ = 8.0 * ((double)c->cfg.nex * c->cfg.ney * c->cfg.nez) / (c->cfg.Lx * c->cfg.Ly * c->cfg.Lz);
         for (size_t I = 0; I < Ng && rect; ++I) {
           const double wf = w3[m.csr_idx[m.csr_off[I]] % Np];
           for (int32_t t = m.csr_off[I] + 1; t < m.csr_off[I + 1]; ++t)
             if (std::fabs(w3[m.csr_idx[t] % Np] - wf) > 1e-14 * wf) rect = false;
-          Minv_r[I] = wf * m.Minv[I];
+          // fixed-point form: w_I / M_I = 1 / (J x element nodes at I), J in closed form like the K_d
+          Minv_r[I] = fx ? rJ / (double)(m.csr_off[I + 1] - m.csr_off[I]) : wf * m.Minv[I];
         }
       }
+      fx = fx && rect;
       up(L.affk, affk.data(), affk.size() * 8);
       if (rect) up(L.Minv_r, Minv_r.data(), Minv_r.size() * 8);
     }
@@ -679,6 +723,9 @@ int numa_bind(numa_ctx* c, void* ws, size_t bytes, void* stream) {
   if (e != cudaSuccess) return cuda_fail(c, e, "numa_bind upload");
   c->L = L;
   c->rect = rect;
+  c->fx = fx;
+  c->fxD = fxD;
+  c->fxexp = fxexp;
   c->slabs = plan_slabs(c->cfg, m, c->nslab_req);
   if (c->slabs.S > 1) {
     e = ensure_slab_streams(c);

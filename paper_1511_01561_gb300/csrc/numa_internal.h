@@ -81,6 +81,7 @@ struct DevLayout {
   double* nrm = nullptr;     // [3][Ng] (shell)
   double* D64 = nullptr;     // [P*P]
   double* affk = nullptr;    // FP64 / pairs affine elements: [3][Ne] K_d = -J dxi_d/dx_d per element
+  int2* fxD = nullptr;       // FP64 rectilinear form: K_d D as fixed-point even/odd tables [3][kFxEntries]
   float* D32 = nullptr;      // [P*P]
   double* F64 = nullptr;     // [P*P] 1D filter matrix (FP64, pairs)
   float* F32 = nullptr;      // [P*P] the same in FP32 (FP32 form)
@@ -89,6 +90,16 @@ struct DevLayout {
   int* flags = nullptr;      // [64]: 0 = non-finite
   size_t bytes = 0;
 };
+
+// Entries of one direction's fixed-point table at the largest order.
+constexpr int kFxEntries = 40;
+// (a b / c) D (one direction's derivative matrix times its metric factor) as
+// the even/odd fixed-point table of fx_line (fixed64.cuh): entries
+// 2^s (a b / c) D as (low 29 bits, rest), D evaluated beyond FP64 and rounded
+// once.  Returns the number of entries.
+int fx_table_host(int P, double a, double b, double c, int s, int2* out);
+// Elements per position of a ragged volume launch (RaggedGroup::elem_prefix).
+int volume_chunk(int N, int precision, int form);
 
 size_t layout_workspace(const numa_config& c, const HostMesh& m, char* base, DevLayout* L);
 size_t residual_bytes(const numa_config& c, const HostMesh& m);  // bytes of the re scratch
@@ -124,6 +135,10 @@ struct VolumeArgs {
   const float2* D2;    // pairs mode
   void* re;            // [5][Nl] output
   const double* affk;   // rectilinear form (FP64, pairs): [3][Ne] -J dxi_d/dx_d
+  const int2* fxD;      // FP64 rectilinear form: fixed-point tables of K_d D, one after the other (nullptr:
+                        // K_d outside the fixed-point range, the elements take plain FP64)
+  const int2* fxD_host; // the same tables in host memory (kernel parameters of the single-mesh launch)
+  int fxexp;            // the exponent that goes with fxD
   long long Ng, Nl;
   int Ne;
   int ebeg, ecnt;      // the launch covers elements [ebeg, ebeg + ecnt) (a slab, or all: 0, Ne)
@@ -260,7 +275,7 @@ struct MemberDesc {
 struct RaggedGroup {
   int n;
   int pad;
-  long long elem_prefix[kMaxMembers + 1];
+  long long elem_prefix[kMaxMembers + 1];   // chunks of volume_chunk elements (each member's padded to whole chunks)
   long long block_prefix[kMaxMembers + 1];  // blocks of kDssBlock global nodes (each member's padded to whole blocks)
   int member[kMaxMembers];
 };
@@ -296,6 +311,9 @@ struct numa_ctx {
   bool bound = false;
   bool prim_valid = false;  // L.prim holds the primitive fields of L.q
   bool rect = false;        // FP64, affine and every element rectilinear: the folded element kernel
+  bool fx = false;          // FP64: L.fxD and fxD hold the mesh's fixed-point tables, with exponent fxexp
+  std::vector<int2> fxD;
+  int fxexp = 0;
   int nslab_req = 0;        // slabs asked for by numa_set_slabs (0: automatic)
   numa::SlabPlan slabs;     // the plan in use (made at bind and by numa_set_slabs)
   cudaStream_t side = nullptr;  // the second stream of the slab pipeline

@@ -248,7 +248,8 @@ void rebuild_tables(numa_sched* s) {
     RaggedGroup& G = s->h_groups[g];
     const int m = G.n++;
     G.member[m] = r.slot;
-    G.elem_prefix[m + 1] = G.elem_prefix[m] + r.ctx->mesh.Ne;
+    const int chunk = volume_chunk(r.cfg.N, r.cfg.precision, volume_form(r.ctx));
+    G.elem_prefix[m + 1] = G.elem_prefix[m] + (r.ctx->mesh.Ne + chunk - 1) / chunk;
     G.block_prefix[m + 1] = G.block_prefix[m] + (r.ctx->mesh.Ng + kDssBlock - 1) / kDssBlock;
   }
   s->tables_dirty = true;

@@ -1,0 +1,91 @@
+"""The FP64 element kernels' fixed-point contractions against the oracle, at
+the sizes and magnitudes where they could go wrong: every order with element
+counts that leave the last CTA partly filled, equation groups of very
+different magnitude, values beyond the fixed-point range (plain FP64 then),
+and non-finite elements beside finite ones.
+
+Bar: 1e-12 of the largest tendency of each variable, the FP64 bar of one
+right-hand side (the integers hold 58 bits of each group's largest value, so
+the contraction adds less than FP64's own rounding)."""
+import numpy as np
+import pytest
+
+from paper_1511_01561_gb300 import inputs as I
+
+from .helpers import scaled_random_state
+
+pytestmark = pytest.mark.gpu
+
+TOL = 1e-12
+
+
+@pytest.fixture(scope="module")
+def numa():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1511_01561_gb300 import build
+    build.build()
+    from paper_1511_01561_gb300 import numa as mod
+    return mod
+
+
+def _rhs(numa, cfg, q):
+    s = numa.Solver(cfg, "fp64")
+    try:
+        return s.rhs(q).cpu().numpy()
+    finally:
+        s.close()
+
+
+def _check(Rg, Ro):
+    scale = np.abs(Ro).max(axis=1)
+    scale[1:4] = scale[1:4].max()
+    err = np.abs(Rg - Ro).max(axis=1) / np.where(scale > 0.0, scale, 1.0)
+    assert err.max() <= TOL, err
+
+
+# element counts that are no multiple of any number of elements per CTA, one
+# element, thin slabs of unlike widths
+@pytest.mark.parametrize("N", range(1, 9))
+@pytest.mark.parametrize("ne,per", [((3, 1, 1), (0, 0, 0)), ((1, 1, 1), (0, 1, 0)), ((2, 3, 3), (1, 0, 0))])
+def test_rect_orders_and_remainders(numa, orc, N, ne, per):
+    cfg = I.box(ne, N, L=(3000.0, 700.0, 900.0), periodic=per)
+    m = orc.Mesh(cfg)
+    q = scaled_random_state(m.Ng, m.ref()[0], m.ref()[1], seed=N)
+    _check(_rhs(numa, cfg, q), m.rhs(q))
+
+
+@pytest.mark.parametrize("N", [2, 4, 7])
+@pytest.mark.parametrize("scale", [1e-30, 1e-200, 1e-310])
+def test_rect_small_momentum(numa, orc, N, scale):
+    """The mass equation is linear in U: a momentum far below the other groups
+    (1e-30), below the fixed-point range (1e-200) and subnormal (1e-310)."""
+    cfg = I.box((3, 2, 2), N)
+    m = orc.Mesh(cfg)
+    q = np.zeros((5, m.Ng))
+    q[1:4] = np.random.default_rng(N).uniform(-1.0, 1.0, (3, m.Ng)) * scale
+    Rg, Ro = _rhs(numa, cfg, q)[0], m.rhs(q)[0]
+    tiny = 64 * 5e-324 if scale < 1e-300 else 0.0  # subnormal sums are rounded to whole units of 5e-324
+    assert np.abs(Rg - Ro).max() <= TOL * np.abs(Ro).max() + tiny
+
+
+@pytest.mark.parametrize("bad", [np.nan, np.inf, -np.inf])
+def test_rect_nonfinite_elements(numa, orc, bad):
+    """One node's x momentum is not finite: the mass tendency is not finite on
+    its x line inside its element and nowhere else (K_d D has no other term
+    with U_x), and the nodes of the other elements are untouched."""
+    cfg = I.box((4, 3, 3), 4)
+    m = orc.Mesh(cfg)
+    q = scaled_random_state(m.Ng, m.ref()[0], m.ref()[1], seed=11)
+    R0 = _rhs(numa, cfg, q)
+    g = 5 + 17 * (6 + 13 * 6)
+    q[1, g] = bad
+    Rg = _rhs(numa, cfg, q)
+    line = np.zeros(m.Ng, dtype=bool)
+    line[g - 1:g + 4] = True  # ix = 4 .. 8
+    assert np.array_equal(~np.isfinite(Rg[0]), line)
+    e = m.l2g().reshape(-1, 125)
+    near = np.unique(e[(e == g).any(axis=1)])
+    far = np.setdiff1d(np.arange(m.Ng), near)
+    assert np.array_equal(Rg[:, far], R0[:, far])
