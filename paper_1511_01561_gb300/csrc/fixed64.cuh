@@ -23,7 +23,19 @@ namespace {
 
 constexpr int kFxBits = 29;                       // bits of a low part
 constexpr unsigned kFxMask = (1u << kFxBits) - 1;
-constexpr unsigned kFxMinExp = 400, kFxMaxExp = 1600;  // biased exponents of a group's largest value
+constexpr long long kFxHalf = 1ll << (kFxBits - 1);  // half a unit of the high part: where a middle accumulator starts
+// biased exponents of a group's largest value, and of a metric row's
+constexpr unsigned kFxMinExp = 400, kFxMaxExp = 1600;
+constexpr int kFxMetMin = 1023 - 200, kFxMetMax = 1023 + 200;
+
+// Entry i of a table of small integers, 4 bits per point of a line.
+__device__ __forceinline__ int fx_nibble(unsigned long long t, int i) { return (int)((t >> (4 * i)) & 15ull); }
+
+// The power of two taken out of node (i, j, k)'s quadrature weight: the sum of
+// its three points' exponents (negated in fxw).
+__device__ __forceinline__ int fx_weight_exp(unsigned long long fxw, int i, int j, int k) {
+  return -(fx_nibble(fxw, i) + fx_nibble(fxw, j) + fx_nibble(fxw, k));
+}
 
 // x as a 58-bit integer in units of 2^(E - 1022 - 58), E the biased exponent
 // of the group's largest magnitude: (low 29 bits, signed rest).  Exact for
@@ -71,7 +83,10 @@ __device__ __forceinline__ bool fx_in_range(uint4 k) {
 }
 
 // (high, middle) accumulators += D * f, D = Dh 2^29 + Dl, f = fh 2^29 + fl;
-// the product of the low parts (2^-58 of the full scale) is left out.
+// the product of the low parts (2^-58 of the full scale) is left out.  The
+// middle accumulator starts at half a unit of the high one, so that
+// h + (m >> 29) is rounded, not cut: a cut would leave every derivative half a
+// unit low, an error that does not average out over a mesh.
 __device__ __forceinline__ void fx_mac(long long& h, long long& m, int2 D, int fl, int fh) {
   h += (long long)D.y * fh;
   m += (long long)D.y * fl;
@@ -114,7 +129,7 @@ __device__ __forceinline__ void fx_line(const int2* __restrict__ F, int stride, 
   }
 #pragma unroll
   for (int i = 0; i < H; ++i) {
-    long long ah = 0, am = 0, bh = 0, bm = 0;
+    long long ah = 0, am = kFxHalf, bh = 0, bm = kFxHalf;
 #pragma unroll
     for (int j = 0; j < H + O; ++j) fx_mac(ah, am, D[i * (H + O) + j], el[j], eh[j]);
 #pragma unroll
@@ -124,17 +139,55 @@ __device__ __forceinline__ void fx_line(const int2* __restrict__ F, int stride, 
     out[N - i] = B - A;
   }
   if constexpr (O) {
-    long long h = 0, m = 0;
+    long long h = 0, m = kFxHalf;
 #pragma unroll
     for (int j = 0; j < H; ++j) fx_mac(h, m, D[H * (H + O) + H * H + j], ol[j], oh[j]);
     out[H] = h + (m >> kFxBits);
   }
 }
 
-// Elements per CTA and threads: the contractions of the rectilinear form are
-// 5 (N+1)^2 lines per direction and element, one per thread and direction.
-// At N = 4 an element's 125 lines and 125 nodes fill 128 threads; the small
-// orders take several elements so that their lines fill whole warps.
+// Shared-memory layout of an element's nodes: node (i, j, k) at i + A j + B k.
+// The lines of a direction are read one per lane; at N = 3 and N = 7 the
+// natural pitches put whole warps on a few banks (a direction's reads take 2.3
+// and 2.8 times the wavefronts), so the planes and rows are padded there.
+template <int N>
+__host__ __device__ constexpr int fx_row() {
+  return N == 7 ? 9 : N + 1;
+}
+template <int N>
+__host__ __device__ constexpr int fx_plane() {
+  return N == 3 ? 19 : fx_row<N>() * (N + 1);
+}
+template <int N>
+__host__ __device__ constexpr int fx_pitch() {  // one element
+  return fx_plane<N>() * (N + 1);
+}
+// Shared index of node l of the CTA's elements.
+template <int N>
+__device__ __forceinline__ int fx_index(int l) {
+  constexpr int P = N + 1, PP = P * P, NP = PP * P;
+  if constexpr (fx_pitch<N>() == NP) return l;
+  else {
+    const int el = l / NP, m = l - el * NP;
+    return el * fx_pitch<N>() + m % P + fx_row<N>() * ((m / P) % P) + fx_plane<N>() * (m / PP);
+  }
+}
+// First node and stride of line r along direction d.
+template <int N>
+__device__ __forceinline__ int fx_line_base(int d, int r) {
+  constexpr int P = N + 1, A = fx_row<N>(), B = fx_plane<N>();
+  const int lo = r % P, hi = r / P;
+  return d == 0 ? A * lo + B * hi : d == 1 ? lo + B * hi : lo + A * hi;
+}
+template <int N>
+__device__ __forceinline__ constexpr int fx_line_stride(int d) {
+  return d == 0 ? 1 : d == 1 ? fx_row<N>() : fx_plane<N>();
+}
+
+// Elements per CTA and threads of the rectilinear form: 5 (N+1)^2 lines per
+// direction and element, one per thread.  At N = 4 an element's 125 lines and
+// 125 nodes fill 128 threads; the small orders take several elements so that
+// their lines fill whole warps.
 template <int N>
 __host__ __device__ constexpr int fx_rect_epb() {
   return N == 1 ? 8 : N == 2 ? 2 : N == 3 ? 2 : 1;
@@ -143,22 +196,44 @@ template <int N>
 __host__ __device__ constexpr int fx_rect_threads() {
   return (fx_rect_epb<N>() * 5 * (N + 1) * (N + 1) + 31) / 32 * 32;
 }
+// Slots of the groups' magnitudes: one per warp of a CTA with one element, or one per element.
+template <int EPB, int NT>
+__host__ __device__ constexpr int fx_slots() {
+  return EPB == 1 ? NT / 32 : EPB;
+}
 template <int N>
 constexpr size_t fx_rect_smem() {
-  constexpr int NN = fx_rect_epb<N>() * (N + 1) * (N + 1) * (N + 1);
-  return 8 * (size_t)(kLF + 10) * NN + 16 * (size_t)(fx_rect_epb<N>() == 1 ? fx_rect_threads<N>() / 32 : fx_rect_epb<N>());
+  constexpr int EPB = fx_rect_epb<N>();
+  return 8 * (size_t)(kLF + 10) * EPB * fx_pitch<N>() + 16 * fx_slots<EPB, fx_rect_threads<N>()>();
 }
 
-// The three directions' tables of one mesh.
+// The per-node form: one thread per node, several elements for the small
+// orders (their 12 (N+1)^2 lines per direction go round the threads).
 template <int N>
+__host__ __device__ constexpr int fx_nodal_epb() {
+  return N == 1 ? 16 : N == 2 ? 4 : N == 3 ? 2 : 1;
+}
+template <int N>
+__host__ __device__ constexpr int fx_nodal_threads() {
+  return (fx_nodal_epb<N>() * (N + 1) * (N + 1) * (N + 1) + 31) / 32 * 32;
+}
+template <int N>
+constexpr size_t fx_nodal_smem() {
+  constexpr int EPB = fx_nodal_epb<N>();
+  return 8 * (size_t)(2 * kLF) * EPB * fx_pitch<N>() + 16 * fx_slots<EPB, fx_nodal_threads<N>()>();
+}
+
+// A mesh's tables as a kernel parameter: K_d D for the three directions
+// (rectilinear form), or D alone (per-node form).
+template <int N, int DIRS>
 struct FxTables {
-  int2 d[3 * fx_table_entries<N>()];
+  int2 d[DIRS * fx_table_entries<N>()];
 };
 
 // The rectilinear residual of one element by plain FP64 arithmetic, nothing
 // staged: for elements the fixed-point form cannot hold.
 template <int N>
-__device__ __noinline__ void rect_plain(const VolumeArgs& a, long long e) {
+__device__ __forceinline__ void rect_plain(const VolumeArgs& a, long long e) {
   constexpr int P = N + 1, NP = P * P * P;
   const long long Nl = a.Nl, Ng = a.Ng;
   const double* w = static_cast<const double*>(a.prim);
@@ -193,6 +268,72 @@ __host__ __device__ constexpr int fx_slot(int f) {
        : f == lTxy ? sTxy : f == lTxz ? sTxz : f == lTyz ? sTyz : f == lHx ? sHx : f == lHy ? sHy : sHz;
 }
 
+// Gathers the 12 flux fields of the nn element nodes from n0 into F as
+// fixed-point integers, one thread per element node.  The largest magnitude of
+// each equation group (x, mass: U; y, momentum: U u + p' I; z, theta: theta U)
+// in an element gives the group's exponent: left per element in gmax
+// (EPB > 1), or returned in gm (EPB = 1).  False (uniform over the CTA) if the
+// integers cannot hold some group.
+template <int N, int EPB, int NT>
+__device__ __forceinline__ bool fx_stage(const VolumeArgs& a, long long n0, int nn, uint4* gmax, int2* F, uint4& gm) {
+  constexpr int NP = (N + 1) * (N + 1) * (N + 1), NN = EPB * NP, IT = (NN + NT - 1) / NT;
+  constexpr int FP = EPB * fx_pitch<N>(), SLOTS = fx_slots<EPB, NT>();
+  const int tid = threadIdx.x;
+  if constexpr (EPB > 1) {
+    if (tid < EPB) gmax[tid] = make_uint4(0u, 0u, 0u, 0u);
+    __syncthreads();
+  }
+  uint4 gw = make_uint4(0u, 0u, 0u, 0u);
+  FluxState64 z[IT];
+#pragma unroll
+  for (int it = 0; it < IT; ++it) {
+    const int l = tid + it * NT;
+    unsigned g0 = 0, g1 = 0, g2 = 0;
+    if (l < nn) {
+      z[it] = gather_fluxes64(a, n0 + l);
+      g0 = fx_group_key(z[it].f + lUx, 3);
+      g1 = fx_group_key(z[it].f + lTxx, 6);
+      g2 = fx_group_key(z[it].f + lHx, 3);
+    }
+    if constexpr (EPB == 1) {
+      gw = make_uint4(max(gw.x, g0), max(gw.y, g1), max(gw.z, g2), 0u);
+    } else if (l < nn) {
+      unsigned* g = reinterpret_cast<unsigned*>(gmax + l / NP);
+      atomicMax(&g[0], g0);
+      atomicMax(&g[1], g1);
+      atomicMax(&g[2], g2);
+    }
+  }
+  if constexpr (EPB == 1) {
+    gw.x = __reduce_max_sync(0xffffffffu, gw.x);
+    gw.y = __reduce_max_sync(0xffffffffu, gw.y);
+    gw.z = __reduce_max_sync(0xffffffffu, gw.z);
+    if ((tid & 31) == 0) gmax[tid >> 5] = gw;
+  }
+  __syncthreads();
+  bool ok = true;
+  gm = make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll
+  for (int t = 0; t < SLOTS; ++t) {
+    const uint4 w = gmax[t];
+    if constexpr (EPB == 1) gm = make_uint4(max(gm.x, w.x), max(gm.y, w.y), max(gm.z, w.z), 0u);
+    else ok &= fx_in_range(w);
+  }
+  if constexpr (EPB == 1) ok = fx_in_range(gm);
+  if (!ok) return false;
+#pragma unroll
+  for (int it = 0; it < IT; ++it) {
+    const int l = tid + it * NT;
+    if (l < nn) {
+      const uint4 g = EPB == 1 ? gm : gmax[l / NP];
+      const int E0 = (int)(g.x >> 20), E1 = (int)(g.y >> 20), E2 = (int)(g.z >> 20), o = fx_index<N>(l);
+#pragma unroll
+      for (int f = 0; f < kLF; ++f) F[fx_slot(f) * FP + o] = fx_of(z[it].f[f], f <= lUz ? E0 : f <= lTyz ? E1 : E2);
+    }
+  }
+  return true;
+}
+
 // create_rhs of up to fx_rect_epb<N>() rectilinear elements e0 .. e0 + ne - 1
 // in fixed point: the residual sum_d K_d (D F_d) without its weight
 // w_i w_j w_k (which the update applies with the inverse mass).
@@ -216,88 +357,32 @@ __host__ __device__ constexpr int fx_slot(int f) {
 template <int N>
 __device__ __forceinline__ void volume_fx_rect(const VolumeArgs& a, const int2* T, long long e0, int ne,
                                                unsigned char* smem_raw) {
-  constexpr int P = N + 1, PP = P * P, NP = PP * P, EPB = fx_rect_epb<N>(), NN = EPB * NP;
-  constexpr int NT = fx_rect_threads<N>(), IT = (NN + NT - 1) / NT;
-  // the largest magnitudes of the three groups: one slot per warp (EPB = 1), or per element
-  constexpr int SLOTS = EPB == 1 ? NT / 32 : EPB;
-  uint4* gmax = reinterpret_cast<uint4*>(smem_raw);              // [SLOTS] (first: 16-byte aligned)
-  int2* F = reinterpret_cast<int2*>(gmax + SLOTS);               // [kLF][NN]
-  long long* part = reinterpret_cast<long long*>(F + kLF * NN);  // [2][5][NN]
+  constexpr int P = N + 1, PP = P * P, NP = PP * P, EPB = fx_rect_epb<N>(), NT = fx_rect_threads<N>();
+  constexpr int EP = fx_pitch<N>(), FP = EPB * EP, M = fx_table_entries<N>(), B = fx_plane<N>();
+  uint4* gmax = reinterpret_cast<uint4*>(smem_raw);                // (first: 16-byte aligned)
+  int2* F = reinterpret_cast<int2*>(gmax + fx_slots<EPB, NT>());  // [kLF][FP]
+  long long* part = reinterpret_cast<long long*>(F + kLF * FP);    // [2][5][FP]
   const int tid = threadIdx.x;
-  const long long Nl = a.Nl, n0 = e0 * NP;
-  const int nn = ne * NP;
-  if constexpr (EPB > 1) {
-    if (tid < EPB) gmax[tid] = make_uint4(0u, 0u, 0u, 0u);
-    __syncthreads();
-  }
-  uint4 gw = make_uint4(0u, 0u, 0u, 0u);
-  FluxState64 z[IT];
-#pragma unroll
-  for (int it = 0; it < IT; ++it) {
-    const int l = tid + it * NT;
-    unsigned g0 = 0, g1 = 0, g2 = 0;
-    if (l < nn) {
-      z[it] = gather_fluxes64(a, n0 + l);
-      g0 = fx_group_key(z[it].f + lUx, 3);
-      g1 = fx_group_key(z[it].f + lTxx, 6);
-      g2 = fx_group_key(z[it].f + lHx, 3);
-    }
-    if constexpr (EPB == 1) {
-      gw = make_uint4(max(gw.x, g0), max(gw.y, g1), max(gw.z, g2), 0u);
-    } else if (l < nn) {
-      unsigned* gm = reinterpret_cast<unsigned*>(gmax + l / NP);
-      atomicMax(&gm[0], g0);
-      atomicMax(&gm[1], g1);
-      atomicMax(&gm[2], g2);
-    }
-  }
-  if constexpr (EPB == 1) {
-    gw.x = __reduce_max_sync(0xffffffffu, gw.x);
-    gw.y = __reduce_max_sync(0xffffffffu, gw.y);
-    gw.z = __reduce_max_sync(0xffffffffu, gw.z);
-    if ((tid & 31) == 0) gmax[tid >> 5] = gw;
-  }
-  __syncthreads();
-  // biased exponents of the groups; (uniform over the CTA) any group outside
-  // the range: every element plain
-  bool plain = a.fxD == nullptr;
-  uint4 gm = make_uint4(0u, 0u, 0u, 0u);
-#pragma unroll
-  for (int t = 0; t < SLOTS; ++t) {
-    const uint4 w = gmax[t];
-    if constexpr (EPB == 1) gm = make_uint4(max(gm.x, w.x), max(gm.y, w.y), max(gm.z, w.z), 0u);
-    else plain |= !fx_in_range(w);
-  }
-  if constexpr (EPB == 1) plain |= !fx_in_range(gm);
-  if (plain) {
+  const long long n0 = e0 * NP;
+  uint4 gm;
+  if (a.fxD == nullptr || !fx_stage<N, EPB, NT>(a, n0, ne * NP, gmax, F, gm)) {  // uniform over the CTA
     for (int t = 0; t < ne; ++t) rect_plain<N>(a, e0 + t);
     return;
-  }
-#pragma unroll
-  for (int it = 0; it < IT; ++it) {
-    const int l = tid + it * NT;
-    if (l < nn) {
-      if constexpr (EPB > 1) gm = gmax[l / NP];
-      const int E0 = (int)(gm.x >> 20), E1 = (int)(gm.y >> 20), E2 = (int)(gm.z >> 20);
-#pragma unroll
-      for (int f = 0; f < kLF; ++f) F[fx_slot(f) * NN + l] = fx_of(z[it].f[f], f <= lUz ? E0 : f <= lTyz ? E1 : E2);
-    }
   }
   __syncthreads();
   const bool act = tid < ne * 5 * PP;
   const int el = EPB == 1 ? 0 : tid / (5 * PP), tt = tid - el * 5 * PP;
   const int v = tt / PP, r = tt - v * PP;
-  constexpr int M = fx_table_entries<N>();
   if (act) {
 #pragma unroll
     for (int d = 0; d < 2; ++d) {
       // the field of equation v along x, y (four bits each)
       constexpr unsigned fy = sUy | sTxy << 4 | sTyy << 8 | sTyz << 12 | sHy << 16;
       const int f = d == 0 ? v : (int)((fy >> (4 * v)) & 15u);
-      const int base = el * NP + (d == 0 ? P * r : r % P + PP * (r / P)), st = d == 0 ? 1 : P;
+      const int base = el * EP + fx_line_base<N>(d, r), st = fx_line_stride<N>(d);
       long long out[P];
-      fx_line<N>(F + f * NN + base, st, T + d * M, out);
-      long long* o = part + (d * 5 + v) * NN + base;
+      fx_line<N>(F + f * FP + base, st, T + d * M, out);
+      long long* o = part + (d * 5 + v) * FP + base;
 #pragma unroll
       for (int m = 0; m < P; ++m) o[m * st] = out[m];
     }
@@ -305,37 +390,190 @@ __device__ __forceinline__ void volume_fx_rect(const VolumeArgs& a, const int2* 
   __syncthreads();
   if (act) {
     constexpr unsigned fz = sUz | sTxz << 4 | sTyz << 8 | sTzz << 12 | sHz << 16;
-    const int f = (int)((fz >> (4 * v)) & 15u), base = el * NP + r;
+    const int f = (int)((fz >> (4 * v)) & 15u), base = el * EP + fx_line_base<N>(2, r);
     long long out[P];
-    fx_line<N>(F + f * NN + base, PP, T + 2 * M, out);
-    const long long* o = part + v * NN + base;
+    fx_line<N>(F + f * FP + base, B, T + 2 * M, out);
+    const long long* o = part + v * FP + base;
     if constexpr (EPB > 1) gm = gmax[el];
     const int kexp = (int)((v == 0 ? gm.x : v == 4 ? gm.z : gm.y) >> 20) + a.fxexp;
-    double* re = static_cast<double*>(a.re) + v * Nl + n0 + base;
+    double* re = static_cast<double*>(a.re) + v * a.Nl + n0 + el * NP + r;
 #pragma unroll
-    for (int m = 0; m < P; ++m) re[m * PP] = fx_to_double(out[m] + o[m * PP] + o[5 * NN + m * PP], kexp);
+    for (int m = 0; m < P; ++m) re[m * PP] = fx_to_double(out[m] + o[m * B] + o[5 * FP + m * B], kexp);
   }
 }
 
+// The per-node residual of one element by plain FP64 arithmetic (see
+// rect_plain), with the metric terms read back from their integers.
 template <int N>
-__global__ void __launch_bounds__(fx_rect_threads<N>())
-    volume_fx_rect_kernel(const __grid_constant__ VolumeArgs a, const __grid_constant__ FxTables<N> T) {
+__device__ __forceinline__ void nodal_plain(const VolumeArgs& a, long long e) {
+  constexpr int P = N + 1, PP = P * P, NP = PP * P;
+  const long long Nl = a.Nl, Ng = a.Ng;
+  const double* w = static_cast<const double*>(a.prim);
+  double* re = static_cast<double*>(a.re);
+  const int4 eb = a.fxE[e];
+  for (int l = threadIdx.x; l < NP; l += blockDim.x) {
+    const int i = l % P, j = (l / P) % P, k = l / PP;
+#pragma unroll 1
+    for (int v = 0; v < 5; ++v) {
+      double t = 0.0;
+#pragma unroll 1
+      for (int d = 0; d < 3; ++d) {
+        const int row = d == 0 ? i : d == 1 ? j : k, st = d == 0 ? 1 : d == 1 ? P : PP;
+#pragma unroll 1
+        for (int c = 0; c < 3; ++c) {
+          // the field of equation v along c: U, the symmetric U u + p' I, theta U
+          const int p = v - 1, lo = min(p, c), hi = max(p, c);
+          const int s = v == 0 ? -1 : v == 4 ? 6 + c : lo == hi ? lo : lo + hi + 2;
+          const double* f = s < 0 ? a.q + (1 + c) * Ng : w + s * Ng;
+          double x = 0.0;
+#pragma unroll 1
+          for (int m = 0; m < P; ++m) x = fma(a.D64[row * P + m], f[a.l2g[e * NP + l + (m - row) * st]], x);
+          // eb.w: the metric terms of this element stayed doubles
+          const long long at = (3 * d + c) * Nl + e * NP + l;
+          double b = a.met64[at];
+          if (!eb.w) {
+            const int2 h = reinterpret_cast<const int2*>(a.met64)[at];
+            const int E = d == 0 ? eb.x : d == 1 ? eb.y : eb.z;
+            b = scalbn((double)(((long long)h.y << kFxBits) + h.x), E - 1022 - 2 * kFxBits + fx_weight_exp(a.fxw, i, j, k));
+          }
+          t = fma(b, x, t);
+        }
+      }
+      re[v * Nl + e * NP + l] = t;
+    }
+  }
+}
+
+// create_rhs of up to fx_nodal_epb<N>() elements of any shape in fixed point,
+// the per-node form of Eq. 5.  Per reference direction d:
+//   1. each thread takes one line and every G-th field on it (fx_line) and
+//      leaves the derivatives in shared memory;
+//   2. one thread per node multiplies the 12 derivatives by the direction's
+//      row of -Jw dxi_d/dx_c (58-bit integers relative to the row's largest
+//      value in the element, fx_metric_kernel) into the five equations.
+// Every row of D is scaled to its own row sum (an end row's is up to 16 times
+// an inner one's).  The directions' sums are aligned by the exponents of their
+// rows, added as integers and rounded once.
+// On the 6x30x30x8 shell at N = 4: 2.068 ms as FP64 (225 operations a node, its
+// pipe 96% busy), 0.505 ms here; 21x17x13 at N = 3: 0.105 -> 0.037 ms.  The 405
+// integer multiply-adds a thread keep their pipe 40% busy and the 2200
+// instructions a warp 61% of the issue slots; both at 8 CTAs an SM (64
+// registers).  Going round all lines of a direction with a division per line
+// instead of one line per thread: 0.570 ms.
+template <int N>
+__device__ __forceinline__ void volume_fx_nodal(const VolumeArgs& a, const int2* T, long long e0, int ne,
+                                                unsigned char* smem_raw) {
+  constexpr int P = N + 1, PP = P * P, NP = PP * P, EPB = fx_nodal_epb<N>(), NT = fx_nodal_threads<N>();
+  constexpr int EP = fx_pitch<N>(), FP = EPB * EP;
+  uint4* gmax = reinterpret_cast<uint4*>(smem_raw);                // (first: 16-byte aligned)
+  int2* F = reinterpret_cast<int2*>(gmax + fx_slots<EPB, NT>());  // [kLF][FP]
+  long long* S = reinterpret_cast<long long*>(F + kLF * FP);       // [kLF][FP]: the direction's derivatives
+  const int tid = threadIdx.x, nn = ne * NP;
+  const long long Nl = a.Nl, n0 = e0 * NP;
+  const bool node = tid < nn;
+  const int nel = EPB == 1 ? 0 : tid / NP;
+  // the elements' metric exponents (w: the element takes plain FP64)
+  const int4 eb = a.fxE[e0 + (node ? nel : 0)];
+  uint4 gm;
+  bool ok = fx_stage<N, EPB, NT>(a, n0, nn, gmax, F, gm);
+  if (__syncthreads_or(!ok || eb.w)) {
+    for (int t = 0; t < ne; ++t) nodal_plain<N>(a, e0 + t);
+    return;
+  }
+  const int at = fx_index<N>(tid);
+  const int2* met = reinterpret_cast<const int2*>(a.met64) + n0 + tid;
+  // the exponents of the node's three directions: the metric row's less that
+  // taken out of its row of D; the sums are kept in units of the largest
+  const int l = tid - nel * NP;
+  const int x0 = eb.x - fx_nibble(a.fxr, l % P), x1 = eb.y - fx_nibble(a.fxr, (l / P) % P);
+  const int x2 = eb.z - fx_nibble(a.fxr, l / PP), xm = max(x0, max(x1, x2));
+  long long sum[5] = {0, 0, 0, 0, 0};
+  // thread's line of every direction, and its first field; the threads of a
+  // line's group take every G-th field
+  constexpr int LN = EPB * PP, G = NT / LN;
+  static_assert(G >= 1, "a thread per line");
+  const int g = tid / LN, q = tid - g * LN, lel = EPB == 1 ? 0 : q / PP, r = q - lel * PP;
+  const int f0 = g < G && lel < ne ? g : kLF;
+  auto direction = [&](auto dir) {
+    constexpr int d = decltype(dir)::value, st = fx_line_stride<N>(d);
+    int2 B[3];
+    if (node) {
+#pragma unroll
+      for (int c = 0; c < 3; ++c) B[c] = met[(3 * d + c) * Nl];
+    }
+    const int base = lel * EP + fx_line_base<N>(d, r);
+    for (int f = f0; f < kLF; f += G) {
+      long long out[P];
+      fx_line<N>(F + f * FP + base, st, T, out);
+#pragma unroll
+      for (int m = 0; m < P; ++m) S[f * FP + base + m * st] = out[m];
+    }
+    __syncthreads();
+    if (node) {
+      const int sh = min(xm - (d == 0 ? x0 : d == 1 ? x1 : x2), 63);
+      auto use = [&](long long& h, long long& m, int slot, int c) {
+        const long long x = S[slot * FP + at];
+        fx_mac(h, m, B[c], (int)((unsigned)x & kFxMask), (int)(x >> kFxBits));
+      };
+      auto eq = [&](int v, int s0, int s1, int s2) {
+        long long h = 0, m = kFxHalf;
+        use(h, m, s0, 0);
+        use(h, m, s1, 1);
+        use(h, m, s2, 2);
+        sum[v] += (h + (m >> kFxBits)) >> sh;
+      };
+      eq(0, sUx, sUy, sUz);
+      eq(1, sTxx, sTxy, sTxz);
+      eq(2, sTxy, sTyy, sTyz);
+      eq(3, sTxz, sTyz, sTzz);
+      eq(4, sHx, sHy, sHz);
+    }
+    if (d < 2) __syncthreads();
+  };
+  direction(std::integral_constant<int, 0>());
+  direction(std::integral_constant<int, 1>());
+  direction(std::integral_constant<int, 2>());
+  if (!node) return;
+  if constexpr (EPB > 1) gm = gmax[nel];
+  const int kx = xm + a.fxexp + fx_weight_exp(a.fxw, l % P, (l / P) % P, l / PP);
+  double* re = static_cast<double*>(a.re) + n0 + tid;
+#pragma unroll
+  for (int v = 0; v < 5; ++v)
+    re[v * Nl] = fx_to_double(sum[v], kx + (int)((v == 0 ? gm.x : v == 4 ? gm.z : gm.y) >> 20));
+}
+
+// CTAs an SM holds at r registers a thread.
+__host__ __device__ constexpr int fx_blocks(int threads, int r) { return 65536 / (threads * r); }
+
+template <int N>
+__global__ void __launch_bounds__(fx_rect_threads<N>(), fx_blocks(fx_rect_threads<N>(), N < 5 ? 48 : 64))
+    volume_fx_rect_kernel(const __grid_constant__ VolumeArgs a, const __grid_constant__ FxTables<N, 3> T) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   constexpr int EPB = fx_rect_epb<N>();
   const int e = (int)blockIdx.x * EPB;
   volume_fx_rect<N>(a, T.d, a.ebeg + (long long)e, min(EPB, a.ecnt - e), smem_raw);
 }
 
-// Ragged form: positions of the group are chunks of fx_rect_epb<N>() elements
-// of one member.
 template <int N>
-__global__ void __launch_bounds__(fx_rect_threads<N>())
-    volume_fx_rect_ragged(const MemberDesc* __restrict__ d, const RaggedGroup* __restrict__ g) {
+__global__ void __launch_bounds__(fx_nodal_threads<N>(), fx_blocks(fx_nodal_threads<N>(), N < 7 ? 64 : 80))
+    volume_fx_nodal_kernel(const __grid_constant__ VolumeArgs a, const __grid_constant__ FxTables<N, 1> T) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  constexpr int EPB = fx_nodal_epb<N>();
+  const int e = (int)blockIdx.x * EPB;
+  volume_fx_nodal<N>(a, T.d, a.ebeg + (long long)e, min(EPB, a.ecnt - e), smem_raw);
+}
+
+// Ragged forms: positions of the group are chunks of EPB elements of one
+// member, whose tables are copied to shared memory.
+template <int N, bool RECT>
+__global__ void __launch_bounds__(RECT ? fx_rect_threads<N>() : fx_nodal_threads<N>(),
+                                  fx_blocks(RECT ? fx_rect_threads<N>() : fx_nodal_threads<N>(), N < 7 ? 64 : 80))
+    volume_fx_ragged(const MemberDesc* __restrict__ d, const RaggedGroup* __restrict__ g) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  constexpr int EPB = RECT ? fx_rect_epb<N>() : fx_nodal_epb<N>(), ENT = (RECT ? 3 : 1) * fx_table_entries<N>();
   __shared__ int s_m;
   __shared__ long long s_e;
-  __shared__ int2 s_T[3 * fx_table_entries<N>()];
-  constexpr int EPB = fx_rect_epb<N>();
+  __shared__ int2 s_T[ENT];
   const int n = g->n;
   const long long total = n > 0 ? g->elem_prefix[n] : 0;
   for (long long w = blockIdx.x; w < total; w += gridDim.x) {
@@ -348,11 +586,52 @@ __global__ void __launch_bounds__(fx_rect_threads<N>())
     // (uniform across the CTA) guard against a table that disagrees with the member
     if (s_m >= 0 && s_m < kMaxMembers && s_e >= 0 && s_e < d[s_m].va.Ne) {
       const VolumeArgs& a = d[s_m].va;
-      if (a.fxD)  // (read after the barriers of volume_fx_rect)
-        for (int t = threadIdx.x; t < 3 * fx_table_entries<N>(); t += blockDim.x) s_T[t] = a.fxD[t];
-      volume_fx_rect<N>(a, s_T, s_e, (int)min((long long)EPB, a.Ne - s_e), smem_raw);
+      if (a.fxD)  // (read after the barriers of the gather)
+        for (int t = threadIdx.x; t < ENT; t += blockDim.x) s_T[t] = a.fxD[t];
+      const int ne = (int)min((long long)EPB, a.Ne - s_e);
+      if constexpr (RECT) volume_fx_rect<N>(a, s_T, s_e, ne, smem_raw);
+      else volume_fx_nodal<N>(a, s_T, s_e, ne, smem_raw);
     }
     __syncthreads();
+  }
+}
+
+// At bind: rows 0..8 of one element's metric array, dxi_d/dx_c, become
+// -Jw dxi_d/dx_c as 58-bit integers (fx_of) relative to the largest of their
+// direction in the element, after division by the power of two
+// fx_weight_exp of the node's quadrature weight (the weights of a corner and
+// of the centre differ by up to 2^13 at N = 8); their biased exponents go to
+// fxE.  Elements whose values the integers cannot hold keep doubles (w = 1).
+template <int UNUSED = 0>
+__global__ void __launch_bounds__(128)
+    fx_metric_kernel(double* met, int4* fxE, long long Nl, int P, unsigned long long fxw) {
+  __shared__ unsigned s_key[3];
+  const int NP = P * P * P;
+  const long long n0 = (long long)blockIdx.x * NP;
+  if (threadIdx.x < 3) s_key[threadIdx.x] = 0u;
+  __syncthreads();
+  for (int l = threadIdx.x; l < NP; l += blockDim.x) {
+    const double jw = -met[9 * Nl + n0 + l];
+    const int we = fx_weight_exp(fxw, l % P, (l / P) % P, l / (P * P));
+    for (int t = 0; t < 9; ++t) {
+      const double b = met[t * Nl + n0 + l] * jw;
+      met[t * Nl + n0 + l] = b;
+      const double x = scalbn(b, -we);
+      atomicMax(&s_key[t / 3], (unsigned)__double2hiint(x) & 0x7fffffffu);
+    }
+  }
+  __syncthreads();
+  const int E[3] = {(int)(s_key[0] >> 20), (int)(s_key[1] >> 20), (int)(s_key[2] >> 20)};
+  bool ok = true;
+  for (int d = 0; d < 3; ++d) ok &= E[d] >= kFxMetMin && E[d] <= kFxMetMax;
+  if (threadIdx.x == 0) fxE[blockIdx.x] = make_int4(E[0], E[1], E[2], ok ? 0 : 1);
+  if (!ok) return;
+  for (int l = threadIdx.x; l < NP; l += blockDim.x) {
+    const int we = fx_weight_exp(fxw, l % P, (l / P) % P, l / (P * P));
+    for (int t = 0; t < 9; ++t) {
+      double* m = met + t * Nl + n0 + l;
+      *reinterpret_cast<int2*>(m) = fx_of(scalbn(*m, -we), E[t / 3]);
+    }
   }
 }
 

@@ -370,107 +370,28 @@ __host__ __device__ constexpr int line_group() {
   return 3 * W32 <= NT ? W32 : P2;
 }
 
-// ---- FP64 element kernels with fewer FP64 instructions ---------------------
-// GB300 issues 2 FP64 FMAs per SM per clock, so the FP64 element kernels are
-// bound by their FP64 instruction count.  Exact rearrangements cut it:
-//
+// ---- the FP64 element kernels' rearrangements of Eq. 4 / Eq. 5 ---------------
 // (1) Per-node form (any element): the pressure is added into the diagonal
 //     momentum fluxes before they are differentiated (12 fields instead of
 //     13) and the metric terms are stored pre-multiplied by -Jw, so the chain
-//     rule is three FMAs per use of a field and no final weighting remains.
+//     rule is three products per use of a field and no final weighting remains.
 // (2) Rectilinear affine elements (every element of an unwarped box): the
 //     metric terms dxi_d/dx_c vanish for c != d and J is constant over the
 //     element, so -Jw div F at node (i,j,k) is w_i w_j w_k sum_d K_d (D F_d)
-//     along xi_d, with K_d = -J dxi_d/dx_d per element.  Folding K_d into the
-//     direction's copy of D leaves the 12 unweighted flux fields of (1) and 15
-//     contractions, with no metric or Jw load per node; in FP64 these run in
-//     fixed point on the integer pipe (fixed64.cuh).  The weight w_i w_j w_k is the same at every element
-//     node of a global node (the Lobatto weights are symmetric and the box's
-//     elements meet face to face), so it moves out of the element kernel
-//     into the inverse mass of the DSS: the kernel writes
-//     sum_d K_d (D F_d), and the update multiplies the sum over element
-//     nodes by w_i w_j w_k / M (Minv_r) instead of 1 / M.
+//     along xi_d, with K_d = -J dxi_d/dx_d.  Folding K_d into the direction's
+//     copy of D leaves the 12 unweighted flux fields of (1) and 15
+//     contractions, with no metric or Jw load per node.  The weight
+//     w_i w_j w_k is the same at every element node of a global node (the
+//     Lobatto weights are symmetric and the box's elements meet face to
+//     face), so it moves out of the element kernel into the inverse mass of
+//     the DSS: the kernel writes sum_d K_d (D F_d), and the update multiplies
+//     the sum over element nodes by w_i w_j w_k / M (Minv_r) instead of 1 / M.
 // (3) Both forms: the nine flux components besides U (U_c u_c + p', the
 //     symmetric U_c u_d, Theta u) are formed once per global node by the
 //     update that writes the state (write_prim) and gathered as they are, not
 //     formed again at each of the global node's element nodes.
-
-// create_rhs of element e in FP64, per-node form of Eq. 5 (any element,
-// curved included), one thread per element node.  The metric terms arrive
-// pre-multiplied by -Jw (rows 0..8 of met64 hold -Jw dxi_d/dx_c for this
-// form), and the pressure sits in the diagonal momentum fluxes, so each of
-// the 12 staged flux fields (kLF) is differentiated along xi, eta and zeta
-// (15 FMAs) and folded into the divergence of every equation that uses it
-// with three FMAs: 180 + 45 FP64 operations per node at N = 4 (the update
-// formed the flux components once per global node).  The
-// result is the weighted residual -Jw div F of Eq. 4.  smem_raw holds
-// 12 (N+1)^3 + (N+1)^2 doubles.
-template <int N>
-__device__ __forceinline__ void volume_element_nodal64(const VolumeArgs& a, long long e, unsigned char* smem_raw) {
-  constexpr int P = N + 1, NP = P * P * P;
-  double* F = reinterpret_cast<double*>(smem_raw);  // [kLF][NP]
-  double* Ds = F + kLF * NP;                         // [P][P]
-  const double* met = a.met64;
-  const int l = threadIdx.x;
-  for (int t = l; t < P * P; t += blockDim.x) Ds[t] = a.D64[t];
-  const long long Nl = a.Nl, n = (long long)e * NP + l;
-  double B[9];  // -Jw dxi_d/dx_c at this node, [3d + c]
-  if (l < NP) {
-#pragma unroll
-    for (int t = 0; t < 9; ++t) B[t] = met[t * Nl + n];
-    const FluxState64 z = gather_fluxes64(a, n);
-#pragma unroll
-    for (int f = 0; f < kLF; ++f) F[f * NP + l] = z.f[f];
-  }
-  __syncthreads();
-  if (l >= NP) return;
-  const int i = l % P, j = (l / P) % P, k = l / (P * P);
-  double dx[P], dy[P], dz[P];
-#pragma unroll
-  for (int m = 0; m < P; ++m) {
-    dx[m] = Ds[i * P + m];
-    dy[m] = Ds[j * P + m];
-    dz[m] = Ds[k * P + m];
-  }
-  const int bx = P * (j + P * k), by = i + P * P * k, bz = i + P * j;
-  // reference-space derivatives of field f along xi, eta, zeta (Eq. 5)
-  auto dref = [&](int f, double& s0, double& s1, double& s2) {
-    const double* Ff = F + f * NP;
-    s0 = dx[0] * Ff[bx];
-    s1 = dy[0] * Ff[by];
-    s2 = dz[0] * Ff[bz];
-#pragma unroll
-    for (int m = 1; m < P; ++m) {
-      s0 = fma(dx[m], Ff[bx + m], s0);
-      s1 = fma(dy[m], Ff[by + P * m], s1);
-      s2 = fma(dz[m], Ff[bz + P * P * m], s2);
-    }
-  };
-  // chain rule into the weighted divergence: acc += -Jw d/dx_c of the field
-  auto first = [&](int c, double s0, double s1, double s2) { return fma(s2, B[6 + c], fma(s1, B[3 + c], s0 * B[c])); };
-  auto add = [&](double& acc, int c, double s0, double s1, double s2) {
-    acc = fma(s2, B[6 + c], fma(s1, B[3 + c], fma(s0, B[c], acc)));
-  };
-  double s0, s1, s2, dr, dxm, dym, dzm, dt;
-  dref(lUx, s0, s1, s2); dr = first(0, s0, s1, s2);
-  dref(lUy, s0, s1, s2); add(dr, 1, s0, s1, s2);
-  dref(lUz, s0, s1, s2); add(dr, 2, s0, s1, s2);
-  dref(lTxx, s0, s1, s2); dxm = first(0, s0, s1, s2);
-  dref(lTyy, s0, s1, s2); dym = first(1, s0, s1, s2);
-  dref(lTzz, s0, s1, s2); dzm = first(2, s0, s1, s2);
-  dref(lTxy, s0, s1, s2); add(dxm, 1, s0, s1, s2); add(dym, 0, s0, s1, s2);
-  dref(lTxz, s0, s1, s2); add(dxm, 2, s0, s1, s2); add(dzm, 0, s0, s1, s2);
-  dref(lTyz, s0, s1, s2); add(dym, 2, s0, s1, s2); add(dzm, 1, s0, s1, s2);
-  dref(lHx, s0, s1, s2); dt = first(0, s0, s1, s2);
-  dref(lHy, s0, s1, s2); add(dt, 1, s0, s1, s2);
-  dref(lHz, s0, s1, s2); add(dt, 2, s0, s1, s2);
-  double* re = static_cast<double*>(a.re);
-  re[n] = dr;
-  re[Nl + n] = dxm;
-  re[2 * Nl + n] = dym;
-  re[3 * Nl + n] = dzm;
-  re[4 * Nl + n] = dt;
-}
+// The contractions and the chain rule run in fixed point on the integer pipe
+// (fixed64.cuh); the pairs mode follows the same forms in float pairs.
 
 // create_rhs of element e in the FP32 form, organised by 1D lines of nodes
 // (Eq. 5 is a contraction along xi, eta and zeta).  Thread t < 3W takes one
@@ -634,7 +555,7 @@ __device__ __forceinline__ void volume_element_lines(const VolumeArgs& a, long l
 }
 
 // create_rhs of element e in the pairs mode: the steps of
-// volume_element_nodal64 (12 flux fields with the pressure on the diagonal,
+// the FP64 per-node form (12 flux fields with the pressure on the diagonal,
 // metric terms pre-multiplied by -Jw: rows 0..8 of met2 hold -Jw dxi_d/dx_c
 // for this form), every value and product carried as a (hi, lo) float pair.
 // The fluxes are differentiated less their values at element node 0, and
@@ -916,7 +837,6 @@ template <int N, typename T, bool AFF>
 constexpr size_t element_smem_bytes() {
   constexpr int P = N + 1, NP = P * P * P;
   if constexpr (std::is_same<T, float>::value) return sizeof(float) * (kNF > 15 ? kNF : 15) * NP;
-  if constexpr (std::is_same<T, double>::value) return sizeof(T) * (kLF * NP + P * P);
   if constexpr (AFF) return sizeof(T) * (15 * NP + P * P + 15);
   return sizeof(T) * (kLF * NP + P * P + kLF);
 }
@@ -932,11 +852,9 @@ __device__ __forceinline__ void element_rhs(const VolumeArgs& a, long long e, un
     } else {
       volume_element_pairs<N>(a, e, smem_raw);
     }
-  } else if constexpr (std::is_same<T, float>::value) {
-    volume_element_lines<N, AFF>(a, e, smem_raw);
   } else {
-    static_assert(!AFF, "rectilinear elements in FP64 take volume_fx_rect; other affine meshes the per-node form");
-    volume_element_nodal64<N>(a, e, smem_raw);
+    static_assert(std::is_same<T, float>::value, "the FP64 element kernels are in fixed64.cuh");
+    volume_element_lines<N, AFF>(a, e, smem_raw);
   }
 }
 

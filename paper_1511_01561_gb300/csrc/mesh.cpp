@@ -87,6 +87,41 @@ void diffmat(const std::vector<double>& x, std::vector<double>& D) {
   }
 }
 
+// Lobatto points and D of order N in 113-bit arithmetic (the same IEEE format
+// on both host architectures).
+#if __LDBL_MANT_DIG__ == 113
+typedef long double Quad;
+#else
+typedef __float128 Quad;
+#endif
+
+void diffmat_quad(int N, std::vector<Quad>& D) {
+  const int P = N + 1;
+  std::vector<double> xd, wd;
+  lobatto(N, xd, wd);
+  std::vector<Quad> x(xd.begin(), xd.end()), lam(P, Quad(1));
+  for (int i = 1; i < N; ++i)
+    for (int it = 0; it < 4; ++it) {  // Newton on x P_N - P_{N-1} from the double roots
+      Quad a = 1, b = x[i];
+      for (int k = 2; k <= N; ++k) {
+        const Quad c = ((2 * k - 1) * x[i] * b - (k - 1) * a) / k;
+        a = b;
+        b = c;
+      }
+      x[i] -= (x[i] * b - a) / ((N + 1) * b);
+    }
+  for (int j = 0; j < P; ++j)
+    for (int k = 0; k < P; ++k)
+      if (k != j) lam[j] *= x[j] - x[k];
+  D.assign(P * P, Quad(0));
+  for (int i = 0; i < P; ++i)
+    for (int j = 0; j < P; ++j)
+      if (j != i) {
+        D[i * P + j] = (lam[i] / lam[j]) / (x[i] - x[j]);
+        D[i * P + i] -= D[i * P + j];
+      }
+}
+
 // Right-handed cube-panel frames (e_a, e_b, e_n) of the gnomonic cubed sphere.
 const int kFrame[6][3][3] = {
     {{0, 1, 0}, {0, 0, 1}, {1, 0, 0}},  {{-1, 0, 0}, {0, 0, 1}, {0, 1, 0}},
@@ -278,53 +313,21 @@ void filter_matrix_host(int N, const double* xi, const double* w, int s, double 
     }
 }
 
-// Lobatto points and D of order N in 113-bit arithmetic (the same IEEE format
-// on both host architectures), so that the fixed-point tables carry no
-// rounding of D.
-#if __LDBL_MANT_DIG__ == 113
-typedef long double Quad;
-#else
-typedef __float128 Quad;
-#endif
-
-static void lobatto_quad(int N, std::vector<Quad>& x) {
-  std::vector<double> xd, wd;
-  lobatto(N, xd, wd);
-  x.assign(xd.begin(), xd.end());
-  for (int i = 1; i < N; ++i)
-    for (int it = 0; it < 4; ++it) {  // Newton on x P_N - P_{N-1} from the double roots
-      Quad a = 1, b = x[i];
-      for (int k = 2; k <= N; ++k) {
-        const Quad c = ((2 * k - 1) * x[i] * b - (k - 1) * a) / k;
-        a = b;
-        b = c;
-      }
-      x[i] -= (x[i] * b - a) / ((N + 1) * b);
-    }
-}
-
 // The order of fx_line (fixed64.cuh): with H = P/2 and O = P%2, rows i < H of
 // (D_ij + D_i,N-j)/2 (j < H) and D_i,mid, rows i < H of (D_ij - D_i,N-j)/2,
 // and for odd P the middle row D_mid,j (j < H).  D 1 = 0 holds exactly in the
 // integers: a row's even part takes the rounding in its last entry (the
 // middle one), or for even P in its largest.
-int fx_table_host(int P, double a, double b, double c, int s, int2* out) {
+int fx_table_host(int P, const double* D64, double a, double b, double c, int s, unsigned long long rows,
+                  int2* out) {
   const int N = P - 1, H = P / 2, O = P % 2;
-  std::vector<Quad> x, lam(P, Quad(1)), D(P * P, Quad(0));
-  lobatto_quad(N, x);
-  for (int j = 0; j < P; ++j)
-    for (int k = 0; k < P; ++k)
-      if (k != j) lam[j] *= x[j] - x[k];
+  std::vector<Quad> D;
+  if (D64) D.assign(D64, D64 + P * P);
+  else diffmat_quad(N, D);
   Quad scale = (Quad)a * (Quad)b / (Quad)c;
   for (int t = 0; t < s; ++t) scale *= 2;
   for (int t = 0; t > s; --t) scale /= 2;
-  for (int i = 0; i < P; ++i) {
-    for (int j = 0; j < P; ++j)
-      if (j != i) {
-        D[i * P + j] = (lam[i] / lam[j]) / (x[i] - x[j]) * scale;
-        D[i * P + i] -= D[i * P + j];
-      }
-  }
+  for (int t = 0; t < P * P; ++t) D[t] *= scale * (Quad)(1 << ((rows >> (4 * (t / P))) & 15));
   auto whole = [](Quad v) { return (long long)(v < 0 ? v - Quad(0.5) : v + Quad(0.5)); };
   int n = 0;
   auto put = [&](long long v) {
@@ -361,6 +364,19 @@ bool build_host_mesh(const numa_config& c, HostMesh& m, std::string& err) {
   m.Np = m.P * m.P * m.P;
   lobatto(m.N, m.xi, m.w);
   diffmat(m.xi, m.D);
+  if (c.precision != NUMA_FP32_MIXED) {
+    // FP64 and pairs: D correctly rounded and with D_{N-i,N-j} = -D_ij exactly,
+    // as the even/odd tables of the fixed-point kernels hold it; the metric
+    // terms below come from the D the fields are differentiated with, so that
+    // its rounding cancels between them on smooth fields
+    const int P = m.P;
+    std::vector<Quad> D;
+    diffmat_quad(m.N, D);
+    for (int t = 0; t < P * P; ++t) {
+      const int u = P * P - 1 - t;  // (N-i, N-j)
+      m.D[t] = u > t ? (double)D[t] : u < t ? -m.D[u] : 0.0;
+    }
+  }
   std::vector<double> X;
   // element nodes from the configuration alone, so that a mesh beyond the
   // 32-bit indices is refused before any of its arrays is built (each global

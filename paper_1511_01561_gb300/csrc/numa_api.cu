@@ -70,6 +70,9 @@ VolumeArgs volume_args(const numa_ctx* c, const double* q, const void* prim, voi
   a.fxD = c->fx ? c->L.fxD : nullptr;
   a.fxD_host = c->fx ? c->fxD.data() : nullptr;
   a.fxexp = c->fxexp;
+  a.fxE = c->L.fxE;
+  a.fxw = c->fxw;
+  a.fxr = c->fxr;
   a.Ng = c->mesh.Ng;
   a.Nl = c->mesh.Nl;
   a.Ne = (int)c->mesh.Ne;
@@ -365,16 +368,6 @@ cudaError_t enqueue_rk_step(numa_ctx* c, double dt, cudaStream_t s, cudaEvent_t*
   return cudaSuccess;
 }
 
-// The per-node FP64 form reads -Jw dxi_d/dx_c: rows 0..8 of the uploaded
-// metric array times -Jw (row 9), in place.
-__global__ void __launch_bounds__(256) weight_metric_kernel(double* met, long long Nl) {
-  const long long n = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (n >= Nl) return;
-  const double mjw = -met[9 * Nl + n];
-#pragma unroll
-  for (int t = 0; t < 9; ++t) met[t * Nl + n] *= mjw;
-}
-
 // Slabs of a box along z for the pipelined RK step (see SlabPlan).  A plan
 // needs CG storage, walls at the bottom and top (a periodic seam would tie
 // the first node slab to the last element slab), element slabs at least two
@@ -481,7 +474,10 @@ size_t layout_workspace(const numa_config& c, const HostMesh& m, char* base, Dev
   if ((c.precision == NUMA_FP64 || c.precision == NUMA_FP64_PAIRS) && affine_elements(c)) {
     d.affk = (double*)take(3 * (size_t)m.Ne * 8);
     d.Minv_r = (double*)take(Ng * 8);
+  }
+  if (c.precision == NUMA_FP64) {
     d.fxD = (int2*)take(3 * kFxEntries * sizeof(int2));
+    d.fxE = (int4*)take((size_t)m.Ne * sizeof(int4));
   }
   d.D32 = (float*)take(PP * 4);
   d.D2 = (float2*)take(PP * 8);
@@ -632,6 +628,7 @@ int numa_bind(numa_ctx* c, void* ws, size_t bytes, void* stream) {
   std::vector<int2> fxD;
   bool rect = false, fx = false;
   int fxexp = 0;
+  unsigned long long fxw = 0, fxr = 0;
   if (c->cfg.precision == NUMA_FP64 || c->cfg.precision == NUMA_FP64_PAIRS) {
     if (affine_elements(c->cfg)) {
       const int P = m.P;
@@ -676,7 +673,7 @@ int numa_bind(numa_ctx* c, void* ws, size_t bytes, void* stream) {
         if (fx) {
           fxD.resize(3 * kFxEntries);
           int n = 0;
-          for (int d = 0; d < 3; ++d) n += fx_table_host(P, num[d][0], num[d][1], den[d], s2, fxD.data() + n);
+          for (int d = 0; d < 3; ++d) n += fx_table_host(P, nullptr, num[d][0], num[d][1], den[d], s2, 0, fxD.data() + n);
           fxexp = 64 - s2;
           up(L.fxD, fxD.data(), (size_t)n * sizeof(int2));
         }
@@ -702,9 +699,28 @@ int numa_bind(numa_ctx* c, void* ws, size_t bytes, void* stream) {
       if (rect) up(L.Minv_r, Minv_r.data(), Minv_r.size() * 8);
     }
     if (c->cfg.precision == NUMA_FP64 && !rect) {
-      if (e == cudaSuccess && Nl)
-        weight_metric_kernel<<<(unsigned)((Nl + 255) / 256), 256, 0, s>>>(L.met64, (long long)Nl);
-      if (e == cudaSuccess) e = cudaGetLastError();
+      // the per-node form: D's table, its row sums scaled to [2^58, 2^59) (a
+      // node's sum of nine products of 2^59 and 2^58 stays below 2^63), the
+      // weights' powers of two, and the metric terms as integers
+      int e2[kMaxN + 1], top = -100;
+      for (int i = 0; i < m.P; ++i) {
+        double row = 0.0;
+        for (int j = 0; j < m.P; ++j) row += std::fabs(m.D[i * m.P + j]);
+        std::frexp(row, &e2[i]);  // row < 2^e2
+        top = std::max(top, e2[i]);
+      }
+      for (int i = 0; i < m.P; ++i) fxr |= (unsigned long long)std::min(15, top - std::max(e2[i], e2[m.N - i])) << (4 * i);
+      fxD.resize(kFxEntries);
+      const int n = fx_table_host(m.P, m.D.data(), 1.0, 1.0, 1.0, 59 - top, fxr, fxD.data());
+      up(L.fxD, fxD.data(), (size_t)n * sizeof(int2));
+      fx = true;
+      fxexp = -958 - (59 - top);
+      for (int i = 0; i < m.P; ++i) {
+        int we = 0;
+        std::frexp(m.w[i], &we);  // w in [2^(we-1), 2^we), at most 4/3
+        fxw |= (unsigned long long)(1 - we) << (4 * i);
+      }
+      if (e == cudaSuccess) e = launch_fx_metric(L.met64, L.fxE, m.Ne, m.N, fxw, s);
     }
   }
   up(L.l2g, m.l2g.data(), Nl * 4);
@@ -726,6 +742,8 @@ int numa_bind(numa_ctx* c, void* ws, size_t bytes, void* stream) {
   c->fx = fx;
   c->fxD = fxD;
   c->fxexp = fxexp;
+  c->fxw = fxw;
+  c->fxr = fxr;
   c->slabs = plan_slabs(c->cfg, m, c->nslab_req);
   if (c->slabs.S > 1) {
     e = ensure_slab_streams(c);

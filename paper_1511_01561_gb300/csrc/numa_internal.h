@@ -64,7 +64,7 @@ struct DevLayout {
   void* prim = nullptr;      // primitive fields (scratch) [kPrimBytesPerNode * Ng]
   void* re = nullptr;        // element residuals -Jw div F (scratch): double or float [5][Nl]
   double* met64 = nullptr;   // [10][Nl] FP64 metric terms and Jw; for the per-node form rows 0..8
-                             // hold -Jw dxi_d/dx_c (the weighted metric of volume_element_nodal64)
+                             // hold -Jw dxi_d/dx_c as integers (fx_metric_kernel)
   float* met32 = nullptr;    // [10][Nl] FP32 copy (mixed-precision form)
   float2* met2 = nullptr;    // [10][Nl] (hi, lo) pairs (pairs mode)
   float2* D2 = nullptr;      // [P*P] (hi, lo) pairs (pairs mode)
@@ -81,7 +81,8 @@ struct DevLayout {
   double* nrm = nullptr;     // [3][Ng] (shell)
   double* D64 = nullptr;     // [P*P]
   double* affk = nullptr;    // FP64 / pairs affine elements: [3][Ne] K_d = -J dxi_d/dx_d per element
-  int2* fxD = nullptr;       // FP64 rectilinear form: K_d D as fixed-point even/odd tables [3][kFxEntries]
+  int2* fxD = nullptr;       // FP64: K_d D (rectilinear form) or D as fixed-point even/odd tables [3][kFxEntries]
+  int4* fxE = nullptr;       // FP64 per-node form: [Ne] exponents of the metric rows (fx_metric_kernel)
   float* D32 = nullptr;      // [P*P]
   double* F64 = nullptr;     // [P*P] 1D filter matrix (FP64, pairs)
   float* F32 = nullptr;      // [P*P] the same in FP32 (FP32 form)
@@ -95,9 +96,10 @@ struct DevLayout {
 constexpr int kFxEntries = 40;
 // (a b / c) D (one direction's derivative matrix times its metric factor) as
 // the even/odd fixed-point table of fx_line (fixed64.cuh): entries
-// 2^s (a b / c) D as (low 29 bits, rest), D evaluated beyond FP64 and rounded
-// once.  Returns the number of entries.
-int fx_table_host(int P, double a, double b, double c, int s, int2* out);
+// 2^s (a b / c) D as (low 29 bits, rest), rounded once; D64 = nullptr: D
+// evaluated beyond FP64.  With rows (4 bits per row, low row first) row i is
+// scaled by 2^(s + rows_i), rows_i = rows_{N-i}.  Returns the number of entries.
+int fx_table_host(int P, const double* D64, double a, double b, double c, int s, unsigned long long rows, int2* out);
 // Elements per position of a ragged volume launch (RaggedGroup::elem_prefix).
 int volume_chunk(int N, int precision, int form);
 
@@ -135,10 +137,13 @@ struct VolumeArgs {
   const float2* D2;    // pairs mode
   void* re;            // [5][Nl] output
   const double* affk;   // rectilinear form (FP64, pairs): [3][Ne] -J dxi_d/dx_d
-  const int2* fxD;      // FP64 rectilinear form: fixed-point tables of K_d D, one after the other (nullptr:
-                        // K_d outside the fixed-point range, the elements take plain FP64)
+  const int2* fxD;      // FP64: fixed-point tables of K_d D (rectilinear form, one after the other; nullptr:
+                        // K_d outside the fixed-point range, the elements take plain FP64) or of D (per-node form)
   const int2* fxD_host; // the same tables in host memory (kernel parameters of the single-mesh launch)
   int fxexp;            // the exponent that goes with fxD
+  const int4* fxE;      // FP64 per-node form: [Ne] exponents of the metric rows' integers
+  unsigned long long fxw, fxr;  // and the powers of two taken out of the quadrature weights (fx_weight_exp)
+                                // and put into the rows of D, 4 bits per point of a line
   long long Ng, Nl;
   int Ne;
   int ebeg, ecnt;      // the launch covers elements [ebeg, ebeg + ecnt) (a slab, or all: 0, Ne)
@@ -246,9 +251,11 @@ cudaError_t upload_d32_constant(int N, const float* D, cudaStream_t s);
 cudaError_t launch_volume(int N, int precision, const VolumeArgs& a, cudaStream_t s);
 // the element kernels of one precision (volume_fp64.cu, volume_fp32.cu,
 // volume_pairs.cu); launch_volume and launch_volume_ragged dispatch to them
-cudaError_t launch_volume_fp64(int N, bool affine, const VolumeArgs& a, cudaStream_t s);
+cudaError_t launch_volume_fp64(int N, bool rect, const VolumeArgs& a, cudaStream_t s);
 cudaError_t launch_volume_fp32(int N, bool affine, const VolumeArgs& a, cudaStream_t s);
 cudaError_t launch_volume_pairs(int N, bool affine, const VolumeArgs& a, cudaStream_t s);
+// the metric terms of the FP64 per-node form as integers, in place
+cudaError_t launch_fx_metric(double* met, int4* fxE, long long Ne, int N, unsigned long long fxw, cudaStream_t s);
 cudaError_t launch_update(int precision, const UpdateArgs& a, cudaStream_t s);
 // the element part of the filter (filter.cu); mode 3 of launch_update does the DSS
 cudaError_t launch_filter(int N, int precision, const FilterArgs& a, cudaStream_t s);
@@ -282,7 +289,7 @@ struct RaggedGroup {
 
 cudaError_t launch_volume_ragged(int N, int precision, bool affine, const MemberDesc* d, const RaggedGroup* g,
                                  cudaStream_t s);
-cudaError_t launch_volume_ragged_fp64(int N, bool affine, const MemberDesc* d, const RaggedGroup* g, cudaStream_t s);
+cudaError_t launch_volume_ragged_fp64(int N, bool rect, const MemberDesc* d, const RaggedGroup* g, cudaStream_t s);
 cudaError_t launch_volume_ragged_fp32(int N, bool affine, const MemberDesc* d, const RaggedGroup* g, cudaStream_t s);
 cudaError_t launch_volume_ragged_pairs(int N, bool affine, const MemberDesc* d, const RaggedGroup* g, cudaStream_t s);
 cudaError_t launch_update_ragged(int precision, bool shell, int stage, const MemberDesc* d, const RaggedGroup* g,
@@ -314,6 +321,7 @@ struct numa_ctx {
   bool fx = false;          // FP64: L.fxD and fxD hold the mesh's fixed-point tables, with exponent fxexp
   std::vector<int2> fxD;
   int fxexp = 0;
+  unsigned long long fxw = 0, fxr = 0;  // FP64 per-node form: VolumeArgs::fxw, fxr
   int nslab_req = 0;        // slabs asked for by numa_set_slabs (0: automatic)
   numa::SlabPlan slabs;     // the plan in use (made at bind and by numa_set_slabs)
   cudaStream_t side = nullptr;  // the second stream of the slab pipeline

@@ -52,7 +52,7 @@ cudaError_t launch_prim(const PrimArgs& a, cudaStream_t s) {
 cudaError_t launch_volume(int N, int precision, const VolumeArgs& a, cudaStream_t s) {
   if (precision == NUMA_FP64_PAIRS) return launch_volume_pairs(N, a.affine != 0, a, s);
   if (precision == NUMA_FP32_MIXED) return launch_volume_fp32(N, a.affine != 0, a, s);
-  return launch_volume_fp64(N, a.affine != 0, a, s);
+  return launch_volume_fp64(N, a.affine == 2, a, s);
 }
 
 cudaError_t launch_update(int precision, const UpdateArgs& a, cudaStream_t s) {

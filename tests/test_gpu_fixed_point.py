@@ -56,12 +56,25 @@ def test_rect_orders_and_remainders(numa, orc, N, ne, per):
     _check(_rhs(numa, cfg, q), m.rhs(q))
 
 
+# the per-node form: warped boxes and the box's elements taken as curved, with
+# rows of the metric 100 times apart
+@pytest.mark.parametrize("N", range(1, 9))
+@pytest.mark.parametrize("over", [dict(warp=0.04), dict(metric_form="nodal")], ids=["warped", "nodal"])
+@pytest.mark.parametrize("ne,per", [((3, 1, 1), (0, 0, 0)), ((2, 3, 3), (1, 0, 0))])
+def test_nodal_orders_and_remainders(numa, orc, N, ne, per, over):
+    cfg = I.box(ne, N, L=(30000.0, 700.0, 900.0), periodic=per, **over)
+    m = orc.Mesh(cfg)
+    q = scaled_random_state(m.Ng, m.ref()[0], m.ref()[1], seed=N)
+    _check(_rhs(numa, cfg, q), m.rhs(q))
+
+
 @pytest.mark.parametrize("N", [2, 4, 7])
+@pytest.mark.parametrize("over", [dict(), dict(warp=0.03)], ids=["rect", "warped"])
 @pytest.mark.parametrize("scale", [1e-30, 1e-200, 1e-310])
-def test_rect_small_momentum(numa, orc, N, scale):
+def test_small_momentum(numa, orc, N, over, scale):
     """The mass equation is linear in U: a momentum far below the other groups
     (1e-30), below the fixed-point range (1e-200) and subnormal (1e-310)."""
-    cfg = I.box((3, 2, 2), N)
+    cfg = I.box((3, 2, 2), N, **over)
     m = orc.Mesh(cfg)
     q = np.zeros((5, m.Ng))
     q[1:4] = np.random.default_rng(N).uniform(-1.0, 1.0, (3, m.Ng)) * scale
