@@ -4,8 +4,8 @@
 // GB300 issues 2 FP64 operations per SM per clock and 32 32x32+64-bit integer
 // multiply-adds (IMAD.WIDE), so a product of two 58-bit numbers in three of
 // them costs 3 cycles of the SM per warp against 16 for an FP64 FMA.  Every
-// field of an element is written as a 58-bit integer relative to the largest
-// magnitude of its equation group in the element (a power of two), D as a
+// field of an element is a 58- or 59-bit integer relative to the largest magnitude
+// of its equation group in the element (a power of two), D as a
 // 60-bit integer relative to its largest row sum, and their products are
 // summed exactly in 64-bit accumulators.  What is dropped is below 2^-58 of
 // (largest field) x (row sum of |D|), the size whose 2^-53 an FP64 chain
@@ -37,10 +37,9 @@ __device__ __forceinline__ int fx_weight_exp(unsigned long long fxw, int i, int 
   return -(fx_nibble(fxw, i) + fx_nibble(fxw, j) + fx_nibble(fxw, k));
 }
 
-// x as a 58-bit integer in units of 2^(E - 1022 - 58), E the biased exponent
-// of the group's largest magnitude: (low 29 bits, signed rest).  Exact for
-// values within 2^5 of the largest; below, truncated towards zero.
-__device__ __forceinline__ int2 fx_of(double x, int E) {
+// x as a 58-bit integer in units of 2^(E - 1022 - 58), |x| < 2^(E - 1022).
+// Exact for values within 2^5 of that; below, truncated towards zero.
+__device__ __forceinline__ long long fx_of(double x, int E) {
   const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
   const unsigned m = (hi & 0xfffffu) | 0x100000u;
   const int e = (int)((hi >> 20) & 0x7ffu);
@@ -48,8 +47,15 @@ __device__ __forceinline__ int2 fx_of(double x, int E) {
   unsigned long long q = ((unsigned long long)__funnelshift_l(lo, m, 10) << 32) | (lo << 10);
   q >>= sh;
   const long long sg = (long long)((int)hi >> 31);
-  const long long s = (long long)(q ^ (unsigned long long)sg) - sg;
-  return make_int2((int)((unsigned)s & kFxMask), (int)(s >> kFxBits));
+  return (long long)(q ^ (unsigned long long)sg) - sg;
+}
+
+// s as l + 2^29 h, l from -2^28 to 2^28 - 1: signed, so that the products of low
+// parts that fx_mac leaves out have no mean (with l from 0 their mean, the
+// same at every node of a row of D, is half a unit of a derivative).
+__device__ __forceinline__ int2 fx_split(long long s) {
+  s += kFxHalf;
+  return make_int2((int)((unsigned)s & kFxMask) - (int)kFxHalf, (int)(s >> kFxBits));
 }
 
 // S 2^(kexp - 1086) rounded to nearest: the double whose biased exponent is
@@ -76,14 +82,35 @@ __device__ __forceinline__ unsigned fx_group_key(const double* x, int n) {
   return max(k, low ? 1u : 0u);
 }
 
-// Whether the fixed-point form holds a CTA's groups (keys x, y, z).
+// The biased exponents of an element's equation groups, |field| <
+// 2^(exponent - 1022), from the magnitude keys of U, u, theta and p' (x, y, z,
+// w): mass: U; momentum: U u + p' I; theta: theta U.  A group of zeros gets an
+// exponent (kFxZero) at which fx_of shifts every bit of a zero out.
+struct FxExp {
+  int U, m, t;
+};
+// U u and p' each stay below 2^(m - 1022), their sum below twice that: a
+// 59-bit integer.
+constexpr int kFxZero = 100;
+__device__ __forceinline__ FxExp fx_exps(uint4 k) {
+  const int U = max((int)(k.x >> 20), kFxZero);
+  // whether the product of the largest U and u carries into the next power of two
+  const unsigned mU = (k.x & 0xfffffu) + 0x100001u, mu = (k.y & 0xfffffu) + 0x100001u;
+  const int Uu = U + (int)(k.y >> 20) - 1023 + ((unsigned long long)mU * mu > (1ull << 41));
+  return {U, max(max(Uu, (int)(k.w >> 20)), kFxZero), U + (int)(k.z >> 20) - 1022};
+}
+
+// Whether the fixed-point form holds an element with these keys: every field
+// and, unless U is zero (and with it every product), every group.
 __device__ __forceinline__ bool fx_in_range(uint4 k) {
-  auto ok = [](unsigned key) { return key == 0u || ((key >> 20) - kFxMinExp <= kFxMaxExp - kFxMinExp); };
-  return ok(k.x) && ok(k.y) && ok(k.z);
+  auto in = [](int E) { return (unsigned)E - kFxMinExp <= kFxMaxExp - kFxMinExp; };
+  auto ok = [&](unsigned key) { return key == 0u || in((int)(key >> 20)); };
+  const FxExp e = fx_exps(k);
+  return ok(k.x) && ok(k.y) && ok(k.z) && ok(k.w) && (k.x == 0u || ((k.y == 0u || in(e.m)) && (k.z == 0u || in(e.t))));
 }
 
 // (high, middle) accumulators += D * f, D = Dh 2^29 + Dl, f = fh 2^29 + fl;
-// the product of the low parts (2^-58 of the full scale) is left out.  The
+// the product of the low parts (below half a unit of the high one) is left out.  The
 // middle accumulator starts at half a unit of the high one, so that
 // h + (m >> 29) is rounded, not cut: a cut would leave every derivative half a
 // unit low, an error that does not average out over a mesh.
@@ -91,6 +118,13 @@ __device__ __forceinline__ void fx_mac(long long& h, long long& m, int2 D, int f
   h += (long long)D.y * fh;
   m += (long long)D.y * fl;
   m += (long long)D.x * fh;
+}
+
+// a b 2^-58, rounded but for the product of the low parts.
+__device__ __forceinline__ long long fx_mul(int2 a, int2 b) {
+  long long h = 0, m = kFxHalf;
+  fx_mac(h, m, a, b.x, b.y);
+  return h + (m >> kFxBits);
 }
 
 // Entries of a direction's even/odd table (see fx_line).
@@ -230,13 +264,23 @@ struct FxTables {
   int2 d[DIRS * fx_table_entries<N>()];
 };
 
+// The flux of equation v along c at global node g, plain FP64: U, the
+// symmetric U u + p' I, theta U.
+__device__ __forceinline__ double plain_flux(const VolumeArgs& a, int v, int c, int g) {
+  const double* U = a.q + a.Ng + g;
+  const double* w = static_cast<const double*>(a.prim) + g;
+  if (v == 0) return U[c * a.Ng];
+  if (v == 4) return w[3 * a.Ng] * U[c * a.Ng];
+  const int lo = min(v - 1, c), hi = max(v - 1, c);
+  return fma(U[lo * a.Ng], w[hi * a.Ng], lo == hi ? w[4 * a.Ng] : 0.0);
+}
+
 // The rectilinear residual of one element by plain FP64 arithmetic, nothing
 // staged: for elements the fixed-point form cannot hold.
 template <int N>
 __device__ __forceinline__ void rect_plain(const VolumeArgs& a, long long e) {
   constexpr int P = N + 1, NP = P * P * P;
-  const long long Nl = a.Nl, Ng = a.Ng;
-  const double* w = static_cast<const double*>(a.prim);
+  const long long Nl = a.Nl;
   double* re = static_cast<double*>(a.re);
   for (int l = threadIdx.x; l < NP; l += blockDim.x) {
     const int i = l % P, j = (l / P) % P, k = l / (P * P);
@@ -247,12 +291,9 @@ __device__ __forceinline__ void rect_plain(const VolumeArgs& a, long long e) {
       for (int d = 0; d < 3; ++d) {
         const int row = d == 0 ? i : d == 1 ? j : k, st = d == 0 ? 1 : d == 1 ? P : P * P;
         const double K = a.affk[d * (long long)a.Ne + e];
-        // the field of equation v along d: U, the symmetric U u + p' I, theta U
-        const int s = v == 0 ? -1 - d : v == 4 ? 6 + d : v - 1 == d ? d : (v - 1) + d + 2;
-        const double* f = s < 0 ? a.q + (1 + d) * Ng : w + s * Ng;
 #pragma unroll 1
         for (int m = 0; m < P; ++m)
-          t = fma(K * a.D64[row * P + m], f[a.l2g[e * NP + l + (m - row) * st]], t);
+          t = fma(K * a.D64[row * P + m], plain_flux(a, v, d, a.l2g[e * NP + l + (m - row) * st]), t);
       }
       re[v * Nl + e * NP + l] = t;
     }
@@ -268,14 +309,13 @@ __host__ __device__ constexpr int fx_slot(int f) {
        : f == lTxy ? sTxy : f == lTxz ? sTxz : f == lTyz ? sTyz : f == lHx ? sHx : f == lHy ? sHy : sHz;
 }
 
-// Gathers the 12 flux fields of the nn element nodes from n0 into F as
-// fixed-point integers, one thread per element node.  The largest magnitude of
-// each equation group (x, mass: U; y, momentum: U u + p' I; z, theta: theta U)
-// in an element gives the group's exponent: left per element in gmax
-// (EPB > 1), or returned in gm (EPB = 1).  False (uniform over the CTA) if the
-// integers cannot hold some group.
+// Gathers U, u, theta and p' at the nn element nodes from n0, one thread per
+// element node, and leaves the 12 flux fields in F as fixed-point integers.
+// The largest magnitudes in an element give its groups' exponents: left as
+// keys per element in gmax (EPB > 1), or returned in ge (EPB = 1).  False
+// (uniform over the CTA) if the integers cannot hold some element.
 template <int N, int EPB, int NT>
-__device__ __forceinline__ bool fx_stage(const VolumeArgs& a, long long n0, int nn, uint4* gmax, int2* F, uint4& gm) {
+__device__ __forceinline__ bool fx_stage(const VolumeArgs& a, long long n0, int nn, uint4* gmax, int2* F, FxExp& ge) {
   constexpr int NP = (N + 1) * (N + 1) * (N + 1), NN = EPB * NP, IT = (NN + NT - 1) / NT;
   constexpr int FP = EPB * fx_pitch<N>(), SLOTS = fx_slots<EPB, NT>();
   const int tid = threadIdx.x;
@@ -284,51 +324,74 @@ __device__ __forceinline__ bool fx_stage(const VolumeArgs& a, long long n0, int 
     __syncthreads();
   }
   uint4 gw = make_uint4(0u, 0u, 0u, 0u);
-  FluxState64 z[IT];
+  NodeState64 z[IT];
 #pragma unroll
   for (int it = 0; it < IT; ++it) {
     const int l = tid + it * NT;
-    unsigned g0 = 0, g1 = 0, g2 = 0;
     if (l < nn) {
-      z[it] = gather_fluxes64(a, n0 + l);
-      g0 = fx_group_key(z[it].f + lUx, 3);
-      g1 = fx_group_key(z[it].f + lTxx, 6);
-      g2 = fx_group_key(z[it].f + lHx, 3);
-    }
-    if constexpr (EPB == 1) {
-      gw = make_uint4(max(gw.x, g0), max(gw.y, g1), max(gw.z, g2), 0u);
-    } else if (l < nn) {
-      unsigned* g = reinterpret_cast<unsigned*>(gmax + l / NP);
-      atomicMax(&g[0], g0);
-      atomicMax(&g[1], g1);
-      atomicMax(&g[2], g2);
+      z[it] = gather_node64(a, n0 + l);
+      const uint4 k = make_uint4(fx_group_key(z[it].U, 3), fx_group_key(z[it].u, 3), fx_group_key(&z[it].th, 1),
+                                 fx_group_key(&z[it].pp, 1));
+      if constexpr (EPB == 1) {
+        gw = make_uint4(max(gw.x, k.x), max(gw.y, k.y), max(gw.z, k.z), max(gw.w, k.w));
+      } else {
+        unsigned* g = reinterpret_cast<unsigned*>(gmax + l / NP);
+        atomicMax(&g[0], k.x);
+        atomicMax(&g[1], k.y);
+        atomicMax(&g[2], k.z);
+        atomicMax(&g[3], k.w);
+      }
     }
   }
   if constexpr (EPB == 1) {
     gw.x = __reduce_max_sync(0xffffffffu, gw.x);
     gw.y = __reduce_max_sync(0xffffffffu, gw.y);
     gw.z = __reduce_max_sync(0xffffffffu, gw.z);
+    gw.w = __reduce_max_sync(0xffffffffu, gw.w);
     if ((tid & 31) == 0) gmax[tid >> 5] = gw;
   }
   __syncthreads();
   bool ok = true;
-  gm = make_uint4(0u, 0u, 0u, 0u);
+  uint4 gm = make_uint4(0u, 0u, 0u, 0u);
 #pragma unroll
   for (int t = 0; t < SLOTS; ++t) {
     const uint4 w = gmax[t];
-    if constexpr (EPB == 1) gm = make_uint4(max(gm.x, w.x), max(gm.y, w.y), max(gm.z, w.z), 0u);
+    if constexpr (EPB == 1) gm = make_uint4(max(gm.x, w.x), max(gm.y, w.y), max(gm.z, w.z), max(gm.w, w.w));
     else ok &= fx_in_range(w);
   }
-  if constexpr (EPB == 1) ok = fx_in_range(gm);
+  if constexpr (EPB == 1) {
+    ok = fx_in_range(gm);
+    ge = fx_exps(gm);
+  }
   if (!ok) return false;
 #pragma unroll
   for (int it = 0; it < IT; ++it) {
     const int l = tid + it * NT;
     if (l < nn) {
-      const uint4 g = EPB == 1 ? gm : gmax[l / NP];
-      const int E0 = (int)(g.x >> 20), E1 = (int)(g.y >> 20), E2 = (int)(g.z >> 20), o = fx_index<N>(l);
+      if constexpr (EPB > 1) gm = gmax[l / NP];
+      const FxExp e = fx_exps(gm);
+      int2* f = F + fx_index<N>(l);
+      // u in the unit that makes U u one of the momentum group's, p' in the group's own
+      int2 U[3], u[3];
 #pragma unroll
-      for (int f = 0; f < kLF; ++f) F[fx_slot(f) * FP + o] = fx_of(z[it].f[f], f <= lUz ? E0 : f <= lTyz ? E1 : E2);
+      for (int c = 0; c < 3; ++c) {
+        U[c] = fx_split(fx_of(z[it].U[c], e.U));
+        u[c] = fx_split(fx_of(z[it].u[c], max(e.m - e.U + 1022, kFxZero)));
+      }
+      const int2 th = fx_split(fx_of(z[it].th, max((int)(gm.z >> 20), kFxZero)));
+      const long long p = fx_of(z[it].pp, e.m);
+      f[sUx * FP] = U[0];
+      f[sUy * FP] = U[1];
+      f[sUz * FP] = U[2];
+      f[sTxx * FP] = fx_split(fx_mul(U[0], u[0]) + p);
+      f[sTyy * FP] = fx_split(fx_mul(U[1], u[1]) + p);
+      f[sTzz * FP] = fx_split(fx_mul(U[2], u[2]) + p);
+      f[sTxy * FP] = fx_split(fx_mul(U[0], u[1]));
+      f[sTxz * FP] = fx_split(fx_mul(U[0], u[2]));
+      f[sTyz * FP] = fx_split(fx_mul(U[1], u[2]));
+      f[sHx * FP] = fx_split(fx_mul(U[0], th));
+      f[sHy * FP] = fx_split(fx_mul(U[1], th));
+      f[sHz * FP] = fx_split(fx_mul(U[2], th));
     }
   }
   return true;
@@ -337,23 +400,21 @@ __device__ __forceinline__ bool fx_stage(const VolumeArgs& a, long long n0, int 
 // create_rhs of up to fx_rect_epb<N>() rectilinear elements e0 .. e0 + ne - 1
 // in fixed point: the residual sum_d K_d (D F_d) without its weight
 // w_i w_j w_k (which the update applies with the inverse mass).
-//   1. one thread per element node gathers the 12 flux fields; the largest
-//      magnitude of each equation group (mass: U; momentum: U u + p' I;
-//      theta: theta U) gives the group's exponent;
-//   2. the fields go to shared memory as fixed-point pairs;
-//   3. thread t takes line t of the 5 (N+1)^2 lines along x (equation
+//   1. the 12 flux fields go to shared memory (fx_stage);
+//   2. thread t takes line t of the 5 (N+1)^2 lines along x (equation
 //      v = t / (N+1)^2), then along y (fx_line), and leaves the derivatives in
 //      shared memory;
-//   4. it then takes its line along z, adds the x and y derivatives at the
+//   3. it then takes its line along z, adds the x and y derivatives at the
 //      line's nodes as integers and converts the sums to FP64, rounded once.
 // On 32^3 elements at N = 4: 0.529 ms as FP64 (its pipe 97% busy: 75
-// operations a node at 16 cycles a warp), 0.216 ms here; 19x23x17 at N = 6:
-// 0.460 -> 0.148 ms.  108 integer multiply-adds a thread keep their pipe 21%
-// busy; shared memory and the scattered gather (54% of the load/store unit's
-// wavefronts) and the 845 instructions a warp are what is left.  D in the
-// kernel parameters instead of global memory: 0.256 -> 0.226 ms; the z lines
-// finishing the nodes (10 shared accesses a node fewer, ten CTAs an SM
-// instead of eight): 0.226 -> 0.216 ms.
+// operations a node at 16 cycles a warp), 0.186 ms here; 19x23x17 at N = 6:
+// 0.460 -> 0.137 ms.  135 integer multiply-adds a thread keep their pipe a
+// quarter busy; shared memory, the scattered gather and the instructions
+// beside the products are what is left.  D in the kernel parameters instead
+// of global memory: 0.256 -> 0.226 ms; the z lines finishing the nodes (10
+// shared accesses a node fewer, ten CTAs an SM instead of eight): 0.226 ->
+// 0.216 ms; the products formed here from 8 gathered fields instead of 12
+// gathered fluxes: 0.216 -> 0.186 ms (and the update 0.199 -> 0.169 ms).
 template <int N>
 __device__ __forceinline__ void volume_fx_rect(const VolumeArgs& a, const int2* T, long long e0, int ne,
                                                unsigned char* smem_raw) {
@@ -364,8 +425,8 @@ __device__ __forceinline__ void volume_fx_rect(const VolumeArgs& a, const int2* 
   long long* part = reinterpret_cast<long long*>(F + kLF * FP);    // [2][5][FP]
   const int tid = threadIdx.x;
   const long long n0 = e0 * NP;
-  uint4 gm;
-  if (a.fxD == nullptr || !fx_stage<N, EPB, NT>(a, n0, ne * NP, gmax, F, gm)) {  // uniform over the CTA
+  FxExp ge;
+  if (a.fxD == nullptr || !fx_stage<N, EPB, NT>(a, n0, ne * NP, gmax, F, ge)) {  // uniform over the CTA
     for (int t = 0; t < ne; ++t) rect_plain<N>(a, e0 + t);
     return;
   }
@@ -394,8 +455,8 @@ __device__ __forceinline__ void volume_fx_rect(const VolumeArgs& a, const int2* 
     long long out[P];
     fx_line<N>(F + f * FP + base, B, T + 2 * M, out);
     const long long* o = part + v * FP + base;
-    if constexpr (EPB > 1) gm = gmax[el];
-    const int kexp = (int)((v == 0 ? gm.x : v == 4 ? gm.z : gm.y) >> 20) + a.fxexp;
+    if constexpr (EPB > 1) ge = fx_exps(gmax[el]);
+    const int kexp = (v == 0 ? ge.U : v == 4 ? ge.t : ge.m) + a.fxexp;
     double* re = static_cast<double*>(a.re) + v * a.Nl + n0 + el * NP + r;
 #pragma unroll
     for (int m = 0; m < P; ++m) re[m * PP] = fx_to_double(out[m] + o[m * B] + o[5 * FP + m * B], kexp);
@@ -407,8 +468,7 @@ __device__ __forceinline__ void volume_fx_rect(const VolumeArgs& a, const int2* 
 template <int N>
 __device__ __forceinline__ void nodal_plain(const VolumeArgs& a, long long e) {
   constexpr int P = N + 1, PP = P * P, NP = PP * P;
-  const long long Nl = a.Nl, Ng = a.Ng;
-  const double* w = static_cast<const double*>(a.prim);
+  const long long Nl = a.Nl;
   double* re = static_cast<double*>(a.re);
   const int4 eb = a.fxE[e];
   for (int l = threadIdx.x; l < NP; l += blockDim.x) {
@@ -421,13 +481,10 @@ __device__ __forceinline__ void nodal_plain(const VolumeArgs& a, long long e) {
         const int row = d == 0 ? i : d == 1 ? j : k, st = d == 0 ? 1 : d == 1 ? P : PP;
 #pragma unroll 1
         for (int c = 0; c < 3; ++c) {
-          // the field of equation v along c: U, the symmetric U u + p' I, theta U
-          const int p = v - 1, lo = min(p, c), hi = max(p, c);
-          const int s = v == 0 ? -1 : v == 4 ? 6 + c : lo == hi ? lo : lo + hi + 2;
-          const double* f = s < 0 ? a.q + (1 + c) * Ng : w + s * Ng;
           double x = 0.0;
 #pragma unroll 1
-          for (int m = 0; m < P; ++m) x = fma(a.D64[row * P + m], f[a.l2g[e * NP + l + (m - row) * st]], x);
+          for (int m = 0; m < P; ++m)
+            x = fma(a.D64[row * P + m], plain_flux(a, v, c, a.l2g[e * NP + l + (m - row) * st]), x);
           // eb.w: the metric terms of this element stayed doubles
           const long long at = (3 * d + c) * Nl + e * NP + l;
           double b = a.met64[at];
@@ -455,11 +512,12 @@ __device__ __forceinline__ void nodal_plain(const VolumeArgs& a, long long e) {
 // an inner one's).  The directions' sums are aligned by the exponents of their
 // rows, added as integers and rounded once.
 // On the 6x30x30x8 shell at N = 4: 2.068 ms as FP64 (225 operations a node, its
-// pipe 96% busy), 0.505 ms here; 21x17x13 at N = 3: 0.105 -> 0.037 ms.  The 405
-// integer multiply-adds a thread keep their pipe 40% busy and the 2200
-// instructions a warp 61% of the issue slots; both at 8 CTAs an SM (64
-// registers).  Going round all lines of a direction with a division per line
-// instead of one line per thread: 0.570 ms.
+// pipe 96% busy), 0.540 ms here; 21x17x13 at N = 3: 0.105 -> 0.039 ms.  The 430
+// integer multiply-adds a thread keep their pipe 40% busy and the 2300
+// instructions a warp 60% of the issue slots, at 8 CTAs an SM (64 registers).
+// With the fluxes formed in the update it took 0.505 ms, and the update 0.335
+// instead of 0.294 ms.  Going round all lines of a direction with a division per line
+// instead of one line per thread: 0.570 against 0.505 ms.
 template <int N>
 __device__ __forceinline__ void volume_fx_nodal(const VolumeArgs& a, const int2* T, long long e0, int ne,
                                                 unsigned char* smem_raw) {
@@ -474,8 +532,8 @@ __device__ __forceinline__ void volume_fx_nodal(const VolumeArgs& a, const int2*
   const int nel = EPB == 1 ? 0 : tid / NP;
   // the elements' metric exponents (w: the element takes plain FP64)
   const int4 eb = a.fxE[e0 + (node ? nel : 0)];
-  uint4 gm;
-  bool ok = fx_stage<N, EPB, NT>(a, n0, nn, gmax, F, gm);
+  FxExp ge;
+  bool ok = fx_stage<N, EPB, NT>(a, n0, nn, gmax, F, ge);
   if (__syncthreads_or(!ok || eb.w)) {
     for (int t = 0; t < ne; ++t) nodal_plain<N>(a, e0 + t);
     return;
@@ -510,17 +568,18 @@ __device__ __forceinline__ void volume_fx_nodal(const VolumeArgs& a, const int2*
     }
     __syncthreads();
     if (node) {
-      const int sh = min(xm - (d == 0 ? x0 : d == 1 ? x1 : x2), 63);
+      const int sh = min(xm + 1 - (d == 0 ? x0 : d == 1 ? x1 : x2), 62);
+      const long long half = 1ll << (sh - 1);  // the shift below rounds
       auto use = [&](long long& h, long long& m, int slot, int c) {
-        const long long x = S[slot * FP + at];
+        const long long x = S[slot * FP + at];  // (its low part from 0: the metric's has no mean)
         fx_mac(h, m, B[c], (int)((unsigned)x & kFxMask), (int)(x >> kFxBits));
       };
       auto eq = [&](int v, int s0, int s1, int s2) {
-        long long h = 0, m = kFxHalf;
+        long long h = half, m = kFxHalf;
         use(h, m, s0, 0);
         use(h, m, s1, 1);
         use(h, m, s2, 2);
-        sum[v] += (h + (m >> kFxBits)) >> sh;
+        sum[v] += (h + (m >> kFxBits)) >> sh;  // (nine products below 2^60, halved: below 2^63)
       };
       eq(0, sUx, sUy, sUz);
       eq(1, sTxx, sTxy, sTxz);
@@ -534,12 +593,12 @@ __device__ __forceinline__ void volume_fx_nodal(const VolumeArgs& a, const int2*
   direction(std::integral_constant<int, 1>());
   direction(std::integral_constant<int, 2>());
   if (!node) return;
-  if constexpr (EPB > 1) gm = gmax[nel];
-  const int kx = xm + a.fxexp + fx_weight_exp(a.fxw, l % P, (l / P) % P, l / PP);
+  if constexpr (EPB > 1) ge = fx_exps(gmax[nel]);
+  const int kx = xm + 1 + a.fxexp + fx_weight_exp(a.fxw, l % P, (l / P) % P, l / PP);
   double* re = static_cast<double*>(a.re) + n0 + tid;
 #pragma unroll
   for (int v = 0; v < 5; ++v)
-    re[v * Nl] = fx_to_double(sum[v], kx + (int)((v == 0 ? gm.x : v == 4 ? gm.z : gm.y) >> 20));
+    re[v * Nl] = fx_to_double(sum[v], kx + (v == 0 ? ge.U : v == 4 ? ge.t : ge.m));
 }
 
 // CTAs an SM holds at r registers a thread.
@@ -630,7 +689,7 @@ __global__ void __launch_bounds__(128)
     const int we = fx_weight_exp(fxw, l % P, (l / P) % P, l / (P * P));
     for (int t = 0; t < 9; ++t) {
       double* m = met + t * Nl + n0 + l;
-      *reinterpret_cast<int2*>(m) = fx_of(scalbn(*m, -we), E[t / 3]);
+      *reinterpret_cast<int2*>(m) = fx_split(fx_of(scalbn(*m, -we), E[t / 3]));
     }
   }
 }

@@ -185,8 +185,7 @@ __device__ __forceinline__ double eos_ratio(double x, const PrimArgs& a) {
 
 // Primitive fields of state (rp, U, Tp) at global node I (reference from a.ref):
 // rho = rho0 + rho', u = U / rho, theta = (Theta0 + Theta') / rho,
-// p' = p0 ((1 + Theta'/Theta0)^gamma - 1); in FP64 the flux components
-// built from them (the element kernels' gathered input).
+// p' = p0 ((1 + Theta'/Theta0)^gamma - 1).
 // F32: the FP32-mixed form (known at compile time, so that its kernels carry
 // none of the FP64 form's code); otherwise FP64 or pairs by a.precision.
 template <bool F32>
@@ -221,22 +220,13 @@ __device__ __forceinline__ void write_prim(const PrimArgs& a, long long I, doubl
     w[6 * Ng + I] = split64(Th * r);
     w[7 * Ng + I] = split64(p0 * eos_ratio(Tp * iTh0, a));
   } else {
-    // FP64: the nine flux components the element kernels need besides U,
-    // formed once per global node (kFlux64 slots): U_c u_c + p' on the
-    // diagonal, the symmetric U_c u_d once, and theta U = Theta u
     double* w = static_cast<double*>(a.prim);
     const double r = rcp64(rho);
-    const double ux = Ux * r, uy = Uy * r, uz = Uz * r;
-    const double pp = p0 * eos_ratio(Tp * iTh0, a);
-    w[I] = fma(Ux, ux, pp);
-    w[Ng + I] = fma(Uy, uy, pp);
-    w[2 * Ng + I] = fma(Uz, uz, pp);
-    w[3 * Ng + I] = Ux * uy;
-    w[4 * Ng + I] = Ux * uz;
-    w[5 * Ng + I] = Uy * uz;
-    w[6 * Ng + I] = Th * ux;
-    w[7 * Ng + I] = Th * uy;
-    w[8 * Ng + I] = Th * uz;
+    w[I] = Ux * r;
+    w[Ng + I] = Uy * r;
+    w[2 * Ng + I] = Uz * r;
+    w[3 * Ng + I] = Th * r;
+    w[4 * Ng + I] = p0 * eos_ratio(Tp * iTh0, a);
   }
   }
 }
@@ -254,7 +244,7 @@ struct NodeState {
 
 template <typename T>
 __device__ __forceinline__ NodeState<T> gather_node(const VolumeArgs& a, long long n) {
-  static_assert(sizeof(T) == 4, "the FP64 kernels gather flux components (gather_fluxes64)");
+  static_assert(sizeof(T) == 4, "the FP64 kernels gather with gather_node64");
   const int g = a.l2g[n];
   NodeState<T> z;
   {
@@ -325,29 +315,25 @@ __device__ __forceinline__ void stage_fluxes_affine(const VolumeArgs& a, long lo
 // symmetric part stored once), F_Theta = theta U.
 enum : int { lUx = 0, lUy, lUz, lTxx, lTyy, lTzz, lTxy, lTxz, lTyz, lHx, lHy, lHz, kLF };
 
-// The 12 flux fields at the global node behind element node n, FP64: U from
-// the state, the other nine as the update kernel formed them (write_prim).
-struct FluxState64 {
-  double f[kLF];
+// The state at the global node behind element node n, FP64: U from the state,
+// u, theta and p' as the update left them (write_prim).
+struct NodeState64 {
+  double U[3], u[3], th, pp;
 };
 
-__device__ __forceinline__ FluxState64 gather_fluxes64(const VolumeArgs& a, long long n) {
+__device__ __forceinline__ NodeState64 gather_node64(const VolumeArgs& a, long long n) {
   const long long Ng = a.Ng;
   const int g = a.l2g[n];
-  const double* w = static_cast<const double*>(a.prim);
-  FluxState64 z;
-  z.f[lUx] = a.q[Ng + g];
-  z.f[lUy] = a.q[2 * Ng + g];
-  z.f[lUz] = a.q[3 * Ng + g];
-  z.f[lTxx] = w[g];
-  z.f[lTyy] = w[Ng + g];
-  z.f[lTzz] = w[2 * Ng + g];
-  z.f[lTxy] = w[3 * Ng + g];
-  z.f[lTxz] = w[4 * Ng + g];
-  z.f[lTyz] = w[5 * Ng + g];
-  z.f[lHx] = w[6 * Ng + g];
-  z.f[lHy] = w[7 * Ng + g];
-  z.f[lHz] = w[8 * Ng + g];
+  const double* q = a.q + Ng + g;
+  const double* w = static_cast<const double*>(a.prim) + g;
+  NodeState64 z;
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    z.U[c] = q[c * Ng];
+    z.u[c] = w[c * Ng];
+  }
+  z.th = w[3 * Ng];
+  z.pp = w[4 * Ng];
   return z;
 }
 
@@ -386,11 +372,10 @@ __host__ __device__ constexpr int line_group() {
 //     face), so it moves out of the element kernel into the inverse mass of
 //     the DSS: the kernel writes sum_d K_d (D F_d), and the update multiplies
 //     the sum over element nodes by w_i w_j w_k / M (Minv_r) instead of 1 / M.
-// (3) Both forms: the nine flux components besides U (U_c u_c + p', the
-//     symmetric U_c u_d, Theta u) are formed once per global node by the
-//     update that writes the state (write_prim) and gathered as they are, not
-//     formed again at each of the global node's element nodes.
-// The contractions and the chain rule run in fixed point on the integer pipe
+// (3) Both forms: the products of the fluxes are formed in the element kernel,
+//     where one costs three integer multiply-adds; in the update, once per
+//     global node, the nine cost as many operations on the FP64 pipe.
+// The products, contractions and chain rule run in fixed point on the integer pipe
 // (fixed64.cuh); the pairs mode follows the same forms in float pairs.
 
 // create_rhs of element e in the FP32 form, organised by 1D lines of nodes

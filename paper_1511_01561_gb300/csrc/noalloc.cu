@@ -11,9 +11,9 @@
 // buffers with a scratch array that is part of the library image: nothing
 // is allocated per call.
 //
-// The array is 16 MiB.  Per global node the primitive fields take 72 bytes
-// (FP64: nine flux components), 32 (FP32-mixed) or 64 (FP64-pairs); per
-// element node the residuals take 40 (FP64, pairs) or 20 (FP32-mixed).  At
+// The array is 16 MiB.  Per global node 72 bytes are counted in FP64 (40 used),
+// 32 in FP32-mixed and 64 in FP64-pairs; per element node the residuals take 40
+// (FP64, pairs) or 20 (FP32-mixed).  At
 // N=4 the largest cubic boxes that fit are 11^3 elements in FP64, 12^3 in
 // the pairs mode and 15^3 in FP32-mixed.  Every GPU that loads this library keeps the array until the
 // process exits.  All calls share it: two calls whose work overlaps on the

@@ -502,8 +502,11 @@ int rhs_with_scratch(numa_ctx* c, const double* q_dev, double* r_dev, double* sc
   if (!c || !q_dev || !r_dev || !scratch) return NUMA_EINVAL;
   if (!c->bound) return fail(c, NUMA_ESTATE, "numa_rhs_static_scratch before numa_bind");
   if ((const void*)q_dev == (const void*)r_dev) return fail(c, NUMA_EINVAL, "q and r must not alias");
+  // the accepted sizes count 72, 32 or 64 bytes a node (FP64, FP32-mixed,
+  // pairs), at least what the kernels use
+  const size_t per_node = c->cfg.precision == NUMA_FP64 ? 72 : prim_bytes_per_node(c->cfg.precision);
   const size_t prim_bytes = align_up(prim_bytes_per_node(c->cfg.precision) * (size_t)c->mesh.Ng);
-  const size_t need = prim_bytes + residual_bytes(c->cfg, c->mesh);
+  const size_t need = align_up(per_node * (size_t)c->mesh.Ng) + residual_bytes(c->cfg, c->mesh);
   if (need > 8 * (size_t)scratch_doubles)
     return fail(c, NUMA_EINVAL, "mesh needs " + std::to_string(need) + " bytes of scratch; the static array holds " +
                                     std::to_string(8 * scratch_doubles));

@@ -47,14 +47,12 @@ bool init_state_host(const numa_config& c, const HostMesh& m, int kind, const do
 // Per-global-node primitive fields that the volume kernel gathers, written by
 // the stage update (or the primitive pass) for the state the next create_rhs
 // differentiates:
-//   FP64 mode  : double [9][Ng] = the flux components U_x u_x + p', U_y u_y + p',
-//                U_z u_z + p', U_x u_y, U_x u_z, U_y u_z, Theta u_x, Theta u_y,
-//                Theta u_z (U comes from q), formed once per global node
+//   FP64 mode  : double [5][Ng] = u_x, u_y, u_z, theta, p' (U comes from q)
 //   FP32 mode  : float  [Ng][8] = (U_x, U_y, U_z, u_x), (u_y, u_z, theta, p') per node,
 //                two float4 (one 32-byte sector per node for the gather)
 //   pairs mode : float2 [8][Ng] = the same eight, each as a (hi, lo) pair
 inline int prim_bytes_per_node(int precision) {
-  return precision == NUMA_FP32_MIXED ? 32 : precision == NUMA_FP64_PAIRS ? 64 : 72;
+  return precision == NUMA_FP32_MIXED ? 32 : precision == NUMA_FP64_PAIRS ? 64 : 40;
 }
 
 // Device workspace carved from the caller's buffer.
