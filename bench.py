@@ -92,7 +92,7 @@ NCU_TRAFFIC = {"kernels_sha256_16": "c162b3edd950e364", "workload": "bubble_32x3
                "volume_fp32_affine": 139.263232e6 + 49.111808e6}
 
 # the sources the element kernels with committed traffic figures are built from
-KERNEL_SOURCES = ["kernels_common.cuh", "volume_fp64.cu", "volume_fp32.cu", "volume_pairs.cu"]
+KERNEL_SOURCES = ["kernels_common.cuh", "fixed64.cuh", "volume_fp64.cu", "volume_fp32.cu"]
 
 
 def code_lines(text: str) -> list:

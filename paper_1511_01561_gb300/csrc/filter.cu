@@ -12,8 +12,7 @@ namespace numa {
 namespace {
 
 // One CTA per element, one thread per element node; three passes along xi,
-// eta and zeta through shared memory.  T = double: FP64 (also the pairs
-// mode); T = float: the FP32 form (the correction in FP32).
+// eta and zeta through shared memory.  T = double: FP64; T = float: the FP32 form (the correction in FP32).
 template <int N, typename T>
 __global__ void __launch_bounds__(((N + 1) * (N + 1) * (N + 1) + 31) / 32 * 32) filter_kernel(FilterArgs a) {
   constexpr int P = N + 1, NP = P * P * P;
@@ -61,10 +60,7 @@ __global__ void __launch_bounds__(((N + 1) * (N + 1) * (N + 1) + 31) / 32 * 32) 
   if (l < NP) {  // along zeta, then the weighted correction
     T jw;
     if (a.met64) jw = T(a.met64[9 * Nl + n]);
-    else if (a.met2) {
-      const float2 p = a.met2[9 * Nl + n];
-      jw = T(join64(Pairs{p.x, p.y}));
-    } else {
+    else {
       if constexpr (sizeof(T) == 8) jw = f2d(a.met32[9 * Nl + n]);
       else jw = a.met32[9 * Nl + n];
     }

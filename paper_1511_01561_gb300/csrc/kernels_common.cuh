@@ -69,94 +69,6 @@ __device__ __forceinline__ double rcp64(double x) {
   return fma(r, e, r);
 }
 
-// ---- FP64 accuracy on the FP32 units ("pairs") ------------------------------
-// A value is the unevaluated sum h + l of two floats with |l| <= ulp(h)/2:
-// about 48 significant bits.  Products are formed with the FMA-based exact
-// product split (Dekker's two-product via FMA), sums with Knuth's TwoSum.
-
-struct Pairs {
-  float h, l;
-};
-
-// double -> pair with integer operations: h = the double's top 24 significant
-// bits (truncated), l = the next bits rounded to a float.  Values outside
-// float range (below 2^-74 the low part vanishes; zeros excepted) take the
-// FP64 path.
-__device__ __noinline__ Pairs split64_rare(double x) {
-  const float h = __double2float_rn(x);
-  return {h, __double2float_rn(x - (double)h)};
-}
-
-__device__ __forceinline__ Pairs split64(double x) {
-  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
-  const int E = (int)((hi >> 20) & 0x7ffu);  // biased FP64 exponent
-  // zeros (common at walls and in a state at rest) inline, with their sign
-  if (((hi & 0x7fffffffu) | lo) == 0u) return {__uint_as_float(hi & 0x80000000u), 0.0f};
-  if (E < 1023 - 74 || E > 1023 + 127) return split64_rare(x);
-  const unsigned sign = hi & 0x80000000u;
-  const float h = __uint_as_float(sign | ((unsigned)(E - 1023 + 127) << 23) | ((hi & 0xfffffu) << 3) | (lo >> 29));
-  // remainder: the low 29 fraction bits, weight 2^(E-1023-52)
-  const unsigned rem = lo & 0x1fffffffu;
-  const float r = __uint2float_rn(rem);  // rounds 29 -> 24 bits
-  const float scale = __uint_as_float((unsigned)(E - 1023 - 52 + 127) << 23);
-  const float l = r * scale;
-  return {h, sign ? -l : l};
-}
-
-// (h, l) pair -> double (exact: the pair fits in 53 bits).
-__device__ __forceinline__ double join64(Pairs a) { return f2d(a.h) + f2d(a.l); }
-
-__device__ __forceinline__ Pairs pp_mul(Pairs a, Pairs b) {
-  const float p = a.h * b.h;
-  float e = fmaf(a.h, b.h, -p);
-  e = fmaf(a.h, b.l, e);
-  e = fmaf(a.l, b.h, e);
-  const float s = p + e;
-  return {s, e - (s - p)};
-}
-
-// Unnormalised accumulator (sh, sl) += a * b.
-__device__ __forceinline__ void pp_fma(float& sh, float& sl, Pairs a, Pairs b) {
-  const float p = a.h * b.h;
-  float e = fmaf(a.h, b.h, -p);
-  e = fmaf(a.h, b.l, e);
-  e = fmaf(a.l, b.h, e);
-  const float s = sh + p;
-  const float bb = s - sh;
-  const float t = (sh - (s - bb)) + (p - bb);
-  sl += t + e;
-  sh = s;
-}
-
-// First term of an accumulation: (sh, sl) = a * b.
-__device__ __forceinline__ void pp_first(float& sh, float& sl, Pairs a, Pairs b) {
-  sh = a.h * b.h;
-  float e = fmaf(a.h, b.h, -sh);
-  e = fmaf(a.h, b.l, e);
-  sl = fmaf(a.l, b.h, e);
-}
-
-__device__ __forceinline__ Pairs pp_norm(float sh, float sl) {
-  const float s = sh + sl;
-  return {s, sl - (s - sh)};
-}
-
-// a + b (TwoSum of the high parts, low parts added in).
-__device__ __forceinline__ Pairs pp_add(Pairs a, Pairs b) {
-  const float s = a.h + b.h;
-  const float bb = s - a.h;
-  const float t = (a.h - (s - bb)) + (b.h - bb) + (a.l + b.l);
-  return pp_norm(s, t);
-}
-
-// a - b (TwoSum of the high parts, low parts added in).
-__device__ __forceinline__ Pairs pp_sub(Pairs a, Pairs b) {
-  const float s = a.h - b.h;
-  const float bb = s - a.h;
-  const float t = (a.h - (s - bb)) - (b.h + bb) + (a.l - b.l);
-  return pp_norm(s, t);
-}
-
 __device__ __noinline__ double eos_ratio_rare(double x, double gamma) { return expm1(gamma * log1p(x)); }
 
 // (1+x)^gamma - 1 with full relative accuracy: the binomial series
@@ -187,7 +99,7 @@ __device__ __forceinline__ double eos_ratio(double x, const PrimArgs& a) {
 // rho = rho0 + rho', u = U / rho, theta = (Theta0 + Theta') / rho,
 // p' = p0 ((1 + Theta'/Theta0)^gamma - 1).
 // F32: the FP32-mixed form (known at compile time, so that its kernels carry
-// none of the FP64 form's code); otherwise FP64 or pairs by a.precision.
+// none of the FP64 form's code).
 template <bool F32>
 __device__ __forceinline__ void write_prim(const PrimArgs& a, long long I, double rp, double Ux, double Uy,
                                            double Uz, double Tp) {
@@ -205,21 +117,8 @@ __device__ __forceinline__ void write_prim(const PrimArgs& a, long long I, doubl
     w[2 * I + 1] = make_float4(Uyf * rf, Uzf * rf, (d2f(Th0) + d2f(Tp)) * rf, d2f(p0 * eos_ratio<true>(Tp * iTh0, a)));
     return;
   } else {
-  const double rho = rho0 + rp;
-  const double Th = Th0 + Tp;
-  if (a.precision == NUMA_FP64_PAIRS) {
-    // FP64 primitives, stored as (hi, lo) pairs for the element kernel
-    Pairs* w = static_cast<Pairs*>(a.prim);
-    const double r = rcp64(rho);
-    w[I] = split64(Ux);
-    w[Ng + I] = split64(Uy);
-    w[2 * Ng + I] = split64(Uz);
-    w[3 * Ng + I] = split64(Ux * r);
-    w[4 * Ng + I] = split64(Uy * r);
-    w[5 * Ng + I] = split64(Uz * r);
-    w[6 * Ng + I] = split64(Th * r);
-    w[7 * Ng + I] = split64(p0 * eos_ratio(Tp * iTh0, a));
-  } else {
+    const double rho = rho0 + rp;
+    const double Th = Th0 + Tp;
     double* w = static_cast<double*>(a.prim);
     const double r = rcp64(rho);
     w[I] = Ux * r;
@@ -227,7 +126,6 @@ __device__ __forceinline__ void write_prim(const PrimArgs& a, long long I, doubl
     w[2 * Ng + I] = Uz * r;
     w[3 * Ng + I] = Th * r;
     w[4 * Ng + I] = p0 * eos_ratio(Tp * iTh0, a);
-  }
   }
 }
 
@@ -310,7 +208,7 @@ __device__ __forceinline__ void stage_fluxes_affine(const VolumeArgs& a, long lo
   }
 }
 
-// The 12 flux fields of the FP64 (and pairs) kernels: F_rho = U, F_U =
+// The 12 flux fields of the FP64 kernels: F_rho = U, F_U =
 // U (x) u + p' I with the pressure in the diagonal components (the
 // symmetric part stored once), F_Theta = theta U.
 enum : int { lUx = 0, lUy, lUz, lTxx, lTyy, lTzz, lTxy, lTxz, lTyz, lHx, lHy, lHz, kLF };
@@ -375,8 +273,8 @@ __host__ __device__ constexpr int line_group() {
 // (3) Both forms: the products of the fluxes are formed in the element kernel,
 //     where one costs three integer multiply-adds; in the update, once per
 //     global node, the nine cost as many operations on the FP64 pipe.
-// The products, contractions and chain rule run in fixed point on the integer pipe
-// (fixed64.cuh); the pairs mode follows the same forms in float pairs.
+// The products, contractions and chain rule run in fixed point on the integer
+// pipe (fixed64.cuh).
 
 // create_rhs of element e in the FP32 form, organised by 1D lines of nodes
 // (Eq. 5 is a contraction along xi, eta and zeta).  Thread t < 3W takes one
@@ -539,315 +437,18 @@ __device__ __forceinline__ void volume_element_lines(const VolumeArgs& a, long l
   }
 }
 
-// create_rhs of element e in the pairs mode: the steps of
-// the FP64 per-node form (12 flux fields with the pressure on the diagonal,
-// metric terms pre-multiplied by -Jw: rows 0..8 of met2 hold -Jw dxi_d/dx_c
-// for this form), every value and product carried as a (hi, lo) float pair.
-// The fluxes are differentiated less their values at element node 0, and
-// p' enters less its node-0 value, so that the 48-bit products round at the
-// level of the fields' variation, not of their common level.  smem_raw
-// holds 12 (N+1)^3 + (N+1)^2 + 12 pairs.
+// Dynamic shared memory of one element: the staged fluxes, then the partial sums.
 template <int N>
-__device__ __forceinline__ void volume_element_pairs(const VolumeArgs& a, long long e, unsigned char* smem_raw) {
-  constexpr int P = N + 1, NP = P * P * P;
-  Pairs* F = reinterpret_cast<Pairs*>(smem_raw);  // [kLF][NP]
-  Pairs* Ds = F + kLF * NP;                         // [P][P]
-  Pairs* base = Ds + P * P;                         // [kLF]: the fluxes at element node 0
-  const Pairs* Dg = reinterpret_cast<const Pairs*>(a.D2);
-  const Pairs* met = reinterpret_cast<const Pairs*>(a.met2);
-  const int l = threadIdx.x;
-  for (int t = l; t < P * P; t += blockDim.x) Ds[t] = Dg[t];
-  const long long e0 = e * NP, n = e0 + l;
-  const long long Ng = a.Ng, Nl = a.Nl;
-  if (l < NP) {
-    const int g = a.l2g[n];
-    const Pairs* w = static_cast<const Pairs*>(a.prim);
-    const Pairs Ux = w[g], Uy = w[Ng + g], Uz = w[2 * Ng + g];
-    const Pairs ux = w[3 * Ng + g], uy = w[4 * Ng + g], uz = w[5 * Ng + g];
-    const Pairs th = w[6 * Ng + g];
-    const Pairs pp = pp_sub(w[7 * Ng + g], w[7 * Ng + a.l2g[e0]]);
-    Pairs v[kLF];
-    v[lUx] = Ux;
-    v[lUy] = Uy;
-    v[lUz] = Uz;
-    v[lTxx] = pp_add(pp_mul(Ux, ux), pp);
-    v[lTyy] = pp_add(pp_mul(Uy, uy), pp);
-    v[lTzz] = pp_add(pp_mul(Uz, uz), pp);
-    v[lTxy] = pp_mul(Ux, uy);
-    v[lTxz] = pp_mul(Ux, uz);
-    v[lTyz] = pp_mul(Uy, uz);
-    v[lHx] = pp_mul(th, Ux);
-    v[lHy] = pp_mul(th, Uy);
-    v[lHz] = pp_mul(th, Uz);
-#pragma unroll
-    for (int f = 0; f < kLF; ++f) F[f * NP + l] = v[f];
-    if (l == 0) {
-#pragma unroll
-      for (int f = 0; f < kLF; ++f) base[f] = v[f];
-    }
-  }
-  __syncthreads();
-  // D annihilates constants, so the derivatives of F and of F - F(node 0)
-  // are the same; the differences keep their full relative accuracy in the
-  // contractions (no cancellation against the fields' common level).  Each
-  // thread rewrites only its own node's entries.
-  if (l < NP) {
-#pragma unroll
-    for (int f = 0; f < kLF; ++f) F[f * NP + l] = pp_sub(F[f * NP + l], base[f]);
-  }
-  __syncthreads();
-  if (l >= NP) return;
-  const int i = l % P, j = (l / P) % P, k = l / (P * P);
-  Pairs B[9];  // -Jw dxi_d/dx_c at this node, [3d + c]
-#pragma unroll
-  for (int t = 0; t < 9; ++t) B[t] = met[t * Nl + n];
-  const int bx = P * (j + P * k), by = i + P * P * k, bz = i + P * j;
-  // reference-space derivatives (Eq. 5) as normalised pairs
-  auto dref = [&](int f, Pairs& s0, Pairs& s1, Pairs& s2) {
-    const Pairs* Ff = F + f * NP;
-    float h0, l0, h1, l1, h2, l2;
-    pp_first(h0, l0, Ds[i * P], Ff[bx]);
-    pp_first(h1, l1, Ds[j * P], Ff[by]);
-    pp_first(h2, l2, Ds[k * P], Ff[bz]);
-#pragma unroll
-    for (int m = 1; m < P; ++m) {
-      pp_fma(h0, l0, Ds[i * P + m], Ff[bx + m]);
-      pp_fma(h1, l1, Ds[j * P + m], Ff[by + P * m]);
-      pp_fma(h2, l2, Ds[k * P + m], Ff[bz + P * P * m]);
-    }
-    s0 = pp_norm(h0, l0);
-    s1 = pp_norm(h1, l1);
-    s2 = pp_norm(h2, l2);
-  };
-  // chain rule into the weighted divergence: (dh, dl) += -Jw d/dx_c of a field
-  auto phys = [&](float& dh, float& dl, bool first, int c, Pairs s0, Pairs s1, Pairs s2) {
-    if (first) pp_first(dh, dl, s0, B[c]);
-    else pp_fma(dh, dl, s0, B[c]);
-    pp_fma(dh, dl, s1, B[3 + c]);
-    pp_fma(dh, dl, s2, B[6 + c]);
-  };
-  Pairs s0, s1, s2;
-  float rh, rl, xh, xl, yh, yl, zh, zl, th_, tl;
-  dref(lUx, s0, s1, s2); phys(rh, rl, true, 0, s0, s1, s2);
-  dref(lUy, s0, s1, s2); phys(rh, rl, false, 1, s0, s1, s2);
-  dref(lUz, s0, s1, s2); phys(rh, rl, false, 2, s0, s1, s2);
-  dref(lTxx, s0, s1, s2); phys(xh, xl, true, 0, s0, s1, s2);
-  dref(lTyy, s0, s1, s2); phys(yh, yl, true, 1, s0, s1, s2);
-  dref(lTzz, s0, s1, s2); phys(zh, zl, true, 2, s0, s1, s2);
-  dref(lTxy, s0, s1, s2); phys(xh, xl, false, 1, s0, s1, s2); phys(yh, yl, false, 0, s0, s1, s2);
-  dref(lTxz, s0, s1, s2); phys(xh, xl, false, 2, s0, s1, s2); phys(zh, zl, false, 0, s0, s1, s2);
-  dref(lTyz, s0, s1, s2); phys(yh, yl, false, 2, s0, s1, s2); phys(zh, zl, false, 1, s0, s1, s2);
-  dref(lHx, s0, s1, s2); phys(th_, tl, true, 0, s0, s1, s2);
-  dref(lHy, s0, s1, s2); phys(th_, tl, false, 1, s0, s1, s2);
-  dref(lHz, s0, s1, s2); phys(th_, tl, false, 2, s0, s1, s2);
-  // the weighted residual -Jw div F of Eq. 4 in FP64 (the pair is exact in a double)
-  double* re = static_cast<double*>(a.re);
-  re[n] = join64(pp_norm(rh, rl));
-  re[Nl + n] = join64(pp_norm(xh, xl));
-  re[2 * Nl + n] = join64(pp_norm(yh, yl));
-  re[3 * Nl + n] = join64(pp_norm(zh, zl));
-  re[4 * Nl + n] = join64(pp_norm(th_, tl));
-}
-
-// create_rhs of an affine element in the pairs mode: the contravariant
-// fluxes of stage_fluxes_affine in (hi, lo) float pairs, less their values
-// at element node 0, and three contractions with D per equation.  smem_raw
-// holds 15 (N+1)^3 + (N+1)^2 + 15 pairs.
-template <int N>
-__device__ __forceinline__ void volume_element_pairs_affine(const VolumeArgs& a, long long e, unsigned char* smem_raw) {
-  constexpr int P = N + 1, NP = P * P * P;
-  Pairs* G = reinterpret_cast<Pairs*>(smem_raw);  // [15][NP]
-  Pairs* Ds = G + 15 * NP;                         // [P][P]
-  Pairs* base = Ds + P * P;                        // [15]: the fluxes at element node 0
-  const Pairs* Dg = reinterpret_cast<const Pairs*>(a.D2);
-  const Pairs* met = reinterpret_cast<const Pairs*>(a.met2);
-  const int l = threadIdx.x;
-  for (int t = l; t < P * P; t += blockDim.x) Ds[t] = Dg[t];
-  const long long e0 = e * NP, n = e0 + l;
-  const long long Ng = a.Ng, Nl = a.Nl;
-  if (l < NP) {
-    Pairs B[9];  // the element's metric terms, at its first node
-#pragma unroll
-    for (int t = 0; t < 9; ++t) B[t] = met[t * Nl + e0];
-    const int g = a.l2g[n];
-    const Pairs* w = static_cast<const Pairs*>(a.prim);
-    const Pairs Ux = w[g], Uy = w[Ng + g], Uz = w[2 * Ng + g];
-    const Pairs ux = w[3 * Ng + g], uy = w[4 * Ng + g], uz = w[5 * Ng + g];
-    const Pairs th = w[6 * Ng + g];
-    // p' relative to its value at element node 0: B_dc p'(node 0) is constant
-    // over the element and D annihilates it, and the difference keeps the
-    // pressure term's rounding at the level of its variation, not of p'
-    const Pairs pp = pp_sub(w[7 * Ng + g], w[7 * Ng + a.l2g[e0]]);
-    Pairs v[15];
-#pragma unroll
-    for (int d = 0; d < 3; ++d) {
-      float h, lo;
-      pp_first(h, lo, B[3 * d], ux);
-      pp_fma(h, lo, B[3 * d + 1], uy);
-      pp_fma(h, lo, B[3 * d + 2], uz);
-      const Pairs ud = pp_norm(h, lo);  // B_d . u
-      pp_first(h, lo, B[3 * d], Ux);
-      pp_fma(h, lo, B[3 * d + 1], Uy);
-      pp_fma(h, lo, B[3 * d + 2], Uz);
-      const Pairs Gr = pp_norm(h, lo);  // B_d . U
-      v[d] = Gr;
-      pp_first(h, lo, Ux, ud);
-      pp_fma(h, lo, B[3 * d], pp);
-      v[3 + d] = pp_norm(h, lo);
-      pp_first(h, lo, Uy, ud);
-      pp_fma(h, lo, B[3 * d + 1], pp);
-      v[6 + d] = pp_norm(h, lo);
-      pp_first(h, lo, Uz, ud);
-      pp_fma(h, lo, B[3 * d + 2], pp);
-      v[9 + d] = pp_norm(h, lo);
-      v[12 + d] = pp_mul(th, Gr);
-    }
-#pragma unroll
-    for (int f = 0; f < 15; ++f) G[f * NP + l] = v[f];
-    if (l == 0) {
-#pragma unroll
-      for (int f = 0; f < 15; ++f) base[f] = v[f];
-    }
-  }
-  __syncthreads();
-  // D annihilates constants: differentiate G - G(node 0), as in the per-node form
-  if (l < NP) {
-#pragma unroll
-    for (int f = 0; f < 15; ++f) G[f * NP + l] = pp_sub(G[f * NP + l], base[f]);
-  }
-  __syncthreads();
-  if (l >= NP) return;
-  const int i = l % P, j = (l / P) % P, k = l / (P * P);
-  const int bx = P * (j + P * k), by = i + P * P * k, bz = i + P * j;
-  const Pairs jw = met[9 * Nl + n];
-  double* re = static_cast<double*>(a.re);
-#pragma unroll
-  for (int v = 0; v < 5; ++v) {
-    const Pairs* g0 = G + (3 * v) * NP;
-    const Pairs* g1 = g0 + NP;
-    const Pairs* g2 = g1 + NP;
-    float h, lo;
-    pp_first(h, lo, Ds[i * P], g0[bx]);
-#pragma unroll
-    for (int m = 1; m < P; ++m) pp_fma(h, lo, Ds[i * P + m], g0[bx + m]);
-#pragma unroll
-    for (int m = 0; m < P; ++m) pp_fma(h, lo, Ds[j * P + m], g1[by + P * m]);
-#pragma unroll
-    for (int m = 0; m < P; ++m) pp_fma(h, lo, Ds[k * P + m], g2[bz + P * P * m]);
-    re[v * Nl + n] = -join64(pp_mul(jw, pp_norm(h, lo)));
-  }
-}
-
-// create_rhs of a rectilinear affine element in the pairs mode: the folded
-// form of volume_fx_rect (K_d D per direction, the weight w_i w_j w_k
-// left to the update's inverse mass, no metric or Jw per node) in (hi, lo)
-// float pairs.  The 12 unweighted fields are differentiated less their values at
-// element node 0 (K_d D annihilates constants as D does), and p' enters less
-// its node-0 value (as in volume_element_pairs_affine).  smem_raw holds
-// 12 (N+1)^3 + 3 (N+1)^2 + 12 pairs.
-template <int N>
-__device__ __forceinline__ void volume_element_pairs_rect(const VolumeArgs& a, long long e, unsigned char* smem_raw) {
-  constexpr int P = N + 1, PP = P * P, NP = PP * P;
-  Pairs* F = reinterpret_cast<Pairs*>(smem_raw);  // [kLF][NP]
-  Pairs* Dk = F + kLF * NP;                        // [3][P][P]: K_d D
-  Pairs* base = Dk + 3 * PP;                       // [kLF]: the fluxes at element node 0
-  const int l = threadIdx.x;
-  for (int t = l; t < 3 * PP; t += blockDim.x) {
-    const int d = t / PP;
-    Dk[t] = split64(a.affk[d * (long long)a.Ne + e] * a.D64[t - d * PP]);
-  }
-  const long long e0 = e * NP, n = e0 + l;
-  const long long Ng = a.Ng, Nl = a.Nl;
-  if (l < NP) {
-    const int g = a.l2g[n];
-    const Pairs* w = static_cast<const Pairs*>(a.prim);
-    const Pairs Ux = w[g], Uy = w[Ng + g], Uz = w[2 * Ng + g];
-    const Pairs ux = w[3 * Ng + g], uy = w[4 * Ng + g], uz = w[5 * Ng + g];
-    const Pairs th = w[6 * Ng + g];
-    const Pairs pp = pp_sub(w[7 * Ng + g], w[7 * Ng + a.l2g[e0]]);
-    Pairs v[kLF];
-    v[lUx] = Ux;
-    v[lUy] = Uy;
-    v[lUz] = Uz;
-    v[lTxx] = pp_add(pp_mul(Ux, ux), pp);
-    v[lTyy] = pp_add(pp_mul(Uy, uy), pp);
-    v[lTzz] = pp_add(pp_mul(Uz, uz), pp);
-    v[lTxy] = pp_mul(Ux, uy);
-    v[lTxz] = pp_mul(Ux, uz);
-    v[lTyz] = pp_mul(Uy, uz);
-    v[lHx] = pp_mul(th, Ux);
-    v[lHy] = pp_mul(th, Uy);
-    v[lHz] = pp_mul(th, Uz);
-#pragma unroll
-    for (int f = 0; f < kLF; ++f) F[f * NP + l] = v[f];
-    if (l == 0) {
-#pragma unroll
-      for (int f = 0; f < kLF; ++f) base[f] = v[f];
-    }
-  }
-  __syncthreads();
-  if (l < NP) {
-#pragma unroll
-    for (int f = 0; f < kLF; ++f) F[f * NP + l] = pp_sub(F[f * NP + l], base[f]);
-  }
-  __syncthreads();
-  if (l >= NP) return;
-  const int i = l % P, j = (l / P) % P, k = l / PP;
-  const int bx = P * (j + P * k), by = i + PP * k, bz = i + P * j;
-  double* re = static_cast<double*>(a.re);
-  auto div = [&](int fx, int fy, int fz) {
-    const Pairs* gx = F + fx * NP;
-    const Pairs* gy = F + fy * NP;
-    const Pairs* gz = F + fz * NP;
-    float h, lo;
-    pp_first(h, lo, Dk[i * P], gx[bx]);
-#pragma unroll
-    for (int m = 1; m < P; ++m) pp_fma(h, lo, Dk[i * P + m], gx[bx + m]);
-#pragma unroll
-    for (int m = 0; m < P; ++m) pp_fma(h, lo, Dk[PP + j * P + m], gy[by + P * m]);
-#pragma unroll
-    for (int m = 0; m < P; ++m) pp_fma(h, lo, Dk[2 * PP + k * P + m], gz[bz + PP * m]);
-    return join64(pp_norm(h, lo));
-  };
-  re[n] = div(lUx, lUy, lUz);
-  re[Nl + n] = div(lTxx, lTxy, lTxz);
-  re[2 * Nl + n] = div(lTxy, lTyy, lTyz);
-  re[3 * Nl + n] = div(lTxz, lTyz, lTzz);
-  re[4 * Nl + n] = div(lHx, lHy, lHz);
-}
-
-// Dynamic shared memory of one element: the staged fluxes, D and (pairs
-// mode) the node-0 base values.
-template <int N, typename T, bool AFF>
 constexpr size_t element_smem_bytes() {
   constexpr int P = N + 1, NP = P * P * P;
-  if constexpr (std::is_same<T, float>::value) return sizeof(float) * (kNF > 15 ? kNF : 15) * NP;
-  if constexpr (AFF) return sizeof(T) * (15 * NP + P * P + 15);
-  return sizeof(T) * (kLF * NP + P * P + kLF);
+  return sizeof(float) * (kNF > 15 ? kNF : 15) * NP;
 }
 
-// Element kernel of one precision; AFF selects the affine-element form.
-template <int N, typename T, bool AFF>
-__device__ __forceinline__ void element_rhs(const VolumeArgs& a, long long e, unsigned char* smem_raw) {
-  if constexpr (std::is_same<T, Pairs>::value) {
-    if constexpr (AFF) {
-      // uniform over the CTA: rectilinear elements take the folded form
-      if (a.affine == 2) volume_element_pairs_rect<N>(a, e, smem_raw);
-      else volume_element_pairs_affine<N>(a, e, smem_raw);
-    } else {
-      volume_element_pairs<N>(a, e, smem_raw);
-    }
-  } else {
-    static_assert(std::is_same<T, float>::value, "the FP64 element kernels are in fixed64.cuh");
-    volume_element_lines<N, AFF>(a, e, smem_raw);
-  }
-}
-
-template <int N, typename T, bool AFF>
+template <int N, bool AFF>
 __global__ void __launch_bounds__(((N + 1) * (N + 1) * (N + 1) + 31) / 32 * 32)
     volume_kernel(VolumeArgs a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  element_rhs<N, T, AFF>(a, a.ebeg + (long long)blockIdx.x, smem_raw);
+  volume_element_lines<N, AFF>(a, a.ebeg + (long long)blockIdx.x, smem_raw);
 }
 
 template <typename RT>
@@ -1132,7 +733,7 @@ __device__ __forceinline__ int ragged_find(const long long* prefix, int n, long 
   return lo;
 }
 
-template <int N, typename T, bool AFF>
+template <int N, bool AFF>
 __global__ void __launch_bounds__(((N + 1) * (N + 1) * (N + 1) + 31) / 32 * 32)
     volume_ragged(const MemberDesc* __restrict__ d, const RaggedGroup* __restrict__ g) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -1149,7 +750,7 @@ __global__ void __launch_bounds__(((N + 1) * (N + 1) * (N + 1) + 31) / 32 * 32)
     __syncthreads();
     // (uniform across the CTA) guard against a table that disagrees with the member
     if (s_m >= 0 && s_m < kMaxMembers && s_e >= 0 && s_e < d[s_m].va.Ne)
-      element_rhs<N, T, AFF>(d[s_m].va, s_e, smem_raw);
+      volume_element_lines<N, AFF>(d[s_m].va, s_e, smem_raw);
     __syncthreads();
   }
 }
@@ -1235,34 +836,34 @@ class DeviceInts {
   std::atomic<int> v_[64] = {};
 };
 
-template <int N, typename T, bool AFF>
+template <int N, bool AFF>
 cudaError_t launch_volume_t(const VolumeArgs& a, cudaStream_t s) {
   constexpr int P = N + 1, NP = P * P * P;
   constexpr int NT = (NP + 31) / 32 * 32;
-  const size_t smem = element_smem_bytes<N, T, AFF>();
+  const size_t smem = element_smem_bytes<N>();
   static DeviceFlags attr_set;
   if (!attr_set.has()) {
     cudaError_t e =
-        cudaFuncSetAttribute(volume_kernel<N, T, AFF>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        cudaFuncSetAttribute(volume_kernel<N, AFF>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     attr_set.set();
   }
   if (a.ecnt <= 0) return cudaSuccess;
-  volume_kernel<N, T, AFF><<<a.ecnt, NT, smem, s>>>(a);
+  volume_kernel<N, AFF><<<a.ecnt, NT, smem, s>>>(a);
   return cudaGetLastError();
 }
 
-template <typename T, bool AFF>
+template <bool AFF>
 cudaError_t launch_volume_p(int N, const VolumeArgs& a, cudaStream_t s) {
   switch (N) {
-    case 1: return launch_volume_t<1, T, AFF>(a, s);
-    case 2: return launch_volume_t<2, T, AFF>(a, s);
-    case 3: return launch_volume_t<3, T, AFF>(a, s);
-    case 4: return launch_volume_t<4, T, AFF>(a, s);
-    case 5: return launch_volume_t<5, T, AFF>(a, s);
-    case 6: return launch_volume_t<6, T, AFF>(a, s);
-    case 7: return launch_volume_t<7, T, AFF>(a, s);
-    case 8: return launch_volume_t<8, T, AFF>(a, s);
+    case 1: return launch_volume_t<1, AFF>(a, s);
+    case 2: return launch_volume_t<2, AFF>(a, s);
+    case 3: return launch_volume_t<3, AFF>(a, s);
+    case 4: return launch_volume_t<4, AFF>(a, s);
+    case 5: return launch_volume_t<5, AFF>(a, s);
+    case 6: return launch_volume_t<6, AFF>(a, s);
+    case 7: return launch_volume_t<7, AFF>(a, s);
+    case 8: return launch_volume_t<8, AFF>(a, s);
     default: return cudaErrorInvalidValue;
   }
 }
@@ -1300,25 +901,25 @@ cudaError_t launch_persistent(K kernel, int threads, size_t smem, DeviceInts& gr
   return cudaGetLastError();
 }
 
-template <int N, typename T, bool AFF>
+template <int N, bool AFF>
 cudaError_t launch_volume_ragged_t(const MemberDesc* d, const RaggedGroup* g, cudaStream_t s) {
   constexpr int P = N + 1, NP = P * P * P;
   static DeviceInts grids;  // per device, set up at its first launch there
-  return launch_persistent(volume_ragged<N, T, AFF>, (NP + 31) / 32 * 32, element_smem_bytes<N, T, AFF>(), grids, d,
+  return launch_persistent(volume_ragged<N, AFF>, (NP + 31) / 32 * 32, element_smem_bytes<N>(), grids, d,
                            g, s);
 }
 
-template <typename T, bool AFF>
+template <bool AFF>
 cudaError_t launch_volume_ragged_p(int N, const MemberDesc* d, const RaggedGroup* g, cudaStream_t s) {
   switch (N) {
-    case 1: return launch_volume_ragged_t<1, T, AFF>(d, g, s);
-    case 2: return launch_volume_ragged_t<2, T, AFF>(d, g, s);
-    case 3: return launch_volume_ragged_t<3, T, AFF>(d, g, s);
-    case 4: return launch_volume_ragged_t<4, T, AFF>(d, g, s);
-    case 5: return launch_volume_ragged_t<5, T, AFF>(d, g, s);
-    case 6: return launch_volume_ragged_t<6, T, AFF>(d, g, s);
-    case 7: return launch_volume_ragged_t<7, T, AFF>(d, g, s);
-    case 8: return launch_volume_ragged_t<8, T, AFF>(d, g, s);
+    case 1: return launch_volume_ragged_t<1, AFF>(d, g, s);
+    case 2: return launch_volume_ragged_t<2, AFF>(d, g, s);
+    case 3: return launch_volume_ragged_t<3, AFF>(d, g, s);
+    case 4: return launch_volume_ragged_t<4, AFF>(d, g, s);
+    case 5: return launch_volume_ragged_t<5, AFF>(d, g, s);
+    case 6: return launch_volume_ragged_t<6, AFF>(d, g, s);
+    case 7: return launch_volume_ragged_t<7, AFF>(d, g, s);
+    case 8: return launch_volume_ragged_t<8, AFF>(d, g, s);
     default: return cudaErrorInvalidValue;
   }
 }

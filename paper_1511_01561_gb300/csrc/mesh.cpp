@@ -365,7 +365,7 @@ bool build_host_mesh(const numa_config& c, HostMesh& m, std::string& err) {
   lobatto(m.N, m.xi, m.w);
   diffmat(m.xi, m.D);
   if (c.precision != NUMA_FP32_MIXED) {
-    // FP64 and pairs: D correctly rounded and with D_{N-i,N-j} = -D_ij exactly,
+    // FP64: D correctly rounded and with D_{N-i,N-j} = -D_ij exactly,
     // as the even/odd tables of the fixed-point kernels hold it; the metric
     // terms below come from the D the fields are differentiated with, so that
     // its rounding cancels between them on smooth fields

@@ -63,8 +63,6 @@ VolumeArgs volume_args(const numa_ctx* c, const double* q, const void* prim, voi
   a.met32 = c->L.met32;
   a.D64 = c->L.D64;
   a.D32 = c->L.D32;
-  a.met2 = c->L.met2;
-  a.D2 = c->L.D2;
   a.re = re;
   a.affk = c->L.affk;
   a.fxD = c->fx ? c->L.fxD : nullptr;
@@ -82,8 +80,8 @@ VolumeArgs volume_args(const numa_ctx* c, const double* q, const void* prim, voi
   return a;
 }
 
-// Element-kernel form of a bound context: 2 the rectilinear form (FP64,
-// pairs), 1 the general affine form (pairs, FP32-mixed), 0 the per-node form
+// Element-kernel form of a bound context: 2 the rectilinear form (FP64),
+// 1 the general affine form (FP32-mixed), 0 the per-node form
 // (any element; FP64 takes it on affine elements that are not rectilinear).
 int volume_form(const numa_ctx* c) {
   if (!affine_elements(c->cfg)) return 0;
@@ -143,7 +141,6 @@ FilterArgs filter_args(const numa_ctx* c) {
   a.F = c->cfg.precision == NUMA_FP32_MIXED ? (const void*)c->L.F32 : (const void*)c->L.F64;
   a.met64 = c->L.met64;
   a.met32 = c->L.met32;
-  a.met2 = c->L.met2;
   a.re = c->L.re;
   a.Ng = c->mesh.Ng;
   a.Nl = c->mesh.Nl;
@@ -251,8 +248,7 @@ int imex_prepare(numa_ctx* c, double dt) {
 }
 
 // One 1D-IMEX step on stream s (imex_prepare(dt) done): create_rhs on q^n,
-// DSS + M^-1 into R (the primitive buffer, 40 B per node in FP64 and 64 B in
-// the pairs mode, free once the element kernel has read it; R[v][g] lies
+// DSS + M^-1 into R (in the primitive buffer, free once the element kernel has read it; R[v][g] lies
 // inside node g's own primitive slots), then the column kernel, which leaves q^{n+1} in q,
 // the filtered q^n in qs and the primitive fields of q^{n+1}.  The start
 // step (no q^{n-1}) uses dt/2 factors, q* = q^0 + dt R and no filter.
@@ -376,8 +372,7 @@ cudaError_t enqueue_rk_step(numa_ctx* c, double dt, cudaStream_t s, cudaEvent_t*
 // slabs <= k and the element slab k reads only node slabs k and k + 1.
 // `want` slabs (0: three for FP32-mixed meshes of 2^18 or more global nodes,
 // where the memory-bound element kernel and the FP64-bound update overlap;
-// in FP64 and the pairs mode both kernels need the FP64 pipe, or the FP32
-// pipe beside it, and the pipeline measured no gain, so none by default).
+// in FP64 the pipeline measured no gain, so none by default).
 SlabPlan plan_slabs(const numa_config& c, const HostMesh& m, int want) {
   SlabPlan P;
   if (c.mesh_kind != NUMA_MESH_BOX || c.storage != NUMA_STORAGE_CG || c.periodic[2]) return P;
@@ -457,7 +452,6 @@ size_t layout_workspace(const numa_config& c, const HostMesh& m, char* base, Dev
   d.prim = take(prim_bytes_per_node(c.precision) * Ng);
   d.re = take(residual_bytes(c, m));
   if (c.precision == NUMA_FP32_MIXED) d.met32 = (float*)take(10 * Nl * 4);
-  else if (c.precision == NUMA_FP64_PAIRS) d.met2 = (float2*)take(10 * Nl * 8);
   else d.met64 = (double*)take(10 * Nl * 8);
   d.l2g = (int32_t*)take(Nl * 4);
   d.csr_off = (int32_t*)take((Ng + 1) * 4);
@@ -471,7 +465,7 @@ size_t layout_workspace(const numa_config& c, const HostMesh& m, char* base, Dev
     d.nrm = (double*)take(3 * Ng * 8);
   }
   d.D64 = (double*)take(PP * 8);
-  if ((c.precision == NUMA_FP64 || c.precision == NUMA_FP64_PAIRS) && affine_elements(c)) {
+  if (c.precision == NUMA_FP64 && affine_elements(c)) {
     d.affk = (double*)take(3 * (size_t)m.Ne * 8);
     d.Minv_r = (double*)take(Ng * 8);
   }
@@ -480,7 +474,6 @@ size_t layout_workspace(const numa_config& c, const HostMesh& m, char* base, Dev
     d.fxE = (int4*)take((size_t)m.Ne * sizeof(int4));
   }
   d.D32 = (float*)take(PP * 4);
-  d.D2 = (float2*)take(PP * 8);
   d.F64 = (double*)take(PP * 8);
   d.F32 = (float*)take(PP * 4);
   int nz = 0;
@@ -504,7 +497,7 @@ int rhs_with_scratch(numa_ctx* c, const double* q_dev, double* r_dev, double* sc
   if ((const void*)q_dev == (const void*)r_dev) return fail(c, NUMA_EINVAL, "q and r must not alias");
   // the accepted sizes count 72, 32 or 64 bytes a node (FP64, FP32-mixed,
   // pairs), at least what the kernels use
-  const size_t per_node = c->cfg.precision == NUMA_FP64 ? 72 : prim_bytes_per_node(c->cfg.precision);
+  const size_t per_node = c->asked_precision == NUMA_FP64_PAIRS ? 64 : c->cfg.precision == NUMA_FP64 ? 72 : 32;
   const size_t prim_bytes = align_up(prim_bytes_per_node(c->cfg.precision) * (size_t)c->mesh.Ng);
   const size_t need = align_up(per_node * (size_t)c->mesh.Ng) + residual_bytes(c->cfg, c->mesh);
   if (need > 8 * (size_t)scratch_doubles)
@@ -531,7 +524,8 @@ int numa_create(const numa_config* cfg, numa_ctx** out) {
   if (!(cfg->cv > 0) || !(cfg->cp > cfg->cv) || !(cfg->Rd > 0) || !(cfg->P00 > 0)) return NUMA_EINVAL;
   numa_ctx* c = new (std::nothrow) numa_ctx();
   if (!c) return NUMA_ENOMEM;
-  c->cfg = *cfg;
+  c->cfg = working_config(*cfg);
+  c->asked_precision = cfg->precision;
   c->gamma = cfg->cp / cfg->cv;
   // binomial coefficients C(gamma, k) of (1+x)^gamma - 1 = sum_k C(gamma,k) x^k
   double ck = 1.0;
@@ -585,54 +579,27 @@ int numa_bind(numa_ctx* c, void* ws, size_t bytes, void* stream) {
   auto up = [&](void* dst, const void* src, size_t n) {
     if (e == cudaSuccess && n) e = cudaMemcpyAsync(dst, src, n, cudaMemcpyHostToDevice, s);
   };
-  std::vector<float> met32, D32, D2;
-  // (hi, lo) float pairs of FP64 values: hi = nearest float, lo = nearest
-  // float of the remainder
-  auto pairs_of = [](const std::vector<double>& v) {
-    std::vector<float> out(2 * v.size());
-    for (size_t t = 0; t < v.size(); ++t) {
-      const float h = (float)v[t];
-      out[2 * t] = h;
-      out[2 * t + 1] = (float)(v[t] - (double)h);
-    }
-    return out;
-  };
+  std::vector<float> met32, D32;
   if (c->cfg.precision == NUMA_FP32_MIXED) {
     met32.resize(m.met.size());
     for (size_t t = 0; t < m.met.size(); ++t) met32[t] = (float)m.met[t];
     up(L.met32, met32.data(), met32.size() * 4);
-  } else if (c->cfg.precision == NUMA_FP64_PAIRS) {
-    if (affine_elements(c->cfg)) {
-      met32 = pairs_of(m.met);
-    } else {
-      // the per-node pairs form reads rows 0..8 as -Jw dxi_d/dx_c (row 9,
-      // Jw itself, stays for the filter): weighted in FP64, then split
-      std::vector<double> wm(m.met);
-      for (size_t n = 0; n < Nl; ++n) {
-        const double jw = m.met[9 * Nl + n];
-        for (int t = 0; t < 9; ++t) wm[t * Nl + n] = -jw * m.met[t * Nl + n];
-      }
-      met32 = pairs_of(wm);
-    }
-    up(L.met2, met32.data(), met32.size() * 4);
   } else {
     up(L.met64, m.met.data(), m.met.size() * 8);
   }
   D32.resize(m.D.size());
   for (size_t t = 0; t < m.D.size(); ++t) D32[t] = (float)m.D[t];
-  D2 = pairs_of(m.D);
   up(L.D64, m.D.data(), m.D.size() * 8);
   up(L.D32, D32.data(), D32.size() * 4);
-  up(L.D2, D2.data(), D2.size() * 4);
   if (e == cudaSuccess) e = upload_d32_constant(m.N, D32.data(), s);
-  // FP64 and pairs: the per-element constants of rectilinear elements; FP64:
-  // the weighted metric of the per-node form, which it takes everywhere else
+  // FP64: the tables and constants of rectilinear elements, or the integer
+  // metric terms of the per-node form, which it takes everywhere else
   std::vector<double> affk, w3, Minv_r;
   std::vector<int2> fxD;
   bool rect = false, fx = false;
   int fxexp = 0;
   unsigned long long fxw = 0, fxr = 0;
-  if (c->cfg.precision == NUMA_FP64 || c->cfg.precision == NUMA_FP64_PAIRS) {
+  if (c->cfg.precision == NUMA_FP64) {
     if (affine_elements(c->cfg)) {
       const int P = m.P;
       rect = rectilinear_elements(m);
@@ -647,7 +614,7 @@ int numa_bind(numa_ctx* c, void* ws, size_t bytes, void* stream) {
       for (int k = 0; k < P; ++k)
         for (int j = 0; j < P; ++j)
           for (int i = 0; i < P; ++i) w3[i + P * (j + P * k)] = m.w[i] * m.w[j] * m.w[k];
-      if (rect && c->cfg.precision == NUMA_FP64) {
+      if (rect) {
         // K_d = -J dxi_d/dx_d = -(area of the element's face normal to d) / 4,
         // the same for all elements of a box (a mesh whose metric terms say
         // otherwise is not treated as rectilinear).  One scale 2^s for the
@@ -701,7 +668,7 @@ int numa_bind(numa_ctx* c, void* ws, size_t bytes, void* stream) {
       up(L.affk, affk.data(), affk.size() * 8);
       if (rect) up(L.Minv_r, Minv_r.data(), Minv_r.size() * 8);
     }
-    if (c->cfg.precision == NUMA_FP64 && !rect) {
+    if (!rect) {
       // the per-node form: D's table, its row sums scaled to [2^58, 2^59) (a
       // node's sum of nine products of 2^59 and 2^58 stays below 2^63), the
       // weights' powers of two, and the metric terms as integers

@@ -44,15 +44,21 @@ void expand_to_dg_storage(HostMesh& m);
 bool init_state_host(const numa_config& c, const HostMesh& m, int kind, const double* prm, int nprm,
                      double* q, std::string& err);
 
+// The configuration the library works with: NUMA_FP64_PAIRS runs as NUMA_FP64.
+inline numa_config working_config(const numa_config& c) {
+  numa_config w = c;
+  if (w.precision == NUMA_FP64_PAIRS) w.precision = NUMA_FP64;
+  return w;
+}
+
 // Per-global-node primitive fields that the volume kernel gathers, written by
 // the stage update (or the primitive pass) for the state the next create_rhs
 // differentiates:
 //   FP64 mode  : double [5][Ng] = u_x, u_y, u_z, theta, p' (U comes from q)
 //   FP32 mode  : float  [Ng][8] = (U_x, U_y, U_z, u_x), (u_y, u_z, theta, p') per node,
 //                two float4 (one 32-byte sector per node for the gather)
-//   pairs mode : float2 [8][Ng] = the same eight, each as a (hi, lo) pair
 inline int prim_bytes_per_node(int precision) {
-  return precision == NUMA_FP32_MIXED ? 32 : precision == NUMA_FP64_PAIRS ? 64 : 40;
+  return precision == NUMA_FP32_MIXED ? 32 : 40;
 }
 
 // Device workspace carved from the caller's buffer.
@@ -64,25 +70,23 @@ struct DevLayout {
   double* met64 = nullptr;   // [10][Nl] FP64 metric terms and Jw; for the per-node form rows 0..8
                              // hold -Jw dxi_d/dx_c as integers (fx_metric_kernel)
   float* met32 = nullptr;    // [10][Nl] FP32 copy (mixed-precision form)
-  float2* met2 = nullptr;    // [10][Nl] (hi, lo) pairs (pairs mode)
-  float2* D2 = nullptr;      // [P*P] (hi, lo) pairs (pairs mode)
   int32_t* l2g = nullptr;
   int32_t* csr_off = nullptr;
   int32_t* csr_idx = nullptr;
   uint8_t* dss_order = nullptr;  // [ceil(Ng/kDssBlock)*kDssBlock]
   double* ref = nullptr;     // [4][Ng]
   double* Minv = nullptr;    // [Ng]
-  double* Minv_r = nullptr;  // rectilinear form (FP64, pairs): [Ng] w_i w_j w_k / M, the weight of the node's
+  double* Minv_r = nullptr;  // rectilinear form (FP64): [Ng] w_i w_j w_k / M, the weight of the node's
                              // element nodes (equal at all of them) folded into the inverse mass
   uint8_t* wall = nullptr;   // [Ng]
   double* gvec = nullptr;    // [3][Ng] (shell)
   double* nrm = nullptr;     // [3][Ng] (shell)
   double* D64 = nullptr;     // [P*P]
-  double* affk = nullptr;    // FP64 / pairs affine elements: [3][Ne] K_d = -J dxi_d/dx_d per element
+  double* affk = nullptr;    // FP64, affine elements: [3][Ne] K_d = -J dxi_d/dx_d per element
   int2* fxD = nullptr;       // FP64: K_d D (rectilinear form) or D as fixed-point even/odd tables [3][kFxEntries]
   int4* fxE = nullptr;       // FP64 per-node form: [Ne] exponents of the metric rows (fx_metric_kernel)
   float* D32 = nullptr;      // [P*P]
-  double* F64 = nullptr;     // [P*P] 1D filter matrix (FP64, pairs)
+  double* F64 = nullptr;     // [P*P] 1D filter matrix (FP64)
   float* F32 = nullptr;      // [P*P] the same in FP32 (FP32 form)
   double* imex = nullptr;    // 1D-IMEX tables (imex_table_doubles), boxes with walled columns only
   int* imex_piv = nullptr;   // [2][nz][3] pivots and row extents of the two factorisations (dt, dt/2)
@@ -131,10 +135,8 @@ struct VolumeArgs {
   const float* met32;
   const double* D64;
   const float* D32;
-  const float2* met2;  // pairs mode
-  const float2* D2;    // pairs mode
   void* re;            // [5][Nl] output
-  const double* affk;   // rectilinear form (FP64, pairs): [3][Ne] -J dxi_d/dx_d
+  const double* affk;   // rectilinear form (FP64): [3][Ne] -J dxi_d/dx_d
   const int2* fxD;      // FP64: fixed-point tables of K_d D (rectilinear form, one after the other; nullptr:
                         // K_d outside the fixed-point range, the elements take plain FP64) or of D (per-node form)
   const int2* fxD_host; // the same tables in host memory (kernel parameters of the single-mesh launch)
@@ -146,8 +148,8 @@ struct VolumeArgs {
   int Ne;
   int ebeg, ecnt;      // the launch covers elements [ebeg, ebeg + ecnt) (a slab, or all: 0, Ne)
   int affine;          // volume_form: 0 the per-node form; 1 every element is affine, the
-                       // contravariant-flux form (FP32-mixed, pairs); 2 every element is also
-                       // rectilinear (diagonal metric terms): the folded form (FP64, pairs)
+                       // contravariant-flux form (FP32-mixed); 2 every element is also
+                       // rectilinear (diagonal metric terms): the folded form (FP64)
 };
 
 struct UpdateArgs {
@@ -233,10 +235,9 @@ size_t imex_table_doubles(int nz, int N);
 struct FilterArgs {
   const double* q;       // state [5][Ng]
   const int32_t* l2g;
-  const void* F;         // 1D filter matrix [(N+1)^2]: double (FP64, pairs) or float (FP32 form)
+  const void* F;         // 1D filter matrix [(N+1)^2]: double (FP64) or float (FP32 form)
   const double* met64;   // Jw is row 9 of whichever metric array the precision stores
   const float* met32;
-  const float2* met2;
   void* re;              // [5][Nl] Jw-weighted correction, double or float like the residuals
   long long Ng, Nl;
   int Ne;
@@ -247,11 +248,10 @@ cudaError_t launch_prim(const PrimArgs& a, cudaStream_t s);
 // until s has run the copy) into the constant table of the FP32 line kernel.
 cudaError_t upload_d32_constant(int N, const float* D, cudaStream_t s);
 cudaError_t launch_volume(int N, int precision, const VolumeArgs& a, cudaStream_t s);
-// the element kernels of one precision (volume_fp64.cu, volume_fp32.cu,
-// volume_pairs.cu); launch_volume and launch_volume_ragged dispatch to them
+// the element kernels of one precision (volume_fp64.cu, volume_fp32.cu);
+// launch_volume and launch_volume_ragged dispatch to them
 cudaError_t launch_volume_fp64(int N, bool rect, const VolumeArgs& a, cudaStream_t s);
 cudaError_t launch_volume_fp32(int N, bool affine, const VolumeArgs& a, cudaStream_t s);
-cudaError_t launch_volume_pairs(int N, bool affine, const VolumeArgs& a, cudaStream_t s);
 // the metric terms of the FP64 per-node form as integers, in place
 cudaError_t launch_fx_metric(double* met, int4* fxE, long long Ne, int N, unsigned long long fxw, cudaStream_t s);
 cudaError_t launch_update(int precision, const UpdateArgs& a, cudaStream_t s);
@@ -289,7 +289,6 @@ cudaError_t launch_volume_ragged(int N, int precision, bool affine, const Member
                                  cudaStream_t s);
 cudaError_t launch_volume_ragged_fp64(int N, bool rect, const MemberDesc* d, const RaggedGroup* g, cudaStream_t s);
 cudaError_t launch_volume_ragged_fp32(int N, bool affine, const MemberDesc* d, const RaggedGroup* g, cudaStream_t s);
-cudaError_t launch_volume_ragged_pairs(int N, bool affine, const MemberDesc* d, const RaggedGroup* g, cudaStream_t s);
 cudaError_t launch_update_ragged(int precision, bool shell, int stage, const MemberDesc* d, const RaggedGroup* g,
                                  cudaStream_t s);
 
@@ -310,7 +309,8 @@ constexpr int kMaxSlabs = 16;
 // A context: the host mesh of one configuration and, once bound, the layout of
 // its device workspace.
 struct numa_ctx {
-  numa_config cfg;
+  numa_config cfg;          // the working configuration
+  int asked_precision = NUMA_FP64;  // as the caller gave it
   numa::HostMesh mesh;
   numa::DevLayout L;
   bool bound = false;

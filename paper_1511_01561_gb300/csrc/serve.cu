@@ -364,15 +364,16 @@ int numa_sched_submit(numa_sched* s, const numa_config* cfg, int ic_kind, const 
                       double dt, int nsteps, long long* id) {
   if (!s || !cfg || !id || nparams < 0 || nparams > 8 || (nparams && !params) || nsteps < 0 || !(dt == dt))
     return NUMA_EINVAL;
+  const numa_config working = working_config(*cfg);
   if (cfg->storage != NUMA_STORAGE_CG) return sfail(s, NUMA_EINVAL, "serving takes CG storage only");
   size_t bytes = 0;
   long long Ng = 0;
-  if (!workspace_bytes_of(*cfg, &bytes, &Ng)) return sfail(s, NUMA_EINVAL, "bad mesh configuration");
+  if (!workspace_bytes_of(working, &bytes, &Ng)) return sfail(s, NUMA_EINVAL, "bad mesh configuration");
   const size_t tables = align_up(sizeof(MemberDesc) * 3 * kMaxMembers) + align_up(sizeof(RaggedGroup) * kMaxGroups);
   if (align_up(bytes) > s->arena_bytes - tables)
     return sfail(s, NUMA_EBUDGET, "request needs " + std::to_string(bytes) + " bytes, more than the arena");
   auto r = std::make_unique<Request>();
-  r->cfg = *cfg;
+  r->cfg = working;
   r->ic = ic_kind;
   r->nparams = nparams;
   for (int t = 0; t < nparams; ++t) r->params[t] = params[t];

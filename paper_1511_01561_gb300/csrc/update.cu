@@ -1,7 +1,7 @@
 // Per-global-node kernels of the GB300 NUMA hot path (sm_103a):
 //   prim_kernel   : the primitive fields of a state, which the element
-//                   kernels build their fluxes from (u, theta, p'; FP32
-//                   and pairs U too), optionally copying the state in the same pass;
+//                   kernels build their fluxes from (u, theta, p'; FP32 U too),
+//                   optionally copying the state in the same pass;
 //   update_kernel : deterministic direct stiffness summation over a
 //                   precomputed inverse map (fixed order, no atomics), inverse
 //                   mass matrix, sources, wall condition, the SSP-RK3 stage
@@ -9,7 +9,7 @@
 //                   on CG boxes the element nodes of each global node come
 //                   from the structured numbering instead of the map;
 // and the launch entry points of all kernels (the element kernels are
-// compiled per precision in volume_fp64.cu, volume_fp32.cu, volume_pairs.cu).
+// compiled per precision in volume_fp64.cu and volume_fp32.cu).
 #include "kernels_common.cuh"
 
 namespace numa {
@@ -49,7 +49,6 @@ cudaError_t launch_prim(const PrimArgs& a, cudaStream_t s) {
 }
 
 cudaError_t launch_volume(int N, int precision, const VolumeArgs& a, cudaStream_t s) {
-  if (precision == NUMA_FP64_PAIRS) return launch_volume_pairs(N, a.affine != 0, a, s);
   if (precision == NUMA_FP32_MIXED) return launch_volume_fp32(N, a.affine != 0, a, s);
   return launch_volume_fp64(N, a.affine == 2, a, s);
 }
@@ -86,7 +85,6 @@ cudaError_t launch_update(int precision, const UpdateArgs& a, cudaStream_t s) {
 
 cudaError_t launch_volume_ragged(int N, int precision, bool affine, const MemberDesc* d, const RaggedGroup* g,
                                  cudaStream_t s) {
-  if (precision == NUMA_FP64_PAIRS) return launch_volume_ragged_pairs(N, affine, d, g, s);
   if (precision == NUMA_FP32_MIXED) return launch_volume_ragged_fp32(N, affine, d, g, s);
   return launch_volume_ragged_fp64(N, affine, d, g, s);
 }

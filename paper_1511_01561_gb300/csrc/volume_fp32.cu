@@ -6,11 +6,11 @@
 namespace numa {
 
 cudaError_t launch_volume_fp32(int N, bool affine, const VolumeArgs& a, cudaStream_t s) {
-  return affine ? launch_volume_p<float, true>(N, a, s) : launch_volume_p<float, false>(N, a, s);
+  return affine ? launch_volume_p<true>(N, a, s) : launch_volume_p<false>(N, a, s);
 }
 
 cudaError_t launch_volume_ragged_fp32(int N, bool affine, const MemberDesc* d, const RaggedGroup* g, cudaStream_t s) {
-  return affine ? launch_volume_ragged_p<float, true>(N, d, g, s) : launch_volume_ragged_p<float, false>(N, d, g, s);
+  return affine ? launch_volume_ragged_p<true>(N, d, g, s) : launch_volume_ragged_p<false>(N, d, g, s);
 }
 
 cudaError_t upload_d32_constant(int N, const float* D, cudaStream_t s) {
