@@ -50,7 +50,12 @@ PrimArgs prim_args(const numa_ctx* c, const double* q, void* prim) {
   a.Ng = c->mesh.Ng;
   a.precision = c->cfg.precision;
   a.gamma = c->gamma;
-  for (int k = 0; k < kEosTerms; ++k) a.eos[k] = c->eos[k];
+  a.eos_soft = c->gamma > 1.0 && c->gamma < 2.0;
+  for (int k = 0; k < kEosTerms; ++k) {
+    a.eos[k] = c->eos[k];
+    a.eosH[k] = a.eos_soft ? (int)std::lrint(std::ldexp(c->eos[k], 29)) : 0;
+    if (k < kEosFull) a.eosI[k] = a.eos_soft ? std::llrint(std::ldexp(c->eos[k], 58)) : 0;
+  }
   return a;
 }
 

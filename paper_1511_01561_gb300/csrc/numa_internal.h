@@ -13,6 +13,7 @@
 namespace numa {
 
 constexpr int kMaxN = 8;
+constexpr int kEosFull = 6;    // terms of it that soft_pressure sums in full width
 constexpr int kEosTerms = 12;  // binomial-series terms of (1+x)^gamma - 1 for |x| <= 1/32
 constexpr int kDssBlock = 128;  // threads of the update kernel; the DSS order is sorted within such blocks
 
@@ -119,6 +120,9 @@ struct PrimArgs {
   int precision;
   double gamma;
   double eos[kEosTerms];  // binomial coefficients C(gamma, k), k = 1..kEosTerms
+  long long eosI[kEosFull];  // the first ones in units of 2^-58
+  int eosH[kEosTerms];       // all in units of 2^-29
+  int eos_soft;              // 1 < gamma < 2: they fit
 };
 
 // Every element of the mesh maps affinely onto the reference cube (a box
