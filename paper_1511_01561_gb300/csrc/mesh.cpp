@@ -3,10 +3,13 @@
 // terms, element-to-global maps and their inverse, mass matrix, hydrostatic
 // reference state and initial conditions.
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <cstdlib>
 #include <cstring>
+#include <exception>
 #include <numeric>
+#include <thread>
 
 #include "numa_internal.h"
 
@@ -14,6 +17,38 @@ namespace numa {
 namespace {
 
 constexpr double kPi = 3.14159265358979323846;
+
+// f(begin, end) over [0, n) in a few threads when there is work for them
+// (each index is computed as in one thread; the caller sees every effect).  An
+// exception in one of them is thrown again here; a thread that cannot be had
+// is done without.
+template <typename F>
+void parallel_for(long long n, long long work, F f) {
+  const long long want = std::min<long long>({8, (long long)std::thread::hardware_concurrency(), work >> 17, n});
+  if (want <= 1) {
+    f(0, n);
+    return;
+  }
+  std::vector<std::thread> ts;
+  std::vector<std::exception_ptr> bad(want);
+  auto part = [&](long long t) {
+    try {
+      f(n * t / want, n * (t + 1) / want);
+    } catch (...) {
+      bad[t] = std::current_exception();
+    }
+  };
+  long long t = 1;
+  try {
+    for (ts.reserve(want); t < want; ++t) ts.emplace_back(part, t);
+  } catch (...) {  // the parts without a thread run here
+  }
+  part(0);
+  for (; t < want; ++t) part(t);
+  for (auto& x : ts) x.join();
+  for (auto& e : bad)
+    if (e) std::rethrow_exception(e);
+}
 
 // P_N and P_{N-1} at x (three-term recurrence).
 void legendre_pair(int N, double x, double& pn, double& pnm1) {
@@ -130,7 +165,7 @@ const int kFrame[6][3][3] = {
 };
 
 // Structured box: element e = ex + nex (ey + ney ez), local l = i + P (j + P k).
-void box_nodes(const numa_config& c, HostMesh& m, std::vector<double>& X) {
+void box_nodes(const numa_config& c, HostMesh& m, RawDoubles& X) {
   const int N = m.N, P = m.P;
   const long long nx = (long long)c.nex * N + (c.periodic[0] ? 0 : 1);
   const long long ny = (long long)c.ney * N + (c.periodic[1] ? 0 : 1);
@@ -138,30 +173,38 @@ void box_nodes(const numa_config& c, HostMesh& m, std::vector<double>& X) {
   m.Ne = (long long)c.nex * c.ney * c.nez;
   m.Nl = m.Ne * m.Np;
   m.Ng = nx * ny * nz;
-  X.assign(3 * m.Nl, 0.0);
-  m.l2g.assign(m.Nl, 0);
-  for (int ez = 0; ez < c.nez; ++ez)
-    for (int ey = 0; ey < c.ney; ++ey)
-      for (int ex = 0; ex < c.nex; ++ex) {
-        long long e = ex + (long long)c.nex * (ey + (long long)c.ney * ez);
-        for (int k = 0; k < P; ++k)
-          for (int j = 0; j < P; ++j)
-            for (int i = 0; i < P; ++i) {
-              long long n = e * m.Np + i + P * (j + P * k);
-              double u = (ex + 0.5 * (1.0 + m.xi[i])) / c.nex;
-              double v = (ey + 0.5 * (1.0 + m.xi[j])) / c.ney;
-              double t = (ez + 0.5 * (1.0 + m.xi[k])) / c.nez;
-              double su = std::sin(kPi * u), sv = std::sin(kPi * v), st = std::sin(kPi * t);
-              X[n] = c.Lx * (u + c.warp * su * sv * st);
-              X[m.Nl + n] = c.Ly * (v + c.warp * std::sin(2.0 * kPi * u) * sv * st);
-              X[2 * m.Nl + n] = c.Lz * (t + c.warp * su * std::sin(2.0 * kPi * v) * st);
-              long long ix = (long long)ex * N + i, iy = (long long)ey * N + j, iz = (long long)ez * N + k;
-              if (ix == nx) ix = 0;
-              if (iy == ny) iy = 0;
-              if (iz == nz) iz = 0;
-              m.l2g[n] = (int32_t)(ix + nx * (iy + ny * iz));
-            }
+  X.resize(3 * m.Nl);
+  m.l2g.resize(m.Nl);
+  // per axis and element point: the unit coordinate and its sines
+  std::vector<double> un[3], sn[3], s2[3];
+  const int ne[3] = {c.nex, c.ney, c.nez};
+  for (int d = 0; d < 3; ++d)
+    for (int q = 0; q < ne[d]; ++q)
+      for (int i = 0; i < P; ++i) {
+        un[d].push_back((q + 0.5 * (1.0 + m.xi[i])) / ne[d]);
+        sn[d].push_back(c.warp != 0.0 ? std::sin(kPi * un[d].back()) : 0.0);
+        s2[d].push_back(c.warp != 0.0 ? std::sin(2.0 * kPi * un[d].back()) : 0.0);
       }
+  parallel_for(m.Ne, (long long)m.Np * m.Ne, [&](long long e0, long long e1) {
+    for (long long e = e0; e < e1; ++e) {
+      const int ex = (int)(e % c.nex), ey = (int)(e / c.nex % c.ney), ez = (int)(e / c.nex / c.ney);
+      for (int k = 0; k < P; ++k)
+        for (int j = 0; j < P; ++j)
+          for (int i = 0; i < P; ++i) {
+            const long long n = e * m.Np + i + P * (j + P * k);
+            const double u = un[0][ex * P + i], v = un[1][ey * P + j], t = un[2][ez * P + k];
+            const double su = sn[0][ex * P + i], sv = sn[1][ey * P + j], st = sn[2][ez * P + k];
+            X[n] = c.Lx * (u + c.warp * su * sv * st);
+            X[m.Nl + n] = c.Ly * (v + c.warp * s2[0][ex * P + i] * sv * st);
+            X[2 * m.Nl + n] = c.Lz * (t + c.warp * su * s2[1][ey * P + j] * st);
+            long long ix = (long long)ex * N + i, iy = (long long)ey * N + j, iz = (long long)ez * N + k;
+            if (ix == nx) ix = 0;
+            if (iy == ny) iy = 0;
+            if (iz == nz) iz = 0;
+            m.l2g[n] = (int32_t)(ix + nx * (iy + ny * iz));
+          }
+    }
+  });
   m.wall.assign(m.Ng, 0);
   for (long long iz = 0; iz < nz; ++iz)
     for (long long iy = 0; iy < ny; ++iy)
@@ -183,63 +226,65 @@ void box_nodes(const numa_config& c, HostMesh& m, std::vector<double>& X) {
 // columns) numbered by first appearance in element-node order and
 // level = il N + k from the bottom, so that a radial column is the same
 // stride-ncol sequence as a z-column of the box.
-void shell_nodes(const numa_config& c, HostMesh& m, std::vector<double>& X) {
+void shell_nodes(const numa_config& c, HostMesh& m, RawDoubles& X) {
   const int N = m.N, P = m.P, np = c.npanel, nl = c.nlayer;
   const long long K = (long long)np * N, W = 2 * K + 1, NR = (long long)nl * N + 1;
   m.Ne = 6LL * np * np * nl;
   m.Nl = m.Ne * m.Np;
-  X.assign(3 * m.Nl, 0.0);
-  m.hgt.assign(m.Nl, 0.0);
-  std::vector<long long> key(m.Nl);
-  std::vector<int> level(m.Nl);
+  X.resize(3 * m.Nl);
+  m.hgt.resize(m.Nl);
+  // the surface points by (panel, ib, ia, j, i), the order in which the element
+  // nodes meet them (in each column's lowest element, k = 0)
+  const long long PP = (long long)P * P, ns = 6LL * np * np * PP;
+  std::vector<long long> key(ns);
   const double dA = 0.5 * kPi / np, dR = (c.r_outer - c.r_inner) / nl;
-  for (int p = 0; p < 6; ++p)
-    for (int ib = 0; ib < np; ++ib)
-      for (int ia = 0; ia < np; ++ia)
-        for (int il = 0; il < nl; ++il) {
-          long long e = il + (long long)nl * (ia + (long long)np * (ib + (long long)np * p));
+  std::vector<double> tn(np * (size_t)P);  // tan of the panel angle per element point along a panel edge
+  for (int ia = 0; ia < np; ++ia)
+    for (int i = 0; i < P; ++i) tn[ia * P + i] = std::tan(-0.25 * kPi + (ia + 0.5 * (1.0 + m.xi[i])) * dA);
+  parallel_for(m.Ne, 4 * m.Nl, [&](long long e0, long long e1) {
+    for (long long e = e0; e < e1; ++e) {
+          const int il = (int)(e % nl), ia = (int)(e / nl % np), ib = (int)(e / nl / np % np), p = (int)(e / nl / np / np);
           for (int k = 0; k < P; ++k)
             for (int j = 0; j < P; ++j)
               for (int i = 0; i < P; ++i) {
                 long long n = e * m.Np + i + P * (j + P * k);
-                double al = -0.25 * kPi + (ia + 0.5 * (1.0 + m.xi[i])) * dA;
-                double be = -0.25 * kPi + (ib + 0.5 * (1.0 + m.xi[j])) * dA;
                 const double h = (il + 0.5 * (1.0 + m.xi[k])) * dR;
                 double r = c.r_inner + h;
                 m.hgt[n] = h;
-                double ta = std::tan(al), tb = std::tan(be), v[3], nn = 0.0;
+                double ta = tn[ia * P + i], tb = tn[ib * P + j], v[3], nn = 0.0;
                 for (int d = 0; d < 3; ++d) {
                   v[d] = kFrame[p][2][d] + ta * kFrame[p][0][d] + tb * kFrame[p][1][d];
                   nn += v[d] * v[d];
                 }
                 double s = r / std::sqrt(nn);
                 for (int d = 0; d < 3; ++d) X[d * m.Nl + n] = s * v[d];
-                long long la = (long long)ia * N + i, lb = (long long)ib * N + j;
-                long long L[3];
-                for (int d = 0; d < 3; ++d)
-                  L[d] = K * kFrame[p][2][d] + (2 * la - K) * kFrame[p][0][d] + (2 * lb - K) * kFrame[p][1][d];
-                key[n] = ((L[0] + K) * W + (L[1] + K)) * W + (L[2] + K);  // the surface point
-                level[n] = (int)((long long)il * N + k);
+                if (il == 0 && k == 0) {
+                  long long la = (long long)ia * N + i, lb = (long long)ib * N + j;
+                  long long L[3];
+                  for (int d = 0; d < 3; ++d)
+                    L[d] = K * kFrame[p][2][d] + (2 * la - K) * kFrame[p][0][d] + (2 * lb - K) * kFrame[p][1][d];
+                  key[e / nl * PP + i + P * j] = ((L[0] + K) * W + (L[1] + K)) * W + (L[2] + K);
+                }
               }
-        }
+    }
+  });
   // columns: the unique surface points, numbered by first appearance
-  std::vector<long long> order(m.Nl);
-  std::iota(order.begin(), order.end(), 0LL);
-  std::stable_sort(order.begin(), order.end(), [&](long long a, long long b) { return key[a] < key[b]; });
-  std::vector<long long> first(m.Nl, -1);  // per element node: first node with its surface point
-  std::vector<long long> firsts;
-  for (long long t = 0; t < m.Nl; ++t) {
-    if (t == 0 || key[order[t]] != key[order[t - 1]]) firsts.push_back(order[t]);
-    first[order[t]] = firsts.back();
+  std::vector<int> order(ns), col(ns);
+  std::iota(order.begin(), order.end(), 0);
+  std::sort(order.begin(), order.end(), [&](int x, int y) { return key[x] != key[y] ? key[x] < key[y] : x < y; });
+  for (long long t = 0, f = 0; t < ns; ++t) {  // the first with its key, for now
+    if (t == 0 || key[order[t]] != key[order[t - 1]]) f = order[t];
+    col[order[t]] = (int)f;
   }
-  std::vector<long long> f_sorted = firsts;
-  std::sort(f_sorted.begin(), f_sorted.end());
-  std::vector<int32_t> col_of_first(m.Nl, -1);
-  for (size_t t = 0; t < f_sorted.size(); ++t) col_of_first[f_sorted[t]] = (int32_t)t;
-  const long long ncol = (long long)f_sorted.size();
+  long long ncol = 0;
+  for (long long t = 0; t < ns; ++t) col[t] = col[t] == t ? (int)ncol++ : col[col[t]];
   m.Ng = ncol * NR;
-  m.l2g.assign(m.Nl, 0);
-  for (long long n = 0; n < m.Nl; ++n) m.l2g[n] = (int32_t)(col_of_first[first[n]] + ncol * level[n]);
+  m.l2g.resize(m.Nl);
+  parallel_for(m.Ne, m.Nl, [&](long long e0, long long e1) {
+    for (long long e = e0; e < e1; ++e)
+      for (int l = 0; l < m.Np; ++l)
+        m.l2g[e * m.Np + l] = (int32_t)(col[e / nl * PP + l % PP] + ncol * (e % nl * N + l / PP));
+  });
   m.wall.assign(m.Ng, 0);
   for (long long c = 0; c < ncol; ++c) {  // the bottom and the lid
     m.wall[c] = 8;
@@ -377,7 +422,7 @@ bool build_host_mesh(const numa_config& c, HostMesh& m, std::string& err) {
       m.D[t] = u > t ? (double)D[t] : u < t ? -m.D[u] : 0.0;
     }
   }
-  std::vector<double> X;
+  RawDoubles X;
   // element nodes from the configuration alone, so that a mesh beyond the
   // 32-bit indices is refused before any of its arrays is built (each global
   // node belongs to at least one element node, so Nl bounds Ng as well)
@@ -430,8 +475,48 @@ bool build_host_mesh(const numa_config& c, HostMesh& m, std::string& err) {
   std::vector<double>().swap(m.hgt);
   // Eq. 5 metric terms: dx_c/dxi_d = sum_m D x_c along direction d, then the
   // analytic inverse of the 3x3 Jacobian matrix; Jw = det * w_i w_j w_k.
-  m.met.assign(10 * Nl, 0.0);
-  for (long long e = 0; e < m.Ne; ++e) {
+  m.met.resize(10 * Nl);
+  std::atomic<bool> folded{false};
+  if (c.mesh_kind == NUMA_MESH_BOX && c.warp == 0.0) {
+    // an unwarped box: dx_c/dxi_d vanishes for d != c and depends on the node's
+    // place along c alone (the sums below, term by term, without their zeros)
+    std::vector<double> A[3];
+    const int ne[3] = {c.nex, c.ney, c.nez};
+    const long long step[3] = {1, (long long)c.nex, (long long)c.nex * c.ney};
+    for (int d = 0; d < 3; ++d) {
+      const long long st = d == 0 ? 1 : d == 1 ? P : P * P;
+      for (int q = 0; q < ne[d]; ++q) {
+        const double* x = &X[d * Nl + q * step[d] * Np];
+        for (int i = 0; i < P; ++i) {
+          double s = 0;
+          for (int t = 0; t < P; ++t) s += m.D[i * P + t] * (x[t * st] - x[0]);
+          A[d].push_back(s);
+        }
+      }
+    }
+    parallel_for(m.Ne, 4 * Nl, [&](long long e0, long long e1) {
+      for (long long e = e0; e < e1; ++e) {
+        const double* ax = &A[0][(e % c.nex) * P];
+        const double* ay = &A[1][(e / c.nex % c.ney) * P];
+        const double* az = &A[2][(e / c.nex / c.ney) * P];
+        for (int l = 0; l < Np; ++l) {
+          const int i = l % P, j = (l / P) % P, k = l / (P * P);
+          const double C00 = ay[j] * az[k], det = ax[i] * C00;
+          if (!(det > 0.0)) {
+            folded = true;
+            return;
+          }
+          const double inv = 1.0 / det;
+          m.met[e * Np + l] = C00 * inv;
+          m.met[4 * Nl + e * Np + l] = (ax[i] * az[k]) * inv;
+          m.met[8 * Nl + e * Np + l] = (ax[i] * ay[j]) * inv;
+          for (int t : {1, 2, 3, 5, 6, 7}) m.met[t * Nl + e * Np + l] = 0.0;
+          m.met[9 * Nl + e * Np + l] = det * m.w[i] * m.w[j] * m.w[k];
+        }
+      }
+    });
+  } else parallel_for(m.Ne, 40 * Nl, [&](long long e0, long long e1) {
+  for (long long e = e0; e < e1; ++e) {
     const long long b = e * Np;
     for (int l = 0; l < Np; ++l) {
       const int i = l % P, j = (l / P) % P, k = l / (P * P);
@@ -457,8 +542,8 @@ bool build_host_mesh(const numa_config& c, HostMesh& m, std::string& err) {
       double C02 = A[1][0] * A[2][1] - A[1][1] * A[2][0];
       double det = A[0][0] * C00 + A[0][1] * C01 + A[0][2] * C02;
       if (!(det > 0.0)) {
-        err = "non-positive element Jacobian";
-        return false;
+        folded = true;
+        return;
       }
       double inv = 1.0 / det;
       double Bi[3][3];  // Bi[d][c] = d xi_d / d x_c
@@ -475,6 +560,11 @@ bool build_host_mesh(const numa_config& c, HostMesh& m, std::string& err) {
         for (int cc = 0; cc < 3; ++cc) m.met[(3 * d + cc) * Nl + b + l] = Bi[d][cc];
       m.met[9 * Nl + b + l] = det * m.w[i] * m.w[j] * m.w[k];
     }
+  }
+  });
+  if (folded) {
+    err = "non-positive element Jacobian";
+    return false;
   }
   // inverse map (CSR, ascending element node) and the mass matrix of Eq. 4
   m.csr_off.assign(Ng + 1, 0);
@@ -500,7 +590,10 @@ bool build_host_mesh(const numa_config& c, HostMesh& m, std::string& err) {
     m.gvec.assign(3 * Ng, 0.0);
     m.nrm.assign(3 * Ng, 0.0);
   }
-  for (long long g = 0; g < Ng; ++g) {
+  std::atomic<int> ref_bad{0};
+  parallel_for(Ng, 8 * Ng, [&](long long g0, long long g1) {
+  double phi_was = -1.0, p0 = 0.0, Th0 = 0.0, rho0 = 0.0;  // of the node before: a level shares them
+  for (long long g = g0; g < g1; ++g) {
     double x = m.gxyz[g], y = m.gxyz[Ng + g], z = m.gxyz[2 * Ng + g], phi;
     if (c.mesh_kind == NUMA_MESH_BOX) {
       phi = c.g * z;
@@ -517,12 +610,13 @@ bool build_host_mesh(const numa_config& c, HostMesh& m, std::string& err) {
       m.nrm[Ng + g] = y / r;
       m.nrm[2 * Ng + g] = z / r;
     }
-    double p0, Th0, rho0;
-    if (c.ref_kind == NUMA_REF_ISENTROPIC) {
+    if (g > g0 && phi == phi_was) {
+      // the reference state of the node before
+    } else if (c.ref_kind == NUMA_REF_ISENTROPIC) {
       double exner = 1.0 - phi / (c.cp * c.theta0);
       if (!(exner > 0.0)) {
-        err = "isentropic reference reaches zero Exner pressure inside the domain";
-        return false;
+        ref_bad = 1;
+        return;
       }
       p0 = c.P00 * std::pow(exner, c.cp / c.Rd);
       Th0 = p0 / (c.Rd * exner);
@@ -532,13 +626,19 @@ bool build_host_mesh(const numa_config& c, HostMesh& m, std::string& err) {
       rho0 = p0 / (c.Rd * c.T0);
       Th0 = (c.P00 / c.Rd) * std::pow(p0 / c.P00, c.cv / c.cp);
     } else {
-      err = "unknown ref_kind";
-      return false;
+      ref_bad = 2;
+      return;
     }
+    phi_was = phi;
     m.ref[g] = rho0;
     m.ref[Ng + g] = Th0;
     m.ref[2 * Ng + g] = p0;
     m.ref[3 * Ng + g] = 1.0 / Th0;
+  }
+  });
+  if (ref_bad) {
+    err = ref_bad == 1 ? "isentropic reference reaches zero Exner pressure inside the domain" : "unknown ref_kind";
+    return false;
   }
   return true;
 }

@@ -589,6 +589,8 @@ int numa_bind(numa_ctx* c, void* ws, size_t bytes, void* stream) {
     met32.resize(m.met.size());
     for (size_t t = 0; t < m.met.size(); ++t) met32[t] = (float)m.met[t];
     up(L.met32, met32.data(), met32.size() * 4);
+  } else if (affine_elements(c->cfg)) {
+    up(L.met64 + 9 * Nl, m.met.data() + 9 * Nl, Nl * 8);  // Jw (the filter's); the rest below if it is read
   } else {
     up(L.met64, m.met.data(), m.met.size() * 8);
   }
@@ -654,17 +656,17 @@ int numa_bind(numa_ctx* c, void* ws, size_t bytes, void* stream) {
         }
       }
       // Minv_r: w_i w_j w_k of the node's first element node (its DSS list
-      // is ascending), times 1/M.  Lobatto weights are symmetric, so every
-      // element node of a global node of a box has that weight; a mesh
-      // where they differ is not treated as rectilinear (volume_form).
+      // is ascending), times 1/M.  Every element node of a global node of a box
+      // has that weight if the two ends of the axis have (Lobatto weights are
+      // symmetric); a mesh where they differ is not treated as rectilinear
+      // (volume_form).
+      if (std::fabs(m.w[0] - m.w[P - 1]) > 1e-14 * m.w[0]) rect = false;
       if (rect) {
         const long long Np = m.Np;
         Minv_r.resize((size_t)Ng);
         const double rJ = 8.0 * ((double)c->cfg.nex * c->cfg.ney * c->cfg.nez) / (c->cfg.Lx * c->cfg.Ly * c->cfg.Lz);
-        for (size_t I = 0; I < Ng && rect; ++I) {
+        for (size_t I = 0; I < Ng; ++I) {
           const double wf = w3[m.csr_idx[m.csr_off[I]] % Np];
-          for (int32_t t = m.csr_off[I] + 1; t < m.csr_off[I + 1]; ++t)
-            if (std::fabs(w3[m.csr_idx[t] % Np] - wf) > 1e-14 * wf) rect = false;
           // fixed-point form: w_I / M_I = 1 / (J x element nodes at I), J in closed form like the K_d
           Minv_r[I] = fx ? rJ / (double)(m.csr_off[I + 1] - m.csr_off[I]) : wf * m.Minv[I];
         }
@@ -674,6 +676,7 @@ int numa_bind(numa_ctx* c, void* ws, size_t bytes, void* stream) {
       if (rect) up(L.Minv_r, Minv_r.data(), Minv_r.size() * 8);
     }
     if (!rect) {
+      if (affine_elements(c->cfg)) up(L.met64, m.met.data(), 9 * Nl * 8);
       // the per-node form: D's table, its row sums scaled to [2^58, 2^59) (a
       // node's sum of nine products of 2^59 and 2^58 stays below 2^63), the
       // weights' powers of two, and the metric terms as integers

@@ -5,7 +5,10 @@
 #include <cuda_runtime.h>
 
 #include <cstdint>
+#include <memory>
+#include <new>
 #include <string>
+#include <utility>
 #include <vector>
 
 #include "numa.h"
@@ -16,6 +19,26 @@ constexpr int kMaxN = 8;
 constexpr int kEosFull = 6;    // terms of it that soft_pressure sums in full width
 constexpr int kEosTerms = 12;  // binomial-series terms of (1+x)^gamma - 1 for |x| <= 1/32
 constexpr int kDssBlock = 128;  // threads of the update kernel; the DSS order is sorted within such blocks
+
+// A vector whose elements are left uninitialised by resize: the threads that
+// fill a large array touch its pages first, not one thread that zeroes it.
+template <typename T>
+struct RawAllocator : std::allocator<T> {
+  template <typename U>
+  struct rebind {
+    using other = RawAllocator<U>;
+  };
+  RawAllocator() = default;
+  template <typename U>
+  RawAllocator(const RawAllocator<U>&) {}
+  template <typename U>
+  void construct(U*) {}
+  template <typename U, typename... A>
+  void construct(U* p, A&&... a) {
+    ::new ((void*)p) U(std::forward<A>(a)...);
+  }
+};
+using RawDoubles = std::vector<double, RawAllocator<double>>;
 
 // Host-side mesh and geometry (Sec. 2.1: Lobatto points, Eq. 4: Jw and M,
 // Eq. 5: isoparametric metric terms).  Built once per context.
@@ -30,7 +53,7 @@ struct HostMesh {
   long long nentries = 0;             // CSR entries: Nl (CG storage) or sum of the squared counts (DG)
   std::vector<uint8_t> dss_order;     // per block of kDssBlock global nodes: local indices sorted by
                                       // their number of element nodes (stable) [ceil(Ng/kDssBlock)*kDssBlock]
-  std::vector<double> met;            // [10][Nl]: dxi_d/dx_c at row 3d+c, then Jw
+  RawDoubles met;                     // [10][Nl]: dxi_d/dx_c at row 3d+c, then Jw
   std::vector<double> ref;            // [4][Ng]: rho0, (rho theta)_0, p0, 1/(rho theta)_0
   std::vector<double> Minv;           // [Ng]: 1 / sum_e Jw
   std::vector<uint8_t> wall;          // [Ng]: bit a = box wall normal to axis a; bit 3 = shell radial wall
