@@ -58,16 +58,17 @@ __device__ __forceinline__ int2 fx_split(long long s) {
   return make_int2((int)((unsigned)s & kFxMask) - (int)kFxHalf, (int)(s >> kFxBits));
 }
 
-// S 2^(kexp - 1086) rounded to nearest: the double whose biased exponent is
-// kexp less the leading zeros of |S|.
+// S 2^(kexp - 1086) rounded to nearest, and fx_of by the FP64 pipe: a conversion
+// and an exact product each, 32 cycles of a pipe that is otherwise idle in
+// place of 24 and 15 integer instructions.  Measured on 32^3 elements, N = 4
+// (rectilinear) and the 6x30x30x8 shell (per-node): all five results so, 0.183
+// -> 0.174 and 0.540 -> 0.526 ms; U and p' of the eight inputs too, 0.183 and
+// 0.519 ms (so in the per-node form only); all eight, 0.213 and 0.520 ms.
 __device__ __forceinline__ double fx_to_double(long long S, int kexp) {
-  const unsigned sg = (unsigned)((unsigned long long)S >> 32) & 0x80000000u;
-  const unsigned long long u = (unsigned long long)(S < 0 ? -S : S);
-  const int lz = __clzll((long long)u);
-  const unsigned long long n = u << lz;  // (u = 0: lz = 64, selected away below)
-  const unsigned long long mant = (n >> 11) + ((n >> 10) & 1ull);  // carries into the exponent
-  const unsigned long long b = mant + ((unsigned long long)(unsigned)(kexp - lz - 1) << 52);
-  return __hiloint2double(u ? (int)((unsigned)(b >> 32) | sg) : 0, u ? (int)(unsigned)b : 0);
+  return __ll2double_rn(S) * __hiloint2double((kexp - 63) << 20, 0);
+}
+__device__ __forceinline__ long long fx_of_pipe(double x, int E) {
+  return __double2ll_rn(x * __hiloint2double((2103 - E) << 20, 0));
 }
 
 // Magnitude key of a group of values: the largest of their high words without
@@ -120,11 +121,17 @@ __device__ __forceinline__ void fx_mac(long long& h, long long& m, int2 D, int f
   m += (long long)D.x * fh;
 }
 
+// h + (m >> 29).  (With m's high word as one more multiply-add, h + 8 m.hi + ...:
+// 5% slower.)
+__device__ __forceinline__ long long fx_sum(long long h, long long m) {
+  return h + (m >> kFxBits);
+}
+
 // a b 2^-58, rounded but for the product of the low parts.
 __device__ __forceinline__ long long fx_mul(int2 a, int2 b) {
   long long h = 0, m = kFxHalf;
   fx_mac(h, m, a, b.x, b.y);
-  return h + (m >> kFxBits);
+  return fx_sum(h, m);
 }
 
 // Entries of a direction's even/odd table (see fx_line).
@@ -168,7 +175,7 @@ __device__ __forceinline__ void fx_line(const int2* __restrict__ F, int stride, 
     for (int j = 0; j < H + O; ++j) fx_mac(ah, am, D[i * (H + O) + j], el[j], eh[j]);
 #pragma unroll
     for (int j = 0; j < H; ++j) fx_mac(bh, bm, D[H * (H + O) + i * H + j], ol[j], oh[j]);
-    const long long A = ah + (am >> kFxBits), B = bh + (bm >> kFxBits);
+    const long long A = fx_sum(ah, am), B = fx_sum(bh, bm);
     out[i] = B + A;
     out[N - i] = B - A;
   }
@@ -176,7 +183,7 @@ __device__ __forceinline__ void fx_line(const int2* __restrict__ F, int stride, 
     long long h = 0, m = kFxHalf;
 #pragma unroll
     for (int j = 0; j < H; ++j) fx_mac(h, m, D[H * (H + O) + H * H + j], ol[j], oh[j]);
-    out[H] = h + (m >> kFxBits);
+    out[H] = fx_sum(h, m);
   }
 }
 
@@ -314,7 +321,7 @@ __host__ __device__ constexpr int fx_slot(int f) {
 // The largest magnitudes in an element give its groups' exponents: left as
 // keys per element in gmax (EPB > 1), or returned in ge (EPB = 1).  False
 // (uniform over the CTA) if the integers cannot hold some element.
-template <int N, int EPB, int NT>
+template <int N, int EPB, int NT, bool PIPE>
 __device__ __forceinline__ bool fx_stage(const VolumeArgs& a, long long n0, int nn, uint4* gmax, int2* F, FxExp& ge) {
   constexpr int NP = (N + 1) * (N + 1) * (N + 1), NN = EPB * NP, IT = (NN + NT - 1) / NT;
   constexpr int FP = EPB * fx_pitch<N>(), SLOTS = fx_slots<EPB, NT>();
@@ -350,6 +357,8 @@ __device__ __forceinline__ bool fx_stage(const VolumeArgs& a, long long n0, int 
     gw.w = __reduce_max_sync(0xffffffffu, gw.w);
     if ((tid & 31) == 0) gmax[tid >> 5] = gw;
   }
+  grid_wait();  // (threads without a node; before any write of the kernel)
+  grid_next();
   __syncthreads();
   bool ok = true;
   uint4 gm = make_uint4(0u, 0u, 0u, 0u);
@@ -375,11 +384,11 @@ __device__ __forceinline__ bool fx_stage(const VolumeArgs& a, long long n0, int 
       int2 U[3], u[3];
 #pragma unroll
       for (int c = 0; c < 3; ++c) {
-        U[c] = fx_split(fx_of(z[it].U[c], e.U));
+        U[c] = fx_split((PIPE ? fx_of_pipe : fx_of)(z[it].U[c], e.U));
         u[c] = fx_split(fx_of(z[it].u[c], max(e.m - e.U + 1022, kFxZero)));
       }
       const int2 th = fx_split(fx_of(z[it].th, max((int)(gm.z >> 20), kFxZero)));
-      const long long p = fx_of(z[it].pp, e.m);
+      const long long p = (PIPE ? fx_of_pipe : fx_of)(z[it].pp, e.m);
       f[sUx * FP] = U[0];
       f[sUy * FP] = U[1];
       f[sUz * FP] = U[2];
@@ -407,14 +416,15 @@ __device__ __forceinline__ bool fx_stage(const VolumeArgs& a, long long n0, int 
 //   3. it then takes its line along z, adds the x and y derivatives at the
 //      line's nodes as integers and converts the sums to FP64, rounded once.
 // On 32^3 elements at N = 4: 0.529 ms as FP64 (its pipe 97% busy: 75
-// operations a node at 16 cycles a warp), 0.186 ms here; 19x23x17 at N = 6:
-// 0.460 -> 0.137 ms.  135 integer multiply-adds a thread keep their pipe a
+// operations a node at 16 cycles a warp), 0.156 ms here; 19x23x17 at N = 6:
+// 0.460 -> 0.135 ms.  135 integer multiply-adds a thread keep their pipe a
 // quarter busy; shared memory, the scattered gather and the instructions
 // beside the products are what is left.  D in the kernel parameters instead
 // of global memory: 0.256 -> 0.226 ms; the z lines finishing the nodes (10
 // shared accesses a node fewer, ten CTAs an SM instead of eight): 0.226 ->
 // 0.216 ms; the products formed here from 8 gathered fields instead of 12
-// gathered fluxes: 0.216 -> 0.186 ms (and the update 0.199 -> 0.169 ms).
+// gathered fluxes: 0.216 -> 0.186 ms (and the update 0.199 -> 0.169 ms); the
+// results converted by the FP64 pipe and 64 registers: 0.186 -> 0.156 ms.
 template <int N>
 __device__ __forceinline__ void volume_fx_rect(const VolumeArgs& a, const int2* T, long long e0, int ne,
                                                unsigned char* smem_raw) {
@@ -426,7 +436,7 @@ __device__ __forceinline__ void volume_fx_rect(const VolumeArgs& a, const int2* 
   const int tid = threadIdx.x;
   const long long n0 = e0 * NP;
   FxExp ge;
-  if (a.fxD == nullptr || !fx_stage<N, EPB, NT>(a, n0, ne * NP, gmax, F, ge)) {  // uniform over the CTA
+  if (a.fxD == nullptr || !fx_stage<N, EPB, NT, false>(a, n0, ne * NP, gmax, F, ge)) {  // uniform over the CTA
     for (int t = 0; t < ne; ++t) rect_plain<N>(a, e0 + t);
     return;
   }
@@ -512,7 +522,7 @@ __device__ __forceinline__ void nodal_plain(const VolumeArgs& a, long long e) {
 // an inner one's).  The directions' sums are aligned by the exponents of their
 // rows, added as integers and rounded once.
 // On the 6x30x30x8 shell at N = 4: 2.068 ms as FP64 (225 operations a node, its
-// pipe 96% busy), 0.540 ms here; 21x17x13 at N = 3: 0.105 -> 0.039 ms.  The 430
+// pipe 96% busy), 0.520 ms here; 21x17x13 at N = 3: 0.105 -> 0.039 ms.  The 430
 // integer multiply-adds a thread keep their pipe 40% busy and the 2300
 // instructions a warp 60% of the issue slots, at 8 CTAs an SM (64 registers).
 // With the fluxes formed in the update it took 0.505 ms, and the update 0.335
@@ -533,7 +543,7 @@ __device__ __forceinline__ void volume_fx_nodal(const VolumeArgs& a, const int2*
   // the elements' metric exponents (w: the element takes plain FP64)
   const int4 eb = a.fxE[e0 + (node ? nel : 0)];
   FxExp ge;
-  bool ok = fx_stage<N, EPB, NT>(a, n0, nn, gmax, F, ge);
+  bool ok = fx_stage<N, EPB, NT, true>(a, n0, nn, gmax, F, ge);
   if (__syncthreads_or(!ok || eb.w)) {
     for (int t = 0; t < ne; ++t) nodal_plain<N>(a, e0 + t);
     return;
@@ -579,7 +589,7 @@ __device__ __forceinline__ void volume_fx_nodal(const VolumeArgs& a, const int2*
         use(h, m, s0, 0);
         use(h, m, s1, 1);
         use(h, m, s2, 2);
-        sum[v] += (h + (m >> kFxBits)) >> sh;  // (nine products below 2^60, halved: below 2^63)
+        sum[v] += fx_sum(h, m) >> sh;  // (nine products below 2^60, halved: below 2^63)
       };
       eq(0, sUx, sUy, sUz);
       eq(1, sTxx, sTxy, sTxz);
@@ -601,20 +611,24 @@ __device__ __forceinline__ void volume_fx_nodal(const VolumeArgs& a, const int2*
     re[v * Nl] = fx_to_double(sum[v], kx + (v == 0 ? ge.U : v == 4 ? ge.t : ge.m));
 }
 
-// CTAs an SM holds at r registers a thread.
+// CTAs an SM holds at r registers a thread.  64 registers for both forms: the
+// rectilinear one at N = 4 took 0.188, 0.177, 0.182 and 0.156 ms with 40, 48, 56
+// and 64 (12 to 8 CTAs an SM); the per-node one 0.531, 0.520, 0.531 and 0.554 ms
+// with 56, 64, 72 and 80 (at N = 3 80 are 4% better).
 __host__ __device__ constexpr int fx_blocks(int threads, int r) { return 65536 / (threads * r); }
 
 template <int N>
-__global__ void __launch_bounds__(fx_rect_threads<N>(), fx_blocks(fx_rect_threads<N>(), N < 5 ? 48 : 64))
+__global__ void __launch_bounds__(fx_rect_threads<N>(), fx_blocks(fx_rect_threads<N>(), 64))
     volume_fx_rect_kernel(const __grid_constant__ VolumeArgs a, const __grid_constant__ FxTables<N, 3> T) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   constexpr int EPB = fx_rect_epb<N>();
   const int e = (int)blockIdx.x * EPB;
+  if (a.fxD == nullptr) grid_wait();
   volume_fx_rect<N>(a, T.d, a.ebeg + (long long)e, min(EPB, a.ecnt - e), smem_raw);
 }
 
 template <int N>
-__global__ void __launch_bounds__(fx_nodal_threads<N>(), fx_blocks(fx_nodal_threads<N>(), N < 7 ? 64 : 80))
+__global__ void __launch_bounds__(fx_nodal_threads<N>(), fx_blocks(fx_nodal_threads<N>(), N == 3 ? 80 : 64))
     volume_fx_nodal_kernel(const __grid_constant__ VolumeArgs a, const __grid_constant__ FxTables<N, 1> T) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   constexpr int EPB = fx_nodal_epb<N>();
@@ -626,7 +640,7 @@ __global__ void __launch_bounds__(fx_nodal_threads<N>(), fx_blocks(fx_nodal_thre
 // member, whose tables are copied to shared memory.
 template <int N, bool RECT>
 __global__ void __launch_bounds__(RECT ? fx_rect_threads<N>() : fx_nodal_threads<N>(),
-                                  fx_blocks(RECT ? fx_rect_threads<N>() : fx_nodal_threads<N>(), N < 7 ? 64 : 80))
+                                  fx_blocks(RECT ? fx_rect_threads<N>() : fx_nodal_threads<N>(), 64))
     volume_fx_ragged(const MemberDesc* __restrict__ d, const RaggedGroup* __restrict__ g) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   constexpr int EPB = RECT ? fx_rect_epb<N>() : fx_nodal_epb<N>(), ENT = (RECT ? 3 : 1) * fx_table_entries<N>();

@@ -21,6 +21,32 @@
 namespace numa {
 namespace {
 
+// ---- launches that overlap the end of the kernel before -----------------------
+// A launch with `early` may begin while the kernel before it on the stream
+// still runs: grid_wait returns once that one is complete and its writes are
+// visible, and comes before any access to what a kernel before wrote or reads
+// (each kernel waits, so all earlier ones are complete too); what is fixed at
+// bind may be read before it.  grid_next, after the wait, lets the next
+// launch begin.  Without `early` both do nothing.
+__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void grid_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+template <typename... K, typename... A>
+cudaError_t launch_kernel(void (*kernel)(K...), unsigned blocks, int threads, size_t smem, cudaStream_t s, bool early,
+                          const A&... args) {
+  cudaLaunchAttribute at;
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(blocks);
+  cfg.blockDim = dim3((unsigned)threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cfg.attrs = &at;
+  cfg.numAttrs = early ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+
 // ---- FP64-pipe-free conversions -------------------------------------------
 // The rare cases (subnormal, infinite, NaN) go through out-of-line functions:
 // an inline fallback would be predicated into every call and issue its FP64
@@ -233,6 +259,7 @@ struct NodeState64 {
 __device__ __forceinline__ NodeState64 gather_node64(const VolumeArgs& a, long long n) {
   const long long Ng = a.Ng;
   const int g = a.l2g[n];
+  grid_wait();
   const double* q = a.q + Ng + g;
   const double* w = static_cast<const double*>(a.prim) + g;
   NodeState64 z;
@@ -459,6 +486,8 @@ template <int N, bool AFF>
 __global__ void __launch_bounds__(((N + 1) * (N + 1) * (N + 1) + 31) / 32 * 32)
     volume_kernel(VolumeArgs a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  grid_wait();
+  grid_next();
   volume_element_lines<N, AFF>(a, a.ebeg + (long long)blockIdx.x, smem_raw);
 }
 
@@ -731,6 +760,8 @@ __global__ void __launch_bounds__(kDssBlock, sizeof(RT) == 8 ? 12 : 16) update_k
   {
     const int lt = a.order[base + threadIdx.x];
     const long long IA = base + lt;
+    grid_wait();
+    grid_next();
     if (IA < a.iend) {
       double s[5];
       if constexpr (BOX) dss_box<RT>(a, IA, s);
@@ -879,8 +910,7 @@ cudaError_t launch_volume_t(const VolumeArgs& a, cudaStream_t s) {
     attr_set.set();
   }
   if (a.ecnt <= 0) return cudaSuccess;
-  volume_kernel<N, AFF><<<a.ecnt, NT, smem, s>>>(a);
-  return cudaGetLastError();
+  return launch_kernel(volume_kernel<N, AFF>, (unsigned)a.ecnt, NT, smem, s, a.early != 0, a);
 }
 
 template <bool AFF>

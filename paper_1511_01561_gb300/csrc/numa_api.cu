@@ -79,6 +79,7 @@ VolumeArgs volume_args(const numa_ctx* c, const double* q, const void* prim, voi
   a.Ng = c->mesh.Ng;
   a.Nl = c->mesh.Nl;
   a.Ne = (int)c->mesh.Ne;
+  a.early = 1;
   a.ebeg = 0;
   a.ecnt = a.Ne;
   a.affine = volume_form(c);
@@ -112,6 +113,7 @@ UpdateArgs update_args(const numa_ctx* c, const void* re, const double* qk, cons
   a.out = out;
   a.Ng = c->mesh.Ng;
   a.Nl = c->mesh.Nl;
+  a.early = 1;
   a.ibeg = 0;
   a.iend = a.Ng;
   a.g = c->cfg.g;
@@ -341,12 +343,14 @@ cudaError_t enqueue_rk_step(numa_ctx* c, double dt, cudaStream_t s, cudaEvent_t*
       for (int k = 0; k < S && e == cudaSuccess; ++k) {
         if (st > 0) e = cudaStreamWaitEvent(s, c->ev_upd[k + 1 < S ? k + 1 : S - 1], 0);
         VolumeArgs va = volume_args(c, qi, c->L.prim, c->L.re);
+        va.early = 0;  // ordered by events with the other stream's kernels
         va.ebeg = P.ebeg[k];
         va.ecnt = P.ebeg[k + 1] - P.ebeg[k];
         if (e == cudaSuccess) e = launch_volume(c->mesh.N, c->cfg.precision, va, s);
         if (e == cudaSuccess) e = cudaEventRecord(c->ev_vol[k], s);
         if (e == cudaSuccess) e = cudaStreamWaitEvent(side, c->ev_vol[k], 0);
         UpdateArgs ua = stage_update(st);
+        ua.early = 0;
         ua.ibeg = P.ibeg[k];
         ua.iend = P.ibeg[k + 1];
         if (e == cudaSuccess) e = launch_update(c->cfg.precision, ua, side);
@@ -359,10 +363,13 @@ cudaError_t enqueue_rk_step(numa_ctx* c, double dt, cudaStream_t s, cudaEvent_t*
   for (int st = 0; st < ns; ++st) {
     const double* qi = ls ? q : qin[st];
     cudaError_t e = ev ? cudaEventRecord(ev[4 * st], s) : cudaSuccess;
-    if (e == cudaSuccess) e = launch_volume(c->mesh.N, c->cfg.precision, volume_args(c, qi, c->L.prim, c->L.re), s);
+    VolumeArgs va = volume_args(c, qi, c->L.prim, c->L.re);
+    UpdateArgs ua = stage_update(st);
+    if (ev) va.early = ua.early = 0;  // each kernel by itself between its events
+    if (e == cudaSuccess) e = launch_volume(c->mesh.N, c->cfg.precision, va, s);
     if (e == cudaSuccess && ev) e = cudaEventRecord(ev[4 * st + 1], s);
     if (e == cudaSuccess && ev) e = cudaEventRecord(ev[4 * st + 2], s);
-    if (e == cudaSuccess) e = launch_update(c->cfg.precision, stage_update(st), s);
+    if (e == cudaSuccess) e = launch_update(c->cfg.precision, ua, s);
     if (e == cudaSuccess && ev) e = cudaEventRecord(ev[4 * st + 3], s);
     if (e != cudaSuccess) return e;
   }

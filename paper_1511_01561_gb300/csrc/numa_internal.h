@@ -173,6 +173,7 @@ struct VolumeArgs {
                                 // and put into the rows of D, 4 bits per point of a line
   long long Ng, Nl;
   int Ne;
+  int early;           // the launch may begin before the kernel before it on the stream has ended
   int ebeg, ecnt;      // the launch covers elements [ebeg, ebeg + ecnt) (a slab, or all: 0, Ne)
   int affine;          // volume_form: 0 the per-node form; 1 every element is affine, the
                        // contravariant-flux form (FP32-mixed); 2 every element is also
@@ -202,6 +203,7 @@ struct UpdateArgs {
                        // write the primitives of out)
   int* flag;           // non-finite flag
   PrimArgs pa;         // primitive output of mode 1 (pa.q unused)
+  int early;           // the launch may begin before the kernel before it on the stream has ended
   // the launch covers global nodes [ibeg, iend): a slab (ibeg a multiple of
   // kDssBlock), or all: 0, Ng
   long long ibeg, iend;

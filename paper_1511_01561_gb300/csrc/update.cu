@@ -33,10 +33,10 @@ __global__ void __launch_bounds__(256) prim_kernel(PrimArgs a) {
 }
 
 template <int MODE, typename RT>
-void launch_update_m(const UpdateArgs& a, unsigned nb, int nt, cudaStream_t s) {
-  if (a.gvec) update_kernel<MODE, true, RT><<<nb, nt, 0, s>>>(a);
-  else if (a.box_N) update_kernel<MODE, false, RT, true><<<nb, nt, 0, s>>>(a);
-  else update_kernel<MODE, false, RT><<<nb, nt, 0, s>>>(a);
+cudaError_t launch_update_m(const UpdateArgs& a, unsigned nb, int nt, cudaStream_t s) {
+  void (*k)(UpdateArgs) = a.gvec ? update_kernel<MODE, true, RT> : a.box_N ? update_kernel<MODE, false, RT, true>
+                                                                           : update_kernel<MODE, false, RT>;
+  return launch_kernel(k, nb, nt, 0, s, a.early != 0, a);
 }
 
 }  // namespace
@@ -59,28 +59,14 @@ cudaError_t launch_update(int precision, const UpdateArgs& a, cudaStream_t s) {
   const int nt = kDssBlock;  // the kernel's block size: one block per DSS-order block
   const unsigned nb = (unsigned)((a.iend - a.ibeg + nt - 1) / nt);
   const bool f32 = precision == NUMA_FP32_MIXED;
-  if (a.mode == 0) {
-    if (f32) launch_update_m<0, float>(a, nb, nt, s);
-    else launch_update_m<0, double>(a, nb, nt, s);
-  } else if (a.mode == 3) {
-    if (f32) launch_update_m<3, float>(a, nb, nt, s);
-    else launch_update_m<3, double>(a, nb, nt, s);
-  } else if (a.mode == 4) {
-    if (a.first_stage) {
-      if (f32) launch_update_m<5, float>(a, nb, nt, s);
-      else launch_update_m<5, double>(a, nb, nt, s);
-    } else {
-      if (f32) launch_update_m<4, float>(a, nb, nt, s);
-      else launch_update_m<4, double>(a, nb, nt, s);
-    }
-  } else if (a.first_stage) {
-    if (f32) launch_update_m<2, float>(a, nb, nt, s);
-    else launch_update_m<2, double>(a, nb, nt, s);
-  } else {
-    if (f32) launch_update_m<1, float>(a, nb, nt, s);
-    else launch_update_m<1, double>(a, nb, nt, s);
-  }
-  return cudaGetLastError();
+  auto go = [&](auto mode) {
+    constexpr int M = decltype(mode)::value;
+    return f32 ? launch_update_m<M, float>(a, nb, nt, s) : launch_update_m<M, double>(a, nb, nt, s);
+  };
+  if (a.mode == 0) return go(std::integral_constant<int, 0>());
+  if (a.mode == 3) return go(std::integral_constant<int, 3>());
+  if (a.mode == 4) return a.first_stage ? go(std::integral_constant<int, 5>()) : go(std::integral_constant<int, 4>());
+  return a.first_stage ? go(std::integral_constant<int, 2>()) : go(std::integral_constant<int, 1>());
 }
 
 cudaError_t launch_volume_ragged(int N, int precision, bool affine, const MemberDesc* d, const RaggedGroup* g,

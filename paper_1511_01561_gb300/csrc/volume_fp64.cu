@@ -25,9 +25,8 @@ cudaError_t launch_fx_t(const VolumeArgs& a, cudaStream_t s) {
   if (a.fxD_host)
     for (int t = 0; t < DIRS * fx_table_entries<N>(); ++t) T.d[t] = a.fxD_host[t];
   const unsigned nb = (unsigned)((a.ecnt + EPB - 1) / EPB);
-  if constexpr (RECT) volume_fx_rect_kernel<N><<<nb, NT, smem, s>>>(a, T);
-  else volume_fx_nodal_kernel<N><<<nb, NT, smem, s>>>(a, T);
-  return cudaGetLastError();
+  if constexpr (RECT) return launch_kernel(volume_fx_rect_kernel<N>, nb, NT, smem, s, a.early != 0, a, T);
+  else return launch_kernel(volume_fx_nodal_kernel<N>, nb, NT, smem, s, a.early != 0, a, T);
 }
 
 template <int N, bool RECT>
