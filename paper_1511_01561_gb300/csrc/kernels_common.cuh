@@ -27,7 +27,8 @@ namespace {
 // visible, and comes before any access to what a kernel before wrote or reads
 // (each kernel waits, so all earlier ones are complete too); what is fixed at
 // bind may be read before it.  grid_next, after the wait, lets the next
-// launch begin.  Without `early` both do nothing.
+// launch begin.  Without `early` both do nothing.  numa_bind asks for it on
+// meshes of a few blocks per SM only (numa_ctx::early).
 __device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void grid_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
