@@ -21,15 +21,26 @@
 // the two vectors whose neighbours the column derivative reads ([2][nz][cols]
 // doubles); values needed only at their own node (q*_rho, s_W, q*_Theta) go
 // back into R, which the same thread reads at the end.  The derivative
-// applications run over all (level, column) pairs of the block; one thread
-// per column runs the banded LU sweeps.
-#include "kernels_common.cuh"
+// applications run over all (level, column) pairs of the block.
+//
+// Columns of up to kImexDense levels (DENSE): y = H^-1 r with the inverse as
+// fixed-point integers, and its derivatives likewise (fixed64.cuh), r in 56
+// bits relative to the largest value of its column.  A level is nz products
+// of three integer multiply-adds, all levels at once, against the 16 to 24
+// FP64 operations of the LU sweeps (16 cycles of an SM a warp each, one thread
+// per column level by level): at 33 levels 99 cycles against 320.  The inverse
+// is refined beyond FP64 on the host.  On the thin box of 64x64x8 elements at
+// N = 4 the DSS and this kernel went from 0.398 to 0.345 ms a step; the FP64
+// pipe is 57% busy and the phases wait for their global reads.  Taller columns take the LU factors, one
+// thread per column running the banded sweeps.
+#include "fixed64.cuh"
 
 namespace numa {
 namespace {
 
 constexpr int kImexThreads = 128;
 constexpr size_t kImexSmemMax = 200 * 1024;
+constexpr int kImexMinExp = 200, kImexMaxExp = 1800;  // biased exponents of a column's r taken as they are
 
 // Band entries [j0, j1] of row k of Dz that can be nonzero: the row of a node
 // inside element e couples to that element's N+1 nodes; a node shared by two
@@ -48,7 +59,7 @@ __device__ __forceinline__ void dz_row_range(int k, int N, int nz, int& j0, int&
 // Column c, level k is global node c + ncol k.  RADIAL = false: z-columns of
 // the box (W = U_z); RADIAL = true: radial columns of the shell (W = U . r_hat,
 // U^{n+1} = U* + (x_W - W*) r_hat).
-template <bool RADIAL>
+template <bool RADIAL, bool DENSE>
 __global__ void __launch_bounds__(kImexThreads) imex_column_kernel(ImexArgs a) {
   extern __shared__ __align__(16) double sm[];
   const int nz = a.nz, CPB = a.cols_per_block, N = a.N, W2 = 2 * a.N + 1, kl = a.kl, US = 1 + 4 * a.N;
@@ -60,9 +71,14 @@ __global__ void __launch_bounds__(kImexThreads) imex_column_kernel(ImexArgs a) {
   double* Ls = EY + plane;                   // [nz][kl]
   double* Us = Ls + (size_t)nz * kl;         // [nz][1 + 4N]
   int* Ps = reinterpret_cast<int*>(Us + (size_t)nz * US);  // [nz][3]
-  for (int t = threadIdx.x; t < nz * kl; t += blockDim.x) Ls[t] = a.Lf[t];
-  for (int t = threadIdx.x; t < nz * US; t += blockDim.x) Us[t] = a.Uf[t];
-  for (int t = threadIdx.x; t < 3 * nz; t += blockDim.x) Ps[t] = a.piv[t];
+  unsigned* key = reinterpret_cast<unsigned*>(EY + plane);  // DENSE: [CPB] largest |r| of each column (high word)
+  if constexpr (DENSE) {
+    if (threadIdx.x < CPB) key[threadIdx.x] = 0u;
+  } else {
+    for (int t = threadIdx.x; t < nz * kl; t += blockDim.x) Ls[t] = a.Lf[t];
+    for (int t = threadIdx.x; t < nz * US; t += blockDim.x) Us[t] = a.Uf[t];
+    for (int t = threadIdx.x; t < 3 * nz; t += blockDim.x) Ps[t] = a.piv[t];
+  }
   double* R = a.R;
   const long long col0 = (long long)blockIdx.x * CPB;
   const double nu = a.nu, tau = a.tau;
@@ -110,15 +126,47 @@ __global__ void __launch_bounds__(kImexThreads) imex_column_kernel(ImexArgs a) {
   // r = e + tau Dz(c2 (s_Theta - q*_Theta)) on the interior rows
   for (int t = threadIdx.x; t < items; t += blockDim.x) {
     const int k = t / CPB, cl = t - k * CPB;
-    if (k == 0 || k == nz - 1) continue;
-    int j0, j1;
-    dz_row_range(k, N, nz, j0, j1);
-    double acc = 0.0;
-    for (int j = j0; j <= j1; ++j) acc = fma(a.Dz[k * W2 + j], UT[(size_t)(k - N + j) * CPB + cl], acc);
-    EY[(size_t)k * CPB + cl] = fma(tau, acc, EY[(size_t)k * CPB + cl]);
+    if (k > 0 && k < nz - 1) {
+      int j0, j1;
+      dz_row_range(k, N, nz, j0, j1);
+      double acc = 0.0;
+      for (int j = j0; j <= j1; ++j) acc = fma(a.Dz[k * W2 + j], UT[(size_t)(k - N + j) * CPB + cl], acc);
+      EY[(size_t)k * CPB + cl] = fma(tau, acc, EY[(size_t)k * CPB + cl]);
+    }
+    if constexpr (DENSE)
+      if (col0 + cl < ncol) atomicMax(&key[cl], (unsigned)__double2hiint(EY[(size_t)k * CPB + cl]) & 0x7fffffffu);
   }
   __syncthreads();
 
+  // exponent of a column's r; above kImexMaxExp (infinities and NaN too) the
+  // column's y is NaN, as the sweeps would make it
+  auto col_exp = [&](int cl) { return key[cl] ? max((int)(key[cl] >> 20), kImexMinExp) : 1023; };
+  int2* Ri = reinterpret_cast<int2*>(EY);           // DENSE: r, then
+  long long* Yi = reinterpret_cast<long long*>(UT);  // y
+  if constexpr (DENSE) {
+    for (int t = threadIdx.x; t < items; t += blockDim.x) {
+      const int cl = t % CPB, E = col_exp(cl);
+      Ri[t] = col0 + cl < ncol && E <= kImexMaxExp ? fx_split(fx_of(EY[t], E + 2)) : make_int2(0, 0);
+    }
+    __syncthreads();
+    // three levels of one column per thread (a warp's lanes are columns)
+    for (int t = threadIdx.x; t < (nz + 2) / 3 * CPB; t += blockDim.x) {
+      const int k = t / CPB * 3, cl = t % CPB;
+      const int2* H0 = a.Hi + (size_t)k * nz;
+      const int2* H1 = k + 1 < nz ? H0 + nz : H0;
+      const int2* H2 = k + 2 < nz ? H0 + 2 * nz : H0;
+      long long h0 = 0, m0 = kFxHalf, h1 = 0, m1 = kFxHalf, h2 = 0, m2 = kFxHalf;
+      for (int j = 0; j < nz; ++j) {
+        const int2 r = Ri[j * CPB + cl];
+        fx_mac(h0, m0, __ldg(H0 + j), r.x, r.y);
+        fx_mac(h1, m1, __ldg(H1 + j), r.x, r.y);
+        fx_mac(h2, m2, __ldg(H2 + j), r.x, r.y);
+      }
+      Yi[k * CPB + cl] = fx_sum(h0, m0);
+      if (k + 1 < nz) Yi[(k + 1) * CPB + cl] = fx_sum(h1, m1);
+      if (k + 2 < nz) Yi[(k + 2) * CPB + cl] = fx_sum(h2, m2);
+    }
+  } else {
   // H y = r: forward elimination with the recorded row swaps, back substitution
   for (int cl = threadIdx.x; cl < CPB; cl += blockDim.x) {
     if (col0 + cl >= ncol) break;
@@ -144,6 +192,7 @@ __global__ void __launch_bounds__(kImexThreads) imex_column_kernel(ImexArgs a) {
   }
   __syncthreads();
   for (int t = threadIdx.x; t < items; t += blockDim.x) UT[t] = a.th0[t / CPB] * EY[t];
+  }
   __syncthreads();
 
   // x_rho = q*_rho - tau G y, x_Theta = q*_Theta - tau G(theta0 y), x_W = s_W + y
@@ -155,18 +204,37 @@ __global__ void __launch_bounds__(kImexThreads) imex_column_kernel(ImexArgs a) {
     const long long g = node(col, k);
     int j0, j1;
     dz_row_range(k, N, nz, j0, j1);
-    double dy = 0.0, dty = 0.0;
-    for (int j = j0; j <= j1; ++j) {
-      const double d = a.Dz[k * W2 + j];
-      const size_t o = (size_t)(k - N + j) * CPB + c;
-      dy = fma(d, EY[o], dy);
-      dty = fma(d, UT[o], dty);
-    }
     const size_t o = (size_t)k * CPB + c;
-    const double yk = EY[o];
+    double dy = 0.0, dty = 0.0, yk, tyk = 0.0;
+    if constexpr (DENSE) {
+      long long h = 0, m = kFxHalf, th = 0, tm = kFxHalf;
+      for (int j = j0; j <= j1; ++j) {
+        const long long y = Yi[(k - N + j) * CPB + c];
+        const int yl = (int)((unsigned)y & kFxMask), yh = (int)(y >> kFxBits);
+        fx_mac(h, m, __ldg(a.DzI + k * W2 + j), yl, yh);
+        fx_mac(th, tm, __ldg(a.DtI + k * W2 + j), yl, yh);
+      }
+      const int E = col_exp(c);
+      const bool bad = E > kImexMaxExp;
+      const int Eu = bad ? 1023 : E;
+      yk = bad ? __hiloint2double(0x7ff80000, 0) : fx_to_double(Yi[o], Eu + a.y_exp);
+      dy = fx_to_double(fx_sum(h, m), Eu + a.d_exp);
+      dty = fx_to_double(fx_sum(th, tm), Eu + a.t_exp);
+      if (bad) dy = dty = yk;
+      if constexpr (RADIAL) tyk = a.th0[k] * yk;
+    } else {
+      for (int j = j0; j <= j1; ++j) {
+        const double d = a.Dz[k * W2 + j];
+        const size_t oj = (size_t)(k - N + j) * CPB + c;
+        dy = fma(d, EY[oj], dy);
+        dty = fma(d, UT[oj], dty);
+      }
+      yk = EY[o];
+      if constexpr (RADIAL) tyk = UT[o];
+    }
     if constexpr (RADIAL) {
       dy = fma(a.r2[k], yk, dy);
-      dty = fma(a.r2[k], UT[o], dty);
+      dty = fma(a.r2[k], tyk, dty);
     }
     const double xr = fma(-tau, dy, R[g]);
     const double xw = R[3 * Ng + g] + yk;
@@ -201,8 +269,12 @@ DeviceFlags imex_attr;
 
 template <bool RADIAL>
 cudaError_t set_imex_attr() {
-  return cudaFuncSetAttribute(imex_column_kernel<RADIAL>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              (int)kImexSmemMax);
+  cudaError_t e = cudaFuncSetAttribute(imex_column_kernel<RADIAL, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)kImexSmemMax);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(imex_column_kernel<RADIAL, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)kImexSmemMax);
+  return e;
 }
 
 }  // namespace
@@ -241,8 +313,15 @@ cudaError_t launch_imex(const ImexArgs& a, cudaStream_t s) {
   if (smem > kImexSmemMax || !imex_attr.has()) return cudaErrorInvalidValue;
   if (a.ncol == 0) return cudaSuccess;
   const long long blocks = (a.ncol + a.cols_per_block - 1) / a.cols_per_block;
-  if (a.nrm) imex_column_kernel<true><<<(unsigned)blocks, kImexThreads, smem, s>>>(a);
-  else imex_column_kernel<false><<<(unsigned)blocks, kImexThreads, smem, s>>>(a);
+  if (a.Hi && a.nz <= kImexDense) {
+    const size_t dense = sizeof(double) * 2 * (size_t)a.nz * a.cols_per_block + sizeof(unsigned) * a.cols_per_block;
+    if (a.nrm) imex_column_kernel<true, true><<<(unsigned)blocks, kImexThreads, dense, s>>>(a);
+    else imex_column_kernel<false, true><<<(unsigned)blocks, kImexThreads, dense, s>>>(a);
+  } else if (a.nrm) {
+    imex_column_kernel<true, false><<<(unsigned)blocks, kImexThreads, smem, s>>>(a);
+  } else {
+    imex_column_kernel<false, false><<<(unsigned)blocks, kImexThreads, smem, s>>>(a);
+  }
   return cudaGetLastError();
 }
 

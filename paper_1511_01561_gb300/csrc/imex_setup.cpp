@@ -43,8 +43,8 @@ bool imex_supported(const numa_config& c, long long* ncol, int* nz, std::string*
 }
 
 size_t imex_table_doubles(int nz, int N) {
-  const size_t n = (size_t)nz;
-  return n * (2 * N + 1) + 4 * n + 2 * (n * 2 * N + n * (1 + 4 * N));
+  const size_t z = (size_t)nz, w = 2 * (size_t)N + 1;
+  return z * w + 4 * z + 2 * (z * 2 * N + z * (1 + 4 * N)) + (nz <= kImexDense ? 2 * z * w + 2 * z * z : 0);
 }
 
 namespace {
@@ -154,16 +154,15 @@ bool imex_operator(const numa_config& c, const HostMesh& m, ImexTables& t, std::
   return true;
 }
 
-bool imex_factor(const ImexTables& t, double tau, std::vector<double>& Lf, std::vector<double>& Uf,
-                 std::vector<int>& piv, int* ku, std::string& err) {
-  const int nz = t.nz, N = t.N, W2 = 2 * N + 1, kl = 2 * N, US = 1 + 4 * N;
+// H = I - tau^2 (Dz C2 G T0 + g G) on the interior rows, identity rows at the walls.
+static std::vector<double> imex_matrix(const ImexTables& t, double tau) {
+  const int nz = t.nz, N = t.N, W2 = 2 * N + 1, kl = 2 * N;
   auto dz = [&](int i, int j) -> double {
     const int d = j - i + N;
     return (d >= 0 && d < W2) ? t.Dz[(size_t)i * W2 + d] : 0.0;
   };
   // G = Dz + diag(2/r): the divergence along the column
   auto gd = [&](int i, int j) -> double { return i == j ? dz(i, j) + t.r2[i] : dz(i, j); };
-  // H = I - tau^2 (Dz C2 G T0 + g G) on the interior rows, identity rows at the walls
   std::vector<double> H((size_t)nz * nz, 0.0);
   for (int i = 0; i < nz; ++i) {
     H[(size_t)i * nz + i] = 1.0;
@@ -175,6 +174,13 @@ bool imex_factor(const ImexTables& t, double tau, std::vector<double>& Lf, std::
       H[(size_t)i * nz + j] -= tau * tau * s;
     }
   }
+  return H;
+}
+
+bool imex_factor(const ImexTables& t, double tau, std::vector<double>& Lf, std::vector<double>& Uf,
+                 std::vector<int>& piv, int* ku, std::string& err) {
+  const int nz = t.nz, N = t.N, kl = 2 * N, US = 1 + 4 * N;
+  std::vector<double> H = imex_matrix(t, tau);
   // Gaussian elimination with partial pivoting inside the band; the row swap
   // of step k acts on the unfinished columns, so the solve applies swap k and
   // then the multipliers of step k, in that order
@@ -219,6 +225,84 @@ bool imex_factor(const ImexTables& t, double tau, std::vector<double>& Lf, std::
       }
   }
   *ku = kumax;
+  return true;
+}
+
+// x += a b in double-double arithmetic.
+static void dd_mac(double& hi, double& lo, double a, double b) {
+  const double p = a * b, e = std::fma(a, b, -p), s = hi + p, t = s - hi;
+  lo += ((hi - (s - t)) + (p - t)) + e;
+  hi = s;
+}
+
+bool imex_dense(const ImexTables& t, double tau, const std::vector<double>& Lf, const std::vector<double>& Uf,
+                const std::vector<int>& piv, ImexDense& out) {
+  const int nz = t.nz, N = t.N, W2 = 2 * N + 1, kl = 2 * N, US = 1 + 4 * N;
+  const std::vector<double> H = imex_matrix(t, tau);
+  auto solve = [&](std::vector<double>& y) {
+    for (int k = 0; k < nz; ++k) {
+      std::swap(y[k], y[piv[3 * k]]);
+      for (int i = 1; i <= piv[3 * k + 1]; ++i) y[k + i] -= Lf[(size_t)k * kl + i - 1] * y[k];
+    }
+    for (int k = nz - 1; k >= 0; --k) {
+      for (int j = 1; j <= piv[3 * k + 2]; ++j) y[k] -= Uf[(size_t)k * US + j] * y[k + j];
+      y[k] *= Uf[(size_t)k * US];
+    }
+  };
+  // columns of H^-1 with one step of refinement, x + dx
+  std::vector<double> X((size_t)nz * nz), dX((size_t)nz * nz), x(nz), r(nz);
+  for (int c = 0; c < nz; ++c) {
+    std::fill(x.begin(), x.end(), 0.0);
+    x[c] = 1.0;
+    solve(x);
+    for (int i = 0; i < nz; ++i) {
+      double hi = i == c ? 1.0 : 0.0, lo = 0.0;
+      for (int j = std::max(0, i - kl); j <= std::min(nz - 1, i + kl); ++j) dd_mac(hi, lo, -H[(size_t)i * nz + j], x[j]);
+      r[i] = hi + lo;
+    }
+    solve(r);
+    for (int i = 0; i < nz; ++i) {
+      X[(size_t)i * nz + c] = x[i];
+      dX[(size_t)i * nz + c] = r[i];
+    }
+  }
+  // rows of x + dx as 2^s times them, (signed low 29 bits, rest); s from the largest row sum
+  auto table = [&](const std::vector<double>& v, const double* dv, int cols, int bits, std::vector<int2>& o, int& s) {
+    double top = 0.0;
+    for (int i = 0; i < nz; ++i) {
+      double row = 0.0;
+      for (int j = 0; j < cols; ++j) row += std::fabs(v[(size_t)i * cols + j]);
+      top = std::max(top, row);
+    }
+    if (!(top > 0.0) || !std::isfinite(top)) return false;
+    int e2 = 0;
+    std::frexp(top, &e2);  // top < 2^e2
+    s = bits - e2;
+    if (s < -150 || s > 250) return false;
+    o.resize((size_t)nz * cols);
+    for (size_t k = 0; k < o.size(); ++k) {
+      // (v scaled has at most 53 bits above its last one: whole part and rest are exact)
+      const double a = std::ldexp(v[k], s), w = std::nearbyint(a);
+      const long long q = (long long)w + std::llrint((a - w) + (dv ? std::ldexp(dv[k], s) : 0.0));
+      const long long h = (q + (1LL << 28)) >> 29;
+      o[k] = make_int2((int)(q - (h << 29)), (int)h);
+    }
+    return true;
+  };
+  std::vector<double> Dt(t.Dz);
+  for (int k = 0; k < nz; ++k)
+    for (int j = 0; j < W2; ++j) {
+      const int l = k - N + j;
+      Dt[(size_t)k * W2 + j] = l >= 0 && l < nz ? t.Dz[(size_t)k * W2 + j] * t.th0[l] : 0.0;
+    }
+  int sH = 0, sD = 0, sT = 0;
+  // (59 bits: with the refinement the row sums stay below 2^60)
+  if (!table(X, dX.data(), nz, 59, out.Hi, sH) || !table(t.Dz, nullptr, W2, 58, out.DzI, sD) ||
+      !table(Dt, nullptr, W2, 58, out.DtI, sT))
+    return false;
+  out.y_exp = 66 - sH;
+  out.d_exp = 124 - sH - sD;
+  out.t_exp = 124 - sH - sT;
   return true;
 }
 

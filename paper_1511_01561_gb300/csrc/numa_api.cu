@@ -201,6 +201,7 @@ int rk_stages(const numa_ctx* c) {
 struct ImexPtrs {
   double *Dz, *c2, *th0, *gl, *r2, *Lf[2], *Uf[2];
   int* piv[2];
+  int2 *DzI, *DtI, *Hi[2];  // columns of up to kImexDense levels
 };
 
 ImexPtrs imex_ptrs(const numa_ctx* c) {
@@ -215,6 +216,10 @@ ImexPtrs imex_ptrs(const numa_ctx* c) {
   p.Uf[0] = p.Lf[0] + (size_t)nz * 2 * N;
   p.Lf[1] = p.Uf[0] + (size_t)nz * (1 + 4 * N);
   p.Uf[1] = p.Lf[1] + (size_t)nz * 2 * N;
+  p.DzI = reinterpret_cast<int2*>(p.Uf[1] + (size_t)nz * (1 + 4 * N));
+  p.DtI = p.DzI + (size_t)nz * (2 * N + 1);
+  p.Hi[0] = p.DtI + (size_t)nz * (2 * N + 1);
+  p.Hi[1] = p.Hi[0] + (size_t)nz * nz;
   p.piv[0] = c->L.imex_piv;
   p.piv[1] = c->L.imex_piv + 3 * nz;
   return p;
@@ -244,6 +249,16 @@ int imex_prepare(numa_ctx* c, double dt) {
     e = cudaMemcpyAsync(p.Lf[f], Lf.data(), Lf.size() * 8, cudaMemcpyHostToDevice, c->stream);
     if (e == cudaSuccess) e = cudaMemcpyAsync(p.Uf[f], Uf.data(), Uf.size() * 8, cudaMemcpyHostToDevice, c->stream);
     if (e == cudaSuccess) e = cudaMemcpyAsync(p.piv[f], piv.data(), 3 * nz * sizeof(int), cudaMemcpyHostToDevice, c->stream);
+    ImexDense d;
+    c->imex_int[f] = t.nz <= kImexDense && imex_dense(t, f == 0 ? dt : 0.5 * dt, Lf, Uf, piv, d);
+    if (c->imex_int[f]) {
+      c->imex_exp[f][0] = d.y_exp;
+      c->imex_exp[f][1] = d.d_exp;
+      c->imex_exp[f][2] = d.t_exp;
+      if (e == cudaSuccess) e = cudaMemcpyAsync(p.Hi[f], d.Hi.data(), d.Hi.size() * 8, cudaMemcpyHostToDevice, c->stream);
+      if (e == cudaSuccess) e = cudaMemcpyAsync(p.DzI, d.DzI.data(), d.DzI.size() * 8, cudaMemcpyHostToDevice, c->stream);
+      if (e == cudaSuccess) e = cudaMemcpyAsync(p.DtI, d.DtI.data(), d.DtI.size() * 8, cudaMemcpyHostToDevice, c->stream);
+    }
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);  // the host vectors are reused
   }
   if (e != cudaSuccess) return cuda_fail(c, e, "1D-IMEX factor upload");
@@ -285,6 +300,12 @@ cudaError_t enqueue_imex_step(numa_ctx* c, double dt, bool start, cudaStream_t s
     a.Lf = p.Lf[f];
     a.Uf = p.Uf[f];
     a.piv = p.piv[f];
+    a.Hi = c->imex_int[f] ? p.Hi[f] : nullptr;
+    a.DzI = p.DzI;
+    a.DtI = p.DtI;
+    a.y_exp = c->imex_exp[f][0];
+    a.d_exp = c->imex_exp[f][1];
+    a.t_exp = c->imex_exp[f][2];
     a.N = c->imex.N;
     a.nz = c->imex.nz;
     a.kl = c->imex.kl;

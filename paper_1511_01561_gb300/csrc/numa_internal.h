@@ -235,6 +235,10 @@ struct ImexArgs {
   const double* Uf;     // [nz][1 + ku]: 1 / U_kk, then U_{k,k+1} .. U_{k,k+ku}
   const int* piv;       // [nz][3]: row swapped with row k at step k, multipliers used (last
                         // nonzero), U entries used (last nonzero) of row k
+  // columns of up to kImexDense levels: H^-1 [nz][nz], Dz and Dz theta0
+  // [nz][2N+1] as fixed-point integers (imex_dense); null: the LU factors
+  const int2 *Hi, *DzI, *DtI;
+  int y_exp, d_exp, t_exp;  // exponents of y, Dz y and Dz(theta0 y)
   int N, nz, kl, ku, cols_per_block;
   long long ncol, Ng;
   double cR, tau, nu;     // q* = qprev + cR R; (I - tau L) correction; filter strength
@@ -259,6 +263,18 @@ bool imex_operator(const numa_config& c, const HostMesh& m, ImexTables& t, std::
 bool imex_factor(const ImexTables& t, double tau, std::vector<double>& Lf, std::vector<double>& Uf,
                  std::vector<int>& piv, int* ku, std::string& err);
 size_t imex_table_doubles(int nz, int N);
+// Columns of at most this many levels are solved with the inverse of the Schur
+// matrix (imex.cu).
+constexpr int kImexDense = 64;
+// The integers of one factored matrix: H^-1 (refined beyond FP64), Dz and
+// Dz theta0, each with its largest row sum scaled below 2^60 (H^-1) or 2^58, and
+// the exponents of their products.  False if they are out of range.
+struct ImexDense {
+  std::vector<int2> Hi, DzI, DtI;
+  int y_exp = 0, d_exp = 0, t_exp = 0;
+};
+bool imex_dense(const ImexTables& t, double tau, const std::vector<double>& Lf, const std::vector<double>& Uf,
+                const std::vector<int>& piv, ImexDense& d);
 
 // One application of the Boyd-Vandeven filter (element part).
 struct FilterArgs {
@@ -380,6 +396,8 @@ struct numa_ctx {
   long long imex_ncol = 0;
   double imex_dt = 0.0;
   int imex_ku[2] = {0, 0};  // upper bandwidths of the factors for dt and dt/2
+  bool imex_int[2] = {false, false};  // their fixed-point inverses are in the workspace, with these exponents
+  int imex_exp[2][3] = {};
   bool imex_factored = false;
   bool imex_started = false;
 };

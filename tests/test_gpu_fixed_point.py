@@ -102,3 +102,29 @@ def test_rect_nonfinite_elements(numa, orc, bad):
     near = np.unique(e[(e == g).any(axis=1)])
     far = np.setdiff1d(np.arange(m.Ng), near)
     assert np.array_equal(Rg[:, far], R0[:, far])
+
+
+# columns of 61 and 64 levels (the tallest solved with the inverse) and of 65
+# and 73 (the LU factors), at a vertical acoustic Courant number of 2 to 4
+@pytest.mark.parametrize("N,nez", [(4, 15), (7, 9), (4, 16), (8, 9)])
+def test_imex_column_heights(numa, orc, N, nez):
+    from oracle import imex
+
+    cfg = I.box((2, 1, nez), N, L=(4000.0, 2000.0, 250.0 * nez))
+    ic = ("bubble", (0.5, 600.0, 2000.0, 1000.0, 120.0 * nez))
+    dt = 3.0 * 250.0 * 0.5 * (1.0 - np.cos(np.pi / N)) / 350.0
+    m = orc.Mesh(cfg)
+    q = m.init_state(*ic)
+    q[1:4] += np.random.default_rng(N).uniform(-0.1, 0.1, (3, m.Ng))
+    qo, _ = imex.run_imex(m, q, dt, 3, 0.1)
+    s = numa.Solver(cfg, "fp64")
+    try:
+        s.set_time_scheme("imex")
+        s.set_robert_asselin(0.1)
+        s.set_state(q)
+        s.run(dt, 3)
+        qg = s.get_state().numpy()
+    finally:
+        s.close()
+    err = np.abs(qg - qo).max(axis=1) / np.maximum(np.abs(qo).max(axis=1), 1e-30)
+    assert err.max() <= 1e-10, err
