@@ -19,9 +19,10 @@
 //
 // One block holds cols_per_block consecutive columns.  Shared memory keeps
 // the two vectors whose neighbours the column derivative reads ([2][nz][cols]
-// doubles); values needed only at their own node (q*_rho, s_W, q*_Theta) go
-// back into R, which the same thread reads at the end.  The derivative
-// applications run over all (level, column) pairs of the block.
+// doubles) and, in the integer form, six values that the same thread needs
+// again at the end (q*_rho, s_W, q*_Theta and the filter's first part); the LU
+// form leaves those in R and qbar^n.  The derivative applications run over
+// all (level, column) pairs of the block.
 //
 // Columns of up to kImexDense levels (DENSE): y = H^-1 r with the inverse as
 // fixed-point integers, and its derivatives likewise (fixed64.cuh), r in 56
@@ -30,15 +31,20 @@
 // FP64 operations of the LU sweeps (16 cycles of an SM a warp each, one thread
 // per column level by level): at 33 levels 99 cycles against 320.  The inverse
 // is refined beyond FP64 on the host.  On the thin box of 64x64x8 elements at
-// N = 4 the DSS and this kernel went from 0.398 to 0.345 ms a step; the FP64
-// pipe is 57% busy and the phases wait for their global reads.  Taller columns take the LU factors, one
-// thread per column running the banded sweeps.
+// N = 4 the DSS and this kernel went from 0.398 to 0.348 ms a step.  All loads
+// of a phase before its first store (0.348 -> 0.322 ms with 128 threads, 0.313
+// with 256), and the six values in shared memory instead of global memory with
+// up to 384 threads, three blocks an SM (0.309 ms; the shell 0.551 -> 0.509);
+// two blocks an SM and no spills: 0.325.  The FP64 operations of the explicit
+// step, the first derivative and the filter (0.154 ms of their pipe) bound it
+// now.  Taller columns take the LU factors, one thread per column running the
+// banded sweeps.
 #include "fixed64.cuh"
 
 namespace numa {
 namespace {
 
-constexpr int kImexThreads = 128;
+constexpr int kImexThreads = 128, kImexDenseThreads = 384;
 constexpr size_t kImexSmemMax = 200 * 1024;
 constexpr int kImexMinExp = 200, kImexMaxExp = 1800;  // biased exponents of a column's r taken as they are
 
@@ -60,7 +66,7 @@ __device__ __forceinline__ void dz_row_range(int k, int N, int nz, int& j0, int&
 // the box (W = U_z); RADIAL = true: radial columns of the shell (W = U . r_hat,
 // U^{n+1} = U* + (x_W - W*) r_hat).
 template <bool RADIAL, bool DENSE>
-__global__ void __launch_bounds__(kImexThreads) imex_column_kernel(ImexArgs a) {
+__global__ void __launch_bounds__(DENSE ? kImexDenseThreads : kImexThreads, DENSE ? 3 : 4) imex_column_kernel(ImexArgs a) {
   extern __shared__ __align__(16) double sm[];
   const int nz = a.nz, CPB = a.cols_per_block, N = a.N, W2 = 2 * a.N + 1, kl = a.kl, US = 1 + 4 * a.N;
   const long long Ng = a.Ng, ncol = a.ncol;
@@ -71,7 +77,10 @@ __global__ void __launch_bounds__(kImexThreads) imex_column_kernel(ImexArgs a) {
   double* Ls = EY + plane;                   // [nz][kl]
   double* Us = Ls + (size_t)nz * kl;         // [nz][1 + 4N]
   int* Ps = reinterpret_cast<int*>(Us + (size_t)nz * US);  // [nz][3]
-  unsigned* key = reinterpret_cast<unsigned*>(EY + plane);  // DENSE: [CPB] largest |r| of each column (high word)
+  // DENSE: q*_rho, s_W, q*_Theta and qbar^n of rho', W, Theta' without x, [6][nz][cols],
+  // then [CPB] largest |r| of each column (high word)
+  double* PK = EY + plane;
+  unsigned* key = reinterpret_cast<unsigned*>(PK + 6 * plane);
   if constexpr (DENSE) {
     if (threadIdx.x < CPB) key[threadIdx.x] = 0u;
   } else {
@@ -92,18 +101,27 @@ __global__ void __launch_bounds__(kImexThreads) imex_column_kernel(ImexArgs a) {
     const long long col = col0 + cl;
     if (col >= ncol) continue;
     const long long g = node(col, k);
-    double qst[5], sv[5];
+    // (all loads before the first store, which the compiler cannot move them over)
+    double qst[5], sv[5], qn[5];
 #pragma unroll
     for (int v = 0; v < 5; ++v) {
-      const double qn = a.q[v * Ng + g], qp = a.qprev[v * Ng + g];
-      qst[v] = fma(a.cR, R[v * Ng + g], qp);
-      sv[v] = fma(2.0, qn, -qp);  // s = 2 q^n - qprev, so qprev - 2 q^n = -s
+      qn[v] = a.q[v * Ng + g];
+      sv[v] = a.qprev[v * Ng + g];
+      qst[v] = R[v * Ng + g];
+    }
+#pragma unroll
+    for (int v = 0; v < 5; ++v) {
+      const double qp = sv[v];
+      qst[v] = fma(a.cR, qst[v], qp);
+      sv[v] = fma(2.0, qn[v], -qp);  // s = 2 q^n - qprev, so qprev - 2 q^n = -s
       if (!RADIAL && (v == 1 || v == 2)) {
         a.q[v * Ng + g] = qst[v];
-        a.qs[v * Ng + g] = fma(nu, qst[v] - sv[v], qn);  // x = q* for U and V
+        a.qs[v * Ng + g] = fma(nu, qst[v] - sv[v], qn[v]);  // x = q* for U and V
       } else {
         if (RADIAL && v >= 1 && v <= 3) a.q[v * Ng + g] = qst[v];
-        a.qs[v * Ng + g] = fma(-nu, sv[v], qn);  // q^n + nu (qprev - 2 q^n)
+        const double b = fma(-nu, sv[v], qn[v]);  // q^n + nu (qprev - 2 q^n)
+        if (DENSE && (v == 0 || v >= 3)) PK[(v == 0 ? 3 : v + 1) * plane + t] = b;
+        else a.qs[v * Ng + g] = b;
       }
     }
     double wst = qst[3], swv = sv[3];
@@ -113,9 +131,15 @@ __global__ void __launch_bounds__(kImexThreads) imex_column_kernel(ImexArgs a) {
       swv = fma(sv[1], nx, fma(sv[2], ny, sv[3] * nz_));
       R[Ng + g] = wst;
     }
-    R[g] = qst[0];
-    R[3 * Ng + g] = swv;
-    R[4 * Ng + g] = qst[4];
+    if constexpr (DENSE) {
+      PK[t] = qst[0];
+      PK[plane + t] = swv;
+      PK[2 * plane + t] = qst[4];
+    } else {
+      R[g] = qst[0];
+      R[3 * Ng + g] = swv;
+      R[4 * Ng + g] = qst[4];
+    }
     const size_t o = (size_t)k * CPB + cl;
     UT[o] = a.c2[k] * (sv[4] - qst[4]);
     const double e = wst - swv;
@@ -202,6 +226,12 @@ __global__ void __launch_bounds__(kImexThreads) imex_column_kernel(ImexArgs a) {
     const long long col = col0 + c;
     if (col >= ncol) continue;
     const long long g = node(col, k);
+    // (loads first, as above)
+    const double R0 = DENSE ? PK[t] : R[g], R3 = DENSE ? PK[plane + t] : R[3 * Ng + g];
+    const double R4 = DENSE ? PK[2 * plane + t] : R[4 * Ng + g];
+    const double s0 = DENSE ? PK[3 * plane + t] : a.qs[g], s3 = DENSE ? PK[4 * plane + t] : a.qs[3 * Ng + g];
+    const double s4 = DENSE ? PK[5 * plane + t] : a.qs[4 * Ng + g];
+    const double q1 = a.q[Ng + g], q2 = a.q[2 * Ng + g];
     int j0, j1;
     dz_row_range(k, N, nz, j0, j1);
     const size_t o = (size_t)k * CPB + c;
@@ -236,32 +266,29 @@ __global__ void __launch_bounds__(kImexThreads) imex_column_kernel(ImexArgs a) {
       dy = fma(a.r2[k], yk, dy);
       dty = fma(a.r2[k], tyk, dty);
     }
-    const double xr = fma(-tau, dy, R[g]);
-    const double xw = R[3 * Ng + g] + yk;
-    const double xt = fma(-tau, dty, R[4 * Ng + g]);
-    a.q[g] = xr;
-    a.q[4 * Ng + g] = xt;
-    a.qs[g] = fma(nu, xr, a.qs[g]);
-    a.qs[4 * Ng + g] = fma(nu, xt, a.qs[4 * Ng + g]);
-    double xu, xv, xz;
+    const double xr = fma(-tau, dy, R0);
+    const double xw = R3 + yk;
+    const double xt = fma(-tau, dty, R4);
+    double xu = q1, xv = q2, xz = xw;
     if constexpr (RADIAL) {
       const double dw = xw - R[Ng + g];  // x_W - W*
-      xu = fma(dw, a.nrm[g], a.q[Ng + g]);
-      xv = fma(dw, a.nrm[Ng + g], a.q[2 * Ng + g]);
+      xu = fma(dw, a.nrm[g], q1);
+      xv = fma(dw, a.nrm[Ng + g], q2);
       xz = fma(dw, a.nrm[2 * Ng + g], a.q[3 * Ng + g]);
+      const double s1 = a.qs[Ng + g], s2 = a.qs[2 * Ng + g];
       a.q[Ng + g] = xu;
       a.q[2 * Ng + g] = xv;
-      a.qs[Ng + g] = fma(nu, xu, a.qs[Ng + g]);
-      a.qs[2 * Ng + g] = fma(nu, xv, a.qs[2 * Ng + g]);
-    } else {
-      xu = a.q[Ng + g];
-      xv = a.q[2 * Ng + g];
-      xz = xw;
+      a.qs[Ng + g] = fma(nu, xu, s1);
+      a.qs[2 * Ng + g] = fma(nu, xv, s2);
     }
-    a.q[3 * Ng + g] = xz;
-    a.qs[3 * Ng + g] = fma(nu, xz, a.qs[3 * Ng + g]);
-    if (nonfinite(xr) | nonfinite(xu) | nonfinite(xv) | nonfinite(xz) | nonfinite(xt)) atomicOr(a.flag, 1);
     write_prim<false>(a.pa, g, xr, xu, xv, xz, xt);
+    a.q[g] = xr;
+    a.q[3 * Ng + g] = xz;
+    a.q[4 * Ng + g] = xt;
+    a.qs[g] = fma(nu, xr, s0);
+    a.qs[3 * Ng + g] = fma(nu, xz, s3);
+    a.qs[4 * Ng + g] = fma(nu, xt, s4);
+    if (nonfinite(xr) | nonfinite(xu) | nonfinite(xv) | nonfinite(xz) | nonfinite(xt)) atomicOr(a.flag, 1);
   }
 }
 
@@ -282,6 +309,8 @@ cudaError_t set_imex_attr() {
 // Columns per block: kImexColsTarget while a block's shared memory stays
 // under kImexSmemMax / 2, fewer for tall columns.
 constexpr int kImexColsTarget = 32;
+// Levels up to which the integer form takes 32 columns a block (72 KB), 16 above.
+constexpr int kImexWide = 36;
 
 int imex_cols_per_block(int nz, int N) {
   for (int c = kImexColsTarget; c >= 32; c /= 2)
@@ -295,6 +324,11 @@ int imex_cols_per_block(int nz, int N) {
 // 2N multipliers and 1 + 4N U entries) and the pivot rows.
 size_t imex_smem_bytes(int nz, int N, int cols_per_block) {
   return sizeof(double) * (size_t)nz * (2 * (size_t)cols_per_block + 2 * N + 1 + 4 * N) + 3 * sizeof(int) * (size_t)nz;
+}
+
+// The integer form: eight vectors per column and a key.
+static size_t imex_dense_smem(int nz, int cols) {
+  return sizeof(double) * 8 * (size_t)nz * cols + sizeof(unsigned) * cols;
 }
 
 cudaError_t imex_kernel_setup() {
@@ -314,9 +348,16 @@ cudaError_t launch_imex(const ImexArgs& a, cudaStream_t s) {
   if (a.ncol == 0) return cudaSuccess;
   const long long blocks = (a.ncol + a.cols_per_block - 1) / a.cols_per_block;
   if (a.Hi && a.nz <= kImexDense) {
-    const size_t dense = sizeof(double) * 2 * (size_t)a.nz * a.cols_per_block + sizeof(unsigned) * a.cols_per_block;
-    if (a.nrm) imex_column_kernel<true, true><<<(unsigned)blocks, kImexThreads, dense, s>>>(a);
-    else imex_column_kernel<false, true><<<(unsigned)blocks, kImexThreads, dense, s>>>(a);
+    ImexArgs d = a;
+    d.cols_per_block = a.nz <= kImexWide ? 32 : 16;
+    const long long items = (long long)a.nz * d.cols_per_block;
+    int warps = 8;  // the count that leaves the fewest lanes idle in the last of its rounds
+    for (int w = 9; w <= kImexDenseThreads / 32; ++w)
+      if ((items + 32 * w - 1) / (32 * w) * w <= (items + 32 * warps - 1) / (32 * warps) * warps) warps = w;
+    const unsigned nb = (unsigned)((a.ncol + d.cols_per_block - 1) / d.cols_per_block);
+    const size_t dense = imex_dense_smem(a.nz, d.cols_per_block);
+    if (a.nrm) imex_column_kernel<true, true><<<nb, 32 * warps, dense, s>>>(d);
+    else imex_column_kernel<false, true><<<nb, 32 * warps, dense, s>>>(d);
   } else if (a.nrm) {
     imex_column_kernel<true, false><<<(unsigned)blocks, kImexThreads, smem, s>>>(a);
   } else {
