@@ -114,7 +114,7 @@ __device__ __forceinline__ double soft_pressure(const PrimArgs& a, double p0, do
   return __hiloint2double(zero ? (int)sign : (int)((unsigned)(b >> 32) | sign), zero ? 0 : (int)(unsigned)b);
 }
 
-// Whether soft_prim takes these values: rho > 0, Theta, U and Theta' zero or
+// Whether the integer form takes these values: rho > 0, Theta, U and Theta' zero or
 // normal and not extreme, |Theta'/Theta0| below 2^-5.
 __device__ __forceinline__ bool soft_ok(const PrimArgs& a, double rho, double Ux, double Uy, double Uz, double Th,
                                         double Tp, double p0, double iTh0) {

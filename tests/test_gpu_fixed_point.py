@@ -128,3 +128,26 @@ def test_imex_column_heights(numa, orc, N, nez):
         s.close()
     err = np.abs(qg - qo).max(axis=1) / np.maximum(np.abs(qo).max(axis=1), 1e-30)
     assert err.max() <= 1e-10, err
+
+
+# the equation of state of the update's primitive pass: |Theta'/Theta0| within
+# a factor 1.5 of 2^-k, both signs, zeros between them, on both sides of every
+# term count and of the end of the integer form (2^-5).  At rest without a
+# density perturbation the momentum tendency is the gradient of p' alone,
+# which is proportional to Theta' for small ratios: its error relative to its
+# own largest value is that of p'.
+@pytest.mark.parametrize("prec", ["fp64", "fp64_pairs"])
+@pytest.mark.parametrize("k", [1, 4, 5, 6, 10, 12, 15, 20, 30, 40, 60, 300, 900])
+def test_pressure_over_magnitudes(numa, orc, prec, k):
+    cfg = I.box((3, 2, 2), 4)
+    m = orc.Mesh(cfg)
+    rng = np.random.default_rng(k)
+    q = np.zeros((5, m.Ng))
+    x = np.ldexp(rng.uniform(0.5, 1.5, m.Ng), -k) * rng.choice([-1.0, 0.0, 1.0], m.Ng)
+    q[4] = x * m.ref()[1]
+    s = numa.Solver(cfg, prec)
+    try:
+        Rg = s.rhs(q).cpu().numpy()
+    finally:
+        s.close()
+    _check(Rg, m.rhs(q))
