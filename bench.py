@@ -80,16 +80,22 @@ def load_peaks():
 # with register-only FMA chains and 1.10 with FP64 mma.sync
 # (profiles/p0_arithmetic_peaks_gb300.md).
 FP64_PEAK_TFLOPS = 1.25
+FP64_PRIM_BYTES = 40  # u, theta, p' of one global node
 FP64_PEAK_SOURCE = "nominal FP64 FMA rate; measured 1.258 TFLOP/s (profiles/p0_arithmetic_peaks_gb300.md)"
+
+# 32x32+64-bit integer multiply-adds of the GB300, the unit the FP64 element
+# kernels form their products on: 152 SMs x 32 per clock x 2070 MHz
+# (register-only chains measured 28 per SM per clock).
+INT_PEAK_TOPS = 10.07
+INT_PEAK_SOURCE = "nominal rate of 32x32+64-bit integer multiply-adds, 32 per SM per clock"
 
 # DRAM bytes (read + write) per launch from one ncu capture of each kernel on
 # this workload (profiles/*_bubble_32x32x32_N4.md), valid only for the kernel
 # sources they were taken on (first 16 hex digits of the sha256 of the kernel
 # sources, see kernel_source_hash).
-NCU_TRAFFIC = {"kernels_sha256_16": "c162b3edd950e364", "workload": "bubble_32x32x32_N4",
-               "volume_fp64_affine": 223.360000e6 + 130.280448e6,
-               "volume_pairs_affine": 154.657536e6 + 122.701056e6,
-               "volume_fp32_affine": 139.263232e6 + 49.111808e6}
+NCU_TRAFFIC = {"kernels_sha256_16": "bbe726f310fc4b3f", "workload": "bubble_32x32x32_N4",
+               "volume_fp64_affine": 153.826560e6 + 123.796224e6,
+               "volume_fp32_affine": 139.233792e6 + 49.506816e6}
 
 # the sources the element kernels with committed traffic figures are built from
 KERNEL_SOURCES = ["kernels_common.cuh", "fixed64.cuh", "volume_fp64.cu", "volume_fp32.cu"]
@@ -138,12 +144,38 @@ def ncu_traffic(key: str, workload: str):
     return NCU_TRAFFIC.get(key)
 
 
+def volume_int_ops(N: int, form: str) -> float:
+    """32x32+64-bit integer multiply-adds per element node of the FP64 element
+    kernel of `form` (csrc/fixed64.cuh): three per product of 58-bit numbers.
+    The even/odd split of D leaves M products per line of N + 1 nodes: 15 lines'
+    worth a node in the rectilinear form, 36 and 45 chain-rule products in the
+    per-node form, and 9 flux products in both."""
+    P, H, O = N + 1, (N + 1) // 2, (N + 1) % 2
+    M = H * (H + O) + H * H + O * H
+    return 3.0 * (15.0 * M / P + 9) if form == "rect" else 3.0 * (36.0 * M / P + 45 + 9)
+
+
+def volume_fp64_roofline(N: int, form: str, Nl: int, t_s: float, nbytes: float, hbm_gbs: float) -> dict:
+    """The FP64 element kernel against the integer pipe its products run on
+    and, beside it, against the HBM time of its algorithmic bytes; the
+    instructions around the products bound it (profiles/).  The algorithmic
+    flops are those of Eq. 4 / Eq. 5 in this form."""
+    ops, fl = volume_int_ops(N, form) * Nl, volume_fp64_cost(N, form)[0] * Nl
+    return {"kernel": f"volume_fx_{form}_kernel<{N}>",
+            "form": "rectilinear (K_d D, w_i w_j w_k)" if form == "rect" else "per-node (Eq. 5)",
+            "bound": "alu", "achieved": ops / t_s / 1e12, "peak": INT_PEAK_TOPS, "unit": "T int multiply-adds/s",
+            "frac": ops / t_s / 1e12 / INT_PEAK_TOPS, "peak_source": INT_PEAK_SOURCE,
+            "int_ops_per_element_node": volume_int_ops(N, form), "algorithmic_flops": fl,
+            "algorithmic_tflops": fl / t_s / 1e12, "algorithmic_bytes": nbytes,
+            "hbm_frac": nbytes / t_s / 1e9 / hbm_gbs, "avg_launch_ms": 1e3 * t_s}
+
+
 def volume_fp64_cost(N: int, form: str) -> tuple:
-    """(flops, FP64 operations) per element node of the FP64 element kernel
-    of `form`.  A flop count takes an FMA as 2; an operation count takes an
-    FMA, a product and a sum as 1 each (each takes one slot of the FP64 pipe).
-    The 12 flux fields (U, the symmetric U (x) u + p' I, theta U) come
-    gathered: the update forms them once per global node.
+    """(flops, operations) per element node of the discrete operator in `form`.
+    A flop count takes an FMA as 2; an operation count takes an FMA, a product
+    and a sum as 1 each.  (The kernels form the products as integers, see
+    volume_int_ops.)  The 12 flux fields (U, the symmetric U (x) u + p' I,
+    theta U) are taken as given.
     - "nodal", the per-node form of Eq. 5 (any element): each field
       differentiated along xi, eta and zeta (3 (N+1) operations, 6 (N+1) - 3
       flops), and 15 uses of a derivative triple folded into their equations
@@ -178,12 +210,10 @@ def filter_flops_per_elem_node(N: int) -> float:
 
 
 def volume_bytes(Nl: int, Ng: int, fp: int, N: int = 4, affine: bool = False, gathered: int = 8) -> float:
-    """Algorithmic DRAM bytes of one volume-kernel launch (fp = 8 for FP64 and
-    the pairs mode, 4 for the FP32-mixed form): metric terms and Jw (10
+    """Algorithmic DRAM bytes of one volume-kernel launch (fp = 8 for FP64, 4 for the FP32-mixed form): metric terms and Jw (10
     values per element node; affine elements: Jw per node and 9 metric terms
     per element), l2g (4 B), the residual write (5 values), and one read per
-    global node of the `gathered` values (FP64: U and the nine flux
-    components, 12; pairs: U and u, theta, p' as pairs, 8; FP32: 8 floats)."""
+    global node of the `gathered` values (U, u, theta, p': 8)."""
     if affine:
         return Nl * (fp + 4 + 5 * fp) + Nl // (N + 1) ** 3 * 9 * fp + Ng * gathered * fp
     return Nl * (10 * fp + 4 + 5 * fp) + Ng * gathered * fp
@@ -194,7 +224,8 @@ def update_bytes(Nl: int, Ng: int, fp: int, stage_reads_qn: float, entries: int 
     4 B per node; `entries` = Nl unless given), residual read (5 values per
     element node, once), M^-1, wall flag, q^k read, q^{k+1} write, q^n on the
     stages that use it, the reference state (4 doubles) and the
-    primitive-field write (`prim` bytes: 72 in FP64, 32 in FP32-mixed)."""
+    primitive-field write (`prim` bytes: 32 in FP32-mixed; FP64 writes u,
+    theta and p', FP64_PRIM_BYTES; 72 unless given: nine flux components)."""
     entries = Nl if entries is None else entries
     prim = (72 if fp == 8 else 32) if prim is None else prim
     return (entries * 4 + Nl * 5 * fp
@@ -489,11 +520,6 @@ def run_mine(args):
     value = whole_job_rate(world, Ng, args.steps, ms)
     nlaunch = STAGES * args.steps
     vol_avg_s = ms_vol * 1e-3 / nlaunch
-    fl_el, ops_el = volume_fp64_cost(N, "rect" if affine else "nodal")
-    flops = fl_el * Nl
-    achieved_tf = flops / vol_avg_s / 1e12
-    # FP64 pipe slots: 2 per SM per clock, i.e. half the FMA flop peak
-    pipe_frac = ops_el * Nl / vol_avg_s / (FP64_PEAK_TFLOPS * 1e12 / 2)
     form_name = "affine" if affine else "nodal"
     line = {
         "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps,
@@ -505,19 +531,12 @@ def run_mine(args):
                    "parallelism": f"replica x{world}" if world > 1 else "single GPU"},
         "e2e": e2e,
         "gpu_launches": 2 * nlaunch,
-        "roofline": {"kernel": f"volume_kernel<{N},double,{form_name}>",
-                     "form": "rectilinear (K_d D, w_i w_j w_k)" if affine else "per-node (Eq. 5)",
-                     "bound": "alu", "achieved": achieved_tf,
-                     "peak": FP64_PEAK_TFLOPS, "unit": "TFLOP/s", "frac": achieved_tf / FP64_PEAK_TFLOPS,
+        "roofline": {**volume_fp64_roofline(N, "rect" if affine else "nodal", Nl, vol_avg_s,
+                                            volume_bytes(Nl, Ng, 8, N, affine), hbm_gbs),
                      "traffic": ncu_traffic(f"volume_fp64_{form_name}", args.workload),
-                     "algorithmic_flops": flops, "fp64_ops_per_element_node": ops_el,
-                     "fp64_pipe_frac": pipe_frac,
-                     "algorithmic_bytes": volume_bytes(Nl, Ng, 8, N, affine, gathered=12),
-                     "peak_source": FP64_PEAK_SOURCE,
-                     "avg_launch_ms": 1e3 * vol_avg_s,
                      "share_of_step": ms_vol / (ms_vol + ms_upd)},
         "kernels": {"volume_ms_avg": 1e3 * vol_avg_s, "update_ms_avg": ms_upd / nlaunch,
-                    "update_hbm_frac": update_bytes(Nl, Ng, 8, 2 / 3) / (ms_upd * 1e-3 / nlaunch) / 1e9 / hbm_gbs,
+                    "update_hbm_frac": update_bytes(Nl, Ng, 8, 2 / 3, prim=FP64_PRIM_BYTES) / (ms_upd * 1e-3 / nlaunch) / 1e9 / hbm_gbs,
                     "stage_hbm_frac": stage_bytes_model(Nl, Ng, 8) / (ms * 1e-3 / nlaunch) / 1e9 / hbm_gbs,
                     "stage_hbm_model": "84 B per element node + 232 B per global node"},
         "clocks": ck,
@@ -543,15 +562,10 @@ def run_mine(args):
         # read and applied at every node), for comparison
         msn, voln, updn, _, _, _, finn, _ = measure("fp64", "nodal")
         voln_s = voln * 1e-3 / nlaunch
-        fl_n = volume_flops_per_elem_node(N, False) * Nl
-        op_n = volume_fp64_cost(N, "nodal")[1] * Nl
         line["fp64_nodal_form"] = {
             "value": world * Ng * STAGES * args.steps / (msn * 1e-3), "unit": UNIT, "ms_per_step": msn / args.steps,
             "finite": finn, "volume_ms_avg": 1e3 * voln_s, "update_ms_avg": updn / nlaunch,
-            "roofline": {"kernel": f"volume_kernel<{N},double,nodal>", "bound": "alu",
-                         "achieved": fl_n / voln_s / 1e12, "peak": FP64_PEAK_TFLOPS, "unit": "TFLOP/s",
-                         "frac": fl_n / voln_s / 1e12 / FP64_PEAK_TFLOPS,
-                         "fp64_pipe_frac": op_n / voln_s / (FP64_PEAK_TFLOPS * 1e12 / 2),
+            "roofline": {**volume_fp64_roofline(N, "nodal", Nl, voln_s, volume_bytes(Nl, Ng, 8), hbm_gbs),
                          "traffic": ncu_traffic("volume_fp64_nodal", args.workload)},
         }
     if not args.no_fp32:
@@ -581,7 +595,7 @@ def run_mine(args):
                 "finite": fin32n, "volume_ms_avg": 1e3 * vol32n_s, "volume_hbm_frac": bn / vol32n_s / 1e9 / hbm_gbs,
                 "traffic": ncu_traffic("volume_fp32_nodal", args.workload)}
     if not args.no_fp32:
-        # FP64-accurate element kernel on the FP32 units ((hi, lo) float pairs)
+        # the pairs precision of the API (runs the FP64 kernels)
         msp, volp, updp, _, _, _, finp, _ = measure("fp64_pairs")
         vp = world * Ng * STAGES * args.steps / (msp * 1e-3)
         volp_s = volp * 1e-3 / nlaunch
@@ -590,7 +604,7 @@ def run_mine(args):
             "value": vp, "unit": UNIT, "ms_per_step": msp / args.steps, "speedup_vs_fp64": vp / value,
             "form": form_name, "finite": finp, "volume_ms_avg": 1e3 * volp_s, "update_ms_avg": updp / nlaunch,
             "volume_fp64_equiv_tflops": volume_flops_per_elem_node(N, affine) * Nl / volp_s / 1e12,
-            "volume_traffic": ncu_traffic(f"volume_pairs_{form_name}", args.workload),
+            "volume_traffic": ncu_traffic(f"volume_fp64_{form_name}", args.workload),
             "volume_hbm_gbs": bp / volp_s / 1e9, "volume_hbm_frac": bp / volp_s / 1e9 / hbm_gbs,
         }
         if affine:
@@ -613,7 +627,8 @@ def run_mine(args):
                 "value": vd, "ms_per_step": msd / args.steps, "vs_cg_storage": vd / ref_v if ref_v else None,
                 "storage_nodes": infod["Ng"], "dss_entries": infod["dss_entries"], "finite": find,
                 "volume_ms_avg": vold / nlaunch, "update_ms_avg": 1e3 * upd_s,
-                "update_hbm_frac": update_bytes(Nl, infod["Ng"], fp, 2 / 3, infod["dss_entries"])
+                "update_hbm_frac": update_bytes(Nl, infod["Ng"], fp, 2 / 3, infod["dss_entries"],
+                                                FP64_PRIM_BYTES if fp == 8 else None)
                 / upd_s / 1e9 / hbm_gbs}
     if not args.no_imex:
         line["imex"] = imex_block(args, numa, torch, dev, barrier, max_ranks)
@@ -630,13 +645,8 @@ def run_mine(args):
             sh[prec] = {"value": whole_job_rate(world, infos["Ng"], args.steps, mss), "ms_per_step": mss / args.steps,
                         "volume_ms_avg": vols / nl, "update_ms_avg": upds / nl, "finite": fins}
             if prec == "fp64":
-                fl_e, op_e = volume_fp64_cost(infos["N"], "nodal")
-                t_s = vols * 1e-3 / nl
-                sh[prec]["roofline"] = {"kernel": f"volume_kernel<{infos['N']},double,nodal>", "bound": "alu",
-                                        "achieved": fl_e * infos["Nl"] / t_s / 1e12, "peak": FP64_PEAK_TFLOPS,
-                                        "unit": "TFLOP/s",
-                                        "frac": fl_e * infos["Nl"] / t_s / 1e12 / FP64_PEAK_TFLOPS,
-                                        "fp64_pipe_frac": op_e * infos["Nl"] / t_s / (FP64_PEAK_TFLOPS * 1e12 / 2)}
+                sh[prec]["roofline"] = volume_fp64_roofline(infos["N"], "nodal", infos["Nl"], vols * 1e-3 / nl,
+                                                            volume_bytes(infos["Nl"], infos["Ng"], 8), hbm_gbs)
             if prec == "fp32_mixed":
                 b32 = volume_bytes(infos["Nl"], infos["Ng"], 4)
                 sh[prec]["speedup_vs_fp64"] = sh[prec]["value"] / sh["fp64"]["value"]
