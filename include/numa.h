@@ -20,7 +20,8 @@
  *   calls on it must be made with that device current.  Contexts on
  *   different devices may be used from one process.  A context is not
  *   thread-safe: calls on one context must not overlap.  Calls on different
- *   contexts may come from different threads.
+ *   contexts may come from different threads.  numa_create builds large
+ *   meshes with up to 8 threads of its own, joined before it returns.
  *
  * Errors
  *   Every call returns an int status: NUMA_OK (0) or a negative NUMA_E* code.
@@ -60,11 +61,13 @@ extern "C" {
 enum numa_mesh_kind { NUMA_MESH_BOX = 0, NUMA_MESH_SHELL = 1 };
 enum numa_ref_kind { NUMA_REF_ISENTROPIC = 0, NUMA_REF_ISOTHERMAL = 1 };
 enum numa_precision {
-  NUMA_FP64 = 0,      /* FP64 throughout: state, primitives and EOS, DSS, inverse
-                          mass and RK as FP64 operations; the element kernel's
-                          products and sums as 58- to 64-bit integers relative
-                          to the largest value of their group in the element,
-                          rounded to FP64 once at the end */
+  NUMA_FP64 = 0,      /* FP64 throughout: state, DSS, inverse mass and RK as FP64
+                          operations; the primitives and EOS as products of
+                          58-bit mantissas; the element kernel's (and short
+                          1D-IMEX columns') products and sums as 58- to 64-bit
+                          integers relative to the largest value of their group
+                          in the element (column), rounded to FP64 once at the
+                          end; values beyond those ranges as FP64 operations */
   NUMA_FP32_MIXED = 1, /* fluxes, metric terms and D contractions in FP32;
                           state, EOS reference subtraction, DSS, inverse mass
                           and the RK combination in FP64 */
@@ -256,12 +259,12 @@ int numa_set_time_scheme(numa_ctx* ctx, int scheme);
  * `nslabs` slabs along z and the global nodes into the matching slabs; within
  * a step the DSS/update of node slab k runs on a second, library-owned stream
  * beside the element kernel of slab k + 1 (the element kernel is bound by
- * memory or FP64 work, the update by FP64 work and latency), ordered by
+ * memory or instruction issue, the update by FP64 work and latency), ordered by
  * events so that every node is computed exactly as without slabs: results are
  * identical bit for bit.  nslabs = 0 (the default) chooses 3 slabs for
  * FP32-mixed meshes of 2^18 or more global nodes (in FP64 and the pairs mode
- * both kernels compete for the same pipes and the pipeline measured no gain,
- * so it stays off there); 1 turns the pipeline off; at most 16.  Where a
+ * both kernels compete for issue slots and the pipeline measured slower, so
+ * it stays off there); 1 turns the pipeline off; at most 16.  Where a
  * mesh cannot be cut (shells, DG storage, periodic in z, slabs thinner than
  * two node planes, planes of fewer than 128 nodes) one slab is used.  *used
  * (may be NULL) receives the slabs in effect (before numa_bind: those that
