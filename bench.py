@@ -98,7 +98,7 @@ NCU_TRAFFIC = {"kernels_sha256_16": "bbe726f310fc4b3f", "workload": "bubble_32x3
                "volume_fp32_affine": 139.233792e6 + 49.506816e6}
 
 # the sources the element kernels with committed traffic figures are built from
-KERNEL_SOURCES = ["kernels_common.cuh", "fixed64.cuh", "volume_fp64.cu", "volume_fp32.cu"]
+KERNEL_SOURCES = ["kernels_common.cuh", "fixed64.cuh", "fixed_int.cuh", "volume_fp64.cu", "volume_fp32.cu"]
 
 
 def code_lines(text: str) -> list:

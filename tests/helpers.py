@@ -52,3 +52,42 @@ def scaled_random_state(Ng: int, rho0: np.ndarray, th0: np.ndarray, seed: int, r
     q[1:4] *= u * rho0
     q[4] *= rel * th0
     return q
+
+
+def lobatto_derivative(N: int) -> list:
+    """The derivative matrix of the Lobatto points of order N as rationals, from
+    points good to 2^-120: Newton on P_N' from the double roots."""
+    from fractions import Fraction
+
+    a, b = [Fraction(1)], [Fraction(0), Fraction(1)]  # P_N in powers of x, by Bonnet's recurrence
+    for k in range(2, N + 1):
+        a, b = b, [Fraction(2 * k - 1, k) * (b[i - 1] if i else 0)
+                   - (Fraction(k - 1, k) * a[i] if i < len(a) else 0) for i in range(k + 1)]
+    c = b
+    d1 = [k * c[k] for k in range(1, len(c))]
+    d2 = [k * d1[k] for k in range(1, len(d1))]
+    ev = lambda p, x: sum(v * x ** k for k, v in enumerate(p))  # noqa: E731
+    roots = np.sort(np.roots([float(v) for v in d1[::-1]]).real) if N > 1 else []
+    x = [Fraction(-1)]
+    for r in roots:
+        t = Fraction(float(r))
+        for _ in range(4):
+            t = t - ev(d1, t) / ev(d2, t)
+            t = Fraction(round(t * 2 ** 140), 2 ** 140)
+        x.append(t)
+    x.append(Fraction(1))
+    P = N + 1
+    lam = []
+    for j in range(P):
+        v = Fraction(1)
+        for k in range(P):
+            if k != j:
+                v *= x[j] - x[k]
+        lam.append(v)
+    D = [[Fraction(0)] * P for _ in range(P)]
+    for i in range(P):
+        for j in range(P):
+            if i != j:
+                D[i][j] = lam[i] / lam[j] / (x[i] - x[j])
+        D[i][i] = -sum(D[i])
+    return D

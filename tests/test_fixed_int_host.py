@@ -1,0 +1,66 @@
+"""The integer arithmetic of the fixed-point FP64 kernels, built for the host
+from the kernels' own header, against exact integers and rationals."""
+import ctypes
+import os
+import subprocess
+from fractions import Fraction
+
+import numpy as np
+import pytest
+
+from .helpers import lobatto_derivative
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+PKG = os.path.join(os.path.dirname(HERE), "paper_1511_01561_gb300")
+
+
+def _cuda_include():
+    nvcc = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
+    return os.path.join(os.path.dirname(os.path.dirname(os.path.realpath(nvcc))), "include")
+
+
+@pytest.fixture(scope="module")
+def fx(tmp_path_factory):
+    lib = str(tmp_path_factory.mktemp("fixed_int") / "fixed_int.so")
+    cmd = ["g++", "-std=c++17", "-O1", "-fwrapv", "-ffp-contract=off", "-shared", "-fPIC", "-Wno-unknown-pragmas", "-I", HERE,
+           "-I", os.path.join(PKG, "csrc"), "-I", os.path.join(os.path.dirname(PKG), "include"), "-I", _cuda_include(),
+           os.path.join(HERE, "fixed_int_host.cpp"), os.path.join(PKG, "csrc", "mesh.cpp"), "-o", lib, "-lpthread"]
+    subprocess.run(cmd, check=True)
+    return ctypes.CDLL(lib)
+
+
+def _ints(n):
+    return (ctypes.c_int * n)()
+
+
+# values within 2^-31 below a power of two, where the diagonal momentum flux
+# comes closest to its bound, and others around them
+@pytest.mark.parametrize("pipe", [0, 1])
+@pytest.mark.parametrize("N", range(1, 9))
+def test_lines_of_extreme_fluxes(fx, N, pipe):
+    """A uniform field's derivative is zero up to one unit a product, and the
+    derivative of a field that changes sign along the line is D F: the sums of
+    two mirrored nodes never leave 32 bits."""
+    D = lobatto_derivative(N)
+    e = int(np.frexp(float(max(sum(abs(v) for v in row) for row in D)))[1])
+    rng = np.random.default_rng(N)
+    near = lambda k: 2.0 ** k * (1.0 - 2.0 ** -rng.integers(31, 48))  # noqa: E731
+    for trial in range(60):
+        u = near(1)
+        p = {0: near(2), 1: near(1), 2: near(3), 3: 0.0}.get(trial % 5, rng.uniform(0.0, 8.0))
+        z = (ctypes.c_double * 8)(u, u, u, u, u, u, 300.0, p)
+        f, g = _ints(24), _ints(3)
+        assert fx.fluxes_of(z, pipe, f, g)
+        for slot in range(12):
+            lo, hi = f[2 * slot], f[2 * slot + 1]
+            F = [lo + (hi << 29)] * (N + 1)
+            if trial % 2:  # the antisymmetric combination
+                F = [-v if m > N // 2 else v for m, v in enumerate(F)]
+            h = [(v + (1 << 28)) >> 29 for v in F]
+            arr = (ctypes.c_int * (2 * N + 2))(*[w for v, t in zip(F, h) for w in (v - (t << 29), t)])
+            out = (ctypes.c_longlong * (N + 1))()
+            fx.line_of(N, arr, e, out)
+            for i in range(N + 1):
+                want = sum(D[i][m] * F[m] for m in range(N + 1)) * Fraction(2) ** (2 - e)
+                # a table entry and a dropped product of low parts, half a unit each, per node; the final rounding
+                assert abs(out[i] - want) <= 2 * (N + 1) + 1, (trial, slot, i)

@@ -151,3 +151,19 @@ def test_pressure_over_magnitudes(numa, orc, prec, k):
     finally:
         s.close()
     _check(Rg, m.rhs(q))
+
+
+# U, u and p' within 2^-31 below powers of two at every node: the diagonal
+# momentum flux at its bound, where sums of two nodes' high halves are largest
+@pytest.mark.parametrize("N", [1, 4, 7])
+@pytest.mark.parametrize("axis", [0, 1])
+@pytest.mark.parametrize("over", [dict(), dict(metric_form="nodal")], ids=["rect", "nodal"])
+def test_momentum_flux_at_its_bound(numa, orc, N, axis, over):
+    cfg = I.box((2, 2, 2), N, periodic=(1, 1, 0), **over)
+    m = orc.Mesh(cfg)
+    rho0, th0, p0 = m.ref()[:3]
+    q = np.zeros((5, m.Ng))
+    q[0] = 1.0 - rho0
+    q[1 + axis] = 2.0 - 2.0 ** -40
+    q[4] = th0 * np.expm1(np.log1p((4.0 - 2.0 ** -34) / p0) * cfg["cv"] / cfg["cp"])
+    _check(_rhs(numa, cfg, q), m.rhs(q))
