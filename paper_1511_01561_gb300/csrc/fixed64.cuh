@@ -13,7 +13,7 @@
 //
 // Elements whose values the integers cannot hold (an infinity or a NaN, or
 // magnitudes near the ends of the FP64 range) go through a plain FP64 form,
-// one element at a time, with the same results as ordinary arithmetic.
+// one element at a time, whichever elements share their CTA.
 #pragma once
 
 #include "fixed_int.cuh"
@@ -146,7 +146,10 @@ __device__ __forceinline__ void rect_plain(const VolumeArgs& a, long long e) {
 // element node, and leaves the 12 flux fields in F as fixed-point integers.
 // The largest magnitudes in an element give its groups' exponents: left as
 // keys per element in gmax (EPB > 1), or returned in ge (EPB = 1).  False
-// (uniform over the CTA) if the integers cannot hold some element.
+// (uniform over the CTA) if the integers cannot hold its one element; with
+// several, the fields of an element they cannot hold (fx_in_range of its key)
+// are left unset, so that no element's result depends on which others share
+// its CTA (a slab launch groups them otherwise).
 template <int N, int EPB, int NT, bool PIPE>
 __device__ __forceinline__ bool fx_stage(const VolumeArgs& a, long long n0, int nn, uint4* gmax, int2* F, FxExp& ge) {
   constexpr int NP = (N + 1) * (N + 1) * (N + 1), NN = EPB * NP, IT = (NN + NT - 1) / NT;
@@ -186,24 +189,24 @@ __device__ __forceinline__ bool fx_stage(const VolumeArgs& a, long long n0, int 
   grid_wait();  // (threads without a node; before any write of the kernel)
   grid_next();
   __syncthreads();
-  bool ok = true;
   uint4 gm = make_uint4(0u, 0u, 0u, 0u);
-#pragma unroll
-  for (int t = 0; t < SLOTS; ++t) {
-    const uint4 w = gmax[t];
-    if constexpr (EPB == 1) gm = make_uint4(max(gm.x, w.x), max(gm.y, w.y), max(gm.z, w.z), max(gm.w, w.w));
-    else ok &= fx_in_range(w);
-  }
   if constexpr (EPB == 1) {
-    ok = fx_in_range(gm);
+#pragma unroll
+    for (int t = 0; t < SLOTS; ++t) {
+      const uint4 w = gmax[t];
+      gm = make_uint4(max(gm.x, w.x), max(gm.y, w.y), max(gm.z, w.z), max(gm.w, w.w));
+    }
+    if (!fx_in_range(gm)) return false;
     ge = fx_exps(gm);
   }
-  if (!ok) return false;
 #pragma unroll
   for (int it = 0; it < IT; ++it) {
     const int l = tid + it * NT;
     if (l < nn) {
-      if constexpr (EPB > 1) gm = gmax[l / NP];
+      if constexpr (EPB > 1) {
+        gm = gmax[l / NP];
+        if (!fx_in_range(gm)) continue;
+      }
       const FxExp e = fx_exps(gm);
       int2* f = F + fx_index<N>(l);
       fx_fluxes<PIPE>(z[it], e, gm.z, [&](int slot, int2 x) { f[slot * FP] = x; });
@@ -271,11 +274,21 @@ __device__ __forceinline__ void volume_fx_rect(const VolumeArgs& a, const int2* 
     long long out[P];
     fx_line<N>(F + f * FP + base, B, T + 2 * M, out);
     const long long* o = part + v * FP + base;
-    if constexpr (EPB > 1) ge = fx_exps(gmax[el]);
-    const int kexp = (v == 0 ? ge.U : v == 4 ? ge.t : ge.m) + a.fxexp;
-    double* re = static_cast<double*>(a.re) + v * a.Nl + n0 + el * NP + r;
+    bool ok = true;
+    if constexpr (EPB > 1) {
+      ok = fx_in_range(gmax[el]);
+      ge = fx_exps(gmax[el]);
+    }
+    if (ok) {
+      const int kexp = (v == 0 ? ge.U : v == 4 ? ge.t : ge.m) + a.fxexp;
+      double* re = static_cast<double*>(a.re) + v * a.Nl + n0 + el * NP + r;
 #pragma unroll
-    for (int m = 0; m < P; ++m) re[m * PP] = fx_to_double(out[m] + o[m * B] + o[5 * FP + m * B], kexp);
+      for (int m = 0; m < P; ++m) re[m * PP] = fx_to_double(out[m] + o[m * B] + o[5 * FP + m * B], kexp);
+    }
+  }
+  if constexpr (EPB > 1) {
+    for (int t = 0; t < ne; ++t)  // (uniform over the CTA)
+      if (!fx_in_range(gmax[t])) rect_plain<N>(a, e0 + t);
   }
 }
 
@@ -349,11 +362,16 @@ __device__ __forceinline__ void volume_fx_nodal(const VolumeArgs& a, const int2*
   // the elements' metric exponents (w: the element takes plain FP64)
   const int4 eb = a.fxE[e0 + (node ? nel : 0)];
   FxExp ge;
-  bool ok = fx_stage<N, EPB, NT, true>(a, n0, nn, gmax, F, ge);
-  if (__syncthreads_or(!ok || eb.w)) {
-    for (int t = 0; t < ne; ++t) nodal_plain<N>(a, e0 + t);
-    return;
+  bool ok = fx_stage<N, EPB, NT, true>(a, n0, nn, gmax, F, ge) && !eb.w;
+  if constexpr (EPB == 1) {  // (uniform over the CTA)
+    if (!ok) {
+      nodal_plain<N>(a, e0);
+      return;
+    }
+  } else {
+    ok = ok && fx_in_range(gmax[nel]);
   }
+  __syncthreads();
   const int at = fx_index<N>(tid);
   const int2* met = reinterpret_cast<const int2*>(a.met64) + n0 + tid;
   // the exponents of the node's three directions: the metric row's less that
@@ -408,13 +426,18 @@ __device__ __forceinline__ void volume_fx_nodal(const VolumeArgs& a, const int2*
   direction(std::integral_constant<int, 0>());
   direction(std::integral_constant<int, 1>());
   direction(std::integral_constant<int, 2>());
-  if (!node) return;
-  if constexpr (EPB > 1) ge = fx_exps(gmax[nel]);
-  const int kx = xm + 1 + a.fxexp + fx_weight_exp(a.fxw, l % P, (l / P) % P, l / PP);
-  double* re = static_cast<double*>(a.re) + n0 + tid;
+  if (node && ok) {
+    if constexpr (EPB > 1) ge = fx_exps(gmax[nel]);
+    const int kx = xm + 1 + a.fxexp + fx_weight_exp(a.fxw, l % P, (l / P) % P, l / PP);
+    double* re = static_cast<double*>(a.re) + n0 + tid;
 #pragma unroll
-  for (int v = 0; v < 5; ++v)
-    re[v * Nl] = fx_to_double(sum[v], kx + (v == 0 ? ge.U : v == 4 ? ge.t : ge.m));
+    for (int v = 0; v < 5; ++v)
+      re[v * Nl] = fx_to_double(sum[v], kx + (v == 0 ? ge.U : v == 4 ? ge.t : ge.m));
+  }
+  if constexpr (EPB > 1) {
+    for (int t = 0; t < ne; ++t)  // (uniform over the CTA)
+      if (a.fxE[e0 + t].w || !fx_in_range(gmax[t])) nodal_plain<N>(a, e0 + t);
+  }
 }
 
 // CTAs an SM holds at r registers a thread.  64 registers for both forms: the

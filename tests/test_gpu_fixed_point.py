@@ -166,4 +166,51 @@ def test_momentum_flux_at_its_bound(numa, orc, N, axis, over):
     q[0] = 1.0 - rho0
     q[1 + axis] = 2.0 - 2.0 ** -40
     q[4] = th0 * np.expm1(np.log1p((4.0 - 2.0 ** -34) / p0) * cfg["cv"] / cfg["cp"])
-    _check(_rhs(numa, cfg, q), m.rhs(q))
+    # uniform fluxes: the tendencies are zero but for the buoyancy, so each variable's
+    # scale is its flux over an element's half edge
+    scale = np.array([2.0, 8.0, 8.0, 8.0, 2.0 * 300.0]) / 250.0
+    err = np.abs(_rhs(numa, cfg, q) - m.rhs(q)).max(axis=1) / scale
+    assert err.max() <= TOL, err
+
+
+# several elements share a CTA at N <= 3: one that the integers cannot hold
+# (momentum of 1e200 at its nodes) leaves the bits of the others alone
+@pytest.mark.parametrize("N", [1, 2, 3])
+@pytest.mark.parametrize("over", [dict(), dict(warp=0.03)], ids=["rect", "warped"])
+def test_elements_of_one_cta_are_independent(numa, orc, N, over):
+    cfg = I.box((11, 3, 3), N, **over)
+    m = orc.Mesh(cfg)
+    q = scaled_random_state(m.Ng, m.ref()[0], m.ref()[1], seed=N)
+    R0 = _rhs(numa, cfg, q)
+    nx = 11 * N + 1
+    g = 4 * N + 1 + nx * (N + (3 * N + 1) * N)  # on an edge between elements in y and z
+    q[1, g] = 1e200
+    Rg = _rhs(numa, cfg, q)
+    e = m.l2g().reshape(-1, (N + 1) ** 3)
+    far = np.setdiff1d(np.arange(m.Ng), np.unique(e[(e == g).any(axis=1)]))
+    assert np.array_equal(Rg[:, far], R0[:, far])
+
+
+# the same through slabs of an odd number of elements, which group the elements
+# of a CTA otherwise: elements with a momentum below the integers' range ahead
+# of a disturbance
+@pytest.mark.parametrize("N,ne", [(1, (13, 11, 6)), (2, (7, 9, 6)), (3, (5, 5, 6))])
+@pytest.mark.parametrize("over", [dict(), dict(warp=0.02)], ids=["rect", "warped"])
+def test_slabs_with_elements_out_of_range(numa, orc, N, ne, over):
+    cfg = I.box(ne, N, **over)
+    m = orc.Mesh(cfg)
+    q = scaled_random_state(m.Ng, m.ref()[0], m.ref()[1], seed=N)
+    ahead = m.coords()[2] > 420.0  # (of 1000)
+    q[:, ahead] = 0.0
+    q[1:4, ahead] = np.random.default_rng(N).uniform(-1e-200, 1e-200, (3, int(ahead.sum())))
+    out = []
+    for slabs in (1, 2, 3):
+        s = numa.Solver(cfg, "fp64")
+        try:
+            assert s.set_slabs(slabs) == slabs
+            s.set_state(q)
+            s.run(1e-3, 1)
+            out.append(s.get_state().numpy().copy())
+        finally:
+            s.close()
+    assert np.array_equal(out[1], out[0]) and np.array_equal(out[2], out[0])
