@@ -187,7 +187,6 @@ __device__ __forceinline__ bool fx_stage(const VolumeArgs& a, long long n0, int 
     if ((tid & 31) == 0) gmax[tid >> 5] = gw;
   }
   grid_wait();  // (threads without a node; before any write of the kernel)
-  grid_next();
   __syncthreads();
   uint4 gm = make_uint4(0u, 0u, 0u, 0u);
   if constexpr (EPB == 1) {

@@ -22,15 +22,25 @@ namespace numa {
 namespace {
 
 // ---- launches that overlap the end of the kernel before -----------------------
-// A launch with `early` may begin while the kernel before it on the stream
-// still runs: grid_wait returns once that one is complete and its writes are
+// A launch with `early` is set up while the kernel before it on the stream
+// still runs, and its blocks are placed as that kernel's last ones end:
+// grid_wait returns once that one is complete and its writes are
 // visible, and comes before any access to what a kernel before wrote or reads
 // (each kernel waits, so all earlier ones are complete too); what is fixed at
-// bind may be read before it.  grid_next, after the wait, lets the next
-// launch begin.  Without `early` both do nothing.  numa_bind asks for it on
-// meshes of a few blocks per SM only (numa_ctx::early).
+// bind may be read before it.  Without `early` (slabs, kernels timed one by
+// one) it does nothing.  A step of 4^3 elements at N = 4 in FP64 takes 29.0 us
+// instead of 31.1 (a right-hand side 12.4 instead of 16.8), of 10^3 elements 47.6
+// instead of 51.3, of 32^3 774 instead of 776; FP32-mixed 30.0 instead of 32.4 on
+// 8^3.  No mesh of 1 to 32 elements an edge, order, form or precision is slower.
+//
+// No kernel lets its successor begin sooner (griddepcontrol.launch_dependents):
+// blocks placed while the first kernel's are resident crowd the SMs that have
+// room, and the FP64 pipe of those SMs then bounds the step.  With the trigger
+// after the kernel's first loads a step took, against plain launches, 53.7
+// against 37.2 us (5^3 elements, N = 8, FP32-mixed), 73.4 against 58.2 (FP64),
+// 43.4 against 27.1 (8^3, N = 1, FP32-mixed) and 61.2 against 52.2 (10^3, N = 4,
+// FP64); as it is 35.0, 55.7, 25.0 and 47.6.
 __device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void grid_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 template <typename... K, typename... A>
 cudaError_t launch_kernel(void (*kernel)(K...), unsigned blocks, int threads, size_t smem, cudaStream_t s, bool early,
@@ -488,7 +498,6 @@ __global__ void __launch_bounds__(((N + 1) * (N + 1) * (N + 1) + 31) / 32 * 32)
     volume_kernel(VolumeArgs a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   grid_wait();
-  grid_next();
   volume_element_lines<N, AFF>(a, a.ebeg + (long long)blockIdx.x, smem_raw);
 }
 
@@ -811,8 +820,7 @@ __global__ void __launch_bounds__(kDssBlock, sizeof(RT) == 8 || BOX ? 12 : 16) u
     const int lt = a.order[base + threadIdx.x];
     const long long IA = base + lt;
     grid_wait();
-    grid_next();
-    if (IA < a.iend) {
+      if (IA < a.iend) {
       double s[5];
       if constexpr (BOX) dss_box<RT>(a, IA, s);
       else dss_node<RT>(a, IA, s);

@@ -79,7 +79,7 @@ VolumeArgs volume_args(const numa_ctx* c, const double* q, const void* prim, voi
   a.Ng = c->mesh.Ng;
   a.Nl = c->mesh.Nl;
   a.Ne = (int)c->mesh.Ne;
-  a.early = c->early;
+  a.early = 1;
   a.ebeg = 0;
   a.ecnt = a.Ne;
   a.affine = volume_form(c);
@@ -113,7 +113,7 @@ UpdateArgs update_args(const numa_ctx* c, const void* re, const double* qk, cons
   a.out = out;
   a.Ng = c->mesh.Ng;
   a.Nl = c->mesh.Nl;
-  a.early = c->early;
+  a.early = 1;
   a.ibeg = 0;
   a.iend = a.Ng;
   a.g = c->cfg.g;
@@ -750,20 +750,6 @@ int numa_bind(numa_ctx* c, void* ws, size_t bytes, void* stream) {
   c->fxexp = fxexp;
   c->fxw = fxw;
   c->fxr = fxr;
-  // Early launches where both kernels of a stage have at most four blocks per
-  // SM: there the gap between launches counts (4^3 elements at N = 4: a
-  // right-hand side 18.4 -> 12.3 us, a step 34.8 -> 30.7 us; 8^3: 42.2 -> 40.5).
-  // On larger grids the blocks that start early are spread unevenly over the
-  // SMs that have room (10^3: 52.2 -> 61.2 us, 32^3: 788 -> 832 us).
-  {
-    int dev = 0, sms = 0;
-    e = cudaGetDevice(&dev);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (e != cudaSuccess) return cuda_fail(c, e, "numa_bind device");
-    const long long chunk = volume_chunk(m.N, c->cfg.precision, volume_form(c));
-    const long long blocks = std::max((m.Ne + chunk - 1) / chunk, (m.Ng + kDssBlock - 1) / kDssBlock);
-    c->early = blocks <= 4LL * sms ? 1 : 0;
-  }
   c->slabs = plan_slabs(c->cfg, m, c->nslab_req);
   if (c->slabs.S > 1) {
     e = ensure_slab_streams(c);

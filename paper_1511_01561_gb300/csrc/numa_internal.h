@@ -365,7 +365,6 @@ struct numa_ctx {
   std::vector<int2> fxD;
   int fxexp = 0;
   unsigned long long fxw = 0, fxr = 0;  // FP64 per-node form: VolumeArgs::fxw, fxr
-  int early = 0;            // kernels may begin before the one before them has ended (small meshes)
   int nslab_req = 0;        // slabs asked for by numa_set_slabs (0: automatic)
   numa::SlabPlan slabs;     // the plan in use (made at bind and by numa_set_slabs)
   cudaStream_t side = nullptr;  // the second stream of the slab pipeline
