@@ -17,6 +17,8 @@
 
 #include <cstdint>
 
+#include "numa_internal.h"
+
 namespace numa {
 namespace {
 
@@ -50,14 +52,24 @@ __device__ __forceinline__ unsigned long long mul58(M58 a, M58 b) {
   return (unsigned long long)a.h * b.h + (m >> 29);
 }
 
+#ifdef __CUDACC__
+// 1/d in FP32, d in [1, 2): within 2^-23.
+__device__ __forceinline__ float rcp_approx(float d) {
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(d));
+  return r;
+}
+#endif
+
 // 1/d 2^58 for d = m 2^-52 in [1, 2): the FP32 reciprocal r0, then
 // r0 (1 + e + e^2) with e = 1 - d r0 formed exactly (its leading bits cancel).
+// The approximation may fall on either side of [1/2, 1), whose exponent R0
+// relies on: next to d = 1 and d = 2 r0 is that interval's end (|e| < 2^-22).
 __device__ __forceinline__ M58 rcp58(double x) {
   const unsigned lo = (unsigned)__double2loint(x), hi = ((unsigned)__double2hiint(x) & 0xfffffu) | 0x100000u;
   const float df = __uint_as_float(0x3f800000u | __funnelshift_l(lo, hi & 0xfffffu, 3));
-  float r;
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(df));
-  const unsigned R0 = (__float_as_uint(fminf(r, 0.99999994f)) & 0x7fffffu) | 0x800000u;  // r0 2^24
+  const float r = fmaxf(fminf(rcp_approx(df), 0.99999994f), 0.5f);
+  const unsigned R0 = (__float_as_uint(r) & 0x7fffffu) | 0x800000u;  // r0 2^24
   // e 2^76 = 2^76 - m R0, exact in the low 64 bits (|e| < 2^-21)
   const long long E = -(long long)((unsigned long long)lo * R0 + ((unsigned long long)(hi * R0) << 32));
   const long long e1 = E >> 16;          // e 2^60

@@ -1,9 +1,14 @@
-// Host build of the fixed-point kernels' integer arithmetic (fixed_int.cuh) for
-// tests/test_fixed_int_host.py.
+// Host build of the fixed-point kernels' integer arithmetic (fixed_int.cuh) and of
+// the integer primitives (soft64.cuh) for tests/test_fixed_int_host.py.
 #include "device_host.h"
+
+// the FP32 reciprocal with an error of its own, in units of 2^-23
+static float rcp_error = 0.0f;
+static float rcp_approx(float d) { return (float)(1.0 / (double)d + (double)rcp_error * 0x1p-23); }
 
 #include "fixed_int.cuh"
 #include "numa_internal.h"
+#include "soft64.cuh"
 
 using namespace numa;
 
@@ -61,4 +66,11 @@ extern "C" void line_of(int N, const int* f, int e, long long* out) {
     case 7: lines<7>(F, D, out); break;
     case 8: lines<8>(F, D, out); break;
   }
+}
+
+// x / rho as the update's primitive pass forms it, with a reciprocal seed that is
+// off by `error` units of 2^-23.
+extern "C" double div_of(double x, double rho, float error) {
+  rcp_error = error;
+  return soft_div(x, rcp58(rho), soft_exp(rho));
 }

@@ -26,7 +26,10 @@ def fx(tmp_path_factory):
            "-I", os.path.join(PKG, "csrc"), "-I", os.path.join(os.path.dirname(PKG), "include"), "-I", _cuda_include(),
            os.path.join(HERE, "fixed_int_host.cpp"), os.path.join(PKG, "csrc", "mesh.cpp"), "-o", lib, "-lpthread"]
     subprocess.run(cmd, check=True)
-    return ctypes.CDLL(lib)
+    fx = ctypes.CDLL(lib)
+    fx.div_of.restype = ctypes.c_double
+    fx.div_of.argtypes = [ctypes.c_double, ctypes.c_double, ctypes.c_float]
+    return fx
 
 
 def _ints(n):
@@ -64,3 +67,18 @@ def test_lines_of_extreme_fluxes(fx, N, pipe):
                 want = sum(D[i][m] * F[m] for m in range(N + 1)) * Fraction(2) ** (2 - e)
                 # a table entry and a dropped product of low parts, half a unit each, per node; the final rounding
                 assert abs(out[i] - want) <= 2 * (N + 1) + 1, (trial, slot, i)
+
+
+# a reciprocal seed anywhere within its documented error, densities on both
+# sides of a power of two, where the exact reciprocal is an end of [1/2, 1)
+@pytest.mark.parametrize("error", [-1.0, -0.5, 0.0, 0.5, 1.0])
+@pytest.mark.parametrize("k", [-2, -1, 0, 3])
+def test_division_next_to_powers_of_two(fx, k, error):
+    rng = np.random.default_rng(k + 5)
+    away = np.concatenate([np.ldexp(rng.uniform(0.5, 1.0, 200), -rng.integers(20, 53, 200)), [0.0, 2.0 ** -52, 2.0 ** -24]])
+    for d in np.concatenate([away, -0.5 * away]):
+        rho, x = float((1.0 + d) * 2.0 ** k), float(rng.uniform(1.0, 2.0))
+        q = fx.div_of(x, rho, error)
+        ulp = Fraction(float(np.spacing(q)))
+        # half an ulp of rounding, and less than 1.5 of the 2^-57 carried, twice (reciprocal, product)
+        assert abs(Fraction(q) - Fraction(x) / Fraction(rho)) <= Fraction(11, 16) * ulp, (d, q, x / rho)

@@ -214,3 +214,16 @@ def test_slabs_with_elements_out_of_range(numa, orc, N, ne, over):
         finally:
             s.close()
     assert np.array_equal(out[1], out[0]) and np.array_equal(out[2], out[0])
+
+
+# densities within 2^-20 of 1, 1/2 and 1/4, on both sides: 1/rho next to the ends
+# of its binade
+@pytest.mark.parametrize("over", [dict(), dict(warp=0.03)], ids=["rect", "warped"])
+def test_densities_next_to_powers_of_two(numa, orc, over):
+    cfg = I.box((4, 3, 3), 4, **over)
+    m = orc.Mesh(cfg)
+    rng = np.random.default_rng(20)
+    q = scaled_random_state(m.Ng, m.ref()[0], m.ref()[1], seed=20)
+    d = np.ldexp(rng.uniform(0.5, 1.0, m.Ng), -rng.integers(20, 53, m.Ng)) * rng.choice([-0.5, 0.0, 1.0], m.Ng)
+    q[0] = (1.0 + d) * rng.choice([1.0, 0.5, 0.25], m.Ng) - m.ref()[0]
+    _check(_rhs(numa, cfg, q), m.rhs(q))
