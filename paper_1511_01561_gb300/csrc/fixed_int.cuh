@@ -48,7 +48,8 @@ __device__ __forceinline__ int2 fx_split(long long s) {
   return make_int2((int)((unsigned)s & kFxMask) - (int)kFxHalf, (int)(s >> kFxBits));
 }
 
-// S 2^(kexp - 1086) rounded to nearest, and fx_of by the FP64 pipe: a conversion
+// S 2^(kexp - 1086) rounded to nearest (kexp - 63 within an FP64's biased
+// exponents: the host's bounds on the tables' and fx_in_range's on the groups'), and fx_of by the FP64 pipe: a conversion
 // and an exact product each, 32 cycles of a pipe that is otherwise idle in
 // place of 24 and 15 integer instructions.  Measured on 32^3 elements, N = 4
 // (rectilinear) and the 6x30x30x8 shell (per-node): all five results so, 0.183
@@ -75,32 +76,33 @@ __device__ __forceinline__ unsigned fx_group_key(const double* x, int n) {
 
 // The biased exponents of an element's equation groups, |field| <
 // 2^(exponent - 1022), from the magnitude keys of U, u, theta and p' (x, y, z,
-// w): mass: U; momentum: U u + p' I; theta: theta U.  A group of zeros gets an
-// exponent (kFxZero) at which fx_of shifts every bit of a zero out.
+// w): mass: U; momentum: U u + p' I; theta: theta U.  A group of zeros has the
+// exponent of 1, so that its zero sums meet a finite factor in fx_to_double.
 struct FxExp {
   int U, m, t;
 };
+constexpr int kFxZero = 1023;
+constexpr int kFxLeast = 100;  // at this exponent and above fx_of shifts every bit of a zero out
 // U u and p' each stay below 2^(m - 1022).  Where their exponents are equal m is
 // one above them, so their sum stays below 1.5 2^(m - 1022): 1.5 2^58 as an
 // integer, whose high part is at most 1.5 2^29, so that fx_line's sums of two
 // of them fit 32 bits.
-constexpr int kFxZero = 100;
 __device__ __forceinline__ FxExp fx_exps(uint4 k) {
-  const int U = max((int)(k.x >> 20), kFxZero);
+  const int U = k.x ? (int)(k.x >> 20) : kFxZero, p = (int)(k.w >> 20);
   // whether the product of the largest U and u carries into the next power of two
   const unsigned mU = (k.x & 0xfffffu) + 0x100001u, mu = (k.y & 0xfffffu) + 0x100001u;
   const int Uu = U + (int)(k.y >> 20) - 1023 + ((unsigned long long)mU * mu > (1ull << 41));
-  const int p = (int)(k.w >> 20);
-  return {U, max(max(Uu, p) + (Uu == p), kFxZero), U + (int)(k.z >> 20) - 1022};
+  const int m = k.x && k.y ? max(Uu, p) + (Uu == p) : k.w ? p : kFxZero;
+  return {U, m, k.x && k.z ? U + (int)(k.z >> 20) - 1022 : kFxZero};
 }
 
 // Whether the fixed-point form holds an element with these keys: every field
-// and, unless U is zero (and with it every product), every group.
+// and every group.
 __device__ __forceinline__ bool fx_in_range(uint4 k) {
   auto in = [](int E) { return (unsigned)E - kFxMinExp <= kFxMaxExp - kFxMinExp; };
   auto ok = [&](unsigned key) { return key == 0u || in((int)(key >> 20)); };
   const FxExp e = fx_exps(k);
-  return ok(k.x) && ok(k.y) && ok(k.z) && ok(k.w) && (k.x == 0u || ((k.y == 0u || in(e.m)) && (k.z == 0u || in(e.t))));
+  return ok(k.x) && ok(k.y) && ok(k.z) && ok(k.w) && in(e.m) && in(e.t);
 }
 
 // (high, middle) accumulators += D * f, D = Dh 2^29 + Dl, f = fh 2^29 + fl;
@@ -140,9 +142,9 @@ __device__ __forceinline__ void fx_fluxes(const Z& z, FxExp e, unsigned thkey, P
 #pragma unroll
   for (int c = 0; c < 3; ++c) {
     U[c] = fx_split((PIPE ? fx_of_pipe : fx_of)(z.U[c], e.U));
-    u[c] = fx_split(fx_of(z.u[c], max(e.m - e.U + 1022, kFxZero)));
+    u[c] = fx_split(fx_of(z.u[c], max(e.m - e.U + 1022, kFxLeast)));
   }
-  const int2 th = fx_split(fx_of(z.th, max((int)(thkey >> 20), kFxZero)));
+  const int2 th = fx_split(fx_of(z.th, max((int)(thkey >> 20), kFxLeast)));
   const long long p = (PIPE ? fx_of_pipe : fx_of)(z.pp, e.m);
   put(sUx, U[0]);
   put(sUy, U[1]);

@@ -82,3 +82,17 @@ def test_division_next_to_powers_of_two(fx, k, error):
         ulp = Fraction(float(np.spacing(q)))
         # half an ulp of rounding, and less than 1.5 of the 2^-57 carried, twice (reciprocal, product)
         assert abs(Fraction(q) - Fraction(x) / Fraction(rho)) <= Fraction(11, 16) * ulp, (d, q, x / rho)
+
+
+# groups of zeros: exponents inside the range of the groups of other values, as
+# the factor that a sum is multiplied by relies on
+@pytest.mark.parametrize("pipe", [0, 1])
+@pytest.mark.parametrize("U,u,th,p", [(0, 0, 300.0, 0), (0, 0, 300.0, 1e4), (0, 0, 0, 0), (2.0, 2.0, 0, 0), (3.0, 0, 1.0, 0)])
+def test_groups_of_zeros(fx, pipe, U, u, th, p):
+    f, e = _ints(24), _ints(3)
+    assert fx.fluxes_of((ctypes.c_double * 8)(U, U, U, u, u, u, th, p), pipe, f, e)
+    assert all(400 <= v <= 1600 for v in e), list(e)
+    want = [U] * 3 + [U * u + p] * 3 + [U * u] * 3 + [U * th] * 3
+    slots = [0, 5, 9, 1, 6, 10, 2, 3, 7, 4, 8, 11]
+    for w, s, k in zip(want, slots, [0] * 3 + [1] * 6 + [2] * 3):
+        assert (f[2 * s] + (f[2 * s + 1] << 29)) * Fraction(2) ** (e[k] - 1080) == Fraction(w)

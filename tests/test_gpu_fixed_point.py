@@ -12,7 +12,7 @@ import pytest
 
 from paper_1511_01561_gb300 import inputs as I
 
-from .helpers import scaled_random_state
+from .helpers import lobatto_derivative, scaled_random_state
 
 pytestmark = pytest.mark.gpu
 
@@ -227,3 +227,15 @@ def test_densities_next_to_powers_of_two(numa, orc, over):
     d = np.ldexp(rng.uniform(0.5, 1.0, m.Ng), -rng.integers(20, 53, m.Ng)) * rng.choice([-0.5, 0.0, 1.0], m.Ng)
     q[0] = (1.0 + d) * rng.choice([1.0, 0.5, 0.25], m.Ng) - m.ref()[0]
     _check(_rhs(numa, cfg, q), m.rhs(q))
+
+
+# a state at rest on meshes whose tables' power of two runs over the range in
+# which a factor of a group of zeros came out as an infinity
+@pytest.mark.parametrize("s2", range(98, 116))
+def test_rest_on_tiny_elements(numa, orc, s2):
+    N = 4
+    row = max(float(sum(abs(v) for v in r)) for r in lobatto_derivative(N))
+    h = np.sqrt(4.0 * 0.75 * 2.0 ** (60 - s2) / row)  # the largest row sum of h^2 / 4 |D|: 0.75 2^(60 - s2)
+    cfg = I.box((3, 2, 2), N, L=(3 * h, 2 * h, 2 * h))
+    R = _rhs(numa, cfg, np.zeros((5, orc.Mesh(cfg).Ng)))
+    assert np.array_equal(R, np.zeros_like(R))
