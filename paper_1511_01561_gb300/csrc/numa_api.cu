@@ -277,11 +277,13 @@ int imex_prepare(numa_ctx* c, double dt) {
 cudaError_t enqueue_imex_step(numa_ctx* c, double dt, bool start, cudaStream_t s, cudaEvent_t* ev = nullptr) {
   double* R = static_cast<double*>(c->L.prim);
   cudaError_t e = ev ? cudaEventRecord(ev[0], s) : cudaSuccess;
-  if (e == cudaSuccess) e = launch_volume(c->mesh.N, c->cfg.precision, volume_args(c, c->L.q, c->L.prim, c->L.re), s);
+  VolumeArgs va = volume_args(c, c->L.q, c->L.prim, c->L.re);
+  UpdateArgs ua = update_args(c, c->L.re, c->L.q, c->L.q, R, 0, 0.0, 1.0, 0.0);
+  if (ev) va.early = ua.early = 0;  // each kernel by itself between its events
+  if (e == cudaSuccess) e = launch_volume(c->mesh.N, c->cfg.precision, va, s);
   if (e == cudaSuccess && ev) e = cudaEventRecord(ev[1], s);
   if (e == cudaSuccess && ev) e = cudaEventRecord(ev[2], s);
-  if (e == cudaSuccess)
-    e = launch_update(c->cfg.precision, update_args(c, c->L.re, c->L.q, c->L.q, R, 0, 0.0, 1.0, 0.0), s);
+  if (e == cudaSuccess) e = launch_update(c->cfg.precision, ua, s);
   if (e == cudaSuccess) {
     const ImexPtrs p = imex_ptrs(c);
     const int f = start ? 1 : 0;
