@@ -82,6 +82,33 @@ bool check_shell_columns(const numa_config& c, const HostMesh& m, long long ncol
 
 }  // namespace
 
+// Rows of v + dv as 2^s times them, (signed low 29 bits, rest); s from the
+// largest row sum of |v| below 2^bits.  False out of range.
+static bool imex_ints(int nz, int cols, const std::vector<double>& v, const double* dv, int bits, std::vector<int2>& o,
+                      int& s) {
+  double top = 0.0;
+  for (int i = 0; i < nz; ++i) {
+    double row = 0.0;
+    for (int j = 0; j < cols; ++j) row += std::fabs(v[(size_t)i * cols + j]);
+    top = std::max(top, row);
+  }
+  if (!(top > 0.0) || !std::isfinite(top)) return false;
+  int e2 = 0;
+  std::frexp(top, &e2);  // top < 2^e2
+  s = bits - e2;
+  if (s < -150 || s > 250) return false;
+  const double scale = std::ldexp(1.0, s);
+  o.resize((size_t)nz * cols);
+  for (size_t k = 0; k < o.size(); ++k) {
+    // (v scaled has at most 53 bits above its last one: whole part and rest are exact)
+    const double a = v[k] * scale, w = std::nearbyint(a);
+    const long long q = (long long)w + (long long)std::nearbyint((a - w) + (dv ? dv[k] * scale : 0.0));
+    const long long h = (q + (1LL << 28)) >> 29;
+    o[k] = make_int2((int)(q - (h << 29)), (int)h);
+  }
+  return true;
+}
+
 bool imex_operator(const numa_config& c, const HostMesh& m, ImexTables& t, std::string& err) {
   long long ncol = 0;
   int nz = 0;
@@ -151,6 +178,15 @@ bool imex_operator(const numa_config& c, const HostMesh& m, ImexTables& t, std::
       t.r2[k] = 0.0;
     }
   }
+  if (nz <= kImexDense) {
+    std::vector<double> Dt(t.Dz);
+    for (int k = 0; k < nz; ++k)
+      for (int j = 0; j < W2; ++j) {
+        const int l = k - N + j;
+        Dt[(size_t)k * W2 + j] = l >= 0 && l < nz ? t.Dz[(size_t)k * W2 + j] * t.th0[l] : 0.0;
+      }
+    t.ints = imex_ints(nz, W2, t.Dz, nullptr, 58, t.DzI, t.sD) && imex_ints(nz, W2, Dt, nullptr, 58, t.DtI, t.sT);
+  }
   return true;
 }
 
@@ -177,10 +213,12 @@ static std::vector<double> imex_matrix(const ImexTables& t, double tau) {
   return H;
 }
 
-bool imex_factor(const ImexTables& t, double tau, std::vector<double>& Lf, std::vector<double>& Uf,
-                 std::vector<int>& piv, int* ku, std::string& err) {
+bool imex_factor(const ImexTables& t, double tau, ImexFactor& out, std::string& err) {
   const int nz = t.nz, N = t.N, kl = 2 * N, US = 1 + 4 * N;
-  std::vector<double> H = imex_matrix(t, tau);
+  out.H = imex_matrix(t, tau);
+  std::vector<double> H = out.H;
+  std::vector<double>&Lf = out.Lf, &Uf = out.Uf;
+  std::vector<int>& piv = out.piv;
   // Gaussian elimination with partial pivoting inside the band; the row swap
   // of step k acts on the unfinished columns, so the solve applies swap k and
   // then the multipliers of step k, in that order
@@ -224,86 +262,69 @@ bool imex_factor(const ImexTables& t, double tau, std::vector<double>& Lf, std::
         return false;
       }
   }
-  *ku = kumax;
+  out.ku = kumax;
   return true;
 }
 
-// x += a b in double-double arithmetic.
-static void dd_mac(double& hi, double& lo, double a, double b) {
-  const double p = a * b, e = std::fma(a, b, -p), s = hi + p, t = s - hi;
-  lo += ((hi - (s - t)) + (p - t)) + e;
-  hi = s;
+// The loops below run along rows of nz values, all columns of the inverse at
+// once, for the host's vector units.
+#pragma GCC push_options
+#pragma GCC optimize("O3")
+
+// y += a x, n columns.
+static void row_mac(double* y, double a, const double* x, int n) {
+  for (int c = 0; c < n; ++c) y[c] += a * x[c];
 }
 
-bool imex_dense(const ImexTables& t, double tau, const std::vector<double>& Lf, const std::vector<double>& Uf,
-                const std::vector<int>& piv, ImexDense& out) {
-  const int nz = t.nz, N = t.N, W2 = 2 * N + 1, kl = 2 * N, US = 1 + 4 * N;
-  const std::vector<double> H = imex_matrix(t, tau);
-  auto solve = [&](std::vector<double>& y) {
+// (hi, lo) += a x in double-double arithmetic, n columns.
+static void row_dd_mac(double* __restrict hi, double* __restrict lo, double a, const double* __restrict x, int n) {
+  for (int c = 0; c < n; ++c) {
+    const double p = a * x[c], e = std::fma(a, x[c], -p), s = hi[c] + p, t = s - hi[c];
+    lo[c] += ((hi[c] - (s - t)) + (p - t)) + e;
+    hi[c] = s;
+  }
+}
+
+bool imex_dense(const ImexTables& t, const ImexFactor& f, std::vector<int2>& Hi, int (&exps)[3]) {
+  const int nz = t.nz, N = t.N, kl = 2 * N, US = 1 + 4 * N;
+  if (!t.ints || nz > kImexDense) return false;
+  // H Y = Y for the nz columns of Y; unit: Y is the identity, whose row k meets
+  // columns up to k + kl only on the way down
+  auto solve = [&](std::vector<double>& Y, bool unit) {
+    double* y = Y.data();
     for (int k = 0; k < nz; ++k) {
-      std::swap(y[k], y[piv[3 * k]]);
-      for (int i = 1; i <= piv[3 * k + 1]; ++i) y[k + i] -= Lf[(size_t)k * kl + i - 1] * y[k];
+      const int n = unit ? std::min(nz, k + kl + 1) : nz, p = f.piv[3 * k];
+      if (p != k) std::swap_ranges(y + (size_t)k * nz, y + (size_t)k * nz + n, y + (size_t)p * nz);
+      for (int i = 1; i <= f.piv[3 * k + 1]; ++i)
+        row_mac(y + (size_t)(k + i) * nz, -f.Lf[(size_t)k * kl + i - 1], y + (size_t)k * nz, n);
     }
     for (int k = nz - 1; k >= 0; --k) {
-      for (int j = 1; j <= piv[3 * k + 2]; ++j) y[k] -= Uf[(size_t)k * US + j] * y[k + j];
-      y[k] *= Uf[(size_t)k * US];
+      double* r = y + (size_t)k * nz;
+      for (int j = 1; j <= f.piv[3 * k + 2]; ++j) row_mac(r, -f.Uf[(size_t)k * US + j], r + (size_t)j * nz, nz);
+      for (int c = 0; c < nz; ++c) r[c] *= f.Uf[(size_t)k * US];
     }
   };
-  // columns of H^-1 with one step of refinement, x + dx
-  std::vector<double> X((size_t)nz * nz), dX((size_t)nz * nz), x(nz), r(nz);
-  for (int c = 0; c < nz; ++c) {
-    std::fill(x.begin(), x.end(), 0.0);
-    x[c] = 1.0;
-    solve(x);
-    for (int i = 0; i < nz; ++i) {
-      double hi = i == c ? 1.0 : 0.0, lo = 0.0;
-      for (int j = std::max(0, i - kl); j <= std::min(nz - 1, i + kl); ++j) dd_mac(hi, lo, -H[(size_t)i * nz + j], x[j]);
-      r[i] = hi + lo;
-    }
-    solve(r);
-    for (int i = 0; i < nz; ++i) {
-      X[(size_t)i * nz + c] = x[i];
-      dX[(size_t)i * nz + c] = r[i];
-    }
+  // H^-1 = x + dx with one step of refinement
+  std::vector<double> X((size_t)nz * nz, 0.0), dX((size_t)nz * nz);
+  for (int i = 0; i < nz; ++i) X[(size_t)i * nz + i] = 1.0;
+  solve(X, true);
+  for (int i = 0; i < nz; ++i) {
+    double hi[kImexDense] = {}, lo[kImexDense] = {};
+    hi[i] = 1.0;
+    for (int j = std::max(0, i - kl); j <= std::min(nz - 1, i + kl); ++j)
+      if (f.H[(size_t)i * nz + j] != 0.0) row_dd_mac(hi, lo, -f.H[(size_t)i * nz + j], &X[(size_t)j * nz], nz);
+    for (int c = 0; c < nz; ++c) dX[(size_t)i * nz + c] = hi[c] + lo[c];
   }
-  // rows of x + dx as 2^s times them, (signed low 29 bits, rest); s from the largest row sum
-  auto table = [&](const std::vector<double>& v, const double* dv, int cols, int bits, std::vector<int2>& o, int& s) {
-    double top = 0.0;
-    for (int i = 0; i < nz; ++i) {
-      double row = 0.0;
-      for (int j = 0; j < cols; ++j) row += std::fabs(v[(size_t)i * cols + j]);
-      top = std::max(top, row);
-    }
-    if (!(top > 0.0) || !std::isfinite(top)) return false;
-    int e2 = 0;
-    std::frexp(top, &e2);  // top < 2^e2
-    s = bits - e2;
-    if (s < -150 || s > 250) return false;
-    o.resize((size_t)nz * cols);
-    for (size_t k = 0; k < o.size(); ++k) {
-      // (v scaled has at most 53 bits above its last one: whole part and rest are exact)
-      const double a = std::ldexp(v[k], s), w = std::nearbyint(a);
-      const long long q = (long long)w + std::llrint((a - w) + (dv ? std::ldexp(dv[k], s) : 0.0));
-      const long long h = (q + (1LL << 28)) >> 29;
-      o[k] = make_int2((int)(q - (h << 29)), (int)h);
-    }
-    return true;
-  };
-  std::vector<double> Dt(t.Dz);
-  for (int k = 0; k < nz; ++k)
-    for (int j = 0; j < W2; ++j) {
-      const int l = k - N + j;
-      Dt[(size_t)k * W2 + j] = l >= 0 && l < nz ? t.Dz[(size_t)k * W2 + j] * t.th0[l] : 0.0;
-    }
-  int sH = 0, sD = 0, sT = 0;
+  solve(dX, false);
+  int sH = 0;
   // (59 bits: with the refinement the row sums stay below 2^60)
-  if (!table(X, dX.data(), nz, 59, out.Hi, sH) || !table(t.Dz, nullptr, W2, 58, out.DzI, sD) ||
-      !table(Dt, nullptr, W2, 58, out.DtI, sT))
-    return false;
-  out.y_exp = 66 - sH;
-  out.d_exp = 124 - sH - sD;
-  out.t_exp = 124 - sH - sT;
+  if (!imex_ints(nz, nz, X, dX.data(), 59, Hi, sH)) return false;
+  exps[0] = 66 - sH;
+  exps[1] = 124 - sH - t.sD;
+  exps[2] = 124 - sH - t.sT;
   return true;
 }
+
+#pragma GCC pop_options
 
 }  // namespace numa

@@ -225,45 +225,51 @@ ImexPtrs imex_ptrs(const numa_ctx* c) {
   return p;
 }
 
-// Host factors of the column matrices for dt and dt/2 into the workspace
-// (when dt changed), with the operator tables; waits for the copies.
+// What 1D-IMEX steps of dt read into the workspace, where it is not there yet:
+// operator tables and the factors for dt and dt/2, and for columns of up to
+// kImexDense levels the inverse for the start step (start) and for the steps
+// after it (rest), each only when such a step follows (an inverse of 64 levels
+// takes the host about as long as a step of a small mesh).  Waits for the copies.
 // NUMA_EINVAL when a matrix cannot be factored, NUMA_ECUDA on a CUDA error.
-int imex_prepare(numa_ctx* c, double dt) {
+int imex_prepare(numa_ctx* c, double dt, bool start, bool rest) {
   cudaError_t e = imex_kernel_setup();
   if (e != cudaSuccess) return cuda_fail(c, e, "1D-IMEX kernel setup");
-  if (c->imex_factored && c->imex_dt == dt) return NUMA_OK;
-  std::string err;
-  ImexPtrs p = imex_ptrs(c);
+  const bool need[2] = {rest, start};
+  const bool same = c->imex_factored && c->imex_dt == dt;
+  if (same && (!rest || c->imex_ready[0]) && (!start || c->imex_ready[1])) return NUMA_OK;
+  const ImexPtrs p = imex_ptrs(c);
   const ImexTables& t = c->imex;
-  std::vector<double> Lf, Uf;
+  std::vector<double> tab;  // the tables as they lie in the workspace
   std::vector<int> piv;
-  const size_t nz = (size_t)t.nz;
-  e = cudaMemcpyAsync(p.Dz, t.Dz.data(), t.Dz.size() * 8, cudaMemcpyHostToDevice, c->stream);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(p.c2, t.c2.data(), nz * 8, cudaMemcpyHostToDevice, c->stream);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(p.th0, t.th0.data(), nz * 8, cudaMemcpyHostToDevice, c->stream);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(p.gl, t.gl.data(), nz * 8, cudaMemcpyHostToDevice, c->stream);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(p.r2, t.r2.data(), nz * 8, cudaMemcpyHostToDevice, c->stream);
-  int ku[2] = {0, 0};
-  for (int f = 0; f < 2 && e == cudaSuccess; ++f) {
-    if (!imex_factor(t, f == 0 ? dt : 0.5 * dt, Lf, Uf, piv, &ku[f], err)) return fail(c, NUMA_EINVAL, err);
-    e = cudaMemcpyAsync(p.Lf[f], Lf.data(), Lf.size() * 8, cudaMemcpyHostToDevice, c->stream);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(p.Uf[f], Uf.data(), Uf.size() * 8, cudaMemcpyHostToDevice, c->stream);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(p.piv[f], piv.data(), 3 * nz * sizeof(int), cudaMemcpyHostToDevice, c->stream);
-    ImexDense d;
-    c->imex_int[f] = t.nz <= kImexDense && imex_dense(t, f == 0 ? dt : 0.5 * dt, Lf, Uf, piv, d);
-    if (c->imex_int[f]) {
-      c->imex_exp[f][0] = d.y_exp;
-      c->imex_exp[f][1] = d.d_exp;
-      c->imex_exp[f][2] = d.t_exp;
-      if (e == cudaSuccess) e = cudaMemcpyAsync(p.Hi[f], d.Hi.data(), d.Hi.size() * 8, cudaMemcpyHostToDevice, c->stream);
-      if (e == cudaSuccess) e = cudaMemcpyAsync(p.DzI, d.DzI.data(), d.DzI.size() * 8, cudaMemcpyHostToDevice, c->stream);
-      if (e == cudaSuccess) e = cudaMemcpyAsync(p.DtI, d.DtI.data(), d.DtI.size() * 8, cudaMemcpyHostToDevice, c->stream);
+  std::vector<int2> Hi[2];
+  if (!same) {
+    c->imex_factored = c->imex_ready[0] = c->imex_ready[1] = false;
+    std::string err;
+    for (int f = 0; f < 2; ++f) {
+      if (!imex_factor(t, f == 0 ? dt : 0.5 * dt, c->imex_f[f], err)) return fail(c, NUMA_EINVAL, err);
+      if (t.nz > kImexDense) std::vector<double>().swap(c->imex_f[f].H);
     }
-    if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);  // the host vectors are reused
+    const ImexFactor* f = c->imex_f;
+    for (const auto* v : {&t.Dz, &t.c2, &t.th0, &t.gl, &t.r2, &f[0].Lf, &f[0].Uf, &f[1].Lf, &f[1].Uf})
+      tab.insert(tab.end(), v->begin(), v->end());
+    if (t.ints) {
+      const size_t n = tab.size();
+      tab.resize(n + t.DzI.size() + t.DtI.size());
+      std::memcpy(tab.data() + n, t.DzI.data(), t.DzI.size() * 8);
+      std::memcpy(tab.data() + n + t.DzI.size(), t.DtI.data(), t.DtI.size() * 8);
+    }
+    for (int k = 0; k < 2; ++k) piv.insert(piv.end(), f[k].piv.begin(), f[k].piv.end());
+    e = cudaMemcpyAsync(p.Dz, tab.data(), tab.size() * 8, cudaMemcpyHostToDevice, c->stream);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(p.piv[0], piv.data(), piv.size() * sizeof(int), cudaMemcpyHostToDevice, c->stream);
   }
+  for (int f = 0; f < 2 && e == cudaSuccess; ++f) {
+    if (!need[f] || c->imex_ready[f]) continue;
+    c->imex_int[f] = imex_dense(t, c->imex_f[f], Hi[f], c->imex_exp[f]);
+    if (c->imex_int[f]) e = cudaMemcpyAsync(p.Hi[f], Hi[f].data(), Hi[f].size() * 8, cudaMemcpyHostToDevice, c->stream);
+  }
+  if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);  // the host vectors end here
   if (e != cudaSuccess) return cuda_fail(c, e, "1D-IMEX factor upload");
-  c->imex_ku[0] = ku[0];
-  c->imex_ku[1] = ku[1];
+  for (int f = 0; f < 2; ++f) c->imex_ready[f] |= need[f];
   c->imex_dt = dt;
   c->imex_factored = true;
   return NUMA_OK;
@@ -311,7 +317,7 @@ cudaError_t enqueue_imex_step(numa_ctx* c, double dt, bool start, cudaStream_t s
     a.N = c->imex.N;
     a.nz = c->imex.nz;
     a.kl = c->imex.kl;
-    a.ku = c->imex_ku[f];
+    a.ku = c->imex_f[f].ku;
     a.cols_per_block = imex_cols_per_block(a.nz, a.N);
     a.ncol = c->imex_ncol;
     a.Ng = c->mesh.Ng;
@@ -851,7 +857,7 @@ int numa_rk_step(numa_ctx* c, double dt) {
   cudaError_t e = ensure_prim(c);
   if (c->rk_scheme == NUMA_LEAPFROG_IMEX) {
     if (e == cudaSuccess) {
-      const int rc = imex_prepare(c, dt);
+      const int rc = imex_prepare(c, dt, !c->imex_started, c->imex_started);
       if (rc != NUMA_OK) return rc;
       e = enqueue_imex_step(c, dt, !c->imex_started, c->stream);
     }
@@ -873,16 +879,19 @@ int numa_run(numa_ctx* c, double dt, int nsteps) {
   if (nsteps < 0 || !std::isfinite(dt)) return fail(c, NUMA_EINVAL, "bad nsteps or dt");
   cudaError_t e = cudaSuccess;
   const bool imex = c->rk_scheme == NUMA_LEAPFROG_IMEX;
+  const bool start = imex && nsteps > 0 && !c->imex_started;
+  const bool rest = imex ? nsteps > (start ? 1 : 0) : true;  // steps of the graph
   if (imex && nsteps > 0) {
-    const int rc = imex_prepare(c, dt);
+    const int rc = imex_prepare(c, dt, start, rest);
     if (rc != NUMA_OK) return rc;
   }
-  if (!c->graph || c->graph_dt != dt || c->graph_q != c->L.q) {
+  if (!c->cap_stream) e = cudaStreamCreateWithFlags(&c->cap_stream, cudaStreamNonBlocking);
+  if (e != cudaSuccess) return cuda_fail(c, e, "numa_run capture stream");
+  if (rest && (!c->graph || c->graph_dt != dt || c->graph_q != c->L.q)) {
     if (c->graph) {
       cudaGraphExecDestroy(c->graph);
       c->graph = nullptr;
     }
-    if (!c->cap_stream) e = cudaStreamCreateWithFlags(&c->cap_stream, cudaStreamNonBlocking);
     cudaGraph_t g = nullptr;
     if (e == cudaSuccess) e = cudaStreamBeginCapture(c->cap_stream, cudaStreamCaptureModeThreadLocal);
     if (e == cudaSuccess) {
@@ -944,7 +953,8 @@ int numa_time_kernels(numa_ctx* c, double dt, int nsteps, double* ms_volume, dou
   for (auto& x : ev)
     if (e == cudaSuccess) e = cudaEventCreate(&x);
   if (c->rk_scheme == NUMA_LEAPFROG_IMEX && e == cudaSuccess && nsteps > 0) {
-    const int rc = imex_prepare(c, dt);
+    const bool start = !c->imex_started;
+    const int rc = imex_prepare(c, dt, start, nsteps > (start ? 1 : 0));
     if (rc != NUMA_OK) {
       for (auto& x : ev)
         if (x) cudaEventDestroy(x);

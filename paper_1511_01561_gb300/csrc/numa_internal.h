@@ -248,11 +248,22 @@ struct ImexArgs {
 
 // Host tables of the vertical operator and the factors of one Schur matrix.
 struct ImexTables {
-  int nz = 0, N = 0, kl = 0, ku = 0;
+  int nz = 0, N = 0, kl = 0;
   std::vector<double> Dz, c2, th0;  // [nz][2N+1], [nz], [nz]
   std::vector<double> gl, r2;       // [nz] g(r) and 2 / r per level (box: g and 0)
-  std::vector<double> Lf, Uf;       // [nz][kl], [nz][1 + 4N] (ku <= 4N used)
-  std::vector<int> piv;             // [nz][3] (see ImexArgs::piv)
+  // Dz and Dz theta0 as integers, 2^sD and 2^sT times them, their largest row sums below 2^58 (columns of up
+  // to kImexDense levels); ints: they are in range
+  std::vector<int2> DzI, DtI;
+  int sD = 0, sT = 0;
+  bool ints = false;
+};
+
+// One Schur matrix of the columns and its factors (see ImexArgs).
+struct ImexFactor {
+  std::vector<double> H;       // [nz][nz]
+  std::vector<double> Lf, Uf;  // [nz][kl], [nz][1 + 4N] (ku <= 4N used)
+  std::vector<int> piv;        // [nz][3]
+  int ku = 0;
 };
 
 // 1D-IMEX: whether the configuration has straight walled vertical columns
@@ -260,21 +271,15 @@ struct ImexTables {
 // column count and height, and the host tables (imex_setup.cpp).
 bool imex_supported(const numa_config& c, long long* ncol, int* nz, std::string* why);
 bool imex_operator(const numa_config& c, const HostMesh& m, ImexTables& t, std::string& err);
-bool imex_factor(const ImexTables& t, double tau, std::vector<double>& Lf, std::vector<double>& Uf,
-                 std::vector<int>& piv, int* ku, std::string& err);
+bool imex_factor(const ImexTables& t, double tau, ImexFactor& f, std::string& err);
 size_t imex_table_doubles(int nz, int N);
 // Columns of at most this many levels are solved with the inverse of the Schur
 // matrix (imex.cu).
 constexpr int kImexDense = 64;
-// The integers of one factored matrix: H^-1 (refined beyond FP64), Dz and
-// Dz theta0, each with its largest row sum scaled below 2^60 (H^-1) or 2^58, and
-// the exponents of their products.  False if they are out of range.
-struct ImexDense {
-  std::vector<int2> Hi, DzI, DtI;
-  int y_exp = 0, d_exp = 0, t_exp = 0;
-};
-bool imex_dense(const ImexTables& t, double tau, const std::vector<double>& Lf, const std::vector<double>& Uf,
-                const std::vector<int>& piv, ImexDense& d);
+// The inverse of a factored matrix as integers (refined beyond FP64, its largest
+// row sum below 2^60), and the exponents of y = H^-1 r, Dz y and Dz(theta0 y).
+// False if they are out of range.
+bool imex_dense(const ImexTables& t, const ImexFactor& f, std::vector<int2>& Hi, int (&exps)[3]);
 
 // One application of the Boyd-Vandeven filter (element part).
 struct FilterArgs {
@@ -394,8 +399,9 @@ struct numa_ctx {
   numa::ImexTables imex;
   long long imex_ncol = 0;
   double imex_dt = 0.0;
-  int imex_ku[2] = {0, 0};  // upper bandwidths of the factors for dt and dt/2
-  bool imex_int[2] = {false, false};  // their fixed-point inverses are in the workspace, with these exponents
+  numa::ImexFactor imex_f[2];  // for dt and dt/2 (the start step)
+  bool imex_ready[2] = {false, false};  // everything that steps with them read is in the workspace
+  bool imex_int[2] = {false, false};  // their fixed-point inverses among it, with these exponents
   int imex_exp[2][3] = {};
   bool imex_factored = false;
   bool imex_started = false;

@@ -239,3 +239,31 @@ def test_rest_on_tiny_elements(numa, orc, s2):
     cfg = I.box((3, 2, 2), N, L=(3 * h, 2 * h, 2 * h))
     R = _rhs(numa, cfg, np.zeros((5, orc.Mesh(cfg).Ng)))
     assert np.array_equal(R, np.zeros_like(R))
+
+
+# 1D-IMEX through run and rk_step in any division into calls, with a new time
+# step in between and a run of no steps first: the same states bit for bit (the
+# columns' inverses are made when a step first needs them)
+@pytest.mark.parametrize("nez", [3, 12, 17])
+def test_imex_calls_in_any_division(numa, nez):
+    cfg = I.box((2, 2, nez), 4, L=(4000.0, 4000.0, 250.0 * nez))
+
+    def go(*calls):
+        s = numa.Solver(cfg, "fp64")
+        try:
+            s.set_time_scheme("imex")
+            s.init_state("bubble", (0.5, 600.0, 2000.0, 2000.0, 120.0 * nez))
+            for dt, n, graph in calls:
+                if graph:
+                    s.run(dt, n)
+                else:
+                    for _ in range(n):
+                        s.rk_step(dt)
+            return s.get_state().numpy().copy()
+        finally:
+            s.close()
+
+    a = go((0.2, 3, True), (0.1, 2, True), (0.2, 1, True))
+    assert np.isfinite(a).all() and np.abs(a).max() > 0.0
+    assert np.array_equal(a, go((0.2, 3, False), (0.1, 2, False), (0.2, 1, False)))
+    assert np.array_equal(a, go((0.2, 0, True), (0.2, 1, True), (0.2, 2, True), (0.1, 1, False), (0.1, 1, True), (0.2, 1, True)))
