@@ -878,8 +878,12 @@ __global__ void __launch_bounds__(((N + 1) * (N + 1) * (N + 1) + 31) / 32 * 32)
 // update_kernel: the member's DSS order within the block (sorted by entry
 // count), the structured box DSS on CG boxes, then the rest in natural
 // order.  Members' node ranges are padded to whole blocks in the table.
+// FP32-mixed shells take 40 registers, 12 blocks an SM, as they did before the
+// stores went behind the loads: with the 55 that took by itself a step of a
+// served shell of 1.5M element nodes at N = 3 rose from 375 to 397 us (371 so), at
+// N = 1 from 437 to 445 (435).  On boxes the registers cost nothing.
 template <int MODE, bool SHELL, typename RT>
-__global__ void __launch_bounds__(kDssBlock) update_ragged(const MemberDesc* __restrict__ d,
+__global__ void __launch_bounds__(kDssBlock, SHELL && sizeof(RT) == 4 ? 12 : 0) update_ragged(const MemberDesc* __restrict__ d,
                                                            const RaggedGroup* __restrict__ g, int stage) {
   __shared__ double sums[5][kDssBlock];
   __shared__ int s_slot;
