@@ -3,13 +3,15 @@
 //
 // GB300 issues 2 FP64 operations per SM per clock and 32 32x32+64-bit integer
 // multiply-adds (IMAD.WIDE), so a product of two 58-bit numbers in three of
-// them costs 3 cycles of the SM per warp against 16 for an FP64 FMA.  Every
-// field of an element is a 58- or 59-bit integer relative to the largest magnitude
-// of its equation group in the element (a power of two), D as a
-// 60-bit integer relative to its largest row sum, and their products are
-// summed exactly in 64-bit accumulators.  What is dropped is below 2^-58 of
-// (largest field) x (row sum of |D|), the size whose 2^-53 an FP64 chain
-// loses at every step.
+// them costs 3 cycles of the SM per warp against 16 for an FP64 FMA.  The flux
+// fields of an element are 58- or 59-bit integers relative to the largest value of
+// their equation in the element (a power of two), with the directions scaled by
+// the size of their metric terms (FxScale); D is a 59- or 60-bit integer relative to
+// its largest row sum, and their products are summed exactly in 64-bit
+// accumulators.  What is dropped is a few units of 2^-58 (2^-56 where equations
+// share a unit, fx_join) of max_c K_c |F_vc| x (row sum of |D|), K_c the metric
+// terms' size along c: the size whose 2^-53 an FP64 chain loses at every step, on
+// elements of any aspect.
 //
 // Elements whose values the integers cannot hold (an infinity or a NaN, or
 // magnitudes near the ends of the FP64 range) go through a plain FP64 form,
@@ -80,7 +82,7 @@ __host__ __device__ constexpr int fx_slots() {
 template <int N>
 constexpr size_t fx_rect_smem() {
   constexpr int EPB = fx_rect_epb<N>();
-  return 8 * (size_t)(kLF + 10) * EPB * fx_pitch<N>() + 16 * fx_slots<EPB, fx_rect_threads<N>()>();
+  return 8 * (size_t)15 * EPB * fx_pitch<N>() + sizeof(FxKeys) * fx_slots<EPB, fx_rect_threads<N>()>();
 }
 
 // The per-node form: one thread per node, several elements for the small
@@ -96,7 +98,7 @@ __host__ __device__ constexpr int fx_nodal_threads() {
 template <int N>
 constexpr size_t fx_nodal_smem() {
   constexpr int EPB = fx_nodal_epb<N>();
-  return 8 * (size_t)(2 * kLF) * EPB * fx_pitch<N>() + 16 * fx_slots<EPB, fx_nodal_threads<N>()>();
+  return 8 * (size_t)(2 * kLF) * EPB * fx_pitch<N>() + sizeof(FxKeys) * fx_slots<EPB, fx_nodal_threads<N>()>();
 }
 
 // A mesh's tables as a kernel parameter: K_d D for the three directions
@@ -142,110 +144,172 @@ __device__ __forceinline__ void rect_plain(const VolumeArgs& a, long long e) {
   }
 }
 
-// Gathers U, u, theta and p' at the nn element nodes from n0, one thread per
-// element node, and leaves the 12 flux fields in F as fixed-point integers.
-// The largest magnitudes in an element give its groups' exponents: left as
-// keys per element in gmax (EPB > 1), or returned in ge (EPB = 1).  False
-// (uniform over the CTA) if the integers cannot hold its one element; with
-// several, the fields of an element they cannot hold (fx_in_range of its key)
-// are left unset, so that no element's result depends on which others share
-// its CTA (a slab launch groups them otherwise).
-template <int N, int EPB, int NT, bool PIPE>
-__device__ __forceinline__ bool fx_stage(const VolumeArgs& a, long long n0, int nn, uint4* gmax, int2* F, FxExp& ge) {
+// An element's scale, ten bits a direction, in the last word of its metric exponents.
+__device__ __forceinline__ FxScale fx_scale_of(int packed) {
+  return {{packed & 1023, (packed >> 10) & 1023, (packed >> 20) & 1023}};
+}
+// The exponents of element t of the CTA (EPB > 1: they take its keys' place).
+__device__ __forceinline__ const FxExp& fx_slot(const FxKeys* keys, int t) {
+  return reinterpret_cast<const FxExp*>(keys)[t];
+}
+
+// Gathers U, u, theta and p' at the nodes of the ne elements from e0, one thread per
+// element node, and leaves their flux fields in F as fixed-point integers (15
+// for the rectilinear form, 12 for the per-node form).  The largest magnitudes
+// in an element give its groups' exponents: returned in ge for the thread's own
+// element node, and with several elements left in shared memory (fx_slot) for
+// every element.  The fields of an element that the integers cannot hold (ok = 0)
+// are left unset: no element's result depends on which others share its CTA (a
+// slab launch groups them otherwise).  w: the scale of the thread's element.
+template <int N, int EPB, int NT, bool RECT>
+__device__ __forceinline__ void fx_stage(const VolumeArgs& a, long long e0, int ne, FxKeys* keys, int2* F,
+                                         const FxScale& w, FxExp& ge) {
   constexpr int NP = (N + 1) * (N + 1) * (N + 1), NN = EPB * NP, IT = (NN + NT - 1) / NT;
   constexpr int FP = EPB * fx_pitch<N>(), SLOTS = fx_slots<EPB, NT>();
-  const int tid = threadIdx.x;
+  static_assert(RECT || IT == 1, "one scale per thread");
+  const int tid = threadIdx.x, nn = ne * NP;
   if constexpr (EPB > 1) {
-    if (tid < EPB) gmax[tid] = make_uint4(0u, 0u, 0u, 0u);
+    if (tid < EPB) keys[tid] = FxKeys();
     __syncthreads();
   }
-  uint4 gw = make_uint4(0u, 0u, 0u, 0u);
+  FxKeys g = FxKeys();
   NodeState64 z[IT];
 #pragma unroll
   for (int it = 0; it < IT; ++it) {
     const int l = tid + it * NT;
     if (l < nn) {
-      z[it] = gather_node64(a, n0 + l);
-      const uint4 k = make_uint4(fx_group_key(z[it].U, 3), fx_group_key(z[it].u, 3), fx_group_key(&z[it].th, 1),
-                                 fx_group_key(&z[it].pp, 1));
-      if constexpr (EPB == 1) {
-        gw = make_uint4(max(gw.x, k.x), max(gw.y, k.y), max(gw.z, k.z), max(gw.w, k.w));
+      z[it] = gather_node64(a, e0 * NP + l);
+      if constexpr (EPB == 1) {  // (without the low words: see below)
+        g.U = max(g.U, fx_high_scaled(z[it].U, w));
+#pragma unroll
+        for (int c = 0; c < 3; ++c) g.u[c] = max(g.u[c], fx_high(z[it].u[c]));
+        g.th = max(g.th, fx_high(z[it].th));
+        g.pp = max(g.pp, fx_high(z[it].pp));
       } else {
-        unsigned* g = reinterpret_cast<unsigned*>(gmax + l / NP);
-        atomicMax(&g[0], k.x);
-        atomicMax(&g[1], k.y);
-        atomicMax(&g[2], k.z);
-        atomicMax(&g[3], k.w);
+        g.U = fx_key_scaled(z[it].U, w);
+#pragma unroll
+        for (int c = 0; c < 3; ++c) g.u[c] = fx_key(z[it].u[c]);
+        g.th = fx_key(z[it].th);
+        g.pp = fx_key(z[it].pp);
+        FxKeys* e = keys + l / NP;
+        atomicMax(&e->U, g.U);
+        atomicMax(&e->th, g.th);
+        atomicMax(&e->pp, g.pp);
+#pragma unroll
+        for (int c = 0; c < 3; ++c) atomicMax(&e->u[c], g.u[c]);
       }
     }
   }
   if constexpr (EPB == 1) {
-    gw.x = __reduce_max_sync(0xffffffffu, gw.x);
-    gw.y = __reduce_max_sync(0xffffffffu, gw.y);
-    gw.z = __reduce_max_sync(0xffffffffu, gw.z);
-    gw.w = __reduce_max_sync(0xffffffffu, gw.w);
-    if ((tid & 31) == 0) gmax[tid >> 5] = gw;
+    g.U = __reduce_max_sync(0xffffffffu, g.U);
+    g.th = __reduce_max_sync(0xffffffffu, g.th);
+    g.pp = __reduce_max_sync(0xffffffffu, g.pp);
+#pragma unroll
+    for (int c = 0; c < 3; ++c) g.u[c] = __reduce_max_sync(0xffffffffu, g.u[c]);
+    if ((tid & 31) == 0) keys[tid >> 5] = g;
   }
   grid_wait();  // (threads without a node; before any write of the kernel)
   __syncthreads();
-  uint4 gm = make_uint4(0u, 0u, 0u, 0u);
   if constexpr (EPB == 1) {
+    // every warp by itself: lane j (of eight) the largest of key j; lanes 4 to 6 the
+    // exponents of the three momentum equations
+    const int lane = tid & 7;
+    const unsigned* q = reinterpret_cast<const unsigned*>(keys) + lane;
+    unsigned k = 0;
 #pragma unroll
-    for (int t = 0; t < SLOTS; ++t) {
-      const uint4 w = gmax[t];
-      gm = make_uint4(max(gm.x, w.x), max(gm.y, w.y), max(gm.z, w.z), max(gm.w, w.w));
+    for (int t = 0; t < SLOTS; ++t) k = max(k, q[8 * t]);
+    const unsigned U = __shfl_sync(0xffffffffu, k, 0), th = __shfl_sync(0xffffffffu, k, 1);
+    const unsigned pp = __shfl_sync(0xffffffffu, k, 2);
+    bool in;
+    const int m = fx_momentum_exp(U, k, pp, lane == 4 ? w.s[0] : lane == 5 ? w.s[1] : w.s[2], in);
+    const bool ok = fx_scalar_exps(ge, U, th, pp);
+    ge.ok = __all_sync(0xffffffffu, ok && (in || lane < 4 || lane == 7));
+#pragma unroll
+    for (int c = 0; c < 3; ++c) ge.m[c] = __shfl_sync(0xffffffffu, m, 4 + c);
+    fx_join(ge, w);
+    if (__any_sync(0xffffffffu, k == 0 && lane != 3 && lane != 7)) {  // (uniform over the CTA)
+      // a group that is zero, or whose values lie below 2^-1042 (plain FP64 then)
+      bool zero[3];
+#pragma unroll
+      for (int c = 0; c < 3; ++c) zero[c] = __shfl_sync(0xffffffffu, k, 4 + c) == 0;
+      unsigned low = 0;
+#pragma unroll
+      for (int it = 0; it < IT; ++it) {
+        if (tid + it * NT < nn) {
+          if (U == 0) low |= fx_key(z[it].U[0]) | fx_key(z[it].U[1]) | fx_key(z[it].U[2]);
+#pragma unroll
+          for (int c = 0; c < 3; ++c)
+            if (zero[c]) low |= fx_key(z[it].u[c]);
+          if (th == 0) low |= fx_key(z[it].th);
+          if (pp == 0) low |= fx_key(z[it].pp);
+        }
+      }
+      if (__syncthreads_or(low != 0)) ge.ok = 0;
     }
-    if (!fx_in_range(gm)) return false;
-    ge = fx_exps(gm);
+  } else {
+    if (tid < ne) {
+      FxScale we = w;
+      if constexpr (!RECT) we = fx_scale_of(a.fxE[e0 + tid].w);
+      const FxExp e = fx_exps(keys[tid], we);
+      *reinterpret_cast<FxExp*>(keys + tid) = e;
+    }
+    __syncthreads();
   }
 #pragma unroll
   for (int it = 0; it < IT; ++it) {
     const int l = tid + it * NT;
     if (l < nn) {
-      if constexpr (EPB > 1) {
-        gm = gmax[l / NP];
-        if (!fx_in_range(gm)) continue;
+      if constexpr (EPB > 1) ge = fx_slot(keys, l / NP);
+      if (ge.ok) {
+        int2* f = F + fx_index<N>(l);
+        auto put = [&](int slot, int2 x) { f[slot * FP] = x; };
+        if constexpr (RECT) fx_fluxes(z[it], ge, w, put);
+        else fx_fluxes_shared(z[it], ge, w, put);
       }
-      const FxExp e = fx_exps(gm);
-      int2* f = F + fx_index<N>(l);
-      fx_fluxes<PIPE>(z[it], e, gm.z, [&](int slot, int2 x) { f[slot * FP] = x; });
     }
   }
-  return true;
 }
 
 // create_rhs of up to fx_rect_epb<N>() rectilinear elements e0 .. e0 + ne - 1
 // in fixed point: the residual sum_d K_d (D F_d) without its weight
 // w_i w_j w_k (which the update applies with the inverse mass).
-//   1. the 12 flux fields go to shared memory (fx_stage);
+//   1. the 15 flux fields (of equation v along direction d: 5 d + v) go to
+//      shared memory (fx_stage);
 //   2. thread t takes line t of the 5 (N+1)^2 lines along x (equation
 //      v = t / (N+1)^2), then along y (fx_line), and leaves the derivatives in
-//      shared memory;
+//      the line's place: each line of a field is read by one thread only;
 //   3. it then takes its line along z, adds the x and y derivatives at the
 //      line's nodes as integers and converts the sums to FP64, rounded once.
-// On 32^3 elements at N = 4: 0.529 ms as FP64 (its pipe 97% busy: 75
-// operations a node at 16 cycles a warp), 0.156 ms here; 19x23x17 at N = 6:
-// 0.460 -> 0.135 ms.  135 integer multiply-adds a thread keep their pipe a
-// quarter busy; shared memory, the scattered gather and the instructions
-// beside the products are what is left.  D in the kernel parameters instead
-// of global memory: 0.256 -> 0.226 ms; the z lines finishing the nodes (10
-// shared accesses a node fewer, ten CTAs an SM instead of eight): 0.226 ->
-// 0.216 ms; the products formed here from 8 gathered fields instead of 12
-// gathered fluxes: 0.216 -> 0.186 ms (and the update 0.199 -> 0.169 ms); the
-// results converted by the FP64 pipe and 64 registers: 0.186 -> 0.156 ms.
+// On 32^3 elements at N = 4: 0.529 ms as FP64 (its pipe 97% busy: 75 operations
+// a node at 16 cycles a warp), 0.164 ms here on the rising bubble (0.172 where the
+// momentum equations' units differ); 19x23x17 at N = 6: 0.460 -> 0.132 ms, 12^3 at
+// N = 8 0.090 ms.  135 to 144 integer multiply-adds a thread; the instructions beside
+// them (1060 a warp and element) and shared memory are what is left.  One unit for
+// all of momentum and one scale took 0.154 ms, with an error that grew with an
+// element's aspect.  D in the kernel parameters instead of global memory: 0.256 ->
+// 0.226 ms; the z lines finishing the nodes (10 shared accesses a node fewer):
+// 0.226 -> 0.216; the products formed here from 8 gathered fields instead of 12
+// gathered fluxes: 0.216 -> 0.186 (and the update 0.199 -> 0.169 ms); the results
+// converted by the FP64 pipe and 64 registers: 0.186 -> 0.156.  Derivatives in the
+// lines' place (15 fields of shared memory, not 22): N = 8 0.132 -> 0.090 ms.
 template <int N>
 __device__ __forceinline__ void volume_fx_rect(const VolumeArgs& a, const int2* T, long long e0, int ne,
                                                unsigned char* smem_raw) {
   constexpr int P = N + 1, PP = P * P, NP = PP * P, EPB = fx_rect_epb<N>(), NT = fx_rect_threads<N>();
   constexpr int EP = fx_pitch<N>(), FP = EPB * EP, M = fx_table_entries<N>(), B = fx_plane<N>();
-  uint4* gmax = reinterpret_cast<uint4*>(smem_raw);                // (first: 16-byte aligned)
-  int2* F = reinterpret_cast<int2*>(gmax + fx_slots<EPB, NT>());  // [kLF][FP]
-  long long* part = reinterpret_cast<long long*>(F + kLF * FP);    // [2][5][FP]
+  FxKeys* keys = reinterpret_cast<FxKeys*>(smem_raw);              // (first: 16-byte aligned)
+  int2* F = reinterpret_cast<int2*>(keys + fx_slots<EPB, NT>());  // [15][FP]
   const int tid = threadIdx.x;
   const long long n0 = e0 * NP;
+  const FxScale w = {{a.fxs[0], a.fxs[1], a.fxs[2]}};
   FxExp ge;
-  if (a.fxD == nullptr || !fx_stage<N, EPB, NT, false>(a, n0, ne * NP, gmax, F, ge)) {  // uniform over the CTA
+  if (a.fxD == nullptr) {
     for (int t = 0; t < ne; ++t) rect_plain<N>(a, e0 + t);
+    return;
+  }
+  fx_stage<N, EPB, NT, true>(a, e0, ne, keys, F, w, ge);
+  if (EPB == 1 && !ge.ok) {  // (uniform over the CTA)
+    rect_plain<N>(a, e0);
     return;
   }
   __syncthreads();
@@ -255,39 +319,31 @@ __device__ __forceinline__ void volume_fx_rect(const VolumeArgs& a, const int2* 
   if (act) {
 #pragma unroll
     for (int d = 0; d < 2; ++d) {
-      // the field of equation v along x, y (four bits each)
-      constexpr unsigned fy = sUy | sTxy << 4 | sTyy << 8 | sTyz << 12 | sHy << 16;
-      const int f = d == 0 ? v : (int)((fy >> (4 * v)) & 15u);
-      const int base = el * EP + fx_line_base<N>(d, r), st = fx_line_stride<N>(d);
+      int2* f = F + (5 * d + v) * FP + el * EP + fx_line_base<N>(d, r);
+      const int st = fx_line_stride<N>(d);
       long long out[P];
-      fx_line<N>(F + f * FP + base, st, T + d * M, out);
-      long long* o = part + (d * 5 + v) * FP + base;
+      fx_line<N>(f, st, T + d * M, out);
 #pragma unroll
-      for (int m = 0; m < P; ++m) o[m * st] = out[m];
+      for (int m = 0; m < P; ++m) f[m * st] = make_int2((int)out[m], (int)(out[m] >> 32));
     }
   }
   __syncthreads();
   if (act) {
-    constexpr unsigned fz = sUz | sTxz << 4 | sTyz << 8 | sTzz << 12 | sHz << 16;
-    const int f = (int)((fz >> (4 * v)) & 15u), base = el * EP + fx_line_base<N>(2, r);
+    const int2* o = F + v * FP + el * EP + fx_line_base<N>(2, r);
     long long out[P];
-    fx_line<N>(F + f * FP + base, B, T + 2 * M, out);
-    const long long* o = part + v * FP + base;
-    bool ok = true;
-    if constexpr (EPB > 1) {
-      ok = fx_in_range(gmax[el]);
-      ge = fx_exps(gmax[el]);
-    }
-    if (ok) {
-      const int kexp = (v == 0 ? ge.U : v == 4 ? ge.t : ge.m) + a.fxexp;
+    fx_line<N>(o + 10 * FP, B, T + 2 * M, out);
+    if constexpr (EPB > 1) ge = fx_slot(keys, el);
+    if (ge.ok) {
+      const int kexp = (v == 0 ? ge.U : v == 4 ? ge.t : ge.m[v == 1 ? 0 : v == 2 ? 1 : 2]) + a.fxexp;
       double* re = static_cast<double*>(a.re) + v * a.Nl + n0 + el * NP + r;
+      auto value = [&](int2 x) { return (long long)x.y << 32 | (unsigned)x.x; };
 #pragma unroll
-      for (int m = 0; m < P; ++m) re[m * PP] = fx_to_double(out[m] + o[m * B] + o[5 * FP + m * B], kexp);
+      for (int m = 0; m < P; ++m) re[m * PP] = fx_to_double(out[m] + value(o[m * B]) + value(o[5 * FP + m * B]), kexp);
     }
   }
   if constexpr (EPB > 1) {
     for (int t = 0; t < ne; ++t)  // (uniform over the CTA)
-      if (!fx_in_range(gmax[t])) rect_plain<N>(a, e0 + t);
+      if (!fx_slot(keys, t).ok) rect_plain<N>(a, e0 + t);
   }
 }
 
@@ -313,12 +369,12 @@ __device__ __forceinline__ void nodal_plain(const VolumeArgs& a, long long e) {
 #pragma unroll 1
           for (int m = 0; m < P; ++m)
             x = fma(a.D64[row * P + m], plain_flux(a, v, c, a.l2g[e * NP + l + (m - row) * st]), x);
-          // eb.w: the metric terms of this element stayed doubles
+          // eb.w < 0: the metric terms of this element stayed doubles
           const long long at = (3 * d + c) * Nl + e * NP + l;
           double b = a.met64[at];
-          if (!eb.w) {
+          if (eb.w >= 0) {
             const int2 h = reinterpret_cast<const int2*>(a.met64)[at];
-            const int E = d == 0 ? eb.x : d == 1 ? eb.y : eb.z;
+            const int E = (d == 0 ? eb.x : d == 1 ? eb.y : eb.z) - fx_scale_of(eb.w).s[c];
             b = scalbn((double)(((long long)h.y << kFxBits) + h.x), E - 1022 - 2 * kFxBits + fx_weight_exp(a.fxw, i, j, k));
           }
           t = fma(b, x, t);
@@ -334,43 +390,46 @@ __device__ __forceinline__ void nodal_plain(const VolumeArgs& a, long long e) {
 //   1. each thread takes one line and every G-th field on it (fx_line) and
 //      leaves the derivatives in shared memory;
 //   2. one thread per node multiplies the 12 derivatives by the direction's
-//      row of -Jw dxi_d/dx_c (58-bit integers relative to the row's largest
-//      value in the element, fx_metric_kernel) into the five equations.
+//      row of -Jw dxi_d/dx_c (58-bit integers, fx_metric_kernel) into the five
+//      equations, those of U_a u_b aligned to the equation's unit (fx_pair).
 // Every row of D is scaled to its own row sum (an end row's is up to 16 times
 // an inner one's).  The directions' sums are aligned by the exponents of their
 // rows, added as integers and rounded once.
 // On the 6x30x30x8 shell at N = 4: 2.068 ms as FP64 (225 operations a node, its
-// pipe 96% busy), 0.520 ms here; 21x17x13 at N = 3: 0.105 -> 0.039 ms.  The 430
-// integer multiply-adds a thread keep their pipe 40% busy and the 2300
-// instructions a warp 60% of the issue slots, at 8 CTAs an SM (64 registers).
-// With the fluxes formed in the update it took 0.505 ms, and the update 0.335
-// instead of 0.294 ms.  Going round all lines of a direction with a division per line
-// instead of one line per thread: 0.570 against 0.505 ms.
+// pipe 96% busy), 0.580 ms here; 21x17x13 at N = 3: 0.105 -> 0.043 ms.  The 421
+// integer multiply-adds a thread keep their pipe 40% busy and the 2580
+// instructions a warp 60% of the issue slots.  One unit for all of momentum and one
+// scale for the directions took 0.517 and 0.039 ms, with the error stated at
+// FxScale; of the difference on the shell, the exponents and keys are 0.017 ms, the
+// alignment 0.011, the choice between U_a u_b and U_b u_a 0.020.  With the fluxes formed in the
+// update the kernel was 0.035 ms shorter, and the update 0.041 longer.  Going round
+// all lines of a direction with a division per line instead of one line per
+// thread: 0.065 ms more.
 template <int N>
 __device__ __forceinline__ void volume_fx_nodal(const VolumeArgs& a, const int2* T, long long e0, int ne,
                                                 unsigned char* smem_raw) {
   constexpr int P = N + 1, PP = P * P, NP = PP * P, EPB = fx_nodal_epb<N>(), NT = fx_nodal_threads<N>();
   constexpr int EP = fx_pitch<N>(), FP = EPB * EP;
-  uint4* gmax = reinterpret_cast<uint4*>(smem_raw);                // (first: 16-byte aligned)
-  int2* F = reinterpret_cast<int2*>(gmax + fx_slots<EPB, NT>());  // [kLF][FP]
+  FxKeys* keys = reinterpret_cast<FxKeys*>(smem_raw);              // (first: 16-byte aligned)
+  int2* F = reinterpret_cast<int2*>(keys + fx_slots<EPB, NT>());  // [kLF][FP]
   long long* S = reinterpret_cast<long long*>(F + kLF * FP);       // [kLF][FP]: the direction's derivatives
   const int tid = threadIdx.x, nn = ne * NP;
   const long long Nl = a.Nl, n0 = e0 * NP;
   const bool node = tid < nn;
   const int nel = EPB == 1 ? 0 : tid / NP;
-  // the elements' metric exponents (w: the element takes plain FP64)
+  // the elements' metric exponents and scale (w < 0: the element takes plain FP64)
   const int4 eb = a.fxE[e0 + (node ? nel : 0)];
+  const FxScale w = fx_scale_of(eb.w);
   FxExp ge;
-  bool ok = fx_stage<N, EPB, NT, true>(a, n0, nn, gmax, F, ge) && !eb.w;
-  if constexpr (EPB == 1) {  // (uniform over the CTA)
-    if (!ok) {
-      nodal_plain<N>(a, e0);
-      return;
-    }
-  } else {
-    ok = ok && fx_in_range(gmax[nel]);
+  fx_stage<N, EPB, NT, false>(a, e0, ne, keys, F, w, ge);
+  const bool ok = ge.ok && eb.w >= 0;
+  if (EPB == 1 && !ok) {  // (uniform over the CTA)
+    nodal_plain<N>(a, e0);
+    return;
   }
   __syncthreads();
+  // (positive: equation a shifts the derivative of U_a u_b, negative: equation b)
+  const int xy = fx_pair(ge, w, 0, 1), xz = fx_pair(ge, w, 0, 2), yz = fx_pair(ge, w, 1, 2);
   const int at = fx_index<N>(tid);
   const int2* met = reinterpret_cast<const int2*>(a.met64) + n0 + tid;
   // the exponents of the node's three directions: the metric row's less that
@@ -403,22 +462,22 @@ __device__ __forceinline__ void volume_fx_nodal(const VolumeArgs& a, const int2*
     if (node) {
       const int sh = min(xm + 1 - (d == 0 ? x0 : d == 1 ? x1 : x2), 62);
       const long long half = 1ll << (sh - 1);  // the shift below rounds
-      auto use = [&](long long& h, long long& m, int slot, int c) {
-        const long long x = S[slot * FP + at];  // (its low part from 0: the metric's has no mean)
+      auto use = [&](long long& h, long long& m, int slot, int c, int by) {
+        const long long x = fx_shift(S[slot * FP + at], by);  // (its low part from 0: the metric's has no mean)
         fx_mac(h, m, B[c], (int)((unsigned)x & kFxMask), (int)(x >> kFxBits));
       };
-      auto eq = [&](int v, int s0, int s1, int s2) {
+      auto eq = [&](int v, int s0, int b0, int s1, int b1, int s2, int b2) {
         long long h = half, m = kFxHalf;
-        use(h, m, s0, 0);
-        use(h, m, s1, 1);
-        use(h, m, s2, 2);
-        sum[v] += fx_sum(h, m) >> sh;  // (nine products below 2^60, halved: below 2^63)
+        use(h, m, s0, 0, b0);
+        use(h, m, s1, 1, b1);
+        use(h, m, s2, 2, b2);
+        sum[v] += fx_sum(h, m) >> sh;  // (nine products below 1.5 2^59, halved: below 2^63)
       };
-      eq(0, sUx, sUy, sUz);
-      eq(1, sTxx, sTxy, sTxz);
-      eq(2, sTxy, sTyy, sTyz);
-      eq(3, sTxz, sTyz, sTzz);
-      eq(4, sHx, sHy, sHz);
+      eq(0, sUx, 0, sUy, 0, sUz, 0);
+      eq(1, sTxx, 0, sTxy, xy, sTxz, xz);
+      eq(2, sTxy, -xy, sTyy, 0, sTyz, yz);
+      eq(3, sTxz, -xz, sTyz, -yz, sTzz, 0);
+      eq(4, sHx, 0, sHy, 0, sHz, 0);
     }
     if (d < 2) __syncthreads();
   };
@@ -426,23 +485,22 @@ __device__ __forceinline__ void volume_fx_nodal(const VolumeArgs& a, const int2*
   direction(std::integral_constant<int, 1>());
   direction(std::integral_constant<int, 2>());
   if (node && ok) {
-    if constexpr (EPB > 1) ge = fx_exps(gmax[nel]);
     const int kx = xm + 1 + a.fxexp + fx_weight_exp(a.fxw, l % P, (l / P) % P, l / PP);
     double* re = static_cast<double*>(a.re) + n0 + tid;
 #pragma unroll
     for (int v = 0; v < 5; ++v)
-      re[v * Nl] = fx_to_double(sum[v], kx + (v == 0 ? ge.U : v == 4 ? ge.t : ge.m));
+      re[v * Nl] = fx_to_double(sum[v], kx + (v == 0 ? ge.U : v == 4 ? ge.t : ge.m[(v + 2) % 3]));
   }
   if constexpr (EPB > 1) {
     for (int t = 0; t < ne; ++t)  // (uniform over the CTA)
-      if (a.fxE[e0 + t].w || !fx_in_range(gmax[t])) nodal_plain<N>(a, e0 + t);
+      if (a.fxE[e0 + t].w < 0 || !fx_slot(keys, t).ok) nodal_plain<N>(a, e0 + t);
   }
 }
 
-// CTAs an SM holds at r registers a thread.  64 registers for both forms: the
-// rectilinear one at N = 4 took 0.188, 0.177, 0.182 and 0.156 ms with 40, 48, 56
-// and 64 (12 to 8 CTAs an SM); the per-node one 0.531, 0.520, 0.531 and 0.554 ms
-// with 56, 64, 72 and 80 (at N = 3 80 are 4% better).
+// CTAs an SM holds at r registers a thread.  64 registers: the rectilinear form
+// at N = 4 took 0.188, 0.177, 0.182 and 0.156 ms with 40, 48, 56 and 64 (12 to 8
+// CTAs an SM; measured with one momentum unit).  The per-node form takes 72 at N = 4 (0.588 ->
+// 0.578 ms on the shell) and 80 at N = 3 (4% better than 64).
 __host__ __device__ constexpr int fx_blocks(int threads, int r) { return 65536 / (threads * r); }
 
 template <int N>
@@ -456,7 +514,7 @@ __global__ void __launch_bounds__(fx_rect_threads<N>(), fx_blocks(fx_rect_thread
 }
 
 template <int N>
-__global__ void __launch_bounds__(fx_nodal_threads<N>(), fx_blocks(fx_nodal_threads<N>(), N == 3 ? 80 : 64))
+__global__ void __launch_bounds__(fx_nodal_threads<N>(), fx_blocks(fx_nodal_threads<N>(), N == 3 ? 80 : N == 4 ? 72 : 64))
     volume_fx_nodal_kernel(const __grid_constant__ VolumeArgs a, const __grid_constant__ FxTables<N, 1> T) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   constexpr int EPB = fx_nodal_epb<N>();
@@ -498,18 +556,20 @@ __global__ void __launch_bounds__(RECT ? fx_rect_threads<N>() : fx_nodal_threads
 }
 
 // At bind: rows 0..8 of one element's metric array, dxi_d/dx_c, become
-// -Jw dxi_d/dx_c as 58-bit integers (fx_of) relative to the largest of their
-// direction in the element, after division by the power of two
+// -Jw dxi_d/dx_c as 58-bit integers, after division by the power of two
 // fx_weight_exp of the node's quadrature weight (the weights of a corner and
-// of the centre differ by up to 2^13 at N = 8); their biased exponents go to
-// fxE.  Elements whose values the integers cannot hold keep doubles (w = 1).
+// of the centre differ by up to 2^13 at N = 8) and multiplication by 2^s_c, which
+// makes the largest of the three terms of each c equal to within a factor of
+// two (FxScale): fx_of relative to the largest of their direction d in the element.
+// The three biased exponents and the scale go to fxE.  Elements whose values the
+// integers cannot hold keep doubles (w = -1).
 template <int UNUSED = 0>
 __global__ void __launch_bounds__(128)
     fx_metric_kernel(double* met, int4* fxE, long long Nl, int P, unsigned long long fxw) {
-  __shared__ unsigned s_key[3];
+  __shared__ unsigned s_key[9];
   const int NP = P * P * P;
   const long long n0 = (long long)blockIdx.x * NP;
-  if (threadIdx.x < 3) s_key[threadIdx.x] = 0u;
+  if (threadIdx.x < 9) s_key[threadIdx.x] = 0u;
   __syncthreads();
   for (int l = threadIdx.x; l < NP; l += blockDim.x) {
     const double jw = -met[9 * Nl + n0 + l];
@@ -518,20 +578,33 @@ __global__ void __launch_bounds__(128)
       const double b = met[t * Nl + n0 + l] * jw;
       met[t * Nl + n0 + l] = b;
       const double x = scalbn(b, -we);
-      atomicMax(&s_key[t / 3], (unsigned)__double2hiint(x) & 0x7fffffffu);
+      atomicMax(&s_key[t], (unsigned)__double2hiint(x) & 0x7fffffffu);
     }
   }
   __syncthreads();
-  const int E[3] = {(int)(s_key[0] >> 20), (int)(s_key[1] >> 20), (int)(s_key[2] >> 20)};
+  int k[9], col[3], E[3] = {0, 0, 0};
   bool ok = true;
+  for (int t = 0; t < 9; ++t) {
+    k[t] = (int)(s_key[t] >> 20);
+    ok &= k[t] <= kFxMetMax;  // (no infinity, no NaN)
+  }
+  for (int c = 0; c < 3; ++c) col[c] = max(k[c], max(k[3 + c], k[6 + c]));
+  const int top = max(col[0], max(col[1], col[2]));
+  // (columns within a factor of four of each other: one scale, see fx_join)
+  if (top - min(col[0], min(col[1], col[2])) <= 1) col[0] = col[1] = col[2] = top;
+  for (int c = 0; c < 3; ++c) {
+    ok &= top - col[c] <= kFxMaxScale;
+    for (int d = 0; d < 3; ++d) E[d] = max(E[d], k[3 * d + c] + top - col[c]);
+  }
   for (int d = 0; d < 3; ++d) ok &= E[d] >= kFxMetMin && E[d] <= kFxMetMax;
-  if (threadIdx.x == 0) fxE[blockIdx.x] = make_int4(E[0], E[1], E[2], ok ? 0 : 1);
+  const int w = (top - col[0]) | (top - col[1]) << 10 | (top - col[2]) << 20;
+  if (threadIdx.x == 0) fxE[blockIdx.x] = make_int4(E[0], E[1], E[2], ok ? w : -1);
   if (!ok) return;
   for (int l = threadIdx.x; l < NP; l += blockDim.x) {
     const int we = fx_weight_exp(fxw, l % P, (l / P) % P, l / (P * P));
     for (int t = 0; t < 9; ++t) {
       double* m = met + t * Nl + n0 + l;
-      *reinterpret_cast<int2*>(m) = fx_split(fx_of(scalbn(*m, -we), E[t / 3]));
+      *reinterpret_cast<int2*>(m) = fx_split(fx_of(scalbn(*m, -we), E[t / 3] - (top - col[t % 3])));
     }
   }
 }

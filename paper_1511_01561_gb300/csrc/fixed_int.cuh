@@ -62,47 +62,106 @@ __device__ __forceinline__ long long fx_of_pipe(double x, int E) {
   return __double2ll_rn(x * __hiloint2double((2103 - E) << 20, 0));
 }
 
-// Magnitude key of a group of values: the largest of their high words without
-// the sign (monotonic in |x|); at least 1 if any value is nonzero.
-__device__ __forceinline__ unsigned fx_group_key(const double* x, int n) {
-  unsigned k = 0, low = 0;
-#pragma unroll
-  for (int t = 0; t < n; ++t) {
-    k = max(k, (unsigned)__double2hiint(x[t]) & 0x7fffffffu);
-    low |= (unsigned)__double2loint(x[t]);
-  }
-  return max(k, low ? 1u : 0u);
+// Magnitude key of a value: its high word without the sign (monotonic in |x|);
+// at least 1 unless the value is zero.
+__device__ __forceinline__ unsigned fx_key(double x) {
+  return max((unsigned)__double2hiint(x) & 0x7fffffffu, min((unsigned)__double2loint(x), 1u));
 }
 
+// Powers of two (s_x, s_y, s_z >= 0) taken out of the three directions of a
+// flux, one of them zero: 2^-s_c F_c are of a size with the terms K_c dF_c / dx_c of
+// Eq. 4 that they lead to (K_c: the size of the metric terms that multiply
+// F_c).  On an element a hundred times wider than high U_z is a hundredth of U_x
+// and K_z a hundred times K_x: with one unit for both, the integers lost a
+// hundred times as much as FP64 sums, whose error follows max_c K_c |F_c|: on smooth
+// flow over elements of 500 to 1 the tendencies of mass and theta were 20 to 40 times
+// as far off as FP64's.  In these units the integers' error follows the same bound.
+struct FxScale {
+  int s[3];
+};
+
+// The same without a look at the low word: 0 for values below 2^-1042 too.
+__device__ __forceinline__ unsigned fx_high(double x) { return (unsigned)__double2hiint(x) & 0x7fffffffu; }
+
+// The key of the vector 2^-s_c x_c from its high words; 0 where those of all components
+// are below 2^(s_c - 1022).
+__device__ __forceinline__ unsigned fx_high_scaled(const double (&x)[3], const FxScale& w) {
+  int k = 0;
+#pragma unroll
+  for (int c = 0; c < 3; ++c) k = max(k, (int)fx_high(x[c]) - (w.s[c] << 20));
+  return (unsigned)k;
+}
+// The key of the vector; at least 1 unless it is zero.
+__device__ __forceinline__ unsigned fx_key_scaled(const double (&x)[3], const FxScale& w) {
+  return max(fx_high_scaled(x, w), min(fx_key(x[0]) | fx_key(x[1]) | fx_key(x[2]), 1u));
+}
+
+// Magnitude keys of an element: of 2^-s_c U_c, theta, p' and each component of u.
+struct alignas(16) FxKeys {
+  unsigned U, th, pp, unused;
+  unsigned u[3], unused2;
+};
+
 // The biased exponents of an element's equation groups, |field| <
-// 2^(exponent - 1022), from the magnitude keys of U, u, theta and p' (x, y, z,
-// w): mass: U; momentum: U u + p' I; theta: theta U.  A group of zeros has the
+// 2^(exponent - 1022): mass: 2^-s_c U_c; momentum equation v: 2^-s_c (U_c u_v +
+// p' I); theta: 2^-s_c theta U_c; and of theta and p' themselves.  A group of zeros has the
 // exponent of 1, so that its zero sums meet a finite factor in fx_to_double.
-struct FxExp {
-  int U, m, t;
+struct alignas(16) FxExp {
+  int U, m[3];
+  int t, th, pp;
+  int ok;  // the integers hold the element
 };
 constexpr int kFxZero = 1023;
 constexpr int kFxLeast = 100;  // at this exponent and above fx_of shifts every bit of a zero out
-// U u and p' each stay below 2^(m - 1022).  Where their exponents are equal m is
-// one above them, so their sum stays below 1.5 2^(m - 1022): 1.5 2^58 as an
-// integer, whose high part is at most 1.5 2^29, so that fx_line's sums of two
-// of them fit 32 bits.
-__device__ __forceinline__ FxExp fx_exps(uint4 k) {
-  const int U = k.x ? (int)(k.x >> 20) : kFxZero, p = (int)(k.w >> 20);
-  // whether the product of the largest U and u carries into the next power of two
-  const unsigned mU = (k.x & 0xfffffu) + 0x100001u, mu = (k.y & 0xfffffu) + 0x100001u;
-  const int Uu = U + (int)(k.y >> 20) - 1023 + ((unsigned long long)mU * mu > (1ull << 41));
-  const int m = k.x && k.y ? max(Uu, p) + (Uu == p) : k.w ? p : kFxZero;
-  return {U, m, k.x && k.z ? U + (int)(k.z >> 20) - 1022 : kFxZero};
-}
 
-// Whether the fixed-point form holds an element with these keys: every field
-// and every group.
-__device__ __forceinline__ bool fx_in_range(uint4 k) {
-  auto in = [](int E) { return (unsigned)E - kFxMinExp <= kFxMaxExp - kFxMinExp; };
-  auto ok = [&](unsigned key) { return key == 0u || in((int)(key >> 20)); };
-  const FxExp e = fx_exps(k);
-  return ok(k.x) && ok(k.y) && ok(k.z) && ok(k.w) && in(e.m) && in(e.t);
+__device__ __forceinline__ bool fx_in(int E) { return (unsigned)E - kFxMinExp <= kFxMaxExp - kFxMinExp; }
+__device__ __forceinline__ bool fx_ok(unsigned key) { return key == 0u || fx_in((int)(key >> 20)); }
+
+// The exponent of momentum equation v from the keys of U, u_v and p', s = s_v;
+// ok: whether u_v and the group are in range.  U_c u_v and p' each stay below
+// 2^(m - 1022).  Where their exponents are equal m is one above them, so their
+// sum stays below 1.5 2^(m - 1022): 1.5 2^58 as an integer, whose high part is at
+// most 1.5 2^29, so that fx_line's sums of two of them fit 32 bits.
+__device__ __forceinline__ int fx_momentum_exp(unsigned U, unsigned u, unsigned pp, int s, bool& ok) {
+  // whether the product of the largest U and u carries into the next power of two
+  const unsigned mU = (U & 0xfffffu) + 0x100001u, mu = (u & 0xfffffu) + 0x100001u;
+  const int Uu = (int)(U >> 20) + (int)(u >> 20) - 1023 + ((unsigned long long)mU * mu > (1ull << 41));
+  const int p = (int)(pp >> 20) - s;
+  const int m = U && u ? max(Uu, p) + (Uu == p) : pp ? p : kFxZero;
+  ok = fx_ok(u) && fx_in(m);
+  return m;
+}
+// The other exponents of e; ok: whether they and the keys of U, theta and p' are in range.
+__device__ __forceinline__ bool fx_scalar_exps(FxExp& e, unsigned U, unsigned th, unsigned pp) {
+  e.U = U ? (int)(U >> 20) : kFxZero;
+  e.t = U && th ? (int)(U >> 20) + (int)(th >> 20) - 1022 : kFxZero;
+  e.th = max((int)(th >> 20), kFxLeast);
+  e.pp = max((int)(pp >> 20), kFxLeast);
+  return fx_ok(U) && fx_ok(th) && fx_ok(pp) && fx_in(e.t);
+}
+// One unit for U_a u_b in both its equations (fx_pair = 0) where that makes no
+// equation's unit larger than four times its own: the 58 bits of a group then
+// keep 56 of the largest of its equation, FP64 sums 53.
+__device__ __forceinline__ void fx_join(FxExp& e, const FxScale& w) {
+  const int m = max(e.m[0] - w.s[0], max(e.m[1] - w.s[1], e.m[2] - w.s[2]));
+  const int least = min(e.m[0] - w.s[0], min(e.m[1] - w.s[1], e.m[2] - w.s[2]));
+  if (m - least <= 2) {
+#pragma unroll
+    for (int v = 0; v < 3; ++v) e.m[v] = m + w.s[v];
+  }
+}
+__device__ __forceinline__ FxExp fx_exps(const FxKeys& k, const FxScale& w) {
+  FxExp e = FxExp();
+  bool ok = fx_scalar_exps(e, k.U, k.th, k.pp);
+#pragma unroll
+  for (int v = 0; v < 3; ++v) {
+    bool in;
+    e.m[v] = fx_momentum_exp(k.U, k.u[v], k.pp, w.s[v], in);
+    ok &= in;
+  }
+  e.ok = ok;
+  fx_join(e, w);
+  return e;
 }
 
 // (high, middle) accumulators += D * f, D = Dh 2^29 + Dl, f = fh 2^29 + fl;
@@ -122,42 +181,112 @@ __device__ __forceinline__ long long fx_sum(long long h, long long m) {
   return h + (m >> kFxBits);
 }
 
-// a b 2^-58, rounded but for the product of the low parts.
-__device__ __forceinline__ long long fx_mul(int2 a, int2 b) {
-  long long h = 0, m = kFxHalf;
+// a b 2^-58 + c, rounded but for the product of the low parts, split as by fx_split.
+__device__ __forceinline__ int2 fx_mul_split(int2 a, int2 b, long long c = 0) {
+  long long h = c + kFxHalf, m = kFxHalf;
   fx_mac(h, m, a, b.x, b.y);
-  return fx_sum(h, m);
+  const long long s = fx_sum(h, m);
+  return make_int2((int)((unsigned)s & kFxMask) - (int)kFxHalf, (int)(s >> kFxBits));
 }
 
-// Shared-memory slots of the 12 flux fields: the five fields differentiated
-// along x in the order of the equations, so that the x lines of all five are
-// one run of memory (no bank conflicts), then the rest.
-enum : int { sUx = 0, sTxx, sTxy, sTxz, sHx, sUy, sTyy, sTyz, sHy, sUz, sTzz, sHz };
-// The 12 flux fields of a node (U, u, theta, p' in z) as integers of their
-// groups: put(slot, value).  thkey: the magnitude key of theta.
-template <bool PIPE, typename Z, typename Put>
-__device__ __forceinline__ void fx_fluxes(const Z& z, FxExp e, unsigned thkey, Put put) {
-  // u in the unit that makes U u one of the momentum group's, p' in the group's own
-  int2 U[3], u[3];
+// The integers of a node (U, u, theta, p' in z): U_c in the unit of the mass
+// group, u_v in the unit that makes U_c u_v one of momentum equation v, theta and
+// p' in their own.
+struct FxNode {
+  int2 U[3], u[3], th;
+  long long pp;
+};
+template <bool PIPE, typename Z>
+__device__ __forceinline__ FxNode fx_node(const Z& z, const FxExp& e, const FxScale& w) {
+  FxNode n;
 #pragma unroll
   for (int c = 0; c < 3; ++c) {
-    U[c] = fx_split((PIPE ? fx_of_pipe : fx_of)(z.U[c], e.U));
-    u[c] = fx_split(fx_of(z.u[c], max(e.m - e.U + 1022, kFxLeast)));
+    n.U[c] = fx_split((PIPE ? fx_of_pipe : fx_of)(z.U[c], e.U + w.s[c]));
+    n.u[c] = fx_split(fx_of(z.u[c], max(e.m[c] - e.U + 1022, kFxLeast)));
   }
-  const int2 th = fx_split(fx_of(z.th, max((int)(thkey >> 20), kFxLeast)));
-  const long long p = (PIPE ? fx_of_pipe : fx_of)(z.pp, e.m);
-  put(sUx, U[0]);
-  put(sUy, U[1]);
-  put(sUz, U[2]);
-  put(sTxx, fx_split(fx_mul(U[0], u[0]) + p));
-  put(sTyy, fx_split(fx_mul(U[1], u[1]) + p));
-  put(sTzz, fx_split(fx_mul(U[2], u[2]) + p));
-  put(sTxy, fx_split(fx_mul(U[0], u[1])));
-  put(sTxz, fx_split(fx_mul(U[0], u[2])));
-  put(sTyz, fx_split(fx_mul(U[1], u[2])));
-  put(sHx, fx_split(fx_mul(U[0], th)));
-  put(sHy, fx_split(fx_mul(U[1], th)));
-  put(sHz, fx_split(fx_mul(U[2], th)));
+  n.th = fx_split(fx_of(z.th, e.th));
+  n.pp = (PIPE ? fx_of_pipe : fx_of)(z.pp, e.pp);
+  return n;
+}
+// p' in momentum equation v along v, in the equation's unit (cut: the derivative of a
+// constant is exactly zero).
+__device__ __forceinline__ long long fx_pressure(const FxNode& n, const FxExp& e, const FxScale& w, int v) {
+  return n.pp >> min(e.m[v] + w.s[v] - e.pp, 63);
+}
+
+// The 15 flux fields of a node for the rectilinear form: put(5 c + v, value) of
+// the flux of equation v along direction c, scaled by 2^-s_c, in equation v's
+// unit.  With one scale and one unit for all (elements of three like edges) U_a u_b
+// serves as the flux of a along b and of b along a, and p' is shifted once.
+template <typename Z, typename Put>
+__device__ __forceinline__ void fx_fluxes(const Z& z, const FxExp& e, const FxScale& w, Put put) {
+  const FxNode n = fx_node<false>(z, e, w);
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    put(5 * c, n.U[c]);
+    put(5 * c + 4, fx_mul_split(n.U[c], n.th));
+  }
+  if (((e.m[0] ^ e.m[1]) | (e.m[0] ^ e.m[2]) | w.s[0] | w.s[1] | w.s[2]) == 0) {
+    const long long p = fx_pressure(n, e, w, 0);
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      put(5 * c + 1 + c, fx_mul_split(n.U[c], n.u[c], p));
+#pragma unroll
+      for (int v = c + 1; v < 3; ++v) {
+        const int2 T = fx_mul_split(n.U[c], n.u[v]);
+        put(5 * c + 1 + v, T);
+        put(5 * v + 1 + c, T);
+      }
+    }
+  } else {
+#pragma unroll
+    for (int c = 0; c < 3; ++c)
+#pragma unroll
+      for (int v = 0; v < 3; ++v)
+        put(5 * c + 1 + v, fx_mul_split(n.U[c], n.u[v], v == c ? fx_pressure(n, e, w, v) : 0));
+  }
+}
+
+// Slots of the 12 flux fields of the per-node form, in which U_a u_b stands for the
+// flux of momentum a along b and of b along a.
+enum : int { sUx = 0, sTxx, sTxy, sTxz, sHx, sUy, sTyy, sTyz, sHy, sUz, sTzz, sHz };
+
+// The two equations' exponents of U_a u_b (a != b), their difference: equation a takes it along b, in the
+// unit m_a + s_b, equation b along a, in m_b + s_a.  The field is held in the
+// smaller unit; the equation of the other shifts its derivative right (fx_shift).
+__device__ __forceinline__ int fx_pair(const FxExp& e, const FxScale& w, int a, int b) {
+  return (e.m[a] + w.s[b]) - (e.m[b] + w.s[a]);
+}
+// x 2^-sh rounded for sh > 0, else x.
+__device__ __forceinline__ long long fx_shift(long long x, int sh) {
+  if (sh > 0) {
+    sh = min(sh, 62);
+    x = (x + (1ll << (sh - 1))) >> sh;
+  }
+  return x;
+}
+
+// The 12 flux fields of a node for the per-node form: put(slot, value).
+template <typename Z, typename Put>
+__device__ __forceinline__ void fx_fluxes_shared(const Z& z, const FxExp& e, const FxScale& w, Put put) {
+  const FxNode n = fx_node<true>(z, e, w);
+  auto diag = [&](int c) { return fx_mul_split(n.U[c], n.u[c], fx_pressure(n, e, w, c)); };
+  auto off = [&](int a, int b) {
+    const bool in_a = fx_pair(e, w, a, b) <= 0;
+    return fx_mul_split(in_a ? n.U[b] : n.U[a], in_a ? n.u[a] : n.u[b]);
+  };
+  put(sUx, n.U[0]);
+  put(sUy, n.U[1]);
+  put(sUz, n.U[2]);
+  put(sTxx, diag(0));
+  put(sTyy, diag(1));
+  put(sTzz, diag(2));
+  put(sTxy, off(0, 1));
+  put(sTxz, off(0, 2));
+  put(sTyz, off(1, 2));
+  put(sHx, fx_mul_split(n.U[0], n.th));
+  put(sHy, fx_mul_split(n.U[1], n.th));
+  put(sHz, fx_mul_split(n.U[2], n.th));
 }
 
 // Entries of a direction's even/odd table (see fx_line).

@@ -73,6 +73,7 @@ VolumeArgs volume_args(const numa_ctx* c, const double* q, const void* prim, voi
   a.fxD = c->fx ? c->L.fxD : nullptr;
   a.fxD_host = c->fx ? c->fxD.data() : nullptr;
   a.fxexp = c->fxexp;
+  for (int d = 0; d < 3; ++d) a.fxs[d] = c->fxs[d];
   a.fxE = c->L.fxE;
   a.fxw = c->fxw;
   a.fxr = c->fxr;
@@ -640,7 +641,7 @@ int numa_bind(numa_ctx* c, void* ws, size_t bytes, void* stream) {
   std::vector<double> affk, w3, Minv_r;
   std::vector<int2> fxD;
   bool rect = false, fx = false;
-  int fxexp = 0;
+  int fxexp = 0, fxs[3] = {0, 0, 0};
   unsigned long long fxw = 0, fxr = 0;
   if (c->cfg.precision == NUMA_FP64) {
     if (affine_elements(c->cfg)) {
@@ -660,11 +661,14 @@ int numa_bind(numa_ctx* c, void* ws, size_t bytes, void* stream) {
       if (rect) {
         // K_d = -J dxi_d/dx_d = -(area of the element's face normal to d) / 4,
         // the same for all elements of a box (a mesh whose metric terms say
-        // otherwise is not treated as rectilinear).  One scale 2^s for the
-        // three directions: the largest row sum of |K_d D| below 2^60.
+        // otherwise is not treated as rectilinear).  Each direction's table with
+        // its own largest row sum of |K_d D| below 2^60; the powers of two
+        // between them scale the fields (FxScale).
         const double Lx[3] = {c->cfg.Lx, c->cfg.Ly, c->cfg.Lz};
         const double ne[3] = {(double)c->cfg.nex, (double)c->cfg.ney, (double)c->cfg.nez};
-        double num[3][2], den[3], top = 0.0;
+        double num[3][2], den[3];
+        int e2[3] = {0, 0, 0};
+        bool ok = rect;
         for (int d = 0; d < 3; ++d) {
           const int p = (d + 1) % 3, r = (d + 2) % 3;
           num[d][0] = -Lx[p];
@@ -673,21 +677,28 @@ int numa_bind(numa_ctx* c, void* ws, size_t bytes, void* stream) {
           const double K = num[d][0] * num[d][1] / den[d];
           for (long long el = 0; el < m.Ne; ++el)
             if (!(std::fabs(affk[d * (size_t)m.Ne + el] - K) <= 1e-9 * std::fabs(K))) rect = false;
+          double top = 0.0;
           for (int i = 0; i < P; ++i) {
             double row = 0.0;
             for (int j = 0; j < P; ++j) row += std::fabs(K * m.D[i * P + j]);
             top = std::max(top, row);
           }
+          std::frexp(top, &e2[d]);  // top < 2^e2
+          ok = ok && top > 0.0 && std::isfinite(top) && e2[d] >= -190 && e2[d] <= 310;
         }
-        int e2 = 0;
-        std::frexp(top, &e2);  // top < 2^e2
-        const int s2 = 60 - e2;
-        fx = rect && top > 0.0 && std::isfinite(top) && s2 >= -250 && s2 <= 250;
+        const int e2max = std::max(e2[0], std::max(e2[1], e2[2]));
+        for (int d = 0; d < 3; ++d) ok = ok && e2max - e2[d] <= kFxMaxScale;
+        // (within a factor of four of each other: one scale, which saves the kernel three products a node)
+        if (e2max - std::min(e2[0], std::min(e2[1], e2[2])) <= 1) e2[0] = e2[1] = e2[2] = e2max;
+        fx = ok && rect;
         if (fx) {
           fxD.resize(3 * kFxEntries);
           int n = 0;
-          for (int d = 0; d < 3; ++d) n += fx_table_host(P, nullptr, num[d][0], num[d][1], den[d], s2, 0, fxD.data() + n);
-          fxexp = 64 - s2;
+          for (int d = 0; d < 3; ++d) {
+            n += fx_table_host(P, nullptr, num[d][0], num[d][1], den[d], 60 - e2[d], 0, fxD.data() + n);
+            fxs[d] = e2max - e2[d];
+          }
+          fxexp = 4 + e2max;
           up(L.fxD, fxD.data(), (size_t)n * sizeof(int2));
         }
       }
@@ -756,6 +767,7 @@ int numa_bind(numa_ctx* c, void* ws, size_t bytes, void* stream) {
   c->fx = fx;
   c->fxD = fxD;
   c->fxexp = fxexp;
+  for (int d = 0; d < 3; ++d) c->fxs[d] = fxs[d];
   c->fxw = fxw;
   c->fxr = fxr;
   c->slabs = plan_slabs(c->cfg, m, c->nslab_req);

@@ -120,6 +120,8 @@ struct DevLayout {
 
 // Entries of one direction's fixed-point table at the largest order.
 constexpr int kFxEntries = 40;
+// Largest power of two between the directions' scales (FxScale).
+constexpr int kFxMaxScale = 200;
 // (a b / c) D (one direction's derivative matrix times its metric factor) as
 // the even/odd fixed-point table of fx_line (fixed64.cuh): entries
 // 2^s (a b / c) D as (low 29 bits, rest), rounded once; D64 = nullptr: D
@@ -168,7 +170,8 @@ struct VolumeArgs {
                         // K_d outside the fixed-point range, the elements take plain FP64) or of D (per-node form)
   const int2* fxD_host; // the same tables in host memory (kernel parameters of the single-mesh launch)
   int fxexp;            // the exponent that goes with fxD
-  const int4* fxE;      // FP64 per-node form: [Ne] exponents of the metric rows' integers
+  int fxs[3];           // rectilinear form: the powers of two taken out of the directions' fluxes (FxScale)
+  const int4* fxE;      // FP64 per-node form: [Ne] exponents of the metric rows' integers, and the element's scale
   unsigned long long fxw, fxr;  // and the powers of two taken out of the quadrature weights (fx_weight_exp)
                                 // and put into the rows of D, 4 bits per point of a line
   long long Ng, Nl;
@@ -368,7 +371,7 @@ struct numa_ctx {
   bool rect = false;        // FP64, affine and every element rectilinear: the folded element kernel
   bool fx = false;          // FP64: L.fxD and fxD hold the mesh's fixed-point tables, with exponent fxexp
   std::vector<int2> fxD;
-  int fxexp = 0;
+  int fxexp = 0, fxs[3] = {0, 0, 0};  // VolumeArgs::fxexp, fxs
   unsigned long long fxw = 0, fxr = 0;  // FP64 per-node form: VolumeArgs::fxw, fxr
   int nslab_req = 0;        // slabs asked for by numa_set_slabs (0: automatic)
   numa::SlabPlan slabs;     // the plan in use (made at bind and by numa_set_slabs)

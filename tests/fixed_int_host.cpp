@@ -2,6 +2,8 @@
 // the integer primitives (soft64.cuh) for tests/test_fixed_int_host.py.
 #include "device_host.h"
 
+#include <cstdlib>
+
 // the FP32 reciprocal with an error of its own, in units of 2^-23
 static float rcp_error = 0.0f;
 static float rcp_approx(float d) { return (float)(1.0 / (double)d + (double)rcp_error * 0x1p-23); }
@@ -18,8 +20,6 @@ struct Node {
   double U[3], u[3], th, pp;
 };
 
-unsigned key1(double x) { return fx_group_key(&x, 1); }
-
 template <int N>
 void lines(const int2* F, const int2* D, long long* out) {
   long long o[N + 1];
@@ -29,25 +29,50 @@ void lines(const int2* F, const int2* D, long long* out) {
 
 }  // namespace
 
-// The 12 flux fields of one node (U, u, theta, p') as the kernels stage them for
-// an element whose nodes all hold it; false if the element is out of range.
-// f: (low, high) per slot; e: the exponents of U, the momentum fluxes and theta U.
-extern "C" int fluxes_of(const double* z, int pipe, int* f, int* e) {
+// The flux fields of one node (U, u, theta, p') as the kernels stage them for an
+// element whose nodes all hold it, with the directions scaled by 2^-s: the 15 of
+// the rectilinear form, or (shared) the 12 of the per-node form; false if the
+// element is out of range.  f: (low, high) per field; e: the exponents of U, the
+// three momentum equations and theta U.
+extern "C" int fluxes_of(const double* z, const int* s, int shared, int* f, int* e) {
   Node n;
   std::memcpy(&n, z, sizeof n);
-  const uint4 k = make_uint4(fx_group_key(n.U, 3), fx_group_key(n.u, 3), key1(n.th), key1(n.pp));
-  if (!fx_in_range(k)) return 0;
-  const FxExp x = fx_exps(k);
+  FxScale w;
+  FxKeys k = FxKeys();
+  for (int c = 0; c < 3; ++c) {
+    w.s[c] = s[c];
+    k.u[c] = fx_key(n.u[c]);
+  }
+  k.U = fx_key_scaled(n.U, w);
+  k.th = fx_key(n.th);
+  k.pp = fx_key(n.pp);
+  const FxExp x = fx_exps(k, w);
+  if (!x.ok) return 0;
   auto put = [&](int slot, int2 v) {
     f[2 * slot] = v.x;
     f[2 * slot + 1] = v.y;
   };
-  if (pipe) fx_fluxes<true>(n, x, k.z, put);
-  else fx_fluxes<false>(n, x, k.z, put);
+  if (shared) fx_fluxes_shared(n, x, w, put);
+  else fx_fluxes(n, x, w, put);
   e[0] = x.U;
-  e[1] = x.m;
-  e[2] = x.t;
+  for (int v = 0; v < 3; ++v) e[1 + v] = x.m[v];
+  e[4] = x.t;
   return 1;
+}
+
+// fx_pair of the equations' exponents m and the scale s.
+extern "C" int pair_of(const int* m, const int* s, int a, int b) {
+  FxExp e = {};
+  FxScale w;
+  for (int c = 0; c < 3; ++c) {
+    e.m[c] = m[c];
+    w.s[c] = s[c];
+  }
+  return fx_pair(e, w, a, b);
+}
+// A derivative as the first (second = 0) or second of the pair's equations takes it.
+extern "C" long long value_of(long long x, int pair, int second) {
+  return fx_shift(x, second ? -pair : pair);
 }
 
 // fx_line of order N over the line's fields (low, high), with the table of

@@ -13,6 +13,7 @@ import pytest
 from paper_1511_01561_gb300 import inputs as I
 
 from .helpers import lobatto_derivative, scaled_random_state
+from .thin_box import thin_flow, thin_rhs
 
 pytestmark = pytest.mark.gpu
 
@@ -267,3 +268,19 @@ def test_imex_calls_in_any_division(numa, nez):
     assert np.isfinite(a).all() and np.abs(a).max() > 0.0
     assert np.array_equal(a, go((0.2, 3, False), (0.1, 2, False), (0.2, 1, False)))
     assert np.array_equal(a, go((0.2, 0, True), (0.2, 1, True), (0.2, 2, True), (0.1, 1, False), (0.1, 1, True), (0.2, 1, True)))
+
+
+# elements much wider than high (or higher than wide), each variable against its
+# own rounding scale u S (thin_box.thin_rhs): FP64 arithmetic in the oracle's
+# order stays within 1.2 u S on these states; the bar is twice u S
+@pytest.mark.parametrize("over", [dict(), dict(metric_form="nodal")], ids=["rect", "nodal"])
+@pytest.mark.parametrize("N", [2, 4, 5, 8])
+@pytest.mark.parametrize("aspect", [0.01, 1.0, 16.0, 100.0, 500.0, 2500.0])
+def test_thin_elements(numa, orc, aspect, N, over):
+    h = 1e4 if aspect > 1.0 else 100.0 if aspect < 1.0 else 1e3
+    cfg = I.box((3, 2, 2), N, L=(3.0 * h, 2.0 * h, 2.0 * h / aspect), **over)
+    m = orc.Mesh(cfg)
+    q = thin_flow(m, cfg)
+    R, S = thin_rhs(m, cfg, q)
+    err = np.abs(_rhs(numa, cfg, q) - R).max(axis=1).astype(float) / (2.0 ** -53 * S)
+    assert err.max() <= 2.0, err
