@@ -63,11 +63,14 @@ enum numa_ref_kind { NUMA_REF_ISENTROPIC = 0, NUMA_REF_ISOTHERMAL = 1 };
 enum numa_precision {
   NUMA_FP64 = 0,      /* FP64 throughout: state, DSS, inverse mass and RK as FP64
                           operations; the primitives and EOS as products of
-                          58-bit mantissas; the element kernel's (and short
-                          1D-IMEX columns') products and sums as 58- to 64-bit
-                          integers relative to the largest value of their group
-                          in the element (column), rounded to FP64 once at the
-                          end; values beyond those ranges as FP64 operations */
+                          58-bit mantissas; the element kernel's products and
+                          sums as 58- to 64-bit integers relative to the largest
+                          value of their equation in the element (with the
+                          directions scaled by their metric terms, so that
+                          elements of any aspect keep FP64's accuracy), rounded
+                          to FP64 once at the end, 1D-IMEX columns of up to 64
+                          levels likewise relative to the column's largest
+                          value; values beyond those ranges as FP64 operations */
   NUMA_FP32_MIXED = 1, /* fluxes, metric terms and D contractions in FP32;
                           state, EOS reference subtraction, DSS, inverse mass
                           and the RK combination in FP64 */
@@ -352,7 +355,9 @@ enum numa_req_status {
 /* Create a scheduler over a caller-owned device arena (256-byte aligned) used
  * for all member workspaces and the scheduler's own tables, the compute
  * stream (cudaStream_t as void*), and build_threads host threads that build
- * meshes in the background.  The library still allocates no device memory. */
+ * meshes in the background (each may start up to eight short-lived ones for a
+ * large mesh, as numa_create does).  The library still allocates no device
+ * memory. */
 int numa_sched_create(void* dev_arena, size_t arena_bytes, void* stream, int build_threads, numa_sched** out);
 
 /* Queue one forecast: mesh/physics/precision config, initial condition (as

@@ -12,7 +12,8 @@ namespace numa {
 namespace {
 
 // One CTA per element, one thread per element node; three passes along xi,
-// eta and zeta through shared memory.  T = double: FP64; T = float: the FP32 form (the correction in FP32).
+// eta and zeta through shared memory.  T = double: FP64; T = float: the FP32
+// form (the correction in FP32).
 template <int N, typename T>
 __global__ void __launch_bounds__(((N + 1) * (N + 1) * (N + 1) + 31) / 32 * 32) filter_kernel(FilterArgs a) {
   constexpr int P = N + 1, NP = P * P * P;

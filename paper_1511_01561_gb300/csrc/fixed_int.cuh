@@ -48,13 +48,14 @@ __device__ __forceinline__ int2 fx_split(long long s) {
   return make_int2((int)((unsigned)s & kFxMask) - (int)kFxHalf, (int)(s >> kFxBits));
 }
 
-// S 2^(kexp - 1086) rounded to nearest (kexp - 63 within an FP64's biased
-// exponents: the host's bounds on the tables' and fx_in_range's on the groups'), and fx_of by the FP64 pipe: a conversion
+// S 2^(kexp - 1086) rounded to nearest, and fx_of by the FP64 pipe: a conversion
 // and an exact product each, 32 cycles of a pipe that is otherwise idle in
-// place of 24 and 15 integer instructions.  Measured on 32^3 elements, N = 4
-// (rectilinear) and the 6x30x30x8 shell (per-node): all five results so, 0.183
-// -> 0.174 and 0.540 -> 0.526 ms; U and p' of the eight inputs too, 0.183 and
-// 0.519 ms (so in the per-node form only); all eight, 0.213 and 0.520 ms.
+// place of 24 and 15 integer instructions.  The host's bounds on the tables and
+// fx_exps' on the groups keep kexp - 63 within an FP64's biased exponents.
+// Measured with one momentum unit on 32^3 elements, N = 4 (rectilinear) and the
+// 6x30x30x8 shell (per-node): all five results so, 0.183 -> 0.174 and 0.540 ->
+// 0.526 ms; U and p' of the eight inputs too, 0.183 and 0.519 ms (so in the
+// per-node form only); all eight, 0.213 and 0.520 ms.
 __device__ __forceinline__ double fx_to_double(long long S, int kexp) {
   return __ll2double_rn(S) * __hiloint2double((kexp - 63) << 20, 0);
 }
@@ -80,7 +81,8 @@ struct FxScale {
   int s[3];
 };
 
-// The same without a look at the low word: 0 for values below 2^-1042 too.
+// The same without a look at the low word: 0 for values below 2^-1042 too.  (With
+// the low words of a node's eight values the kernels take 1% longer at N = 4.)
 __device__ __forceinline__ unsigned fx_high(double x) { return (unsigned)__double2hiint(x) & 0x7fffffffu; }
 
 // The key of the vector 2^-s_c x_c from its high words; 0 where those of all components

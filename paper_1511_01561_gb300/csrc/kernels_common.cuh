@@ -1,10 +1,10 @@
 // Device code shared by the kernel translation units of the GB300 NUMA hot
-// path (sm_103a): FP64-pipe-free conversions, float-pair arithmetic, the
-// equation of state, the element kernels of Eq. 4 / Eq. 5 (per-node, affine
-// and line forms), the per-node DSS / inverse-mass / RK-stage update, the
-// ragged multi-member kernels, and their launch templates.  Everything is in
-// an anonymous namespace: each translation unit instantiates the templates
-// it launches.
+// path (sm_103a): FP64-pipe-free conversions, the equation of state, the FP32
+// element kernels of Eq. 4 / Eq. 5 (per-node and affine forms, organised by
+// lines), the per-node DSS / inverse-mass / RK-stage update, the ragged
+// multi-member kernels, and their launch templates.  Everything is in an
+// anonymous namespace: each translation unit instantiates the templates it
+// launches.
 //
 // GB300 executes FP64 at 1/64 of the FP32 rate, so everything that does not
 // need FP64 stays off the FP64 pipe: float<->double conversions and the
@@ -256,10 +256,10 @@ __device__ __forceinline__ void stage_fluxes_affine(const VolumeArgs& a, long lo
   }
 }
 
-// The 12 flux fields of the FP64 kernels: F_rho = U, F_U =
-// U (x) u + p' I with the pressure in the diagonal components (the
-// symmetric part stored once), F_Theta = theta U.
-enum : int { lUx = 0, lUy, lUz, lTxx, lTyy, lTzz, lTxy, lTxz, lTyz, lHx, lHy, lHz, kLF };
+// Flux fields of the FP64 per-node kernel: F_rho = U, F_U = U (x) u + p' I with
+// the pressure in the diagonal components (the symmetric part stored once),
+// F_Theta = theta U.
+constexpr int kLF = 12;
 
 // The state at the global node behind element node n, FP64: U from the state,
 // u, theta and p' as the update left them (write_prim).
@@ -312,8 +312,9 @@ __host__ __device__ constexpr int line_group() {
 //     metric terms dxi_d/dx_c vanish for c != d and J is constant over the
 //     element, so -Jw div F at node (i,j,k) is w_i w_j w_k sum_d K_d (D F_d)
 //     along xi_d, with K_d = -J dxi_d/dx_d.  Folding K_d into the direction's
-//     copy of D leaves the 12 unweighted flux fields of (1) and 15
-//     contractions, with no metric or Jw load per node.  The weight
+//     copy of D leaves 15 contractions of unweighted fluxes, with no metric or
+//     Jw load per node (15 fields: in fixed point the flux of momentum a along
+//     b and of b along a have units of their own).  The weight
 //     w_i w_j w_k is the same at every element node of a global node (the
 //     Lobatto weights are symmetric and the box's elements meet face to
 //     face), so it moves out of the element kernel into the inverse mass of
@@ -780,13 +781,6 @@ __device__ __forceinline__ void update_node_sums(const UpdateArgs& a, long long 
   }
 }
 
-template <int MODE, bool SHELL, typename RT>
-__device__ __forceinline__ void update_node(const UpdateArgs& a, long long I) {
-  double s[5];
-  dss_node<RT>(a, I, s);
-  update_node_sums<MODE, SHELL, std::is_same<RT, float>::value>(a, I, s[0], s[1], s[2], s[3], s[4]);
-}
-
 // Fetches into L2 the 128-byte lines that the second half of a block's update
 // reads (q^k, q^n, the reference state and the inverse mass: two lines per
 // warp and array, one per lane), while the DSS waits for its gathers.  With 12
@@ -809,7 +803,7 @@ __device__ __forceinline__ void prefetch_update(const UpdateArgs& a, long long b
 // block's precomputed order (nodes sorted by their number of element nodes,
 // so that the lanes of a warp loop equally often) and leaves the sums in
 // shared memory; the rest runs in natural order (coalesced).  Each node's
-// sum is the same as update_node's, bit for bit.  BOX: a CG box, whose DSS
+// sum is in ascending element-node order, the same bits in any block order.  BOX: a CG box, whose DSS
 // finds the element nodes from the structured numbering (dss_box).
 template <int MODE, bool SHELL, typename RT, bool BOX = false>
 __global__ void __launch_bounds__(kDssBlock, sizeof(RT) == 8 || BOX ? 12 : 16) update_kernel(UpdateArgs a) {

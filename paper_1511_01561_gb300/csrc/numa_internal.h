@@ -277,7 +277,11 @@ bool imex_operator(const numa_config& c, const HostMesh& m, ImexTables& t, std::
 bool imex_factor(const ImexTables& t, double tau, ImexFactor& f, std::string& err);
 size_t imex_table_doubles(int nz, int N);
 // Columns of at most this many levels are solved with the inverse of the Schur
-// matrix (imex.cu).
+// matrix (imex.cu).  Against the LU sweeps a step of 32x32 columns' elements at N = 4
+// took 71 / 87 us at 17 levels, 138 / 167 at 33, 199 / 250 at 49 and 292 / 311 at 61; 8x8
+// at 49 levels 43 / 119.  Taller columns measured faster too (1.1 to 2 times at
+// 65 to 97 levels; at 121 to 125 levels from 0.8 to 1.7 times) but keep the sweeps: the
+// host's part of the inverse grows with the cube of the levels (0.06 ms at 64).
 constexpr int kImexDense = 64;
 // The inverse of a factored matrix as integers (refined beyond FP64, its largest
 // row sum below 2^60), and the exponents of y = H^-1 r, Dz y and Dz(theta0 y).
