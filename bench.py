@@ -149,7 +149,8 @@ def volume_int_ops(N: int, form: str) -> float:
     kernel of `form` (csrc/fixed64.cuh): three per product of 58-bit numbers.
     The even/odd split of D leaves M products per line of N + 1 nodes: 15 lines'
     worth a node in the rectilinear form, 36 and 45 chain-rule products in the
-    per-node form, and 9 flux products in both."""
+    per-node form, and 9 flux products in both (12 in the rectilinear form where
+    the momentum equations' units differ, which depends on the state)."""
     P, H, O = N + 1, (N + 1) // 2, (N + 1) % 2
     M = H * (H + O) + H * H + O * H
     return 3.0 * (15.0 * M / P + 9) if form == "rect" else 3.0 * (36.0 * M / P + 45 + 9)

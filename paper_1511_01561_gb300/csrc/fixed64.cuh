@@ -168,7 +168,9 @@ __device__ __forceinline__ void fx_stage(const VolumeArgs& a, long long e0, int 
   constexpr int FP = EPB * fx_pitch<N>(), SLOTS = fx_slots<EPB, NT>();
   static_assert(RECT || IT == 1, "one scale per thread");
   const int tid = threadIdx.x, nn = ne * NP;
+  int packed = 0;  // of the element whose exponents the thread forms below
   if constexpr (EPB > 1) {
+    if (!RECT && tid < ne) packed = a.fxE[e0 + tid].w;
     if (tid < EPB) keys[tid] = FxKeys();
     __syncthreads();
   }
@@ -248,9 +250,8 @@ __device__ __forceinline__ void fx_stage(const VolumeArgs& a, long long e0, int 
     }
   } else {
     if (tid < ne) {
-      FxScale we = w;
-      if constexpr (!RECT) we = fx_scale_of(a.fxE[e0 + tid].w);
-      const FxExp e = fx_exps(keys[tid], we);
+      FxExp e = fx_exps(keys[tid], RECT ? w : fx_scale_of(packed));
+      if (packed < 0) e.ok = 0;
       *reinterpret_cast<FxExp*>(keys + tid) = e;
     }
     __syncthreads();
@@ -284,7 +285,7 @@ __device__ __forceinline__ void fx_stage(const VolumeArgs& a, long long e0, int 
 // a node at 16 cycles a warp), 0.164 ms here on the rising bubble (0.172 where the
 // momentum equations' units differ); 19x23x17 at N = 6: 0.460 -> 0.132 ms, 12^3 at
 // N = 8 0.090 ms.  135 to 144 integer multiply-adds a thread; the instructions beside
-// them (1060 a warp and element) and shared memory are what is left.  One unit for
+// them (1030 a warp) and shared memory are what is left.  One unit for
 // all of momentum and one scale took 0.154 ms, with an error that grew with an
 // element's aspect.  D in the kernel parameters instead of global memory: 0.256 ->
 // 0.226 ms; the z lines finishing the nodes (10 shared accesses a node fewer):
@@ -342,8 +343,10 @@ __device__ __forceinline__ void volume_fx_rect(const VolumeArgs& a, const int2* 
     }
   }
   if constexpr (EPB > 1) {
-    for (int t = 0; t < ne; ++t)  // (uniform over the CTA)
-      if (!fx_slot(keys, t).ok) rect_plain<N>(a, e0 + t);
+    if (__syncthreads_or(act && !ge.ok)) {
+      for (int t = 0; t < ne; ++t)
+        if (!fx_slot(keys, t).ok) rect_plain<N>(a, e0 + t);
+    }
   }
 }
 
@@ -397,7 +400,7 @@ __device__ __forceinline__ void nodal_plain(const VolumeArgs& a, long long e) {
 // rows, added as integers and rounded once.
 // On the 6x30x30x8 shell at N = 4: 2.068 ms as FP64 (225 operations a node, its
 // pipe 96% busy), 0.580 ms here; 21x17x13 at N = 3: 0.105 -> 0.043 ms.  The 421
-// integer multiply-adds a thread keep their pipe 40% busy and the 2580
+// integer multiply-adds a thread keep their pipe 40% busy and the 2515
 // instructions a warp 60% of the issue slots.  One unit for all of momentum and one
 // scale for the directions took 0.517 and 0.039 ms, with the error stated at
 // FxScale; of the difference on the shell, the exponents and keys are 0.017 ms, the
@@ -422,7 +425,7 @@ __device__ __forceinline__ void volume_fx_nodal(const VolumeArgs& a, const int2*
   const FxScale w = fx_scale_of(eb.w);
   FxExp ge;
   fx_stage<N, EPB, NT, false>(a, e0, ne, keys, F, w, ge);
-  const bool ok = ge.ok && eb.w >= 0;
+  const bool ok = ge.ok && (EPB > 1 || eb.w >= 0);
   if (EPB == 1 && !ok) {  // (uniform over the CTA)
     nodal_plain<N>(a, e0);
     return;
@@ -492,8 +495,10 @@ __device__ __forceinline__ void volume_fx_nodal(const VolumeArgs& a, const int2*
       re[v * Nl] = fx_to_double(sum[v], kx + (v == 0 ? ge.U : v == 4 ? ge.t : ge.m[(v + 2) % 3]));
   }
   if constexpr (EPB > 1) {
-    for (int t = 0; t < ne; ++t)  // (uniform over the CTA)
-      if (a.fxE[e0 + t].w < 0 || !fx_slot(keys, t).ok) nodal_plain<N>(a, e0 + t);
+    if (__syncthreads_or(node && !ok)) {
+      for (int t = 0; t < ne; ++t)
+        if (!fx_slot(keys, t).ok) nodal_plain<N>(a, e0 + t);
+    }
   }
 }
 
