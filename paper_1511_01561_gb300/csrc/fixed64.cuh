@@ -153,6 +153,33 @@ __device__ __forceinline__ const FxExp& fx_slot(const FxKeys* keys, int t) {
   return reinterpret_cast<const FxExp*>(keys)[t];
 }
 
+// The largest of a warp's keys, in every lane; keys raised to at least k's.
+__device__ __forceinline__ FxKeys fx_warp_max(FxKeys k) {
+  k.U = __reduce_max_sync(0xffffffffu, k.U);
+  k.th = __reduce_max_sync(0xffffffffu, k.th);
+  k.pp = __reduce_max_sync(0xffffffffu, k.pp);
+#pragma unroll
+  for (int c = 0; c < 3; ++c) k.u[c] = __reduce_max_sync(0xffffffffu, k.u[c]);
+  return k;
+}
+__device__ __forceinline__ void fx_raise(FxKeys* keys, const FxKeys& k) {
+  atomicMax(&keys->U, k.U);
+  atomicMax(&keys->th, k.th);
+  atomicMax(&keys->pp, k.pp);
+#pragma unroll
+  for (int c = 0; c < 3; ++c) atomicMax(&keys->u[c], k.u[c]);
+}
+// The most elements (of NP nodes each, NN in all) that the nodes of one warp belong to.
+template <int NP, int NN>
+__host__ __device__ constexpr int fx_warp_elements() {
+  int most = 0;
+  for (int l = 0; l < NN; l += 32) {
+    const int last = l + 31 < NN ? l + 31 : NN - 1, n = last / NP - l / NP + 1;
+    if (n > most) most = n;
+  }
+  return most;
+}
+
 // Gathers U, u, theta and p' at the nodes of the ne elements from e0, one thread per
 // element node, and leaves their flux fields in F as fixed-point integers (15
 // for the rectilinear form, 12 for the per-node form).  The largest magnitudes
@@ -166,7 +193,7 @@ __device__ __forceinline__ void fx_stage(const VolumeArgs& a, long long e0, int 
                                          const FxScale& w, FxExp& ge) {
   constexpr int NP = (N + 1) * (N + 1) * (N + 1), NN = EPB * NP, IT = (NN + NT - 1) / NT;
   constexpr int FP = EPB * fx_pitch<N>(), SLOTS = fx_slots<EPB, NT>();
-  static_assert(RECT || IT == 1, "one scale per thread");
+  static_assert((RECT && EPB == 1) || IT == 1, "one node per thread");
   const int tid = threadIdx.x, nn = ne * NP;
   int packed = 0;  // of the element whose exponents the thread forms below
   if constexpr (EPB > 1) {
@@ -193,22 +220,24 @@ __device__ __forceinline__ void fx_stage(const VolumeArgs& a, long long e0, int 
         for (int c = 0; c < 3; ++c) g.u[c] = fx_key(z[it].u[c]);
         g.th = fx_key(z[it].th);
         g.pp = fx_key(z[it].pp);
-        FxKeys* e = keys + l / NP;
-        atomicMax(&e->U, g.U);
-        atomicMax(&e->th, g.th);
-        atomicMax(&e->pp, g.pp);
-#pragma unroll
-        for (int c = 0; c < 3; ++c) atomicMax(&e->u[c], g.u[c]);
       }
     }
   }
   if constexpr (EPB == 1) {
-    g.U = __reduce_max_sync(0xffffffffu, g.U);
-    g.th = __reduce_max_sync(0xffffffffu, g.th);
-    g.pp = __reduce_max_sync(0xffffffffu, g.pp);
-#pragma unroll
-    for (int c = 0; c < 3; ++c) g.u[c] = __reduce_max_sync(0xffffffffu, g.u[c]);
+    g = fx_warp_max(g);
     if ((tid & 31) == 0) keys[tid >> 5] = g;
+  } else if constexpr (fx_warp_elements<NP, NN>() <= 2) {
+    // the warp's elements one after the other (an atomic per lane, 27 to 32 of them in
+    // turn on one address: 0.211 ms instead of 0.179 on 50^3 elements at N = 2, 0.228
+    // instead of 0.186 on 40^3 at N = 3)
+#pragma unroll
+    for (int j = 0; j < fx_warp_elements<NP, NN>(); ++j) {
+      const int t = (tid & ~31) / NP + j;
+      const FxKeys k = fx_warp_max(tid < nn && tid / NP == t ? g : FxKeys());
+      if ((tid & 31) == 0 && t < ne) fx_raise(keys + t, k);
+    }
+  } else {
+    if (tid < nn) fx_raise(keys + tid / NP, g);
   }
   grid_wait();  // (threads without a node; before any write of the kernel)
   __syncthreads();
@@ -399,7 +428,7 @@ __device__ __forceinline__ void nodal_plain(const VolumeArgs& a, long long e) {
 // an inner one's).  The directions' sums are aligned by the exponents of their
 // rows, added as integers and rounded once.
 // On the 6x30x30x8 shell at N = 4: 2.068 ms as FP64 (225 operations a node, its
-// pipe 96% busy), 0.580 ms here; 21x17x13 at N = 3: 0.105 -> 0.043 ms.  The 421
+// pipe 96% busy), 0.580 ms here; 21x17x13 at N = 3: 0.105 -> 0.039 ms.  The 421
 // integer multiply-adds a thread keep their pipe 40% busy and the 2515
 // instructions a warp 60% of the issue slots.  One unit for all of momentum and one
 // scale for the directions took 0.517 and 0.039 ms, with the error stated at
