@@ -93,9 +93,9 @@ INT_PEAK_SOURCE = "nominal rate of 32x32+64-bit integer multiply-adds, 32 per SM
 # this workload (profiles/*_bubble_32x32x32_N4.md), valid only for the kernel
 # sources they were taken on (first 16 hex digits of the sha256 of the kernel
 # sources, see kernel_source_hash).
-NCU_TRAFFIC = {"kernels_sha256_16": "6a6d2b8db43e1fb7", "workload": "bubble_32x32x32_N4",
-               "volume_fp64_affine": 153.862400e6 + 126.470144e6,
-               "volume_fp32_affine": 139.232512e6 + 49.094912e6}
+NCU_TRAFFIC = {"kernels_sha256_16": "e61064c9682569e2", "workload": "bubble_32x32x32_N4",
+               "volume_fp64_affine": 153.844224e6 + 126.131456e6,
+               "volume_fp32_affine": 139.232768e6 + 48.967936e6}
 
 # the sources the element kernels with committed traffic figures are built from
 KERNEL_SOURCES = ["kernels_common.cuh", "fixed64.cuh", "fixed_int.cuh", "volume_fp64.cu", "volume_fp32.cu"]
